@@ -260,6 +260,10 @@ static int set_shapes(hom_ctx *ctx, Geometry &g, int nc) {
         t1 = 16;
         while (t1 > 1 && 2ull * g.n1 * nc * t1 * cs > 96 * 1024) t1 >>= 1;
     }
+    // columns of the TMA-staged n2 pass: 128- or 256-byte rows, 64 from 320 up
+    // (the ring's shared memory)
+    if (sizeof(R) == 4 && ctx->staging == 0 && line_tpl(g.n2) && !g.fast[1])
+        t2 = g.n2 >= 320 ? 8 : (g.n2 >= 100 ? 16 : 32);
     if (nc == 6) {
         if (ctx->shape[0] > 0) rows = ctx->shape[0];
         if (ctx->shape[1] > 0) t2 = ctx->shape[1];
@@ -303,18 +307,23 @@ static int set_shapes(hom_ctx *ctx, Geometry &g, int nc) {
     if ((t2 & (t2 - 1)) != 0 || g.threads2 % t2 != 0) return fail(ctx, HOM_EINVAL, "tile2 must be a power of two");
     if (nc == 6 && g.threads1 > 384)
         return fail(ctx, HOM_EINVAL, "launch shape needs more than 384 threads per CTA in the fused n1 pass");
-    g.kvec = (long long)((g.n2 * g.h + t1 - 1) / t1) * g.n1 * nc * t1;
     g.x3r = (sizeof(R) == 4 && nc == 6 && x3r_length(g.n3) && ctx->shape[0] == 0 &&
              x3r_smem(g.n3) + 1024 <= (size_t)dev_smem && (g.n1 * g.n2) % x3r_rows_per_warp(g.n3) == 0) ? 1 : 0;
     g.grid3r = g.x3r ? Launch<R>::x3r_grid(g) : 0;
     if (g.grid3r <= 0) g.x3r = 0;
-    // persistent TMA-staged n2 / n1 passes: FP32, register-FFT lengths <= 256
-    g.tma = 0;
+    // persistent TMA-staged passes (FP32): the unfused n1 pass at the register
+    // engine's n1 in [64, 512], the n2 pass and the fused MINRES n1 pass at
+    // every length of the line engine
+    g.tma = g.x2t = g.grp1l = g.grid1l_tma = 0;
+    g.tile1l = t1;
     g.err = ctx->d_err;
     g.tma_cache = nullptr;
-    if (sizeof(R) == 4 && ctx->staging == 0 && tma_available() && g.fast[0] >= 64 && g.fast[0] <= 512 &&
-        g.fast[1] >= 64 && g.fast[1] <= 512 && g.tile2 % 2 == 0) {
-        g.tma = 1;
+    if (sizeof(R) == 4 && ctx->staging == 0 && tma_available()) {
+        g.box1 = tma_box_rows(g.n1, nc * t1 * (int)cs);
+        g.tma = g.fast[0] >= 64 && g.fast[1] >= 64 && t2 % 2 == 0 && g.box1 > 0;
+        g.smem1_tma = 2ull * nc * t1 * g.n1 * cs;
+        g.smem1d_tma = 2 * g.smem1_tma;
+        if (g.smem1d_tma + 1024 > (size_t)dev_smem) g.tma = 0;
         // n2 ring stages: 3 at n2 >= 256 (0.143 against 0.148 ms per pass at
         // 256^3; 0.280 against 0.36 ms on 256 x 512 x 256), 2 below (at 128^3
         // three were slower: 0.0185 against 0.0165 ms); HOM_X2_STAGES (2..4)
@@ -324,7 +333,11 @@ static int set_shapes(hom_ctx *ctx, Geometry &g, int nc) {
             const int v = e ? atoi(e) : (g.n2 >= 256 ? 3 : 2);
             g.x2_stages = v < 2 ? 2 : (v > kX2MaxStages ? kX2MaxStages : v);
         }
-        g.smem2_tma = (size_t)g.x2_stages * g.n2 * g.tile2 * cs;
+        g.smem2_tma = (size_t)g.x2_stages * g.n2 * t2 * cs;
+        g.threads2t = round32(t2 * line_tpl(g.n2));
+        g.box2 = tma_box_rows(g.n2, t2 * (int)cs);
+        g.x2t = line_tpl(g.n2) > 0 && g.box2 > 0 && g.threads2t <= 512 &&
+                (size_t)g.n2 * t2 * cs % 128 == 0;   // every ring stage on a 128-byte boundary
         // fused n1 pass: bulk L2 prefetch of each tile's u_k and u_{k-1}
         // blocks at the tile's start (0.625 against 0.647 ms at 256^3; the
         // two warp groups' reads of u_{k-1} then both hit L2); HOM_X1_L2PF=0
@@ -333,12 +346,23 @@ static int set_shapes(hom_ctx *ctx, Geometry &g, int nc) {
             const char *e = getenv("HOM_X1_L2PF");
             g.x1_l2pf = e ? atoi(e) : 1;
         }
-        g.smem1_tma = 2ull * nc * g.tile1 * g.n1 * cs;
-        g.smem1d_tma = 2 * g.smem1_tma;
-        if (g.smem1d_tma + 1024 > (size_t)dev_smem || g.smem2_tma + 1024 > (size_t)dev_smem) g.tma = 0;
-        if (g.tma && Launch<R>::tma_grids(g)) g.tma_cache = tma_cache_new();
-        else g.tma = 0;
+        // tiles of as many columns as the transform group has threads for
+        const int tpl = line_tpl(g.n1);
+        if (nc == 6 && tpl > 0) {
+            int t = ctx->shape[2] > 0 ? ctx->shape[2] : std::max(1, std::min(16, kX1Group / (6 * tpl)));
+            while (ctx->shape[2] == 0 && t > 1 && !tma_box_rows(g.n1, 6 * t * (int)cs)) --t;
+            g.box1l = tma_box_rows(g.n1, 6 * t * (int)cs);
+            if (6 * t * tpl <= kX1Group && g.box1l > 0) {
+                g.tile1l = t;
+                g.grp1l = round32(6 * t * tpl);
+                g.stage1l = (6ull * t * g.n1 * cs + 127) / 128 * 128;
+            }
+        }
+        Launch<R>::tma_grids(g);
+        if (!g.grp1l) g.tile1l = t1;
+        if (g.tma || g.x2t || g.grp1l) g.tma_cache = tma_cache_new();
     }
+    g.kvec = (long long)((g.n2 * g.h + g.tile1l - 1) / g.tile1l) * g.n1 * nc * g.tile1l;
     return HOM_OK;
 }
 
@@ -1366,8 +1390,10 @@ static int batch_reserve(hom_ctx *ctx, int nb) {
         np = std::max(np, (long long)Launch<double>::x3_epart_grid(ctx->e64.g));
         np = std::max(np, (long long)Launch<double>::x1_lanczos_grid(ctx->e64.g));
     } else {
-        np = std::max(np, (long long)Launch<float>::x3_epart_grid(ctx->e32.g));
-        np = std::max(np, (long long)Launch<float>::x1_lanczos_grid(ctx->e32.g));
+        Geometry gb = ctx->e32.g;   // the persistent grids grow with the cases
+        gb.nb = nb;
+        np = std::max(np, (long long)Launch<float>::x3_epart_grid(gb));
+        np = std::max(np, (long long)Launch<float>::x1_lanczos_grid(gb));
     }
     CU(cudaMalloc(&ctx->bpart, sizeof(double) * np * nb));
     CU(cudaMalloc(&ctx->bcnt, sizeof(int) * kFoldCounters));
@@ -1437,12 +1463,12 @@ static void capture_bbody(hom_ctx *ctx, Engine<R> &E) {
 // cases); a change of nb drops the cell's stacked graph
 template <typename R>
 static void set_bgeom(hom_ctx *ctx, Engine<R> &E, int nb) {
-    if (ctx->bg.nb == nb && ctx->bg.n1 == E.g.n1 && ctx->bg.mask0 == E.g.mask0 && (ctx->btma || !E.g.tma)) return;
+    if (ctx->bg.nb == nb && ctx->bg.n1 == E.g.n1 && ctx->bg.mask0 == E.g.mask0 && (ctx->btma || !E.g.tma_cache)) return;
     if (ctx->bgraph) cudaGraphExecDestroy(ctx->bgraph);
     ctx->bgraph = nullptr;
     ctx->bgraph_nb = 0;
     tma_cache_free(ctx->btma);
-    ctx->btma = E.g.tma ? tma_cache_new() : nullptr;
+    ctx->btma = E.g.tma_cache ? tma_cache_new() : nullptr;
     ctx->bg = E.g;
     ctx->bg.nb = nb;
     ctx->bg.tma_cache = ctx->btma;

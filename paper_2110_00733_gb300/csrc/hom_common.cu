@@ -302,6 +302,28 @@ struct TmaCache {
 };
 }  // namespace
 
+int tma_box_rows(int n, int rowb) {
+    for (int k = (n + 255) / 256; k <= n; ++k)
+        if (n % k == 0 && (k == 1 || (n / k) * rowb % 128 == 0)) return n / k;
+    return 0;
+}
+
+int line_tpl(int n) {
+    switch (n) {
+#define HOM_LINE_TPL(N) case N: return LinePlan<N>::TPL;
+        HOM_LINE_LENGTHS_A(HOM_LINE_TPL) HOM_LINE_LENGTHS_B(HOM_LINE_TPL) HOM_LINE_LENGTHS_C(HOM_LINE_TPL)
+#undef HOM_LINE_TPL
+        default: return 0;
+    }
+}
+
+void line_kernel_attr(const void *kernel, int optin) {
+    cudaFuncAttributes fa{};
+    cudaFuncGetAttributes(&fa, kernel);
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
+    cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+}
+
 bool tma_available() { return encoder() != nullptr; }
 
 void *tma_cache_new() { return new TmaCache(); }
@@ -317,7 +339,8 @@ void tma_cache_free(void *c) {
 //  TMA_X2: 3-D (6h, n2, n1), box (tile2, n2, 1): one tile2-wide run of
 //          columns over all k2 of one k1 plane.
 //  TMA_X1: 2-D (6 n2 h, n1), box (6 tile1, n1): tile1 (k2,k3) columns with
-//          their 6 components over all k1.
+//          their 6 components over all k1.  TMA_X1L the same with tile1l.
+// Columns longer than a box move in several boxes (tma_box_rows), one copy each.
 const CUtensorMap *tma_map(const Geometry &g, const void *ptr, int kind, int units) {
     TmaCache *tc = static_cast<TmaCache *>(g.tma_cache);
     for (TmaEntry *e : tc->entries)
@@ -333,9 +356,7 @@ const CUtensorMap *tma_map(const Geometry &g, const void *ptr, int kind, int uni
     if (kind == TMA_X2) {
         cuuint64_t dims[3] = {h6, (cuuint64_t)g.n2, (cuuint64_t)g.n1 * g.nb};
         cuuint64_t strides[2] = {h6 * 8, h6 * 8 * g.n2};
-        // box dimensions hold at most 256 elements: longer columns move in
-        // boxes of 256 rows (the kernels issue one copy per box)
-        cuuint32_t box[3] = {(cuuint32_t)(g.tile2 * units), (cuuint32_t)(g.n2 < 256 ? g.n2 : 256), 1};
+        cuuint32_t box[3] = {(cuuint32_t)(g.tile2 * units), (cuuint32_t)g.box2, 1};
         cuuint32_t es[3] = {1, 1, 1};
         r = fn(&e->map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, const_cast<void *>(ptr), dims, strides, box, es,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -343,7 +364,9 @@ const CUtensorMap *tma_map(const Geometry &g, const void *ptr, int kind, int uni
     } else {
         cuuint64_t dims[2] = {h6 * g.n2, (cuuint64_t)g.n1 * g.nb};
         cuuint64_t strides[1] = {h6 * g.n2 * 8};
-        cuuint32_t box[2] = {(cuuint32_t)(g.nc * g.tile1 * units), (cuuint32_t)(g.n1 < 256 ? g.n1 : 256)};
+        const bool fused = kind == TMA_X1L;
+        cuuint32_t box[2] = {(cuuint32_t)(g.nc * (fused ? g.tile1l : g.tile1) * units),
+                             (cuuint32_t)(fused ? g.box1l : g.box1)};
         cuuint32_t es[2] = {1, 1};
         r = fn(&e->map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, const_cast<void *>(ptr), dims, strides, box, es,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,

@@ -9,6 +9,7 @@
 // butterflies (R in {2,3,4,5,8,16}) held in registers; twiddles come from a
 // per-axis table w[t] = exp(-2 pi i t / N) computed on the host in double.
 #pragma once
+#include <initializer_list>
 #include <type_traits>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -147,62 +148,71 @@ template <typename R, int S> __device__ __forceinline__ void dft16(cpx<R> *v) {
     }
 }
 
-// exp(S 2 pi i e / N) for N = 12 or 20 (e known at compile time after
-// unrolling): cosines of multiples of 30 and 18 degrees
-template <typename R, int N> __device__ __forceinline__ R cos_n(int e) {
-    e %= N;
-    if constexpr (N == 12) {
-        const R c30 = (R)0.86602540378443864676;   // cos(pi/6)
-        const R t[12] = {1, c30, (R)0.5, 0, (R)-0.5, -c30, -1, -c30, (R)-0.5, 0, (R)0.5, c30};
-        return t[e];
-    } else {
-        const R a = (R)0.95105651629515357212, b = (R)0.80901699437494742410;   // cos(pi/10), cos(pi/5)
-        const R c = (R)0.58778525229247312917, d = (R)0.30901699437494742410;   // cos(3pi/10), cos(2pi/5)
-        const R t[20] = {1, a, b, c, d, 0, -d, -c, -b, -a, -1, -a, -b, -c, -d, 0, d, c, b, a};
-        return t[e];
-    }
-}
-template <typename R, int S, int N> __device__ __forceinline__ cpx<R> w_n(int e) {
-    // sin(2 pi e / N) = cos(2 pi (e - N/4) / N)
-    return mk<R>(cos_n<R, N>(e), (R)S * cos_n<R, N>(e + 3 * N / 4));
+// exp(S 2 pi i e / 9) for e = 1, 2, 4, the twiddles of the radix-9 butterfly:
+// cosines and sines of 40, 80 and 160 degrees
+template <typename R, int S> __device__ __forceinline__ cpx<R> w9(int e) {
+    const R c1 = (R)0.76604444311897803520, s1 = (R)0.64278760968653932632;
+    const R c2 = (R)0.17364817766693034885, s2 = (R)0.98480775301220805937;
+    const R c4 = (R)-0.93969262078590838405, s4 = (R)0.34202014332566873304;
+    return e == 1 ? mk<R>(c1, (R)S * s1) : (e == 2 ? mk<R>(c2, (R)S * s2) : mk<R>(c4, (R)S * s4));
 }
 
-// Composite DFT of length N1 N2 in registers (Cooley-Tukey): DFT-N1 over n1
-// for each n2 on x[N2 n1 + n2], the twiddle w_N^(n2 k1), DFT-N2 over n2 for
-// each k1, output X[k1 + N1 k2].
-template <typename R, int S, int N1, int N2> __device__ __forceinline__ void dft_ct(cpx<R> *v);
+template <typename R, int S, int RAD> __device__ __forceinline__ void dft(cpx<R> *v);
+
+template <typename R, int S> __device__ __forceinline__ void dft9(cpx<R> *v) {
+    cpx<R> y[3][3];   // y[k1][n2]: DFT-3 over n1 of x[3 n1 + n2], times w9^(n2 k1)
+#pragma unroll
+    for (int n2 = 0; n2 < 3; ++n2) {
+        cpx<R> a[3] = {v[n2], v[3 + n2], v[6 + n2]};
+        dft3<R, S>(a);
+#pragma unroll
+        for (int k1 = 0; k1 < 3; ++k1) y[k1][n2] = n2 * k1 == 0 ? a[k1] : mul<R>(a[k1], w9<R, S>(n2 * k1));
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < 3; ++k1) {
+        dft3<R, S>(y[k1]);
+#pragma unroll
+        for (int k2 = 0; k2 < 3; ++k2) v[k1 + 3 * k2] = y[k1][k2];
+    }
+}
+
+// DFT of length N1 N2, N1 and N2 coprime, in registers without twiddles
+// (Good's prime-factor mapping): inputs x[(N2 n1 + N1 n2) mod N], output
+// X[k] from the DFT-N1 index k mod N1 and the DFT-N2 index k mod N2.
+template <typename R, int S, int N1, int N2> __device__ __forceinline__ void dft_pfa(cpx<R> *v) {
+    constexpr int N = N1 * N2;
+    cpx<R> y[N1][N2];
+#pragma unroll
+    for (int n2 = 0; n2 < N2; ++n2) {
+        cpx<R> a[N1];
+#pragma unroll
+        for (int n1 = 0; n1 < N1; ++n1) a[n1] = v[(N2 * n1 + N1 * n2) % N];
+        dft<R, S, N1>(a);
+#pragma unroll
+        for (int k1 = 0; k1 < N1; ++k1) y[k1][n2] = a[k1];
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < N1; ++k1) dft<R, S, N2>(y[k1]);
+#pragma unroll
+    for (int k = 0; k < N; ++k) v[k] = y[k % N1][k % N2];
+}
 
 template <typename R, int S, int RAD> __device__ __forceinline__ void dft(cpx<R> *v) {
     if constexpr (RAD == 2) dft2<R, S>(v[0], v[1]);
     else if constexpr (RAD == 3) dft3<R, S>(v);
     else if constexpr (RAD == 4) dft4<R, S>(v);
     else if constexpr (RAD == 5) dft5<R, S>(v);
+    else if constexpr (RAD == 6) dft_pfa<R, S, 2, 3>(v);
     else if constexpr (RAD == 8) dft8<R, S>(v);
-    else if constexpr (RAD == 12) dft_ct<R, S, 4, 3>(v);
-    else if constexpr (RAD == 20) dft_ct<R, S, 4, 5>(v);
-    else dft16<R, S>(v);
-}
-
-template <typename R, int S, int N1, int N2> __device__ __forceinline__ void dft_ct(cpx<R> *v) {
-    constexpr int N = N1 * N2;
-    cpx<R> y[N];
-#pragma unroll
-    for (int n2 = 0; n2 < N2; ++n2) {
-        cpx<R> a[N1];
-#pragma unroll
-        for (int n1 = 0; n1 < N1; ++n1) a[n1] = v[N2 * n1 + n2];
-        dft<R, S, N1>(a);
-#pragma unroll
-        for (int k1 = 0; k1 < N1; ++k1) y[N2 * k1 + n2] = (n2 * k1 == 0) ? a[k1] : mul<R>(a[k1], w_n<R, S, N>(n2 * k1));
-    }
-#pragma unroll
-    for (int k1 = 0; k1 < N1; ++k1) {
-        cpx<R> b[N2];
-#pragma unroll
-        for (int n2 = 0; n2 < N2; ++n2) b[n2] = y[N2 * k1 + n2];
-        dft<R, S, N2>(b);
-#pragma unroll
-        for (int k2 = 0; k2 < N2; ++k2) v[k1 + N1 * k2] = b[k2];
+    else if constexpr (RAD == 9) dft9<R, S>(v);
+    else if constexpr (RAD == 10) dft_pfa<R, S, 2, 5>(v);
+    else if constexpr (RAD == 12) dft_pfa<R, S, 4, 3>(v);
+    else if constexpr (RAD == 15) dft_pfa<R, S, 3, 5>(v);
+    else if constexpr (RAD == 18) dft_pfa<R, S, 2, 9>(v);
+    else if constexpr (RAD == 20) dft_pfa<R, S, 4, 5>(v);
+    else {
+        static_assert(RAD == 16, "no butterfly of this radix");
+        dft16<R, S>(v);
     }
 }
 
@@ -371,6 +381,138 @@ __device__ __forceinline__ void fast_fft(cpx<R> *buf, int L, int ES, const cpx<R
     if constexpr (P::NS > 1) fast_stage<R, S, N, P::R1, P::R0, PAD, P>(buf, ES, l, j0, tw, nsync);
     if constexpr (P::NS > 2) fast_stage<R, S, N, P::R2, P::R0 * P::R1, PAD, P>(buf, ES, l, j0, tw, nsync);
     if constexpr (P::NS > 3) fast_stage<R, S, N, P::R3, P::R0 * P::R1 * P::R2, PAD, P>(buf, ES, l, j0, tw, nsync);
+}
+
+// ---------------------------------------------------------------------------
+// Line engine: the register engine above for every length 2^a 3^b 5^c in
+// [16, 512], with two or three stages of any of the butterflies.  TPL threads
+// share a line; a stage of radix RAD has N / RAD butterflies, which the TPL
+// threads take in ceil(N / (RAD TPL)) rounds (idle where they do not divide:
+// 108 = 12 9 with TPL = 12 idles 3 threads of 12 in its radix-12 stage).
+// Measured against the runtime Stockham engine (whose index arithmetic
+// divides at run time and which needs two shared buffers) in the comments of
+// the passes that use it.
+// ---------------------------------------------------------------------------
+struct LinePlanV { int r0, r1, r2, tpl; };
+
+constexpr bool line_radix(int r) {
+    return r == 2 || r == 3 || r == 4 || r == 5 || r == 6 || r == 8 || r == 9 || r == 10 || r == 12 || r == 15 ||
+           r == 16 || r == 18 || r == 20;
+}
+constexpr int kLineMaxElems = 20;
+
+// (complex) elements a thread holds between the barriers of its widest stage
+constexpr int line_elems(int N, int r0, int r1, int r2, int tpl) {
+    const int rs[3] = {r0, r1, r2};
+    int e = 0;
+    for (int i = 0; i < 3; ++i) {
+        const int v = (N / rs[i] + tpl - 1) / tpl * rs[i];
+        if (rs[i] > 1 && v > e) e = v;
+    }
+    return e;
+}
+
+// radices (largest first: a stage's twiddles are N (1 - 1/r)) and threads of a
+// line.  The score weighs the element slots a line passes through (its
+// stages' rounds times TPL threads, idle ones included) against the elements
+// a thread holds; more than 16 of them (32 registers) only where few plans
+// divide N in two stages.  The power-of-two plans are 64 = 8 8, 128 = 16 8,
+// 256 = 16 16 with 8, 8 and 16 threads.
+constexpr LinePlanV line_plan(int N) {
+    LinePlanV best{0, 0, 0, 0};
+    int bc = 1 << 30;
+    for (int r0 = 20; r0 >= 2; --r0) {
+        if (!line_radix(r0) || N % r0) continue;
+        for (int r1 = r0; r1 >= 1; --r1) {
+            if ((r1 > 1 && !line_radix(r1)) || (N / r0) % r1) continue;
+            const int r2 = N / r0 / r1;
+            if (r2 > r1 || (r2 > 1 && !line_radix(r2))) continue;
+            for (int tpl = 2; tpl <= 32; ++tpl) {
+                const int e = line_elems(N, r0, r1, r2, tpl);
+                if (e > kLineMaxElems) continue;
+                int slots = 0;
+                for (int r : {r0, r1, r2})
+                    if (r > 1) slots += (N / r + tpl - 1) / tpl * r * tpl;
+                const int score = slots * 1000 / N + e * 40 + tpl + (e > 16 ? 400 : 0);
+                if (score < bc) {
+                    bc = score;
+                    best = LinePlanV{r0, r1, r2, tpl};
+                }
+            }
+        }
+    }
+    return best;
+}
+// The lengths' kernels are instantiated from these lists (see the passes).
+#define HOM_LINE_LENGTHS_A(X) \
+    X(16) X(18) X(20) X(24) X(25) X(27) X(30) X(32) X(36) X(40) X(45) X(48) X(50) X(54) X(60) X(64) X(72) X(75) X(80)
+#define HOM_LINE_LENGTHS_B(X) \
+    X(81) X(90) X(96) X(100) X(108) X(120) X(125) X(128) X(135) X(144) X(150) X(160) X(162) X(180) X(192) X(200)
+#define HOM_LINE_LENGTHS_C(X) \
+    X(216) X(225) X(240) X(243) X(250) X(256) X(270) X(288) X(300) X(320) X(324) X(360) X(375) X(384) X(400) X(405) \
+    X(432) X(450) X(480) X(486) X(500) X(512)
+
+template <int N> struct LinePlan {
+    static constexpr LinePlanV P = line_plan(N);
+    static constexpr int R0 = P.r0, R1 = P.r1, R2 = P.r2, TPL = P.tpl;
+    static constexpr int E = line_elems(N, P.r0, P.r1, P.r2, P.tpl);
+    static_assert(R0 * R1 * R2 == N, "no plan for this length");
+};
+// threads of a line at run time (0: not a length of the line engine)
+int line_tpl(int n);
+
+template <typename R, int S, int N, int RAD, int NSB, int TPL>
+__device__ __forceinline__ void line_stage(cpx<R> *buf, int ES, int l, int j0, const cpx<R> *__restrict__ tw,
+                                           int nsync) {
+    constexpr int nb = N / RAD;
+    constexpr int BPT = (nb + TPL - 1) / TPL;
+    constexpr bool even = nb % TPL == 0;
+    constexpr int twstep = N / (NSB * RAD);
+    cpx<R> v[BPT][RAD];
+    // idle slots load and transform butterfly 0 and store nothing, so that
+    // only the stores are conditional
+#pragma unroll
+    for (int i = 0; i < BPT; ++i) {
+        const int jj = j0 + i * TPL, j = j0 < TPL && (even || jj < nb) ? jj : 0;
+#pragma unroll
+        for (int r = 0; r < RAD; ++r) v[i][r] = buf[(j + r * nb) * ES + l];
+    }
+    group_sync(nsync);
+#pragma unroll
+    for (int i = 0; i < BPT; ++i) {
+        const int jj = j0 + i * TPL;
+        const bool live = j0 < TPL && (even || jj < nb);
+        const int j = live ? jj : 0;
+        const int jm = nb == NSB ? j : j % NSB;   // nb = NSB in the last stage
+        if constexpr (NSB > 1) {
+#pragma unroll
+            for (int r = 1; r < RAD; ++r) {
+                cpx<R> w = __ldg(&tw[jm * r * twstep]);
+                if (S > 0) w.y = -w.y;
+                v[i][r] = mul<R>(v[i][r], w);
+            }
+        }
+        dft<R, S, RAD>(v[i]);
+        const int o = (j - jm) * RAD + jm;
+        if (live) {
+#pragma unroll
+            for (int r = 0; r < RAD; ++r) buf[(o + r * NSB) * ES + l] = v[i][r];
+        }
+    }
+    group_sync(nsync);
+}
+
+// Transform of L interleaved lines in buf (in place), element e of line l at
+// buf[e * ES + l].  The CTA's threads (nsync = 0), or its first nsync on named
+// barrier 1, all call it; those beyond L * TPL only take part in the barriers.
+template <typename R, int S, int N>
+__device__ __forceinline__ void line_fft(cpx<R> *buf, int L, int ES, const cpx<R> *__restrict__ tw, int nsync = 0) {
+    using P = LinePlan<N>;
+    const int l = (int)threadIdx.x % L;
+    const int j0 = (int)threadIdx.x / L;
+    line_stage<R, S, N, P::R0, 1, P::TPL>(buf, ES, l, j0, tw, nsync);
+    if constexpr (P::R1 > 1) line_stage<R, S, N, P::R1, P::R0, P::TPL>(buf, ES, l, j0, tw, nsync);
+    if constexpr (P::R2 > 1) line_stage<R, S, N, P::R2, P::R0 * P::R1, P::TPL>(buf, ES, l, j0, tw, nsync);
 }
 
 }  // namespace hom

@@ -144,21 +144,29 @@ struct Geometry {
     // predecessor with griddepcontrol before touching memory)
     int pdl = 0;
     int mask0;              // stress-controlled Mandel components (bit c): the projector keeps them at xi = 0
-    // persistent TMA-staged n2 / n1 passes (FP32, register-FFT n in [64, 512]):
-    // enabled flag, persistent grid sizes, shared memory, host-side cache of
-    // tensor maps (never dereferenced on the device) and the device word a
-    // pass sets when a bounded wait gives up
+    // persistent TMA-staged passes (FP32): tma enables the unfused n1 pass
+    // (register-FFT n1 and n2 in [64, 512]); persistent grid sizes, shared
+    // memory, host-side cache of tensor maps (never dereferenced on the
+    // device) and the device word a pass sets when a bounded wait gives up
     int tma;
     // fused MINRES chain: complex elements of one Krylov vector stored in
-    // n1-tile order (tiles of tile1 (k2,k3) columns, each tile a contiguous
-    // n1 x 6 tile1 block laid out as the pass's shared-memory tile)
+    // n1-tile order (tiles of tile1l (k2,k3) columns, each tile a contiguous
+    // n1 x 6 tile1l block laid out as the pass's shared-memory tile)
     long long kvec;
     // register-resident n3 pass (k_x3r: FP32, n3 in {64, 128, 256}) for
     // spectrum-to-spectrum applications
     int x3r;
     int grid2_tma, grid1_tma, grid1d_tma;
-    int grid1l_tma;         // persistent grid of the fused MINRES n1 pass (0: plain-load form)
+    int grid1l_tma = 0;     // persistent grid of the fused MINRES n1 pass (0: plain-load form)
     size_t smem2_tma, smem1_tma, smem1d_tma;
+    // TMA-staged n2 pass and fused n1 pass, every length of the line engine:
+    // x2t enables the n2 pass (threads2t threads); the fused n1 pass has
+    // grp1l transform threads (0: plain-load form), tiles of tile1l columns
+    // and stage1l bytes per shared-memory stage; rows per TMA box
+    int x2t = 0, threads2t = 0, grp1l = 0;
+    int tile1l;             // columns of a Krylov-vector tile (tile1 where the plain-load form runs)
+    size_t stage1l = 0;
+    int box2 = 0, box1 = 0, box1l = 0;
     int grid3r = 0;         // persistent grid of the register n3 pass
     int x2_stages = 2;      // TMA ring stages of the persistent n2 pass
     int x1_l2pf = 1;        // fused n1 pass: L2 prefetch of each tile's u_k, u_{k-1} blocks
@@ -218,7 +226,7 @@ inline void launch_k(int pdl, void (*k)(KArgs...), dim3 grid, dim3 block, size_t
 }
 
 // tensor-map kinds of the TMA passes
-enum TmaKind { TMA_X2 = 0, TMA_X1 = 1 };
+enum TmaKind { TMA_X2 = 0, TMA_X1 = 1, TMA_X1L = 2 };
 // Host: the cached tensor map of `ptr` (a half spectrum of this geometry) for
 // the given pass; nullptr if the driver entry point is unavailable.
 const CUtensorMap *tma_map(const Geometry &g, const void *ptr, int kind, int elem_units);
@@ -236,8 +244,9 @@ enum X1Flags { X1_FWD = 1, X1_GAMMA_IN = 2, X1_GAMMA_OUT = 4, X1_DOT = 8 };
 
 constexpr int kEwBlocks = 152 * 8;   // grid of the element-wise Krylov kernels
 constexpr int kNbMax = 8;            // load cases of one stacked MINRES batch
-// threads of the persistent fused n1 pass: the transform group (the fast
-// lengths' n1 tiles take 192 threads) and the lagged-update warps
+// threads of the persistent fused n1 pass: the most its transform group may
+// have (with the lagged-update warps, two CTAs per SM at 127 registers) and
+// the lagged-update warps
 constexpr int kX1Group = 192;
 constexpr int kX1LagThreads = 64;
 constexpr int kX1LagChunk = 4096;      // bytes of one operand per ring stage
@@ -260,6 +269,19 @@ struct Fold {
     double scale;        // alpha: the partials sum to <u, A^ u> / scale
 };
 constexpr int kFoldCounters = 2 * kNbMax + 1;
+
+// Kernels of the line engine (FP32) for one length; nullptr where it has none.
+using X2LineFn = void (*)(Geometry, CUtensorMap, int, const MinresState *);
+using X1lLineFn = void (*)(Geometry, CUtensorMap, const float2 *, const float2 *, float2 *, const float2 *, float2 *,
+                           float2 *, const MinresState *, double *, Fold);
+X2LineFn x2_line_kernel(int n, int inverse);
+X1lLineFn x1l_line_kernel(int n);
+// shared-memory limit and carve-out of one of them
+void line_kernel_attr(const void *kernel, int optin);
+// rows of a TMA box for tiles of n rows of rowb bytes: the most that divide n,
+// fit a box dimension (256) and keep every box on a 128-byte boundary of
+// shared memory (0: none)
+int tma_box_rows(int n, int rowb);
 
 template <typename R> struct Launch {
     // n3 pass: C2R (SPEC in) or real / macro input, optional material law
@@ -351,7 +373,7 @@ template <typename R> struct Launch {
     // resident CTAs x SMs of the persistent register n3 pass (0: it cannot run)
     static int x3r_grid(const Geometry &g);
     static int x1_grid(const Geometry &g);
-    static int tma_grids(Geometry &g);
+    static void tma_grids(Geometry &g);
 };
 
 // FP64 helpers on spectral vectors (double2) and real fields

@@ -797,23 +797,24 @@ __global__ void HOM_PASS_BOUNDS_NF(R, NF) k_x1(Geometry g, int flags, const cpx<
     }
 }
 
-// A TMA box dimension holds at most 256 elements: a tile of n > 256 rows
-// (n = 512) moves as consecutive boxes of 256 rows; rowb is the bytes of one
-// row of the tile in shared memory.
-constexpr int kBoxRows = 256;
-__device__ __forceinline__ void tma_load_rows_3d(void *dst, const CUtensorMap *tm, int x, int n, int z, int rowb,
-                                                 uint64_t *bar) {
-    for (int y0 = 0; y0 < n; y0 += kBoxRows) tma_load_3d((char *)dst + (size_t)y0 * rowb, tm, x, y0, z, bar);
+// A TMA box dimension holds at most 256 elements: a tile of n > 256 rows moves
+// as n / box consecutive boxes of box rows (tma_box_rows); rowb is the bytes of
+// one row of the tile in shared memory.
+__device__ __forceinline__ void tma_load_rows_3d(void *dst, const CUtensorMap *tm, int x, int n, int box, int z,
+                                                 int rowb, uint64_t *bar) {
+    for (int y0 = 0; y0 < n; y0 += box) tma_load_3d((char *)dst + (size_t)y0 * rowb, tm, x, y0, z, bar);
 }
-__device__ __forceinline__ void tma_store_rows_3d(const CUtensorMap *tm, int x, int n, int z, const void *src, int rowb) {
-    for (int y0 = 0; y0 < n; y0 += kBoxRows) tma_store_3d(tm, x, y0, z, (const char *)src + (size_t)y0 * rowb);
+__device__ __forceinline__ void tma_store_rows_3d(const CUtensorMap *tm, int x, int n, int box, int z, const void *src,
+                                                  int rowb) {
+    for (int y0 = 0; y0 < n; y0 += box) tma_store_3d(tm, x, y0, z, (const char *)src + (size_t)y0 * rowb);
 }
-__device__ __forceinline__ void tma_load_rows_2d(void *dst, const CUtensorMap *tm, int x, int y, int n, int rowb,
-                                                 uint64_t *bar) {
-    for (int y0 = 0; y0 < n; y0 += kBoxRows) tma_load_2d((char *)dst + (size_t)y0 * rowb, tm, x, y + y0, bar);
+__device__ __forceinline__ void tma_load_rows_2d(void *dst, const CUtensorMap *tm, int x, int y, int n, int box,
+                                                 int rowb, uint64_t *bar) {
+    for (int y0 = 0; y0 < n; y0 += box) tma_load_2d((char *)dst + (size_t)y0 * rowb, tm, x, y + y0, bar);
 }
-__device__ __forceinline__ void tma_store_rows_2d(const CUtensorMap *tm, int x, int y, int n, const void *src, int rowb) {
-    for (int y0 = 0; y0 < n; y0 += kBoxRows) tma_store_2d(tm, x, y + y0, (const char *)src + (size_t)y0 * rowb);
+__device__ __forceinline__ void tma_store_rows_2d(const CUtensorMap *tm, int x, int y, int n, int box, const void *src,
+                                                  int rowb) {
+    for (int y0 = 0; y0 < n; y0 += box) tma_store_2d(tm, x, y + y0, (const char *)src + (size_t)y0 * rowb);
 }
 
 // ---------------------------------------------------------------------------
@@ -825,73 +826,6 @@ __device__ __forceinline__ void tma_store_rows_2d(const CUtensorMap *tm, int x, 
 // the failure in *g.err, waits (bounded) for its own load in flight and
 // returns, and the host reports HOM_ETIMEOUT.
 // ---------------------------------------------------------------------------
-template <typename R, int S, int NF>
-__global__ void HOM_PASS_BOUNDS_NF(R, NF) k_x2_tma(Geometry g, const __grid_constant__ CUtensorMap tm, int qtiles,
-                                            const MinresState *state) {
-    pdl_release();
-    pdl_wait();   // predecessor complete (programmatic launch in the MINRES graph)
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t bar[kX2MaxStages];
-    const int N = g.n2, T = g.tile2, NS = g.x2_stages;
-    const int ntiles = g.n1 * g.nb * qtiles;   // stacked cases along k1
-    const int tpc = g.n1 * qtiles;             // tiles per case
-    // next tile of this CTA's sequence whose case is still iterating
-    auto live_from = [&](int t) {
-        while (t < ntiles && skip_case(state, t / tpc)) t += gridDim.x;
-        return t;
-    };
-    cpx<R> *const base = reinterpret_cast<cpx<R> *>(smem_raw);
-    const int per = N * T;   // stage s starts at base + s * per
-    const uint32_t bytes = (uint32_t)(per * sizeof(cpx<R>));
-    const bool leader = threadIdx.x == 0;
-    if (leader) {
-        for (int q = 0; q < NS; ++q) mbar_init(&bar[q], 1);
-        fence_mbar_init();
-    }
-    __syncthreads();
-    // NS-stage ring: the leader keeps NS - 1 tiles in flight ahead of the one
-    // being transformed (tile j of the sequence in stage j mod NS)
-    int tile = live_from(blockIdx.x);
-    int ahead = tile, issued = 0;   // next tile to load, tiles loaded (leader)
-    auto issue = [&]() {
-        const int q = issued % NS;
-        mbar_expect_tx(&bar[q], bytes);
-        tma_load_rows_3d(base + q * per, &tm, (ahead % qtiles) * T, N, ahead / qtiles, T * (int)sizeof(cpx<R>),
-                         &bar[q]);
-        ++issued;
-        ahead = live_from(ahead + gridDim.x);
-    };
-    if (leader)
-        for (int q = 0; q < NS - 1 && ahead < ntiles; ++q) issue();
-    const cpx<R> *tw = reinterpret_cast<const cpx<R> *>(g.ax[1].tw);
-    for (int i = 0; tile < ntiles; ++i) {
-        const int q = i % NS;
-        if (leader && ahead < ntiles) {
-            bulk_wait_read_all();   // the store of the tile that used this stage has read it
-            issue();
-        }
-        const bool ok = mbar_wait_bounded(&bar[q], (uint32_t)(i / NS) & 1u);
-        if (__syncthreads_or(!ok)) {
-            if (leader) {   // record, then wait (bounded) for this CTA's loads in flight
-                atomicExch(g.err, 1);
-                for (int m = i; m < issued; ++m) mbar_wait_bounded(&bar[m % NS], (uint32_t)(m / NS) & 1u);
-                bulk_wait_all();
-            }
-            return;
-        }
-        cpx<R> *buf = base + q * per;
-        fast_fft<R, S, NF>(buf, T, T, tw);
-        fence_proxy_async_smem();
-        __syncthreads();
-        if (leader) {
-            tma_store_rows_3d(&tm, (tile % qtiles) * T, N, tile / qtiles, buf, T * (int)sizeof(cpx<R>));
-            bulk_commit();
-        }
-        tile = live_from(tile + gridDim.x);
-    }
-    if (leader) bulk_wait_all();
-}
-
 // MoDBFFT contraction at frequency (k1, k2, k3) of the 10-component
 // forward transform t (the stress tau and the penalty vector g), eq.
 // (modbfftfop): r = tau xi + g with xi = i 2 pi q, q the integer frequency (0
@@ -1002,8 +936,8 @@ __global__ void HOM_PASS_BOUNDS_NF(R, NF) k_x1_tma(Geometry g, int flags, const 
     __syncthreads();
     auto issue = [&](int t, int s) {
         mbar_expect_tx(&bar[s], bytes);
-        tma_load_rows_2d(base + s * per, &tin, NC * T * t, 0, N, L * (int)sizeof(cpx<R>), &bar[s]);
-        if (dot) tma_load_rows_2d(base + s * per + tile_elems, &tdot, NC * T * t, 0, N, L * (int)sizeof(cpx<R>), &bar[s]);
+        tma_load_rows_2d(base + s * per, &tin, NC * T * t, 0, N, g.box1, L * (int)sizeof(cpx<R>), &bar[s]);
+        if (dot) tma_load_rows_2d(base + s * per + tile_elems, &tdot, NC * T * t, 0, N, g.box1, L * (int)sizeof(cpx<R>), &bar[s]);
     };
     int tile = blockIdx.x;
     if (leader && tile < ntiles) issue(tile, 0);
@@ -1081,7 +1015,7 @@ __global__ void HOM_PASS_BOUNDS_NF(R, NF) k_x1_tma(Geometry g, int flags, const 
         fence_proxy_async_smem();
         __syncthreads();
         if (leader) {
-            tma_store_rows_2d(&tout, NC * T * tile, 0, N, buf, L * (int)sizeof(cpx<R>));
+            tma_store_rows_2d(&tout, NC * T * tile, 0, N, g.box1, buf, L * (int)sizeof(cpx<R>));
             bulk_commit();
         }
     }
@@ -1132,7 +1066,7 @@ __global__ void HOM_PASS_BOUNDS_NF(R, NF) k_x1_tma_expand(Geometry g, const __gr
         fence_proxy_async_smem();
         __syncthreads();
         if (leader) {
-            tma_store_rows_2d(&tout, NC * T * tile, 0, N, buf, L * (int)sizeof(cpx<R>));
+            tma_store_rows_2d(&tout, NC * T * tile, 0, N, g.box1, buf, L * (int)sizeof(cpx<R>));
             bulk_commit();
         }
     }
@@ -1158,6 +1092,15 @@ __global__ void HOM_PASS_BOUNDS_NF(R, NF) k_x1_tma_expand(Geometry g, const __gr
 // w_{k-1} replaces it); the flush after the loop adds what is pending.  The
 // sum is the same as one update per step, rounded in another order.
 // ---------------------------------------------------------------------------
+// The transform along n1 of the plain-load passes: the register engine at its
+// lengths, else the runtime Stockham engine.
+template <typename R, int NF> struct PassFft {
+    template <int S>
+    __device__ static __forceinline__ cpx<R> *run(cpx<R> *buf, cpx<R> *buf2, int L, const AxisPlan &p, int nsync) {
+        return run_fft<R, S, NF>(buf, buf2, L, L, p, nsync);
+    }
+};
+
 template <typename R> struct LzCoef {
     R cp, cu, cv;            // 1/beta_k, -alpha_k/beta_k, -beta_k/beta_{k-1}
     R d, e, ig, tau, ib;     // lagged update of step k-1
@@ -1199,18 +1142,19 @@ __device__ __forceinline__ LzCoef<R> lz_coef(const MinresState *st) {
 // contiguous block.  u_{k+1} goes to un, a third buffer (u_{k-1} stays
 // readable for the lagged update); with LAG the lagged w / x update of step
 // k-1 is done here too, else by other warps (x1_lagged_block).
-template <typename R, int NF, bool LAG>
-__device__ __forceinline__ cpx<R> *x1_lanczos_tile(const Geometry &g, cpx<R> *buf, cpx<R> *buf2, int g0,
+// Fft is the transform along n1 (PassFft here, LineFft in the TMA-staged form).
+template <typename R, typename Fft, bool LAG>
+__device__ __forceinline__ cpx<R> *x1_lanczos_tile(const Geometry &g, int T, cpx<R> *buf, cpx<R> *buf2, int g0,
                                                    const LzCoef<R> &c, const cpx<R> *__restrict__ uk,
                                                    const cpx<R> *__restrict__ um, cpx<R> *__restrict__ un,
                                                    const cpx<R> *__restrict__ wa, cpx<R> *__restrict__ wb,
                                                    cpx<R> *__restrict__ x, Acc<R> &acc, int nsync) {
     constexpr int NC = 6;
-    const int N = g.n1, T = g.tile1, H = g.h, L = NC * T;
+    const int N = g.n1, H = g.h, L = NC * T;
     const int cols = g.n2 * H;
     const int nthr = nsync ? nsync : (int)blockDim.x;
     // 1. forward DFT along n1
-    cpx<R> *res = run_fft<R, -1, NF>(buf, buf2, L, L, g.ax[0], nsync);
+    cpx<R> *res = Fft::template run<-1>(buf, buf2, L, g.ax[0], nsync);
     // 2. per frequency: p = G (.), Lanczos step, lagged update, G u_{k+1}
     const size_t kb = (size_t)(g0 / T) * (size_t)(N * L);
     for (int f = threadIdx.x; f < N * T; f += nthr) {
@@ -1272,7 +1216,7 @@ __device__ __forceinline__ cpx<R> *x1_lanczos_tile(const Geometry &g, cpx<R> *bu
     }
     group_sync(nsync);
     // 3. inverse DFT along n1 of G u_{k+1}
-    return run_fft<R, 1, NF>(res, res == buf ? buf2 : buf, L, L, g.ax[0], nsync);
+    return Fft::template run<1>(res, res == buf ? buf2 : buf, L, g.ax[0], nsync);
 }
 
 // At most 384 threads per CTA (set_shapes enforces it): the fused pass keeps
@@ -1312,7 +1256,7 @@ __global__ void HOM_X1L_BOUNDS(R) k_x1_lanczos(Geometry g, cpx<R> *__restrict__ 
     }
     __syncthreads();
     Acc<R> acc;
-    cpx<R> *res = x1_lanczos_tile<R, NF, true>(g, buf, buf2, g0, c, uk + ko, um + ko, un + ko, wa + ko, wb + ko,
+    cpx<R> *res = x1_lanczos_tile<R, PassFft<R, NF>, true>(g, T, buf, buf2, g0, c, uk + ko, um + ko, un + ko, wa + ko, wb + ko,
                                                x + ko, acc, 0);
     if (live) {
         cpx<R> *dst = spec + (size_t)g0 * NC + lt;
@@ -1326,245 +1270,6 @@ __global__ void HOM_X1L_BOUNDS(R) k_x1_lanczos(Geometry g, cpx<R> *__restrict__ 
             givens_step(fold.st + cs, tot);
             fold.cnt[kNbMax + cs] = 0;
         }
-    }
-}
-
-// OR of a predicate over the n threads that use named barrier ID
-template <int ID>
-__device__ __forceinline__ bool group_or(bool v, int n) {
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.u32 q, %1, 0;\n\t"
-        "bar.red.or.pred p, %2, %3, q;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(r)
-        : "r"((uint32_t)v), "n"(ID), "r"(n)
-        : "memory");
-    return r != 0;
-}
-
-// The lagged update of step k-1 by the lagged-update warps (named barrier
-// 2) of the fused n1 pass, over the Krylov blocks of the CTA's tiles whose
-// case has one:
-//   w_{k-1} = (u_{k-1} / beta_{k-1} - delta w_{k-2} - eps w_{k-3}) / gamma
-// over the slot of w_{k-3}, and on every third step the deferred x update.
-// The blocks are cut into items of kX1LagChunk bytes; one thread brings an
-// item's operands (u_{k-1}, w_{k-2}, w_{k-3}, and x on an x step) into a
-// ring of S stages with untiled bulk copies, S items ahead, and the warps
-// update it from shared memory and store w_{k-1} (and x) to HBM.  The update is the same on every real number,
-// so it runs on 16-byte vectors.  Returns false after a bounded wait ran
-// out (the copies in flight have been waited for, bounded).
-template <typename R, typename LiveFrom>
-__device__ __forceinline__ bool x1_lagged(const Geometry &g, const LzCoef<R> *scoef, LiveFrom live_from, int ntiles,
-                                          int tpc, int per, unsigned char *ring, uint64_t *lbar,
-                                          const cpx<R> *__restrict__ um, const cpx<R> *__restrict__ wa,
-                                          cpx<R> *__restrict__ wb, cpx<R> *__restrict__ x) {
-    using V = typename std::conditional<sizeof(R) == 4, float4, double2>::type;
-    constexpr int NR = 16 / sizeof(R);
-    const int S = g.x1_lag_stages;
-    const int lt = threadIdx.x - kX1Group;
-    const long long pbytes = (long long)per * sizeof(cpx<R>);
-    auto next_tile = [&](int t) {
-        t = live_from(t);
-        while (t < ntiles && !scoef[t / tpc].lagged) t = live_from(t + gridDim.x);
-        return t;
-    };
-    auto base_of = [&](int t) {   // byte offset of tile t's block in each Krylov vector
-        return ((long long)(t / tpc) * g.kvec + (long long)(t % tpc) * per) * (long long)sizeof(cpx<R>);
-    };
-    int pt = next_tile(blockIdx.x), ct = pt;   // producer / consumer cursors (tile, byte offset)
-    long long po = 0, co = 0;
-    int issued = 0;                            // items issued (thread lt = 0)
-    auto issue = [&]() {
-        const int s = issued % S;
-        const uint32_t nb = (uint32_t)(pbytes - po < kX1LagChunk ? pbytes - po : kX1LagChunk);
-        const long long o = base_of(pt) + po;
-        unsigned char *st = ring + (size_t)s * 4 * kX1LagChunk;
-        const bool xs = scoef[pt / tpc].xstep;
-        mbar_expect_tx(&lbar[s], (xs ? 4 : 3) * nb);
-        bulk_load(st, reinterpret_cast<const char *>(um) + o, nb, &lbar[s]);
-        bulk_load(st + kX1LagChunk, reinterpret_cast<const char *>(wa) + o, nb, &lbar[s]);
-        bulk_load(st + 2 * kX1LagChunk, reinterpret_cast<const char *>(wb) + o, nb, &lbar[s]);
-        if (xs) bulk_load(st + 3 * kX1LagChunk, reinterpret_cast<const char *>(x) + o, nb, &lbar[s]);
-        ++issued;
-        po += kX1LagChunk;
-        if (po >= pbytes) {
-            po = 0;
-            pt = next_tile(pt + gridDim.x);
-        }
-    };
-    if (lt == 0)
-        for (int s = 0; s < S && pt < ntiles; ++s) issue();
-    int n = 0;
-    for (; ct < ntiles; ++n) {
-        const int s = n % S;
-        const bool got = mbar_wait_bounded(&lbar[s], (uint32_t)(n / S) & 1u);
-        if (group_or<2>(!got, kX1LagThreads)) {
-            if (lt == 0) {   // record, then wait (bounded) for the items in flight
-                atomicExch(g.err, 1);
-                for (int m = n; m < issued; ++m) mbar_wait_bounded(&lbar[m % S], (uint32_t)(m / S) & 1u);
-            }
-            return false;
-        }
-        const LzCoef<R> c = scoef[ct / tpc];
-        const int nv = (int)((pbytes - co < kX1LagChunk ? pbytes - co : kX1LagChunk) / 16);
-        const long long o = base_of(ct) + co;
-        const V *su = reinterpret_cast<const V *>(ring + (size_t)s * 4 * kX1LagChunk);
-        const V *sa = su + kX1LagChunk / 16, *sb = su + 2 * (kX1LagChunk / 16), *sx = su + 3 * (kX1LagChunk / 16);
-        V *gb = reinterpret_cast<V *>(reinterpret_cast<char *>(wb) + o);
-        V *gx = reinterpret_cast<V *>(reinterpret_cast<char *>(x) + o);
-        if (c.xstep) {
-            for (int j = lt; j < nv; j += kX1LagThreads) {
-                V vu = su[j], va = sa[j], vb = sb[j], vx = sx[j], vn;
-                const R *u = reinterpret_cast<const R *>(&vu);
-                const R *a = reinterpret_cast<const R *>(&va);
-                const R *b = reinterpret_cast<const R *>(&vb);
-                R *wn = reinterpret_cast<R *>(&vn);
-                R *xx = reinterpret_cast<R *>(&vx);
-#pragma unroll
-                for (int r = 0; r < NR; ++r) {
-                    wn[r] = (u[r] * c.ib - c.d * a[r] - c.e * b[r]) * c.ig;
-                    xx[r] += c.t2 * b[r] + c.t1 * a[r] + c.tau * wn[r];
-                }
-                gb[j] = vn;
-                gx[j] = vx;
-            }
-        } else {
-            for (int j = lt; j < nv; j += kX1LagThreads) {
-                V vu = su[j], va = sa[j], vb = sb[j];
-                const R *u = reinterpret_cast<const R *>(&vu);
-                const R *a = reinterpret_cast<const R *>(&va);
-                R *b = reinterpret_cast<R *>(&vb);
-#pragma unroll
-                for (int r = 0; r < NR; ++r) b[r] = (u[r] * c.ib - c.d * a[r] - c.e * b[r]) * c.ig;
-                gb[j] = vb;
-            }
-        }
-        co += kX1LagChunk;
-        if (co >= pbytes) {
-            co = 0;
-            ct = next_tile(ct + gridDim.x);
-        }
-        asm volatile("bar.sync 2, %0;" ::"n"(kX1LagThreads) : "memory");   // stage s is read
-        if (lt == 0 && pt < ntiles) issue();
-    }
-    return true;
-}
-
-// persistent TMA-staged form (FP32, register FFT lengths 64..512), warp-
-// specialised.  The first g.threads1 threads (the transform group, named
-// barrier 1) take the work tiles: each comes and goes by TMA, double-
-// buffered as in k_x1_tma, and the Lanczos step reads u_k and u_{k-1}
-// (bulk-prefetched into L2 at the tile's start) and writes u_{k+1} with
-// plain coalesced accesses.  The last kX1LagThreads threads (two warps) run
-// the lagged w update (and on one step in three the deferred x update) on
-// the same tiles' Krylov blocks, streaming u_{k-1}, w_{k-2}, w_{k-3} (and x)
-// while the transform group works in shared memory; the two groups share no
-// written data (u_{k+1} has its own buffer), so they never wait on each
-// other.  (Prefetching the next tile's blocks into L2 was measured to double
-// the DRAM reads: the lines were evicted before use; the current tile's are
-// used within microseconds.)  Tiles are numbered case-major over the stacked
-// batch; tiles of converged cases are skipped; each transform thread keeps
-// one running sum per case in shared memory, and the CTA writes one partial
-// per case (partials[case * gridDim + block]).
-template <typename R, int NF>
-__global__ void __launch_bounds__(kX1Group + kX1LagThreads, 2)
-    k_x1_lanczos_tma(Geometry g, const __grid_constant__ CUtensorMap tspec, const cpx<R> *__restrict__ uk,
-                     const cpx<R> *__restrict__ um, cpx<R> *__restrict__ un, const cpx<R> *__restrict__ wa,
-                     cpx<R> *__restrict__ wb, cpx<R> *__restrict__ x, const MinresState *state,
-                     double *__restrict__ partials, Fold fold) {
-    pdl_release();
-    pdl_wait();   // predecessor complete (programmatic launch in the MINRES graph)
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t bar[2];
-    __shared__ __align__(8) uint64_t lbar[kX1LagMaxStages];
-    __shared__ double sacc[kNbMax * kX1Group];
-    __shared__ LzCoef<R> scoef[kNbMax];   // each case's coefficients, converted once
-    constexpr int NC = 6;
-    const int N = g.n1, T = g.tile1, L = NC * T;
-    const int cols = g.n2 * g.h;
-    const int tpc = (cols + T - 1) / T;   // tiles per case
-    const int ntiles = tpc * g.nb;
-    const int per = N * L;
-    const uint32_t bytes = (uint32_t)(per * sizeof(cpx<R>));
-    cpx<R> *base = reinterpret_cast<cpx<R> *>(smem_raw);
-    const bool leader = threadIdx.x == 0;
-    const bool xform = threadIdx.x < kX1Group;
-    auto live_from = [&](int t) {
-        while (t < ntiles && skip_case(state, t / tpc)) t += gridDim.x;
-        return t;
-    };
-    if (xform)
-        for (int cc = 0; cc < g.nb; ++cc) sacc[cc * kX1Group + threadIdx.x] = 0.0;
-    if (threadIdx.x < g.nb) scoef[threadIdx.x] = lz_coef<R>(state + threadIdx.x);
-    if (leader) {
-        mbar_init(&bar[0], 1);
-        mbar_init(&bar[1], 1);
-        for (int q = 0; q < kX1LagMaxStages; ++q) mbar_init(&lbar[q], 1);
-        fence_mbar_init();
-    }
-    __syncthreads();
-    if (!xform) {
-        x1_lagged<R>(g, scoef, live_from, ntiles, tpc, per, smem_raw + g.smem1_tma, lbar, um, wa, wb, x);
-    } else {
-        int tile = live_from(blockIdx.x);
-        if (leader && tile < ntiles) {
-            mbar_expect_tx(&bar[0], bytes);
-            tma_load_rows_2d(base, &tspec, NC * T * (tile % tpc), N * (tile / tpc), N, L * (int)sizeof(cpx<R>),
-                             &bar[0]);
-        }
-        for (int i = 0; tile < ntiles; ++i) {
-            const int s = i & 1;
-            const int next = live_from(tile + gridDim.x);
-            if (leader && next < ntiles) {
-                bulk_wait_read_all();   // the store of the tile that used stage s^1 has read it
-                mbar_expect_tx(&bar[s ^ 1], bytes);
-                tma_load_rows_2d(base + (s ^ 1) * per, &tspec, NC * T * (next % tpc), N * (next / tpc), N,
-                                 L * (int)sizeof(cpx<R>), &bar[s ^ 1]);
-            }
-            const bool ok = mbar_wait_bounded(&bar[s], (i >> 1) & 1);
-            if (group_or<1>(!ok, kX1Group)) {
-                if (leader) {   // record, then wait (bounded) for this CTA's loads in flight
-                    atomicExch(g.err, 1);
-                    mbar_wait_bounded(&bar[s], (i >> 1) & 1);
-                    if (next < ntiles) mbar_wait_bounded(&bar[s ^ 1], ((i + 1) >> 1) & 1);
-                }
-                break;
-            }
-            const int cs = tile / tpc, tc = tile - cs * tpc;
-            const size_t ko = (size_t)cs * g.kvec;
-            if (leader && g.x1_l2pf) {   // this tile's u_k and u_{k-1} blocks into L2 for the Lanczos step
-                bulk_prefetch_l2(uk + ko + (size_t)tc * per, bytes);
-                bulk_prefetch_l2(um + ko + (size_t)tc * per, bytes);
-            }
-            const LzCoef<R> c = scoef[cs];
-            Acc<R> acc;
-            cpx<R> *buf = base + s * per;
-            cpx<R> *res = x1_lanczos_tile<R, NF, false>(g, buf, buf, tc * T, c, uk + ko, um + ko, un + ko, wa + ko,
-                                                        wb + ko, x + ko, acc, kX1Group);
-            sacc[cs * kX1Group + threadIdx.x] += acc.value();
-            fence_proxy_async_smem();
-            group_sync(kX1Group);
-            if (leader) {
-                tma_store_rows_2d(&tspec, NC * T * tc, N * cs, N, res, L * (int)sizeof(cpx<R>));
-                bulk_commit();
-            }
-            tile = next;
-        }
-        if (leader) bulk_wait_all();
-    }
-    __syncthreads();   // both groups done
-    for (int cc = 0; cc < g.nb; ++cc) {
-        const double sum = block_sum(xform ? sacc[cc * kX1Group + threadIdx.x] : 0.0);
-        if (threadIdx.x == 0) partials[cc * gridDim.x + blockIdx.x] = sum;
-    }
-    if (fold.cnt && last_of(fold.cnt + 2 * kNbMax, gridDim.x)) {   // Givens step of every case
-        for (int cc = 0; cc < g.nb; ++cc) {
-            const double tot = sum_partials(partials + (size_t)cc * gridDim.x, gridDim.x);
-            if (threadIdx.x == 0) givens_step(fold.st + cc, tot);
-        }
-        if (threadIdx.x == 0) fold.cnt[2 * kNbMax] = 0;
     }
 }
 
@@ -1826,12 +1531,9 @@ void Launch<R>::table_init(const Geometry &) {
     HOM_SET_ATTR(128) HOM_SET_ATTR(160) HOM_SET_ATTR(256) HOM_SET_ATTR(512)
     if constexpr (sizeof(R) == 4) {
 #define HOM_SET_TMA(NF)                   \
-    HOM_SET_ATTR1((k_x2_tma<R, -1, NF>))  \
-    HOM_SET_ATTR1((k_x2_tma<R, 1, NF>))   \
     HOM_SET_ATTR1((k_x1_tma<R, NF>))      \
     HOM_SET_ATTR1((k_x1_tma<R, NF, true>)) \
-    HOM_SET_ATTR1((k_x1_tma_expand<R, NF>)) \
-    HOM_SET_ATTR1((k_x1_lanczos_tma<R, NF>))
+    HOM_SET_ATTR1((k_x1_tma_expand<R, NF>))
         HOM_SET_TMA(64) HOM_SET_TMA(96) HOM_SET_TMA(128) HOM_SET_TMA(160) HOM_SET_TMA(256) HOM_SET_TMA(512)
 #undef HOM_SET_TMA
         HOM_SET_ATTR1((k_x3r<64>))
@@ -1842,75 +1544,71 @@ void Launch<R>::table_init(const Geometry &) {
 #undef HOM_SET_ATTR1
 }
 
-// persistent-grid sizes of the TMA passes: resident CTAs per SM x SMs
+// persistent-grid sizes of the TMA passes: resident CTAs per SM x SMs (a pass
+// that cannot run has its flag cleared: tma, x2t, grid1l_tma)
 template <typename R>
-int Launch<R>::tma_grids(Geometry &g) {
+void Launch<R>::tma_grids(Geometry &g) {
     if constexpr (sizeof(R) != 4) {
-        g.tma = 0;
-        return 0;
+        g.tma = g.x2t = g.grid1l_tma = 0;
     } else {
-        int dev = 0, sms = 0;
+        int dev = 0, sms = 0, optin = 0, smem_sm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        int b2 = 0, b1 = 0, b1d = 0;
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
         auto occ = [&](auto kern, int threads, size_t smem) {
             int nb = 0;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, threads, smem);
+            if (smem + 1024 <= (size_t)optin) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, threads, smem);
             return nb;
         };
-        switch (g.fast[1]) {
-            case 64: b2 = occ(k_x2_tma<R, -1, 64>, g.threads2, g.smem2_tma); break;
-            case 96: b2 = occ(k_x2_tma<R, -1, 96>, g.threads2, g.smem2_tma); break;
-            case 160: b2 = occ(k_x2_tma<R, -1, 160>, g.threads2, g.smem2_tma); break;
-            case 512: b2 = occ(k_x2_tma<R, -1, 512>, g.threads2, g.smem2_tma); break;
-            case 128: b2 = occ(k_x2_tma<R, -1, 128>, g.threads2, g.smem2_tma); break;
-            default: b2 = occ(k_x2_tma<R, -1, 256>, g.threads2, g.smem2_tma); break;
-        }
-        switch (g.fast[0]) {
-            case 64: b1 = occ(k_x1_tma<R, 64>, g.threads1, g.smem1_tma);
-                     b1d = occ(k_x1_tma<R, 64>, g.threads1, g.smem1d_tma); break;
-            case 96: b1 = occ(k_x1_tma<R, 96>, g.threads1, g.smem1_tma);
-                     b1d = occ(k_x1_tma<R, 96>, g.threads1, g.smem1d_tma); break;
-            case 160: b1 = occ(k_x1_tma<R, 160>, g.threads1, g.smem1_tma);
-                      b1d = occ(k_x1_tma<R, 160>, g.threads1, g.smem1d_tma); break;
-            case 512: b1 = occ(k_x1_tma<R, 512>, g.threads1, g.smem1_tma);
-                      b1d = occ(k_x1_tma<R, 512>, g.threads1, g.smem1d_tma); break;
-            case 128: b1 = occ(k_x1_tma<R, 128>, g.threads1, g.smem1_tma);
-                      b1d = occ(k_x1_tma<R, 128>, g.threads1, g.smem1d_tma); break;
-            default: b1 = occ(k_x1_tma<R, 256>, g.threads1, g.smem1_tma);
-                     b1d = occ(k_x1_tma<R, 256>, g.threads1, g.smem1d_tma); break;
-        }
-        if (b2 < 1 || b1 < 1 || b1d < 1) {
-            g.tma = 0;
-            return 0;
-        }
-        // the fused MINRES n1 pass: a transform group of exactly kX1Group
-        // threads plus the lagged-update warps, whose ring takes as many
-        // stages (up to kX1LagMaxStages) as leave room for two CTAs per SM
-        int b1l = 0;
-        if (g.nc == 6 && g.threads1 == kX1Group) {
-            const int t = kX1Group + kX1LagThreads;
-            int smem_sm = 0;
-            cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-            const size_t ring = 4 * (size_t)kX1LagChunk, fixed = 15 * 1024;   // static + reserved per CTA
-            int st = kX1LagMaxStages;
-            while (st > 1 && 2 * (g.smem1_tma + st * ring + fixed) > (size_t)smem_sm) --st;
-            g.x1_lag_stages = st;
-            g.smem1l_tma = g.smem1_tma + st * ring;
+        if (g.tma) {
+            int b1 = 0, b1d = 0;
+#define HOM_OCC1(NF)                                            \
+    b1 = occ(k_x1_tma<R, NF>, g.threads1, g.smem1_tma);         \
+    b1d = occ(k_x1_tma<R, NF>, g.threads1, g.smem1d_tma);
             switch (g.fast[0]) {
-                case 64: b1l = occ(k_x1_lanczos_tma<R, 64>, t, g.smem1l_tma); break;
-                case 96: b1l = occ(k_x1_lanczos_tma<R, 96>, t, g.smem1l_tma); break;
-                case 160: b1l = occ(k_x1_lanczos_tma<R, 160>, t, g.smem1l_tma); break;
-                case 512: b1l = occ(k_x1_lanczos_tma<R, 512>, t, g.smem1l_tma); break;
-                case 128: b1l = occ(k_x1_lanczos_tma<R, 128>, t, g.smem1l_tma); break;
-                default: b1l = occ(k_x1_lanczos_tma<R, 256>, t, g.smem1l_tma); break;
+                case 64: HOM_OCC1(64) break;
+                case 96: HOM_OCC1(96) break;
+                case 128: HOM_OCC1(128) break;
+                case 160: HOM_OCC1(160) break;
+                case 256: HOM_OCC1(256) break;
+                default: HOM_OCC1(512) break;
             }
+#undef HOM_OCC1
+            g.grid1_tma = b1 * sms;
+            g.grid1d_tma = b1d * sms;
+            if (b1 < 1 || b1d < 1) g.tma = 0;
         }
-        g.grid1l_tma = b1l * sms;
-        g.grid2_tma = b2 * sms;
-        g.grid1_tma = b1 * sms;
-        g.grid1d_tma = b1d * sms;
-        return 1;
+        if (g.x2t) {
+            const X2LineFn f = x2_line_kernel(g.n2, 0), fi = x2_line_kernel(g.n2, 1);
+            int b = 0;
+            if (f && fi) {
+                line_kernel_attr((const void *)f, optin);
+                line_kernel_attr((const void *)fi, optin);
+                b = occ(f, g.threads2t, g.smem2_tma);
+            }
+            g.grid2_tma = b * sms;
+            if (b < 1) g.x2t = 0;
+        }
+        // the fused MINRES n1 pass: the transform group plus the lagged-update
+        // warps, whose ring takes as many stages (up to kX1LagMaxStages) as
+        // leave room for two CTAs per SM
+        if (g.grp1l) {
+            const X1lLineFn f = x1l_line_kernel(g.n1);
+            const int t = g.grp1l + kX1LagThreads;
+            const size_t tiles = 2 * g.stage1l, ring = 4 * (size_t)kX1LagChunk, fixed = 15 * 1024;   // static + reserved per CTA
+            int st = kX1LagMaxStages;
+            while (st > 1 && 2 * (tiles + st * ring + fixed) > (size_t)smem_sm) --st;
+            g.x1_lag_stages = st;
+            g.smem1l_tma = tiles + st * ring;
+            int b = 0;
+            if (f) {
+                line_kernel_attr((const void *)f, optin);
+                b = occ(f, t, g.smem1l_tma);
+            }
+            g.grid1l_tma = b * sms;
+            if (b < 1) g.grp1l = 0;
+        }
     }
 }
 
@@ -1955,21 +1653,13 @@ void Launch<R>::x3(const Geometry &g, cudaStream_t st, int in_mode, const void *
 template <typename R>
 void Launch<R>::x2(const Geometry &g, cudaStream_t st, int inverse, cpx<R> *spec, const MinresState *state) {
     if constexpr (sizeof(R) == 4) {
-        if (g.tma) {
+        if (g.x2t) {
             const CUtensorMap *tm = tma_map(g, spec, TMA_X2, 1);
             const int qtiles = (g.nc * g.h + g.tile2 - 1) / g.tile2;
-#define HOM_X2T(NF)                                                                                         \
-    if (inverse) launch_k(g.pdl, k_x2_tma<R, 1, NF>, g.grid2_tma, g.threads2, g.smem2_tma, st, g, *tm, qtiles, state); \
-    else launch_k(g.pdl, k_x2_tma<R, -1, NF>, g.grid2_tma, g.threads2, g.smem2_tma, st, g, *tm, qtiles, state)
-            switch (g.fast[1]) {
-                case 64: HOM_X2T(64); break;
-                case 96: HOM_X2T(96); break;
-                case 160: HOM_X2T(160); break;
-                case 512: HOM_X2T(512); break;
-                case 128: HOM_X2T(128); break;
-                default: HOM_X2T(256); break;
-            }
-#undef HOM_X2T
+            const long long tiles = (long long)g.n1 * g.nb * qtiles;
+            const int grid = tiles < g.grid2_tma ? (int)tiles : g.grid2_tma;
+            launch_k(g.pdl, x2_line_kernel(g.n2, inverse), grid, g.threads2t, g.smem2_tma, st, g, *tm, qtiles,
+                     state);
             return;
         }
     }
@@ -2062,7 +1752,11 @@ bool Launch<R>::x1_modb_expand(const Geometry &g, cudaStream_t st, double alpha,
 // partials per load case written by the fused n1 pass (case c's at c * count)
 template <typename R>
 int Launch<R>::x1_lanczos_grid(const Geometry &g) {
-    return (g.tma && g.grid1l_tma > 0) ? g.grid1l_tma : (g.n2 * g.h + g.tile1 - 1) / g.tile1;
+    if (g.grid1l_tma > 0) {   // no more CTAs than tiles
+        const long long tiles = (long long)((g.n2 * g.h + g.tile1l - 1) / g.tile1l) * g.nb;
+        return tiles < g.grid1l_tma ? (int)tiles : g.grid1l_tma;
+    }
+    return (g.n2 * g.h + g.tile1 - 1) / g.tile1;
 }
 
 template <typename R>
@@ -2070,20 +1764,10 @@ void Launch<R>::x1_lanczos(const Geometry &g, cudaStream_t st, cpx<R> *spec, con
                            cpx<R> *un, const cpx<R> *wa, cpx<R> *wb, cpx<R> *x, const MinresState *state,
                            double *partials, Fold fold) {
     if constexpr (sizeof(R) == 4) {
-        if (g.tma && g.grid1l_tma > 0) {
-            const CUtensorMap *ts = tma_map(g, spec, TMA_X1, 1);
-#define HOM_X1LT(NF)                                                                                         \
-    launch_k(g.pdl, k_x1_lanczos_tma<R, NF>, g.grid1l_tma, kX1Group + kX1LagThreads, g.smem1l_tma, st, g, *ts, uk, um, \
-             un, wa, wb, x, state, partials, fold)
-            switch (g.fast[0]) {
-                case 64: HOM_X1LT(64); break;
-                case 96: HOM_X1LT(96); break;
-                case 160: HOM_X1LT(160); break;
-                case 512: HOM_X1LT(512); break;
-                case 128: HOM_X1LT(128); break;
-                default: HOM_X1LT(256); break;
-            }
-#undef HOM_X1LT
+        if (g.grid1l_tma > 0) {
+            const CUtensorMap *ts = tma_map(g, spec, TMA_X1L, 1);
+            launch_k(g.pdl, x1l_line_kernel(g.n1), x1_lanczos_grid(g), g.grp1l + kX1LagThreads, g.smem1l_tma, st, g, *ts, uk,
+                     um, un, wa, wb, x, state, partials, fold);
             return;
         }
     }
@@ -2098,13 +1782,13 @@ void Launch<R>::x1_lanczos(const Geometry &g, cudaStream_t st, cpx<R> *spec, con
 template <typename R>
 void Launch<R>::to_tiles(const Geometry &g, cudaStream_t st, const cpx<R> *in, cpx<R> *out) {
     const long long n = 6 * g.S;
-    k_tiles<R><<<ew_grid(n), kEwThreads, 0, st>>>(n, g.n1, g.n2 * g.h, g.tile1, 1, in, out);
+    k_tiles<R><<<ew_grid(n), kEwThreads, 0, st>>>(n, g.n1, g.n2 * g.h, g.tile1l, 1, in, out);
 }
 
 template <typename R>
 void Launch<R>::from_tiles(const Geometry &g, cudaStream_t st, const cpx<R> *in, cpx<R> *out) {
     const long long n = 6 * g.S;
-    k_tiles<R><<<ew_grid(n), kEwThreads, 0, st>>>(n, g.n1, g.n2 * g.h, g.tile1, 0, in, out);
+    k_tiles<R><<<ew_grid(n), kEwThreads, 0, st>>>(n, g.n1, g.n2 * g.h, g.tile1l, 0, in, out);
 }
 
 template <typename R>

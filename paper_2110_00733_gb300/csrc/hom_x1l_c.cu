@@ -1,0 +1,13 @@
+// Fused MINRES n1 pass (FP32), line lengths of list C.
+#include "hom_lines.cuh"
+
+namespace hom {
+X1lLineFn x1l_line_kernel_c(int n) {
+    switch (n) {
+#define HOM_CASE(N) case N: return k_x1_lanczos_tma<float, N>;
+        HOM_LINE_LENGTHS_C(HOM_CASE)
+#undef HOM_CASE
+        default: return nullptr;
+    }
+}
+}  // namespace hom
