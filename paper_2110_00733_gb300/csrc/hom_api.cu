@@ -309,8 +309,11 @@ static int set_shapes(hom_ctx *ctx, Geometry &g, int nc) {
         return fail(ctx, HOM_EINVAL, "launch shape needs more than 384 threads per CTA in the fused n1 pass");
     g.x3r = (sizeof(R) == 4 && nc == 6 && x3r_length(g.n3) && ctx->shape[0] == 0 &&
              x3r_smem(g.n3) + 1024 <= (size_t)dev_smem && (g.n1 * g.n2) % x3r_rows_per_warp(g.n3) == 0) ? 1 : 0;
-    g.grid3r = g.x3r ? Launch<R>::x3r_grid(g) : 0;
-    if (g.grid3r <= 0) g.x3r = 0;
+    // else the persistent n3 pass at its lengths; k_x3 for the rest, FP64,
+    // MoDBFFT and an explicit rows3
+    g.x3l = sizeof(R) == 4 && nc == 6 && ctx->shape[0] == 0 && !g.x3r && x3_line_kernel(g.n3).fn;
+    g.grid3r = g.x3r || g.x3l ? Launch<R>::x3r_grid(g) : 0;
+    if (g.grid3r <= 0) g.x3r = g.x3l = 0;
     // persistent TMA-staged passes (FP32): the unfused n1 pass at the register
     // engine's n1 in [64, 512], the n2 pass and the fused MINRES n1 pass at
     // every length of the line engine
@@ -1435,7 +1438,7 @@ static void capture_bbody(hom_ctx *ctx, Engine<R> &E) {
     // voxel-iterations/s either way at 256^3)
     const Fold fold{ctx->bcnt, ctx->d_bst, (double)ctx->V};
     const char *fa = std::getenv("HOM_FOLD_ALPHA");
-    const bool fold_alpha = g.x3r && fa && std::atoi(fa) == 1;
+    const bool fold_alpha = (g.x3r || g.x3l) && fa && std::atoi(fa) == 1;
     const Fold fold3 = fold_alpha ? Fold{ctx->bcnt, ctx->d_bst, (double)ctx->V} : Fold{nullptr, nullptr, 0.0};
     const int np3 = Launch<R>::x3_epart_grid(g);
     cudaStream_t s = ctx->stream;

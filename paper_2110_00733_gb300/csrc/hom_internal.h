@@ -153,9 +153,10 @@ struct Geometry {
     // n1-tile order (tiles of tile1l (k2,k3) columns, each tile a contiguous
     // n1 x 6 tile1l block laid out as the pass's shared-memory tile)
     long long kvec;
-    // register-resident n3 pass (k_x3r: FP32, n3 in {64, 128, 256}) for
+    // register-resident n3 pass (k_x3r: FP32, n3 = 256) for
     // spectrum-to-spectrum applications
     int x3r;
+    int x3l = 0;            // the persistent n3 pass of X3Plan instead (see x3_line_kernel)
     int grid2_tma, grid1_tma, grid1d_tma;
     int grid1l_tma = 0;     // persistent grid of the fused MINRES n1 pass (0: plain-load form)
     size_t smem2_tma, smem1_tma, smem1d_tma;
@@ -176,25 +177,18 @@ struct Geometry {
     int *err;
 };
 
-// register-resident n3 pass (k_x3r): supported lengths, rows per 128-thread
-// CTA, and its shared memory (per row, the transpose slab of 3 lines x Q x
-// (P + 1) complex values, N = P Q)
-__host__ __device__ constexpr bool x3r_length(int n) { return n == 64 || n == 128 || n == 256; }
-// register n3 pass: rows per warp (32 / lanes per row), and per warp the
-// prefetch buffer of a row group (its rows' half spectra, then phi) and one
-// transpose slab per row; four warps per CTA
-__host__ __device__ constexpr int x3r_row_lanes(int n) { return n == 256 ? 16 : 8; }
+// register-resident n3 pass (k_x3r, n3 = 256: the length at which it is faster
+// than the persistent pass of X3Plan): lanes of a row, rows per warp (32 /
+// lanes), and per warp the prefetch buffer of a row group (its rows' half
+// spectra, then phi) and one transpose slab (Q x (P + 1) complex values,
+// N = P Q) per row; four warps per CTA
+__host__ __device__ constexpr bool x3r_length(int n) { return n == 256; }
+__host__ __device__ constexpr int x3r_row_lanes(int) { return 16; }
 __host__ __device__ constexpr int x3r_rows_per_warp(int n) { return 32 / x3r_row_lanes(n); }
 __host__ __device__ constexpr size_t x3r_in_bytes(int n) {
     return (size_t)x3r_rows_per_warp(n) * (n / 2 + 1) * 6 * sizeof(float2);
 }
-// phi is prefetched with the rows except at n = 128, where its 2 KB per
-// warp would leave room for two CTAs per SM instead of three (it is read
-// from L2 there)
-__host__ __device__ constexpr bool x3r_phi_prefetch(int n) { return n != 128; }
-__host__ __device__ constexpr size_t x3r_phi_bytes(int n) {
-    return x3r_phi_prefetch(n) ? (size_t)x3r_rows_per_warp(n) * n * sizeof(float) : 0;
-}
+__host__ __device__ constexpr size_t x3r_phi_bytes(int n) { return (size_t)x3r_rows_per_warp(n) * n * sizeof(float); }
 __host__ __device__ constexpr size_t x3r_slab_elems(int n) {
     return (size_t)(n / x3r_row_lanes(n)) * (x3r_row_lanes(n) + 1);
 }
@@ -276,6 +270,15 @@ using X1lLineFn = void (*)(Geometry, CUtensorMap, const float2 *, const float2 *
                            float2 *, const MinresState *, double *, Fold);
 X2LineFn x2_line_kernel(int n, int inverse);
 X1lLineFn x1l_line_kernel(int n);
+// persistent n3 pass of a length, with its threads, rows per tile and shared
+// memory (fn null: none)
+struct X3Line {
+    void (*fn)(Geometry, const float2 *, float2 *, int, float, float, const float *, const MinresState *, double *,
+               Fold) = nullptr;
+    int threads = 0, rows = 0;
+    size_t smem = 0;
+};
+X3Line x3_line_kernel(int n);
 // shared-memory limit and carve-out of one of them
 void line_kernel_attr(const void *kernel, int optin);
 // rows of a TMA box for tiles of n rows of rowb bytes: the most that divide n,

@@ -11,6 +11,13 @@ X1lLineFn x1l_line_kernel(int n) {
     return f ? f : x1l_line_kernel_c(n);
 }
 
+X3Line x3_line_kernel_a(int n), x3_line_kernel_b(int n), x3_line_kernel_c(int n);
+X3Line x3_line_kernel(int n) {
+    X3Line f = x3_line_kernel_a(n);
+    if (!f.fn) f = x3_line_kernel_b(n);
+    return f.fn ? f : x3_line_kernel_c(n);
+}
+
 X2LineFn x2_line_kernel_a(int n, int inverse), x2_line_kernel_b(int n, int inverse), x2_line_kernel_c(int n, int inverse);
 X2LineFn x2_line_kernel(int n, int inverse) {
     X2LineFn f = x2_line_kernel_a(n, inverse);

@@ -440,7 +440,7 @@ __global__ void HOM_PASS_BOUNDS_N3(R, NF) k_x3(Geometry g, int in_mode, const vo
 }
 
 // ---------------------------------------------------------------------------
-// Register-resident n3 pass (FP32, n3 in {64, 128, 256}, 6-component spectra,
+// Register-resident n3 pass (FP32, n3 = 256, 6-component spectra,
 // spectrum in and out): the C2R of a row, the material law with the strain-
 // energy sums, and the R2C, with the row's data in registers.
 //
@@ -463,9 +463,7 @@ __global__ void HOM_PASS_BOUNDS_N3(R, NF) k_x3(Geometry g, int in_mode, const vo
 // synchronisation is used until the final energy reduction.
 // ---------------------------------------------------------------------------
 template <int N> struct X3RPlan;
-template <> struct X3RPlan<64>  { static constexpr int P = 8,  Q = 8,  ROWS = 16; };
-template <> struct X3RPlan<128> { static constexpr int P = 8,  Q = 16, ROWS = 16; };
-template <> struct X3RPlan<256> { static constexpr int P = 16, Q = 16, ROWS = 8; };
+template <> struct X3RPlan<256> { static constexpr int P = 16, Q = 16; };
 
 
 template <int P>
@@ -506,7 +504,7 @@ __device__ __forceinline__ float2 tw_load(const float2 *p) {
 }
 
 template <int N>
-__global__ void __launch_bounds__(kX3rWarps * 32, N == 64 ? 5 : 3)
+__global__ void __launch_bounds__(kX3rWarps * 32, 3)
     k_x3r(Geometry g, const float2 *__restrict__ in, float2 *__restrict__ out, int material, float lam, float mu2,
           const float *__restrict__ phi, const MinresState *state, double *__restrict__ epart, Fold fold) {
     pdl_release();
@@ -547,7 +545,7 @@ __global__ void __launch_bounds__(kX3rWarps * 32, N == 64 ? 5 : 3)
         constexpr int nin = (int)(x3r_in_bytes(N) / 16);
 #pragma unroll 1
         for (int i = lane; i < nin; i += 32) cp_async16(reinterpret_cast<char *>(inb) + 16 * i, src + 16 * i);
-        if (material && x3r_phi_prefetch(N)) {
+        if (material) {
             const char *ps = reinterpret_cast<const char *>(phi + (size_t)rowc * N);
             constexpr int nph = (int)(x3r_phi_bytes(N) / 16);
 #pragma unroll 1
@@ -617,11 +615,10 @@ __global__ void __launch_bounds__(kX3rWarps * 32, N == 64 ? 5 : 3)
         // ---- material law on voxels j + P m (scaled by 1/V), strain energy
         float en = 0.f;
         if (material) {
-            const float *ph_row = x3r_phi_prefetch(N) ? phb + rw * N
-                                                      : phi + ((size_t)(q - cs * gpc) * RW + rw) * N;
+            const float *ph_row = phb + rw * N;
 #pragma unroll
             for (int m = 0; m < Q; ++m) {
-                const float ph = x3r_phi_prefetch(N) ? ph_row[j + P * m] : __ldg(&ph_row[j + P * m]);
+                const float ph = ph_row[j + P * m];
                 float t[6];
 #pragma unroll
                 for (int p = 0; p < 3; ++p) {
@@ -1458,6 +1455,10 @@ int Launch<R>::x3_grid(const Geometry &g) { return (g.n1 * g.n2 + g.rows3 - 1) /
 // (spectrum in and out): case c's are at [c * count, (c + 1) * count)
 template <typename R>
 int Launch<R>::x3_epart_grid(const Geometry &g) {
+    if (sizeof(R) == 4 && g.x3l) {   // no more CTAs than tiles of rows
+        const int rows = x3_line_kernel(g.n3).rows, tiles = (g.n1 * g.n2 + rows - 1) / rows * g.nb;
+        return tiles < g.grid3r ? tiles : g.grid3r;
+    }
     if (sizeof(R) == 4 && g.x3r) return g.grid3r;
     return x3_grid(g);
 }
@@ -1469,13 +1470,18 @@ int Launch<R>::x3r_grid(const Geometry &g) {
         int dev = 0, sms = 0, nb = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const size_t sm = x3r_smem(g.n3);
-        switch (g.n3) {
-            case 64: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_x3r<64>, kX3rWarps * 32, sm); break;
-            case 128: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_x3r<128>, kX3rWarps * 32, sm); break;
-            case 256: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_x3r<256>, kX3rWarps * 32, sm); break;
-            default: return 0;
+        if (g.x3l) {
+            const X3Line k = x3_line_kernel(g.n3);
+            int optin = 0;
+            cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+            if (!k.fn || k.smem + 1024 > (size_t)optin) return 0;
+            line_kernel_attr((const void *)k.fn, optin);
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k.fn, k.threads, k.smem);
+            return nb * sms;
         }
+        const size_t sm = x3r_smem(g.n3);
+        if (g.n3 != 256) return 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_x3r<256>, kX3rWarps * 32, sm);
         return nb * sms;
     }
 }
@@ -1536,8 +1542,6 @@ void Launch<R>::table_init(const Geometry &) {
     HOM_SET_ATTR1((k_x1_tma_expand<R, NF>))
         HOM_SET_TMA(64) HOM_SET_TMA(96) HOM_SET_TMA(128) HOM_SET_TMA(160) HOM_SET_TMA(256) HOM_SET_TMA(512)
 #undef HOM_SET_TMA
-        HOM_SET_ATTR1((k_x3r<64>))
-        HOM_SET_ATTR1((k_x3r<128>))
         HOM_SET_ATTR1((k_x3r<256>))
     }
 #undef HOM_SET_ATTR
@@ -1617,6 +1621,14 @@ void Launch<R>::x3(const Geometry &g, cudaStream_t st, int in_mode, const void *
                    const double *macro, double scl, int out_mode, void *out, const R *phi,
                    const MinresState *state, double *epart, Fold fold, double *tsum) {
     if constexpr (sizeof(R) == 4) {
+        if (!tsum && g.x3l && g.nc == 6 && in_mode == X3_IN_SPEC && out_mode == X3_OUT_SPEC && scl == 1.0 &&
+            (mid == X3_MID_MATERIAL || mid == X3_MID_NONE)) {
+            const X3Line k = x3_line_kernel(g.n3);
+            launch_k(g.pdl, k.fn, x3_epart_grid(g), k.threads, k.smem, st, g, reinterpret_cast<const float2 *>(in),
+                     reinterpret_cast<float2 *>(out), mid == X3_MID_MATERIAL ? 1 : 0, (float)lam, (float)(2.0 * mu),
+                     (const float *)phi, state, epart, fold);
+            return;
+        }
         if (!tsum && g.x3r && g.nc == 6 && in_mode == X3_IN_SPEC && out_mode == X3_OUT_SPEC && scl == 1.0 &&
             (mid == X3_MID_MATERIAL || mid == X3_MID_NONE)) {
             const int grid = g.grid3r;   // persistent: every case's row groups
@@ -1624,14 +1636,8 @@ void Launch<R>::x3(const Geometry &g, cudaStream_t st, int in_mode, const void *
             const int mat = mid == X3_MID_MATERIAL;
             const float2 *fi = reinterpret_cast<const float2 *>(in);
             float2 *fo = reinterpret_cast<float2 *>(out);
-            switch (g.n3) {
-                case 64: launch_k(g.pdl, k_x3r<64>, grid, 128, sm, st, g, fi, fo, mat, (float)lam, (float)(2.0 * mu),
-                                                          (const float *)phi, state, epart, fold); break;
-                case 128: launch_k(g.pdl, k_x3r<128>, grid, 128, sm, st, g, fi, fo, mat, (float)lam, (float)(2.0 * mu),
-                                                            (const float *)phi, state, epart, fold); break;
-                default: launch_k(g.pdl, k_x3r<256>, grid, 128, sm, st, g, fi, fo, mat, (float)lam, (float)(2.0 * mu),
-                                                            (const float *)phi, state, epart, fold); break;
-            }
+            launch_k(g.pdl, k_x3r<256>, grid, 128, sm, st, g, fi, fo, mat, (float)lam, (float)(2.0 * mu),
+                     (const float *)phi, state, epart, fold);
             return;
         }
     }

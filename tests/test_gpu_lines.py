@@ -53,3 +53,24 @@ def test_fused_n1_pass_matches_plain_loads(hom, n):
             got.append([hom.hom_fields(ctx, k, want=("stress",))[1] for k in range(2)])
     for a, b in zip(*got):
         assert np.linalg.norm(a - b) <= 5e-6 * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("n", LENGTHS)
+def test_n3_pass_matches_the_shared_memory_pass(hom, n):
+    """The persistent n3 pass (law and strain energy) against the pass that an
+    explicit rows3 selects: the operator, and a solve, whose alpha is the
+    pass's energy.  45 rows: ragged last tile."""
+    g = (5, 9, n)
+    phi = ri.random_phi(g, 13)
+    E = np.array([[1e-3, 2e-4, -3e-4, 1e-4, 3e-4, -2e-4], [0, 0, 1e-3, 0, 0, 5e-4]])
+    spec = np.fft.rfftn(ri.random_field(g, 5), axes=(1, 2, 3))
+    spec = np.ascontiguousarray(np.moveaxis(spec, 0, -1)).astype(np.complex64)
+    got = []
+    for rows in (0, 2):
+        with hom.hom_create(g, phi, hom.HOM_INPUT_FRACTION_F64, shape=(rows, 0, 0)) as ctx:
+            out = [hom.hom_apply_spectrum(ctx, spec)]
+            rc, info = hom.hom_solve(ctx, E, tol=1e-12, max_it=7)
+            assert rc == hom.HOM_NOT_CONVERGED and [i["iterations"] for i in info] == [7, 7]
+            got.append(out + [hom.hom_fields(ctx, k, want=("stress",))[1] for k in range(2)])
+    for a, b in zip(*got):
+        assert np.linalg.norm(a - b) <= 5e-6 * np.linalg.norm(b)
