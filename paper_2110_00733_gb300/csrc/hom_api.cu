@@ -162,7 +162,7 @@ struct hom_ctx {
     void *brhs = nullptr;                        // bcap x 6S: right-hand sides, then iterates
     double2 *bb64 = nullptr, *br64 = nullptr;    // bcap x 6S
     MinresState *d_bst = nullptr, *h_bst = nullptr;
-    double *bpart = nullptr;
+    double *bpart = nullptr, *bdsum = nullptr;   // per-CTA partial sums; the stress sums of stress-controlled solves
     int *bcnt = nullptr;                         // kFoldCounters counters of the folded scalar steps
     cudaGraphExec_t bgraph = nullptr;
     int bgraph_nb = 0;
@@ -349,23 +349,20 @@ static int set_shapes(hom_ctx *ctx, Geometry &g, int nc) {
             const char *e = getenv("HOM_X1_L2PF");
             g.x1_l2pf = e ? atoi(e) : 1;
         }
-        // tiles of as many columns as the transform group has threads for
-        const int tpl = line_tpl(g.n1);
-        if (nc == 6 && tpl > 0) {
-            int t = ctx->shape[2] > 0 ? ctx->shape[2] : std::max(1, std::min(16, kX1Group / (6 * tpl)));
-            while (ctx->shape[2] == 0 && t > 1 && !tma_box_rows(g.n1, 6 * t * (int)cs)) --t;
-            g.box1l = tma_box_rows(g.n1, 6 * t * (int)cs);
-            if (6 * t * tpl <= kX1Group && g.box1l > 0) {
-                g.tile1l = t;
-                g.grp1l = round32(6 * t * tpl);
-                g.stage1l = (6ull * t * g.n1 * cs + 127) / 128 * 128;
-            }
+        // the fused pass's tile width is the plan's; an explicit tile1 other
+        // than it selects the plain-load form
+        const int tpl = line_tpl(g.n1), t = tpl > 0 && nc == 6 ? x1l_cols(g.n1, tpl) : 0;
+        if (t > 0 && (ctx->shape[2] == 0 || ctx->shape[2] == t)) {
+            g.box1l = tma_box_rows(g.n1, 48 * t);
+            g.tile1l = t;
+            g.grp1l = x1l_group(g.n1, tpl);
+            g.stage1l = (6ull * t * g.n1 * cs + 127) / 128 * 128;
         }
         Launch<R>::tma_grids(g);
         if (!g.grp1l) g.tile1l = t1;
         if (g.tma || g.x2t || g.grp1l) g.tma_cache = tma_cache_new();
     }
-    g.kvec = (long long)((g.n2 * g.h + g.tile1l - 1) / g.tile1l) * g.n1 * nc * g.tile1l;
+    g.kvec = (long long)((g.n2 * g.h + g.tile1l - 1) / g.tile1l) * krylov_tile(g.n1, g.tile1l);
     return HOM_OK;
 }
 
@@ -1351,13 +1348,14 @@ static void batch_free(hom_ctx *ctx) {
     cudaFree(ctx->br64);
     cudaFree(ctx->d_bst);
     cudaFree(ctx->bpart);
+    cudaFree(ctx->bdsum);
     cudaFree(ctx->bcnt);
     ctx->bcnt = nullptr;
     if (ctx->h_bst) cudaFreeHost(ctx->h_bst);
     ctx->bspec = ctx->bv[0] = ctx->bv[1] = ctx->bv[2] = ctx->bw[0] = ctx->bw[1] = ctx->bx = ctx->brhs = nullptr;
     ctx->bb64 = ctx->br64 = nullptr;
     ctx->d_bst = ctx->h_bst = nullptr;
-    ctx->bpart = nullptr;
+    ctx->bpart = ctx->bdsum = nullptr;
     ctx->bcap = 0;
     ctx->bg.nb = 0;
 }
@@ -1399,6 +1397,7 @@ static int batch_reserve(hom_ctx *ctx, int nb) {
         np = std::max(np, (long long)Launch<float>::x1_lanczos_grid(gb));
     }
     CU(cudaMalloc(&ctx->bpart, sizeof(double) * np * nb));
+    CU(cudaMalloc(&ctx->bdsum, sizeof(double) * 6 * np * nb));
     CU(cudaMalloc(&ctx->bcnt, sizeof(int) * kFoldCounters));
     CU(cudaMemset(ctx->bcnt, 0, sizeof(int) * kFoldCounters));
     ctx->bcap = nb;
@@ -1438,7 +1437,8 @@ static void capture_bbody(hom_ctx *ctx, Engine<R> &E) {
     // voxel-iterations/s either way at 256^3)
     const Fold fold{ctx->bcnt, ctx->d_bst, (double)ctx->V};
     const char *fa = std::getenv("HOM_FOLD_ALPHA");
-    const bool fold_alpha = (g.x3r || g.x3l) && fa && std::atoi(fa) == 1;
+    const bool dc = sizeof(R) == 4 && g.mask0 != 0;   // xi = 0 in FP64, see MinresState
+    const bool fold_alpha = !dc && (g.x3r || g.x3l) && fa && std::atoi(fa) == 1;
     const Fold fold3 = fold_alpha ? Fold{ctx->bcnt, ctx->d_bst, (double)ctx->V} : Fold{nullptr, nullptr, 0.0};
     const int np3 = Launch<R>::x3_epart_grid(g);
     cudaStream_t s = ctx->stream;
@@ -1451,8 +1451,9 @@ static void capture_bbody(hom_ctx *ctx, Engine<R> &E) {
         cpx<R> *wa = odd ? wd : wc, *wb = odd ? wc : wd;
         Launch<R>::x2(g, s, 1, spec, ctx->d_bst);
         Launch<R>::x3(g, s, X3_IN_SPEC, spec, X3_MID_MATERIAL, ctx->lam, ctx->mu, nullptr, 1.0, X3_OUT_SPEC, spec,
-                      E.phi, ctx->d_bst, ctx->bpart, fold3);
-        if (!fold3.cnt) scalar_alpha(s, ctx->d_bst, ctx->bpart, np3, (double)ctx->V, g.nb, g.pdl);
+                      E.phi, ctx->d_bst, ctx->bpart, fold3, dc ? ctx->bdsum : nullptr);
+        if (!fold3.cnt)
+            scalar_alpha(s, ctx->d_bst, ctx->bpart, np3, (double)ctx->V, g.nb, g.pdl, dc ? ctx->bdsum : nullptr);
         Launch<R>::x2(g, s, 0, spec, ctx->d_bst);
         Launch<R>::x1_lanczos(g, s, spec, uk, um, un, wa, wb, x, ctx->d_bst, ctx->bpart, fold);
         ctx->launches += fold3.cnt ? 4 : 5;
@@ -1534,8 +1535,8 @@ static int build_bgraph(hom_ctx *ctx, Engine<R> &E, int nb) {
 // (standard order, solve precision); case j runs with tolerance tol[j] and
 // at most maxit[j] iterations (0: the case sits this sweep out).  In three
 // parts so that several cells can share one graph launch:
-//   batch_begin  per-case norms and FP64 states, Krylov vectors in tile
-//                order, the first inverse n1 transform; *any = some case runs
+//   batch_begin  Krylov vectors, per-case norms and FP64 states, the first
+//                inverse n1 transform; *any = some case runs
 //   (the stacked graph, see build_bgraph / hom_solve_batch)
 //   batch_end    the last lagged update, the iterates back in the standard
 //                order over ctx->brhs (zero for cases that did not run), and
@@ -1545,34 +1546,34 @@ static int batch_begin(hom_ctx *ctx, Engine<R> &E, int nb, const double *tol, co
                        bool *any) {
     cudaStream_t s = ctx->stream;
     const long long n6 = 6 * ctx->S, kv = E.g.kvec;
-    const int npe = Launch<R>::ew_grid(n6);
     cpx<R> *rhs = (cpx<R> *)ctx->brhs, *spec = (cpx<R> *)ctx->bspec;
+    // u_0 = 0, u_1 = rhs (= beta_1 v_1), w_0 = w_{-1} = 0 as Krylov vectors;
+    // the work spectrum enters each step holding F_1^-1 G u_k
+    for (void *p : {ctx->bv[0], ctx->bv[1], ctx->bv[2], ctx->bw[0], ctx->bw[1], ctx->bx})
+        CU(cudaMemsetAsync(p, 0, sizeof(cpx<R>) * kv * nb, s));
+    const int npe = Launch<R>::ew_grid(ctx->S);
     for (int j = 0; j < nb; ++j) {
-        Launch<R>::norm2w(E.g, s, rhs + j * n6, ctx->bpart + (size_t)j * npe);
+        Launch<R>::to_krylov(E.g, s, rhs + j * n6, (cpx<R> *)ctx->bv[1] + j * kv, ctx->bpart + (size_t)j * npe);
         scalar_start(s, ctx->d_bst + j, ctx->bpart + (size_t)j * npe, npe, tol[j], maxit[j], max_bodies);
+        if constexpr (sizeof(R) == 4)
+            if (E.g.mask0) {
+                dc_start(s, ctx->d_bst + j, rhs + j * n6, E.g.mask0);
+                ctx->launches += 1;
+            }
     }
     ctx->launches += 2 * nb;
     CU(cudaMemcpyAsync(ctx->h_bst, ctx->d_bst, sizeof(MinresState) * nb, cudaMemcpyDeviceToHost, s));
     CU(cudaStreamSynchronize(s));
     *any = false;
     for (int j = 0; j < nb; ++j) *any = *any || !ctx->h_bst[j].done;
-    CU(cudaMemsetAsync(ctx->bx, 0, sizeof(cpx<R>) * kv * nb, s));
     if (!*any) return HOM_OK;
     // the folded scalar steps' counters start at zero (each last CTA resets
     // its own; this also clears any left by a sweep that stopped on an error)
     CU(cudaMemsetAsync(ctx->bcnt, 0, sizeof(int) * kFoldCounters, s));
-    // u_0 = 0, u_1 = rhs (= beta_1 v_1), w_0 = w_{-1} = 0, in tile order; the
-    // work spectrum enters each step holding F_1^-1 G u_k
-    CU(cudaMemsetAsync(ctx->bv[0], 0, sizeof(cpx<R>) * kv * nb, s));
-    CU(cudaMemsetAsync(ctx->bv[1], 0, sizeof(cpx<R>) * kv * nb, s));
-    CU(cudaMemsetAsync(ctx->bv[2], 0, sizeof(cpx<R>) * kv * nb, s));
-    CU(cudaMemsetAsync(ctx->bw[0], 0, sizeof(cpx<R>) * kv * nb, s));
-    CU(cudaMemsetAsync(ctx->bw[1], 0, sizeof(cpx<R>) * kv * nb, s));
     for (int j = 0; j < nb; ++j) {
         if (ctx->h_bst[j].done) continue;
-        Launch<R>::to_tiles(E.g, s, rhs + j * n6, (cpx<R> *)ctx->bv[1] + j * kv);
         Launch<R>::x1(E.g, s, X1_GAMMA_IN, rhs + j * n6, spec + j * n6, nullptr, nullptr, nullptr);
-        ctx->launches += 2;
+        ctx->launches += 1;
     }
     return HOM_OK;
 }
@@ -1587,7 +1588,7 @@ static int batch_end(hom_ctx *ctx, Engine<R> &E, int nb, const int *maxit, bool 
                                 (const cpx<R> *)ctx->bv[2], (cpx<R> *)ctx->bw[0], (cpx<R> *)ctx->bw[1], (cpx<R> *)ctx->bx, ctx->d_bst, kv);
         ctx->launches += 1;
     }
-    for (int j = 0; j < nb; ++j) Launch<R>::from_tiles(E.g, s, (const cpx<R> *)ctx->bx + j * kv, rhs + j * n6);
+    for (int j = 0; j < nb; ++j) Launch<R>::from_krylov(E.g, s, (const cpx<R> *)ctx->bx + j * kv, rhs + j * n6, ctx->d_bst + j);
     ctx->launches += nb;
     CU(cudaMemcpyAsync(ctx->h_bst, ctx->d_bst, sizeof(MinresState) * nb, cudaMemcpyDeviceToHost, s));
     CU(cudaStreamSynchronize(s));

@@ -75,12 +75,13 @@ __global__ void k_scalar_start(MinresState *st, const double *partials, int np, 
     st->done = (beta1 == 0.0 || max_it <= 0) ? 1 : 0;
     st->done_update = st->done;
     st->status = 0;
+    st->dc = 0;
     if (!isfinite(beta1)) { st->status = -5; st->done = 1; st->done_update = 1; }
 }
 
 // alpha_k = <v_k, A v_k> = <u_k, A u_k> / beta_k^2; the partials sum to
 // <u_k, A u_k> / scale (scale = V for the strain-energy sums of the n3 pass)
-__global__ void k_scalar_alpha(MinresState *st, const double *partials, int np, double scale) {
+__global__ void k_scalar_alpha(MinresState *st, const double *partials, int np, double scale, const double *tsum) {
     pdl_release();
     pdl_wait();                    // the n3 pass's partials (programmatic launch in the MINRES graph)
     st += blockIdx.x;              // load case of a stacked batch (one CTA each)
@@ -88,6 +89,32 @@ __global__ void k_scalar_alpha(MinresState *st, const double *partials, int np, 
     if (st->done) return;
     const double a = reduce_partials(partials, np);
     if (threadIdx.x == 0) alpha_step(st, a, scale);
+    if (tsum && st->dc) {   // the six sums at once, a group of warps each
+        __shared__ double part[32];
+        const int warp = threadIdx.x >> 5, per = (int)(blockDim.x >> 5) / 6;   // warps of a sum
+        const int c = warp / per;
+        double v = 0.0;
+        if (c < 6) {
+            const double *t = tsum + ((size_t)c * gridDim.x + blockIdx.x) * np;
+            for (int i = threadIdx.x - 32 * c * per; i < np; i += 32 * per) v += t[i];
+        }
+        v = warp_sum(v);
+        if ((threadIdx.x & 31) == 0) part[warp] = v;
+        __syncthreads();
+        if (threadIdx.x < 6) {
+            double t = 0.0;
+            for (int i = 0; i < per; ++i) t += part[threadIdx.x * per + i];
+            st->dc_tau[threadIdx.x] = t;
+        }
+    }
+}
+
+__global__ void k_dc_start(MinresState *st, const float2 *rhs, int mask) {
+    const int c = threadIdx.x;
+    if (c >= 6) return;
+    st->dc_u[c] = (mask >> c) & 1 ? (double)rhs[c].x : 0.0;
+    st->dc_tau[c] = st->dc_um[c] = st->dc_un[c] = st->dc_w1[c] = st->dc_w2[c] = st->dc_x[c] = 0.0;
+    if (c == 0) st->dc = 1;
 }
 
 // MINRES step k: apply the previous Givens rotation to the new column of the
@@ -302,12 +329,6 @@ struct TmaCache {
 };
 }  // namespace
 
-int tma_box_rows(int n, int rowb) {
-    for (int k = (n + 255) / 256; k <= n; ++k)
-        if (n % k == 0 && (k == 1 || (n / k) * rowb % 128 == 0)) return n / k;
-    return 0;
-}
-
 int line_tpl(int n) {
     switch (n) {
 #define HOM_LINE_TPL(N) case N: return LinePlan<N>::TPL;
@@ -441,9 +462,11 @@ void scalar_start(cudaStream_t st, MinresState *s, const double *partials, int n
 void loop_cond(cudaStream_t st, cudaGraphConditionalHandle h, MinresState *s, int nb) {
     k_loop_cond<<<1, 32, 0, st>>>(h, s, nb);
 }
-void scalar_alpha(cudaStream_t st, MinresState *s, const double *partials, int np, double scale, int nb, int pdl) {
-    launch_k(pdl, k_scalar_alpha, nb, 1024, 0, st, s, partials, np, scale);
+void scalar_alpha(cudaStream_t st, MinresState *s, const double *partials, int np, double scale, int nb, int pdl,
+                  const double *tsum) {
+    launch_k(pdl, k_scalar_alpha, nb, 1024, 0, st, s, partials, np, scale, tsum);
 }
+void dc_start(cudaStream_t st, MinresState *s, const float2 *rhs, int mask) { k_dc_start<<<1, 32, 0, st>>>(s, rhs, mask); }
 void scalar_givens(cudaStream_t st, MinresState *s, const double *partials, int np, int nb) {
     k_scalar_givens<<<nb, 1024, 0, st>>>(s, partials, np);
 }

@@ -52,7 +52,55 @@ struct MinresState {
     double est;        // phibar_k / beta_1
     int bodies;        // captured bodies run by the device-side loop
     int max_bodies;    // hard cap of that loop
+    // FP32 fields under stress control (dc != 0): the vectors' values at xi = 0,
+    // the macroscopic strain the load drives, carried in FP64 beside their FP32
+    // entries, with A u at xi = 0 from the n3 pass's FP64 stress sums.  One FP32
+    // rounding of them is a uniform strain, which no average over voxels takes
+    // out: without this the stresses of an uniaxial solve after 50 steps are
+    // 1.4 to 2.7e-6 off an FP64 solve's, with it 1.3 to 1.5e-6 (a numpy
+    // restatement, 48^3 octet).  Six real components each (Mandel).
+    int dc;
+    double dc_tau[6], dc_u[6], dc_um[6], dc_un[6], dc_w1[6], dc_w2[6], dc_x[6];
 };
+
+// the step's w and x at xi = 0, and u_{k+1} in u_k's place (one thread; ib =
+// 1 / beta_k, ig = 1 / gamma; the values are loaded together, one memory
+// latency and not six)
+__device__ __forceinline__ void dc_step(MinresState *st, double ib, double delta, double eps, double ig, double tau) {
+    double u[6], un[6], w1[6], w2[6], x[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        u[c] = st->dc_u[c];
+        un[c] = st->dc_un[c];
+        w1[c] = st->dc_w1[c];
+        w2[c] = st->dc_w2[c];
+        x[c] = st->dc_x[c];
+    }
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        const double w = (u[c] * ib - delta * w1[c] - eps * w2[c]) * ig;
+        st->dc_w2[c] = w1[c];
+        st->dc_w1[c] = w;
+        st->dc_x[c] = x[c] + tau * w;
+        st->dc_um[c] = u[c];
+        st->dc_u[c] = un[c];
+    }
+}
+// u_{k+1} at xi = 0 (one thread of the fused n1 pass); q: its three values
+template <typename R> __device__ __forceinline__ void dc_lanczos(MinresState *st, int mask, cpx<R> *q) {
+    const double ib = 1.0 / st->beta, cu = -st->alpha * ib;
+    const double cv = st->beta_prev > 0.0 ? -st->beta / st->beta_prev : 0.0;
+    double v[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c)
+        v[c] = (mask >> c) & 1 ? st->dc_tau[c] * ib + cu * st->dc_u[c] + cv * st->dc_um[c] : 0.0;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        st->dc_un[c] = v[c];
+        if (c & 1) q[c / 2].y = (R)v[c];
+        else q[c / 2].x = (R)v[c];
+    }
+}
 
 // alpha_k = <v_k, A v_k> = <u_k, A u_k> / beta_k^2 from sum = <u_k, A u_k> / scale
 __device__ __forceinline__ void alpha_step(MinresState *st, double sum, double scale) {
@@ -78,6 +126,7 @@ __device__ __forceinline__ void givens_step(MinresState *st, double bn2) {
     const double cn = gbar / gamma, sn = beta_next / gamma;
     const double tau = cn * st->phibar;
     const double phibar = sn * st->phibar;
+    if (st->dc) dc_step(st, 1.0 / st->beta, delta, st->eps, 1.0 / gamma, tau);
     st->u_delta = delta;
     st->u_eps = st->eps;            // epsilon_k multiplies w_{k-2}
     st->u_inv_gamma = 1.0 / gamma;
@@ -149,9 +198,10 @@ struct Geometry {
     // memory, host-side cache of tensor maps (never dereferenced on the
     // device) and the device word a pass sets when a bounded wait gives up
     int tma;
-    // fused MINRES chain: complex elements of one Krylov vector stored in
-    // n1-tile order (tiles of tile1l (k2,k3) columns, each tile a contiguous
-    // n1 x 6 tile1l block laid out as the pass's shared-memory tile)
+    // fused MINRES chain: complex elements of one Krylov vector, three
+    // components a frequency (gamma_to_q) in n1-tile order: tiles of tile1l
+    // (k2,k3) columns, each krylov_tile(n1, tile1l) values, one plane n1 x
+    // tile1l per component
     long long kvec;
     // register-resident n3 pass (k_x3r: FP32, n3 = 256) for
     // spectrum-to-spectrum applications
@@ -238,17 +288,19 @@ enum X1Flags { X1_FWD = 1, X1_GAMMA_IN = 2, X1_GAMMA_OUT = 4, X1_DOT = 8 };
 
 constexpr int kEwBlocks = 152 * 8;   // grid of the element-wise Krylov kernels
 constexpr int kNbMax = 8;            // load cases of one stacked MINRES batch
-// threads of the persistent fused n1 pass: the most its transform group may
-// have (with the lagged-update warps, two CTAs per SM at 127 registers) and
-// the lagged-update warps
+// persistent fused n1 pass: the most threads its transform group may have, and
+// its lagged-update ring
 constexpr int kX1Group = 192;
-constexpr int kX1LagThreads = 64;
-constexpr int kX1LagChunk = 4096;      // bytes of one operand per ring stage
+constexpr int kX1LagChunk = 2048;      // bytes of one operand per ring stage
 constexpr int kX1LagMaxStages = 3;
 constexpr int kX2MaxStages = 4;        // TMA ring of the persistent n2 pass
 constexpr int kEwThreads = 256;
 
 struct Mac6 { double v[6]; };
+
+// complex values of a Krylov tile of t columns: three planes, padded to 16 bytes
+// for the bulk copies
+__host__ __device__ constexpr int krylov_tile(int n1, int t) { return (3 * n1 * t + 1) / 2 * 2; }
 
 // The MINRES scalar steps folded into the pass that produces their partial
 // sums: every CTA of a group counts itself on a counter after writing its
@@ -272,9 +324,11 @@ X2LineFn x2_line_kernel(int n, int inverse);
 X1lLineFn x1l_line_kernel(int n);
 // persistent n3 pass of a length, with its threads, rows per tile and shared
 // memory (fn null: none)
+// (fn_sums: with the stress sums)
 struct X3Line {
-    void (*fn)(Geometry, const float2 *, float2 *, int, float, float, const float *, const MinresState *, double *,
-               Fold) = nullptr;
+    using Fn = void (*)(Geometry, const float2 *, float2 *, int, float, float, const float *, const MinresState *,
+                        double *, Fold, double *);
+    Fn fn = nullptr, fn_sums = nullptr;
     int threads = 0, rows = 0;
     size_t smem = 0;
 };
@@ -284,7 +338,26 @@ void line_kernel_attr(const void *kernel, int optin);
 // rows of a TMA box for tiles of n rows of rowb bytes: the most that divide n,
 // fit a box dimension (256) and keep every box on a 128-byte boundary of
 // shared memory (0: none)
-int tma_box_rows(int n, int rowb);
+constexpr int tma_box_rows(int n, int rowb) {
+    for (int k = (n + 255) / 256; k <= n; ++k)
+        if (n % k == 0 && (k == 1 || (n / k) * rowb % 128 == 0)) return n / k;
+    return 0;
+}
+// columns of a tile of the TMA-staged fused n1 pass (FP32, six components): as
+// many as its transform group has threads for and its boxes allow (0: none)
+constexpr int x1l_cols(int n, int tpl) {
+    int t = kX1Group / (6 * tpl);
+    for (t = t > 16 ? 16 : t; t > 0; --t)
+        if (tma_box_rows(n, 48 * t)) break;
+    return t;
+}
+// its transform threads, lagged-update threads and both.  One lagged warp
+// beside small groups, so that four CTAs fit at 80 registers (40 against 44 us
+// at 108^3), two beside full ones, which three CTAs leave the registers for
+// (398 against 423 us at 256^3).
+constexpr int x1l_group(int n, int tpl) { return (6 * x1l_cols(n, tpl) * tpl + 31) / 32 * 32; }
+constexpr int x1l_lag_threads(int grp) { return grp > 160 ? 64 : 32; }
+constexpr int x1l_threads(int n, int tpl) { return x1l_group(n, tpl) + x1l_lag_threads(x1l_group(n, tpl)); }
 
 template <typename R> struct Launch {
     // n3 pass: C2R (SPEC in) or real / macro input, optional material law
@@ -293,9 +366,9 @@ template <typename R> struct Launch {
     // epart (6-component spectra only): per-CTA sums of the strain energy
     // e : C : e of the scaled real-space input (x3_grid(g) values).
     // fold: the alpha step folded into the pass (see Fold in hom_passes.cuh)
-    // tsum (shared-memory pass with the material law only): per-CTA partial
-    // sums over the voxels of the six stress components it forms,
-    // tsum[c * x3_grid(g) + block]
+    // tsum (with the material law): per-CTA partial sums over the voxels of
+    // the six stress components it forms, tsum[(c * nb + case) * blocks + block],
+    // blocks a case's partials (x3_epart_grid(g) from spectrum to spectrum)
     static void x3(const Geometry &g, cudaStream_t st, int in_mode, const void *in, int mid, double lam, double mu,
                    const double *macro_mandel, double scale, int out_mode, void *out, const R *phi,
                    const MinresState *state, double *epart = nullptr, Fold fold = Fold{}, double *tsum = nullptr);
@@ -335,10 +408,11 @@ template <typename R> struct Launch {
                            cpx<R> *un, const cpx<R> *wa, cpx<R> *wb, cpx<R> *x, const MinresState *state,
                            double *partials, Fold fold = Fold{});
     static int x1_lanczos_grid(const Geometry &g);
-    // standard half-spectrum order <-> n1-tile order of the fused chain's
-    // Krylov vectors (the tile order's padding is left untouched)
-    static void to_tiles(const Geometry &g, cudaStream_t st, const cpx<R> *in, cpx<R> *out);
-    static void from_tiles(const Geometry &g, cudaStream_t st, const cpx<R> *in, cpx<R> *out);
+    // half spectrum in standard order <-> Krylov vector (its padding is left
+    // untouched); to_krylov returns the number of partials of ||q||^2
+    static int to_krylov(const Geometry &g, cudaStream_t st, const cpx<R> *in, cpx<R> *out, double *partials);
+    // (state: its FP64 values at xi = 0 are taken where it has them)
+    static void from_krylov(const Geometry &g, cudaStream_t st, const cpx<R> *in, cpx<R> *out, const MinresState *state);
     // the lagged update of the last step K after the loop; u_K sits in
     // buffer K mod 3 of (ua, ub, uc), or without uc (two Lanczos buffers) in
     // ub for odd K, in ua for even K; w_{K-1} in wd for even K, wc for odd K
@@ -411,8 +485,12 @@ void loop_cond(cudaStream_t st, cudaGraphConditionalHandle h, MinresState *s, in
 // alpha_k from partials summing to <u_k, A^ u_k> / scale.  The scalar
 // kernels of a stacked batch run one CTA per case c, on s[c] and the
 // partials at c * np.
+// tsum: the stress sums of the n3 pass (see x3), for states with dc set.
 void scalar_alpha(cudaStream_t st, MinresState *s, const double *partials, int np, double scale = 1.0, int nb = 1,
-                  int pdl = 0);
+                  int pdl = 0, const double *tsum = nullptr);
+// the FP64 values at xi = 0 of a stress-controlled FP32 solve start from the
+// right-hand side's
+void dc_start(cudaStream_t st, MinresState *s, const float2 *rhs, int mask);
 void scalar_givens(cudaStream_t st, MinresState *s, const double *partials, int np, int nb = 1);
 // PCG scalars (MoDBFFT): start from <r0,z0>, ||r0||^2; step length; direction
 void scalar_cg_start(cudaStream_t st, CgState *s, const double *partials, int np, double tol, int max_it);

@@ -14,16 +14,95 @@
 
 namespace hom {
 
-template <typename R, int N> struct LineFft {
-    template <int S>
-    __device__ static __forceinline__ cpx<R> *run(cpx<R> *buf, cpx<R> *, int L, const AxisPlan &p, int nsync) {
-        line_fft<R, S, N>(buf, L, L, reinterpret_cast<const cpx<R> *>(p.tw), nsync);
-        return buf;
-    }
-};
+// 1 / sqrt(n2): the hardware's estimate and one Newton step, within an ulp or
+// two of the correctly rounded quotient and a third of its instructions
+__device__ __forceinline__ float inv_norm(float n2) {
+    const float y = rsqrtf(n2);
+    return fmaf(0.5f * y, fmaf(-n2 * y, y, 1.0f), y);
+}
 
+// Steps 1-3 of the fused pass (see k_x1_lanczos) on the tile of columns [g0, g0
+// + T) held in buf, element e of line l at buf[e * L + l], L = 6 T; the GRP
+// threads of the transform group call it.  Everything but n2, n3 is known at
+// compile time, and a thread keeps one column, so that its part of xi (axes 2
+// and 3), the Parseval weight and the addresses are formed once per tile.
+template <typename R, int N, int T, int GRP>
+__device__ __forceinline__ void x1_lanczos_line(const Geometry &g, cpx<R> *buf, int g0, const LzCoef<R> &c,
+                                                const cpx<R> *__restrict__ uk, const cpx<R> *__restrict__ um,
+                                                cpx<R> *__restrict__ un, Acc<R> &acc, MinresState *dst) {
+    constexpr int NC = 6, L = NC * T, NT = N * T, ES = GRP / T;   // ES frequencies at once
+    const cpx<R> *tw = reinterpret_cast<const cpx<R> *>(g.ax[0].tw);
+    line_fft<R, -1, N>(buf, L, L, tw, GRP);
+    const int t = threadIdx.x % T, e0 = threadIdx.x / T;
+    const int col = g0 + t, H = g.h;
+    if (e0 < ES && col < g.n2 * H) {
+        const int k2 = col / H, k3 = col - k2 * H;
+        const R w = (R)pweight(k3, g.n3);
+        // mode of the column: 0 a Nyquist index of axis 2 or 3, else 1
+        const bool nyq = 2 * k2 == g.n2 || 2 * k3 == g.n3;
+        const cpx<R> m1 = __ldg(&reinterpret_cast<const cpx<R> *>(g.M[1])[k2]);
+        const cpx<R> m2 = __ldg(&reinterpret_cast<const cpx<R> *>(g.M[2])[k3]);
+        const cpx<R> m12 = mul<R>(m1, m2);
+        const cpx<R> d1 = mul<R>(__ldg(&reinterpret_cast<const cpx<R> *>(g.D[1])[k2]), m2);
+        const cpx<R> d2 = mul<R>(__ldg(&reinterpret_cast<const cpx<R> *>(g.D[2])[k3]), m1);
+        const cpx<R> *D0 = reinterpret_cast<const cpx<R> *>(g.D[0]);
+        const cpx<R> *M0 = reinterpret_cast<const cpx<R> *>(g.M[0]);
+        const size_t i0 = (size_t)(g0 / T) * krylov_tile(N, T) + t;
+#pragma unroll 1
+        for (int e = e0; e < N; e += ES) {
+            const size_t i = i0 + e * T;
+            cpx<R> *sp = buf + e * L + t * NC;
+            cpx<R> v[NC], q[3], u[3], uo[3];
+#pragma unroll
+            for (int c3 = 0; c3 < 3; ++c3) {
+                u[c3] = uk[i + c3 * NT];
+                uo[c3] = um[i + c3 * NT];
+            }
+            const cpx<R> m0 = __ldg(&M0[e]);
+            GammaE<R> ge;
+            ge.e0 = mul<R>(__ldg(&D0[e]), m12);
+            ge.e1 = mul<R>(d1, m0);
+            ge.e2 = mul<R>(d2, m0);
+            const R n2 = ge.e0.x * ge.e0.x + ge.e0.y * ge.e0.y + ge.e1.x * ge.e1.x + ge.e1.y * ge.e1.y +
+                         ge.e2.x * ge.e2.x + ge.e2.y * ge.e2.y;
+            ge.mode = (nyq || 2 * e == N || !(n2 > (R)0)) ? 0 : 1;
+            if (col == 0 && e == 0) ge.mode = 2;
+            const R inv = inv_norm(n2);
+            ge.e0 = scale<R>(ge.e0, inv);
+            ge.e1 = scale<R>(ge.e1, inv);
+            ge.e2 = scale<R>(ge.e2, inv);
+#pragma unroll
+            for (int p = 0; p < 3; ++p) Six<R>::load_pair(sp, p, v[2 * p], v[2 * p + 1]);
+            gamma_to_q<R>(g, ge, v, q);
+#pragma unroll
+            for (int c3 = 0; c3 < 3; ++c3) {
+                q[c3] = mk<R>(c.cp * q[c3].x + c.cu * u[c3].x + c.cv * uo[c3].x,
+                              c.cp * q[c3].y + c.cu * u[c3].y + c.cv * uo[c3].y);
+            }
+            if (c.dc && ge.mode == 2) dc_lanczos<R>(dst, g.mask0, q);
+#pragma unroll
+            for (int c3 = 0; c3 < 3; ++c3) {
+                acc.add_prod(w * q[c3].x, q[c3].x);
+                acc.add_prod(w * q[c3].y, q[c3].y);
+                un[i + c3 * NT] = q[c3];
+            }
+            gamma_from_q<R>(g, ge, q, v);
+#pragma unroll
+            for (int p = 0; p < 3; ++p) Six<R>::store_pair(sp, p, v[2 * p], v[2 * p + 1]);
+        }
+    }
+    // (the columns beyond the last hold zeros: TMA fills them, and a DFT keeps them)
+    group_sync(GRP);
+    line_fft<R, 1, N>(buf, L, L, tw, GRP);
+}
+
+// Held to 64 registers (CTAs of 128 to 256 threads, as many as the ring's
+// shared memory leaves room for) except where the plan needs more, and from 225
+// up, where that room is two or three CTAs anyway: there the twiddles stay in
+// registers across the loop (141 against 146 us at 256^3, 118 against 127 at
+// 240^3; at 192^3 68 against 66).
 template <typename R, int S, int N>
-__global__ void __launch_bounds__(512, LinePlan<N>::E <= 16 ? 2 : 1) k_x2_tma(Geometry g, const __grid_constant__ CUtensorMap tm, int qtiles,
+__global__ void __launch_bounds__(512, LinePlan<N>::E <= 16 && N < 225 ? 2 : 1) k_x2_tma(Geometry g, const __grid_constant__ CUtensorMap tm, int qtiles,
                                             const MinresState *state) {
     pdl_release();
     pdl_wait();   // predecessor complete (programmatic launch in the MINRES graph)
@@ -115,8 +194,8 @@ __device__ __forceinline__ bool group_or(bool v, int n) {
 // update it from shared memory and store w_{k-1} (and x) to HBM.  The update is the same on every real number,
 // so it runs on 16-byte vectors.  Returns false after a bounded wait ran
 // out (the copies in flight have been waited for, bounded).
-template <typename R, typename LiveFrom>
-__device__ __forceinline__ bool x1_lagged(const Geometry &g, int grp, const LzCoef<R> *scoef, LiveFrom live_from, int ntiles,
+template <typename R, int grp, int NLAG, typename LiveFrom>
+__device__ __forceinline__ bool x1_lagged(const Geometry &g, const LzCoef<R> *scoef, LiveFrom live_from, int ntiles,
                                           int tpc, int per, unsigned char *ring, uint64_t *lbar,
                                           const cpx<R> *__restrict__ um, const cpx<R> *__restrict__ wa,
                                           cpx<R> *__restrict__ wb, cpx<R> *__restrict__ x) {
@@ -160,7 +239,7 @@ __device__ __forceinline__ bool x1_lagged(const Geometry &g, int grp, const LzCo
     for (; ct < ntiles; ++n) {
         const int s = n % S;
         const bool got = mbar_wait_bounded(&lbar[s], (uint32_t)(n / S) & 1u);
-        if (group_or<2>(!got, kX1LagThreads)) {
+        if (group_or<2>(!got, NLAG)) {
             if (lt == 0) {   // record, then wait (bounded) for the items in flight
                 atomicExch(g.err, 1);
                 for (int m = n; m < issued; ++m) mbar_wait_bounded(&lbar[m % S], (uint32_t)(m / S) & 1u);
@@ -175,7 +254,7 @@ __device__ __forceinline__ bool x1_lagged(const Geometry &g, int grp, const LzCo
         V *gb = reinterpret_cast<V *>(reinterpret_cast<char *>(wb) + o);
         V *gx = reinterpret_cast<V *>(reinterpret_cast<char *>(x) + o);
         if (c.xstep) {
-            for (int j = lt; j < nv; j += kX1LagThreads) {
+            for (int j = lt; j < nv; j += NLAG) {
                 V vu = su[j], va = sa[j], vb = sb[j], vx = sx[j], vn;
                 const R *u = reinterpret_cast<const R *>(&vu);
                 const R *a = reinterpret_cast<const R *>(&va);
@@ -191,7 +270,7 @@ __device__ __forceinline__ bool x1_lagged(const Geometry &g, int grp, const LzCo
                 gx[j] = vx;
             }
         } else {
-            for (int j = lt; j < nv; j += kX1LagThreads) {
+            for (int j = lt; j < nv; j += NLAG) {
                 V vu = su[j], va = sa[j], vb = sb[j];
                 const R *u = reinterpret_cast<const R *>(&vu);
                 const R *a = reinterpret_cast<const R *>(&va);
@@ -206,7 +285,7 @@ __device__ __forceinline__ bool x1_lagged(const Geometry &g, int grp, const LzCo
             co = 0;
             ct = next_tile(ct + gridDim.x);
         }
-        asm volatile("bar.sync 2, %0;" ::"n"(kX1LagThreads) : "memory");   // stage s is read
+        asm volatile("bar.sync 2, %0;" ::"n"(NLAG) : "memory");   // stage s is read
         if (lt == 0 && pt < ntiles) issue();
     }
     return true;
@@ -217,7 +296,7 @@ __device__ __forceinline__ bool x1_lagged(const Geometry &g, int grp, const LzCo
 // barrier 1) take the work tiles: each comes and goes by TMA, double-
 // buffered as in k_x1_tma, and the Lanczos step reads u_k and u_{k-1}
 // (bulk-prefetched into L2 at the tile's start) and writes u_{k+1} with
-// plain coalesced accesses.  The last kX1LagThreads threads (two warps) run
+// plain coalesced accesses.  The last one or two warps (x1l_lag_threads) run
 // the lagged w update (and on one step in three the deferred x update) on
 // the same tiles' Krylov blocks, streaming u_{k-1}, w_{k-2}, w_{k-3} (and x)
 // while the transform group works in shared memory; the two groups share no
@@ -229,7 +308,8 @@ __device__ __forceinline__ bool x1_lagged(const Geometry &g, int grp, const LzCo
 // one running sum per case in shared memory, and the CTA writes one partial
 // per case (partials[case * gridDim + block]).
 template <typename R, int N>
-__global__ void __launch_bounds__(kX1Group + kX1LagThreads, 2)
+__global__ void __launch_bounds__(x1l_threads(N, LinePlan<N>::TPL),
+                                  LinePlan<N>::E > 16 ? 2 : (x1l_threads(N, LinePlan<N>::TPL) <= 192 ? 4 : 3))
     k_x1_lanczos_tma(Geometry g, const __grid_constant__ CUtensorMap tspec, const cpx<R> *__restrict__ uk,
                      const cpx<R> *__restrict__ um, cpx<R> *__restrict__ un, const cpx<R> *__restrict__ wa,
                      cpx<R> *__restrict__ wb, cpx<R> *__restrict__ x, const MinresState *state,
@@ -239,16 +319,17 @@ __global__ void __launch_bounds__(kX1Group + kX1LagThreads, 2)
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bar[2];
     __shared__ __align__(8) uint64_t lbar[kX1LagMaxStages];
-    __shared__ double sacc[kNbMax * kX1Group];
+    __shared__ double sacc[kNbMax * (kX1Group / 32)];   // ||u_{k+1}||^2 of each case, one running sum a warp
     __shared__ LzCoef<R> scoef[kNbMax];   // each case's coefficients, converted once
     constexpr int NC = 6;
-    const int T = g.tile1l, L = NC * T, GRP = g.grp1l;
+    constexpr int T = x1l_cols(N, LinePlan<N>::TPL), L = NC * T, GRP = x1l_group(N, LinePlan<N>::TPL);
     const int cols = g.n2 * g.h;
     const int tpc = (cols + T - 1) / T;   // tiles per case
     const int ntiles = tpc * g.nb;
-    const int per = N * L;
-    const int sper = (int)(g.stage1l / sizeof(cpx<R>));   // stage stride: per rounded up to 128 bytes
-    const uint32_t bytes = (uint32_t)(per * sizeof(cpx<R>));
+    constexpr int kper = krylov_tile(N, T);
+    constexpr int sper = (N * L + 15) / 16 * 16;   // stage stride: a multiple of 128 bytes (FP32)
+    constexpr int box = tma_box_rows(N, L * (int)sizeof(cpx<R>));
+    constexpr uint32_t bytes = (uint32_t)(N * L * sizeof(cpx<R>));
     cpx<R> *base = reinterpret_cast<cpx<R> *>(smem_raw);
     const bool leader = threadIdx.x == 0;
     const bool xform = threadIdx.x < GRP;
@@ -256,8 +337,7 @@ __global__ void __launch_bounds__(kX1Group + kX1LagThreads, 2)
         while (t < ntiles && skip_case(state, t / tpc)) t += gridDim.x;
         return t;
     };
-    if (xform)
-        for (int cc = 0; cc < g.nb; ++cc) sacc[cc * kX1Group + threadIdx.x] = 0.0;
+    if (threadIdx.x < kNbMax * (kX1Group / 32)) sacc[threadIdx.x] = 0.0;
     if (threadIdx.x < g.nb) scoef[threadIdx.x] = lz_coef<R>(state + threadIdx.x);
     if (leader) {
         mbar_init(&bar[0], 1);
@@ -267,12 +347,13 @@ __global__ void __launch_bounds__(kX1Group + kX1LagThreads, 2)
     }
     __syncthreads();
     if (!xform) {
-        x1_lagged<R>(g, GRP, scoef, live_from, ntiles, tpc, per, smem_raw + 2 * g.stage1l, lbar, um, wa, wb, x);
+        x1_lagged<R, GRP, x1l_lag_threads(GRP)>(g, scoef, live_from, ntiles, tpc, kper, smem_raw + 2 * g.stage1l, lbar, um, wa, wb, x);
     } else {
+        Acc<R> acc;   // this thread's ||u_{k+1}||^2 of the running case
         int tile = live_from(blockIdx.x);
         if (leader && tile < ntiles) {
             mbar_expect_tx(&bar[0], bytes);
-            tma_load_rows_2d(base, &tspec, NC * T * (tile % tpc), N * (tile / tpc), N, g.box1l, L * (int)sizeof(cpx<R>),
+            tma_load_rows_2d(base, &tspec, NC * T * (tile % tpc), N * (tile / tpc), N, box, L * (int)sizeof(cpx<R>),
                              &bar[0]);
         }
         for (int i = 0; tile < ntiles; ++i) {
@@ -281,7 +362,7 @@ __global__ void __launch_bounds__(kX1Group + kX1LagThreads, 2)
             if (leader && next < ntiles) {
                 bulk_wait_read_all();   // the store of the tile that used stage s^1 has read it
                 mbar_expect_tx(&bar[s ^ 1], bytes);
-                tma_load_rows_2d(base + (s ^ 1) * sper, &tspec, NC * T * (next % tpc), N * (next / tpc), N, g.box1l,
+                tma_load_rows_2d(base + (s ^ 1) * sper, &tspec, NC * T * (next % tpc), N * (next / tpc), N, box,
                                  L * (int)sizeof(cpx<R>), &bar[s ^ 1]);
             }
             const bool ok = mbar_wait_bounded(&bar[s], (i >> 1) & 1);
@@ -296,19 +377,21 @@ __global__ void __launch_bounds__(kX1Group + kX1LagThreads, 2)
             const int cs = tile / tpc, tc = tile - cs * tpc;
             const size_t ko = (size_t)cs * g.kvec;
             if (leader && g.x1_l2pf) {   // this tile's u_k and u_{k-1} blocks into L2 for the Lanczos step
-                bulk_prefetch_l2(uk + ko + (size_t)tc * per, bytes);
-                bulk_prefetch_l2(um + ko + (size_t)tc * per, bytes);
+                bulk_prefetch_l2(uk + ko + (size_t)tc * kper, (uint32_t)(kper * sizeof(cpx<R>)));
+                bulk_prefetch_l2(um + ko + (size_t)tc * kper, (uint32_t)(kper * sizeof(cpx<R>)));
             }
             const LzCoef<R> c = scoef[cs];
-            Acc<R> acc;
             cpx<R> *buf = base + s * sper;
-            cpx<R> *res = x1_lanczos_tile<R, LineFft<R, N>, false>(g, T, buf, buf, tc * T, c, uk + ko, um + ko, un + ko,
-                                                                  wa + ko, wb + ko, x + ko, acc, GRP);
-            sacc[cs * kX1Group + threadIdx.x] += acc.value();
+            x1_lanczos_line<R, N, T, GRP>(g, buf, tc * T, c, uk + ko, um + ko, un + ko, acc, fold.st + cs);
+            if (next >= ntiles || next / tpc != cs) {   // the last tile of the case here
+                const double ws = warp_sum(acc.value());
+                if ((threadIdx.x & 31) == 0) sacc[cs * (kX1Group / 32) + (threadIdx.x >> 5)] += ws;
+                acc = Acc<R>{};
+            }
             fence_proxy_async_smem();
             group_sync(GRP);
             if (leader) {
-                tma_store_rows_2d(&tspec, NC * T * tc, N * cs, N, g.box1l, res, L * (int)sizeof(cpx<R>));
+                tma_store_rows_2d(&tspec, NC * T * tc, N * cs, N, box, buf, L * (int)sizeof(cpx<R>));
                 bulk_commit();
             }
             tile = next;
@@ -321,10 +404,9 @@ __global__ void __launch_bounds__(kX1Group + kX1LagThreads, 2)
     // tiles if one thread takes the cases in turn
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     for (int cc = warp; cc < g.nb; cc += nw) {
-        double v = 0.0;
-        for (int i = lane; i < GRP; i += 32) v += sacc[cc * kX1Group + i];
-        v = warp_sum(v);
         if (lane == 0) {
+            double v = 0.0;
+            for (int i = 0; i < kX1Group / 32; ++i) v += sacc[cc * (kX1Group / 32) + i];
             partials[cc * gridDim.x + blockIdx.x] = v;
             __threadfence();
         }

@@ -42,6 +42,12 @@ template <> struct Acc<float> {
         hi = s;
         lo += err + e;
     }
+    __device__ __forceinline__ void add(float p) {
+        float s = hi + p;
+        float bp = s - hi;
+        lo += (hi - (s - bp)) + (p - bp);
+        hi = s;
+    }
     __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 template <> struct Acc<double> {
@@ -218,6 +224,64 @@ template <typename R>
 __device__ __forceinline__ void gamma_at(const Geometry &g, int k1, int k2, int k3, cpx<R> *t) {
     const GammaE<R> q = gamma_e<R>(g, k1, k2, k3);
     gamma_apply<R>(g, q, t);
+}
+
+// The projector's range at a frequency has three degrees of freedom, and the
+// fused MINRES step keeps its Krylov vectors in them: q with |q| = |strain|
+// (Mandel).  With P x = sqrt2 x + (1 - sqrt2) e (e^H x), |e| = 1,
+//   strain = B q = sym(P q (x) e),   q = B^H tau = P (tau conj(e)),
+// B is an isometry onto the range (|sym(u (x) e)|^2 = (|u|^2 + |e^H u|^2) / 2)
+// and G = B B^H, so MINRES on B^H F C F^-1 B is the iteration on G F C F^-1 G
+// in half the storage.  At xi = 0 the six stress-controlled components are
+// real: two to a value.
+template <typename R>
+__device__ __forceinline__ void gamma_p(const GammaE<R> &ge, cpx<R> *x) {
+    const R s2 = (R)1.41421356237309504880, a = (R)-0.41421356237309504880;
+    const cpx<R> s = add<R>(add<R>(mul<R>(conjc<R>(ge.e0), x[0]), mul<R>(conjc<R>(ge.e1), x[1])),
+                            mul<R>(conjc<R>(ge.e2), x[2]));
+    const cpx<R> as = scale<R>(s, a);
+    x[0] = add<R>(scale<R>(x[0], s2), mul<R>(ge.e0, as));
+    x[1] = add<R>(scale<R>(x[1], s2), mul<R>(ge.e1, as));
+    x[2] = add<R>(scale<R>(x[2], s2), mul<R>(ge.e2, as));
+}
+
+// q = B^H t
+template <typename R>
+__device__ __forceinline__ void gamma_to_q(const Geometry &g, const GammaE<R> &ge, const cpx<R> *t, cpx<R> *q) {
+    if (ge.mode != 1) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            q[c] = ge.mode == 0 ? mk<R>(0, 0) : mk<R>((g.mask0 >> (2 * c)) & 1 ? t[2 * c].x : (R)0,
+                                                      (g.mask0 >> (2 * c + 1)) & 1 ? t[2 * c + 1].x : (R)0);
+        return;
+    }
+    const cpx<R> c0 = conjc<R>(ge.e0), c1 = conjc<R>(ge.e1), c2 = conjc<R>(ge.e2);
+    const R r2 = (R)0.70710678118654752440;   // 1/sqrt(2)
+    const cpx<R> T23 = scale<R>(t[3], r2), T13 = scale<R>(t[4], r2), T12 = scale<R>(t[5], r2);
+    q[0] = add<R>(add<R>(mul<R>(t[0], c0), mul<R>(T12, c1)), mul<R>(T13, c2));
+    q[1] = add<R>(add<R>(mul<R>(T12, c0), mul<R>(t[1], c1)), mul<R>(T23, c2));
+    q[2] = add<R>(add<R>(mul<R>(T13, c0), mul<R>(T23, c1)), mul<R>(t[2], c2));
+    gamma_p<R>(ge, q);
+}
+
+// t = B q
+template <typename R>
+__device__ __forceinline__ void gamma_from_q(const Geometry &g, const GammaE<R> &ge, const cpx<R> *q, cpx<R> *t) {
+    if (ge.mode != 1) {
+#pragma unroll
+        for (int c = 0; c < 6; ++c)
+            t[c] = ge.mode == 0 || !((g.mask0 >> c) & 1) ? mk<R>(0, 0) : mk<R>(c & 1 ? q[c / 2].y : q[c / 2].x, 0);
+        return;
+    }
+    const R r2 = (R)0.70710678118654752440;   // 1/sqrt(2)
+    cpx<R> u[3] = {q[0], q[1], q[2]};
+    gamma_p<R>(ge, u);
+    t[0] = mul<R>(u[0], ge.e0);
+    t[1] = mul<R>(u[1], ge.e1);
+    t[2] = mul<R>(u[2], ge.e2);
+    t[3] = scale<R>(add<R>(mul<R>(u[1], ge.e2), mul<R>(u[2], ge.e1)), r2);
+    t[4] = scale<R>(add<R>(mul<R>(u[0], ge.e2), mul<R>(u[2], ge.e0)), r2);
+    t[5] = scale<R>(add<R>(mul<R>(u[0], ge.e1), mul<R>(u[1], ge.e0)), r2);
 }
 
 // Run the transform of the L lines in buf.  Fast engine: in place, returns
@@ -503,10 +567,11 @@ __device__ __forceinline__ float2 tw_load(const float2 *p) {
     return v;
 }
 
-template <int N>
+template <int N, bool SUMS>
 __global__ void __launch_bounds__(kX3rWarps * 32, 3)
     k_x3r(Geometry g, const float2 *__restrict__ in, float2 *__restrict__ out, int material, float lam, float mu2,
-          const float *__restrict__ phi, const MinresState *state, double *__restrict__ epart, Fold fold) {
+          const float *__restrict__ phi, const MinresState *state, double *__restrict__ epart, Fold fold,
+          double *__restrict__ tsum) {
     pdl_release();
     pdl_wait();   // predecessor complete (programmatic launch in the MINRES graph)
     using PL = X3RPlan<N>;
@@ -516,6 +581,8 @@ __global__ void __launch_bounds__(kX3rWarps * 32, 3)
     static_assert(P == x3r_row_lanes(N) && TS == (int)x3r_slab_elems(N), "x3r layout");
     extern __shared__ __align__(16) unsigned char x3r_smem_raw[];
     __shared__ double sacc[kNbMax * kX3rWarps];
+    // (behind the warps' buffers, as large as the cases need: three CTAs per SM)
+    double *ssum = reinterpret_cast<double *>(x3r_smem_raw + x3r_smem(N));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rw = lane / P, j = lane % P;
     unsigned char *wbase = x3r_smem_raw + (size_t)warp * x3r_warp_bytes(N);
@@ -533,6 +600,8 @@ __global__ void __launch_bounds__(kX3rWarps * 32, 3)
     const int ngroups = gpc * g.nb;
     const int gstride = gridDim.x * kX3rWarps;
     if (threadIdx.x < kNbMax * kX3rWarps) sacc[threadIdx.x] = 0.0;
+    if constexpr (SUMS)
+        for (int i = threadIdx.x; i < 6 * g.nb * kX3rWarps; i += blockDim.x) ssum[i] = 0.0;
     __syncthreads();
     auto live_from = [&](int q) {
         while (q < ngroups && skip_case(state, q / gpc)) q += gstride;
@@ -557,6 +626,7 @@ __global__ void __launch_bounds__(kX3rWarps * 32, 3)
     const int lane0 = lane & ~(P - 1);
     const int partner = lane0 + ((P - j) & (P - 1));
     const float sV = 1.0f / (float)g.V;
+    Acc<float> eacc;   // this lane's energy of the running case
     int q = live_from(blockIdx.x * kX3rWarps + warp);
     if (q < ngroups) prefetch(q);
     while (q < ngroups) {
@@ -613,7 +683,7 @@ __global__ void __launch_bounds__(kX3rWarps * 32, 3)
         for (int p = 0; p < 3; ++p) x3r_stage2<1, P, Q>(tb3 + p * RW * TS, j, z[p]);
         __syncwarp();
         // ---- material law on voxels j + P m (scaled by 1/V), strain energy
-        float en = 0.f;
+        float en = 0.f, ts[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         if (material) {
             const float *ph_row = phb + rw * N;
 #pragma unroll
@@ -632,7 +702,10 @@ __global__ void __launch_bounds__(kX3rWarps * 32, 3)
                 for (int c = 1; c < 6; ++c) ee += t[c] * t[c];
                 en += ph * (tr * sum + mu2 * ee);
 #pragma unroll
-                for (int c = 0; c < 6; ++c) t[c] = ph * ((c < 3 ? tr : 0.f) + mu2 * t[c]);
+                for (int c = 0; c < 6; ++c) {
+                    t[c] = ph * ((c < 3 ? tr : 0.f) + mu2 * t[c]);
+                    if constexpr (SUMS) ts[c] += t[c];
+                }
 #pragma unroll
                 for (int p = 0; p < 3; ++p) z[p][m] = make_float2(t[2 * p], t[2 * p + 1]);
             }
@@ -678,13 +751,31 @@ __global__ void __launch_bounds__(kX3rWarps * 32, 3)
                 }
             }
         }
-        if (epart) {
-            const double ws = warp_sum((double)en);
+        // (reduced over the warp once a case: FP64 adds run at a small rate)
+        eacc.add(en);
+        if (epart && (qn >= ngroups || qn / gpc != cs)) {
+            const double ws = warp_sum(eacc.value());
             if (lane == 0) sacc[cs * kX3rWarps + warp] += ws;
+            eacc = Acc<float>{};
+        }
+        if constexpr (SUMS) {
+#pragma unroll
+            for (int c = 0; c < 6; ++c) {
+                const double ws = warp_sum((double)ts[c]);
+                if (lane == 0) ssum[(c * g.nb + cs) * kX3rWarps + warp] += ws;
+            }
         }
         q = qn;
     }
     cp_async_wait_all();
+    if constexpr (SUMS) {
+        __syncthreads();
+        if (threadIdx.x < 6 * g.nb) {
+            double t = 0.0;
+            for (int w = 0; w < kX3rWarps; ++w) t += ssum[threadIdx.x * kX3rWarps + w];
+            tsum[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = t;   // = tsum[(c * nb + case) * grid + block]
+        }
+    }
     if (epart) {
         __syncthreads();
         if (threadIdx.x < g.nb) {
@@ -1075,13 +1166,15 @@ __global__ void HOM_PASS_BOUNDS_NF(R, NF) k_x1_tma_expand(Geometry g, const __gr
 // spectrum holding F_3 F_2 of tau = C e_k (the forward n3 and n2 passes of
 // A^ u_k) and alpha_k already known from the n3 pass's strain energy, one
 // pass over each n1 tile
-//   1. finishes p = A^ u_k: forward DFT along n1 and the projector G;
+//   1. finishes p = A^ u_k: forward DFT along n1 and B^H (see gamma_to_q: the
+//      Krylov vectors hold three components a frequency, not six);
 //   2. takes the Lanczos step on unnormalised vectors,
 //        u_{k+1} = p / beta_k - (alpha_k / beta_k) u_k - (beta_k / beta_{k-1}) u_{k-1},
 //      into a third buffer, with the weighted partial ||u_{k+1}||^2, and the
 //      lagged w update of step k-1 (w_{k-1} over w_{k-3});
-//   3. starts A^ u_{k+1}: G on u_{k+1} and the inverse DFT along n1, written
-//      back over the tile of the work spectrum for the next step's n2 pass.
+//   3. starts A^ u_{k+1}: the strain B u_{k+1} and the inverse DFT along n1,
+//      written back over the tile of the work spectrum for the next step's n2
+//      pass.
 // p never reaches HBM, and u_k is read once per step instead of three times.
 // x is updated every third step only, with the three newest w at once,
 //   x += tau_{k-3} w_{k-3} + tau_{k-2} w_{k-2} + tau_{k-1} w_{k-1},
@@ -1089,21 +1182,13 @@ __global__ void HOM_PASS_BOUNDS_NF(R, NF) k_x1_tma_expand(Geometry g, const __gr
 // w_{k-1} replaces it); the flush after the loop adds what is pending.  The
 // sum is the same as one update per step, rounded in another order.
 // ---------------------------------------------------------------------------
-// The transform along n1 of the plain-load passes: the register engine at its
-// lengths, else the runtime Stockham engine.
-template <typename R, int NF> struct PassFft {
-    template <int S>
-    __device__ static __forceinline__ cpx<R> *run(cpx<R> *buf, cpx<R> *buf2, int L, const AxisPlan &p, int nsync) {
-        return run_fft<R, S, NF>(buf, buf2, L, L, p, nsync);
-    }
-};
-
 template <typename R> struct LzCoef {
     R cp, cu, cv;            // 1/beta_k, -alpha_k/beta_k, -beta_k/beta_{k-1}
     R d, e, ig, tau, ib;     // lagged update of step k-1
     R t1, t2;                // tau of the two steps before
     bool lagged;
     bool xstep;              // this step updates x
+    bool dc;                 // the state carries xi = 0 in FP64
 };
 
 // x is updated when the iterations done (the state's k) are a multiple of 3
@@ -1125,36 +1210,32 @@ __device__ __forceinline__ LzCoef<R> lz_coef(const MinresState *st) {
     c.t1 = (R)st->u_tau1;
     c.t2 = (R)st->u_tau2;
     c.xstep = minres_xstep(st->k);
+    c.dc = st->dc != 0;
     return c;
 }
 
-// Steps 1-3 on the tile of columns [g0, g0 + T) held in buf (element e of
-// line l at buf[e * L + l], L = 6 T); returns the buffer holding the inverse
-// transform (buf for the register engine).  The CTA's threads (nsync = 0) or
-// its first nsync threads (named barrier 1) call it.  Between the two
-// transforms one loop over the tile's frequencies builds xi once per
-// frequency and applies the projector to p and to u_{k+1}; the Krylov
-// vectors are stored in tile order, so the six components of a frequency
-// are 48 contiguous bytes of each vector and a warp reads and writes a
-// contiguous block.  u_{k+1} goes to un, a third buffer (u_{k-1} stays
-// readable for the lagged update); with LAG the lagged w / x update of step
-// k-1 is done here too, else by other warps (x1_lagged_block).
-// Fft is the transform along n1 (PassFft here, LineFft in the TMA-staged form).
-template <typename R, typename Fft, bool LAG>
-__device__ __forceinline__ cpx<R> *x1_lanczos_tile(const Geometry &g, int T, cpx<R> *buf, cpx<R> *buf2, int g0,
+// Steps 1-3 of the plain-load form on the tile of columns [g0, g0 + T) held in
+// buf (element e of line l at buf[e * L + l], L = 6 T), the lagged w / x update
+// of step k-1 included; returns the buffer holding the inverse transform (buf
+// for the register engine).  Between the two transforms one loop over the
+// tile's frequencies builds xi once per frequency for B^H p and B u_{k+1}; the
+// Krylov vectors are stored in tile order, one plane of n1 T values per
+// component, so that a warp reads and writes contiguous blocks.
+template <typename R, int NF>
+__device__ __forceinline__ cpx<R> *x1_lanczos_tile(const Geometry &g, cpx<R> *buf, cpx<R> *buf2, int g0,
                                                    const LzCoef<R> &c, const cpx<R> *__restrict__ uk,
                                                    const cpx<R> *__restrict__ um, cpx<R> *__restrict__ un,
                                                    const cpx<R> *__restrict__ wa, cpx<R> *__restrict__ wb,
-                                                   cpx<R> *__restrict__ x, Acc<R> &acc, int nsync) {
+                                                   cpx<R> *__restrict__ x, Acc<R> &acc, MinresState *dst) {
     constexpr int NC = 6;
-    const int N = g.n1, H = g.h, L = NC * T;
+    const int N = g.n1, T = g.tile1, H = g.h, L = NC * T;
     const int cols = g.n2 * H;
-    const int nthr = nsync ? nsync : (int)blockDim.x;
     // 1. forward DFT along n1
-    cpx<R> *res = Fft::template run<-1>(buf, buf2, L, g.ax[0], nsync);
-    // 2. per frequency: p = G (.), Lanczos step, lagged update, G u_{k+1}
-    const size_t kb = (size_t)(g0 / T) * (size_t)(N * L);
-    for (int f = threadIdx.x; f < N * T; f += nthr) {
+    cpx<R> *res = run_fft<R, -1, NF>(buf, buf2, L, L, g.ax[0]);
+    // 2. per frequency: q of p, Lanczos step, lagged update, strain of u_{k+1}
+    const int NT = N * T;   // one of the three planes of a Krylov tile
+    const size_t kb = (size_t)(g0 / T) * krylov_tile(N, T);
+    for (int f = threadIdx.x; f < NT; f += blockDim.x) {
         const int e = f / T, t = f - e * T;
         const int col = g0 + t;
         cpx<R> *sp = res + e * L + t * NC;
@@ -1164,60 +1245,56 @@ __device__ __forceinline__ cpx<R> *x1_lanczos_tile(const Geometry &g, int T, cpx
             continue;
         }
         const int k2 = col / H, k3 = col - k2 * H;
-        const size_t i = kb + (size_t)f * NC;
-        cpx<R> v[NC], u[NC], uo[NC];
+        const size_t i = kb + f;
+        cpx<R> v[NC], q[3], u[3], uo[3];
 #pragma unroll
-        for (int p = 0; p < 3; ++p) {
-            Six<R>::load_pair(sp, p, v[2 * p], v[2 * p + 1]);
-            Six<R>::load_pair(uk + i, p, u[2 * p], u[2 * p + 1]);
-            Six<R>::load_pair(um + i, p, uo[2 * p], uo[2 * p + 1]);
+        for (int c3 = 0; c3 < 3; ++c3) {
+            u[c3] = uk[i + c3 * NT];
+            uo[c3] = um[i + c3 * NT];
         }
+#pragma unroll
+        for (int p = 0; p < 3; ++p) Six<R>::load_pair(sp, p, v[2 * p], v[2 * p + 1]);
         const GammaE<R> ge = gamma_e<R>(g, e, k2, k3);
-        gamma_apply<R>(g, ge, v);
+        gamma_to_q<R>(g, ge, v, q);
         const R w = (R)pweight(k3, g.n3);
 #pragma unroll
-        for (int q = 0; q < NC; ++q) {
-            v[q] = mk<R>(c.cp * v[q].x + c.cu * u[q].x + c.cv * uo[q].x, c.cp * v[q].y + c.cu * u[q].y + c.cv * uo[q].y);
-            acc.add_prod(w * v[q].x, v[q].x);
-            acc.add_prod(w * v[q].y, v[q].y);
+        for (int c3 = 0; c3 < 3; ++c3) {
+            q[c3] = mk<R>(c.cp * q[c3].x + c.cu * u[c3].x + c.cv * uo[c3].x,
+                          c.cp * q[c3].y + c.cu * u[c3].y + c.cv * uo[c3].y);
         }
+        if (c.dc && ge.mode == 2) dc_lanczos<R>(dst, g.mask0, q);
 #pragma unroll
-        for (int p = 0; p < 3; ++p) Six<R>::store_pair(un + i, p, v[2 * p], v[2 * p + 1]);
-        if (LAG && c.lagged) {
+        for (int c3 = 0; c3 < 3; ++c3) {
+            acc.add_prod(w * q[c3].x, q[c3].x);
+            acc.add_prod(w * q[c3].y, q[c3].y);
+            un[i + c3 * NT] = q[c3];
+        }
+        if (c.lagged) {
 #pragma unroll
-            for (int p = 0; p < 3; ++p) {
-                cpx<R> a[2], b[2], wn[2];
-                Six<R>::load_pair(wa + i, p, a[0], a[1]);
-                Six<R>::load_pair(wb + i, p, b[0], b[1]);
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const cpx<R> &o = uo[2 * p + q];
-                    wn[q] = mk<R>((o.x * c.ib - c.d * a[q].x - c.e * b[q].x) * c.ig,
-                                  (o.y * c.ib - c.d * a[q].y - c.e * b[q].y) * c.ig);
-                }
-                Six<R>::store_pair(wb + i, p, wn[0], wn[1]);
+            for (int c3 = 0; c3 < 3; ++c3) {
+                const size_t ic = i + c3 * NT;
+                const cpx<R> o = uo[c3], a = wa[ic], b = wb[ic];
+                const cpx<R> wn = mk<R>((o.x * c.ib - c.d * a.x - c.e * b.x) * c.ig,
+                                        (o.y * c.ib - c.d * a.y - c.e * b.y) * c.ig);
+                wb[ic] = wn;
                 if (c.xstep) {
-                    cpx<R> xx[2];
-                    Six<R>::load_pair(x + i, p, xx[0], xx[1]);
-#pragma unroll
-                    for (int q = 0; q < 2; ++q)
-                        xx[q] = mk<R>(xx[q].x + c.t2 * b[q].x + c.t1 * a[q].x + c.tau * wn[q].x,
-                                      xx[q].y + c.t2 * b[q].y + c.t1 * a[q].y + c.tau * wn[q].y);
-                    Six<R>::store_pair(x + i, p, xx[0], xx[1]);
+                    const cpx<R> xx = x[ic];
+                    x[ic] = mk<R>(xx.x + c.t2 * b.x + c.t1 * a.x + c.tau * wn.x,
+                                  xx.y + c.t2 * b.y + c.t1 * a.y + c.tau * wn.y);
                 }
             }
         }
-        gamma_apply<R>(g, ge, v);
+        gamma_from_q<R>(g, ge, q, v);
 #pragma unroll
         for (int p = 0; p < 3; ++p) Six<R>::store_pair(sp, p, v[2 * p], v[2 * p + 1]);
     }
-    group_sync(nsync);
-    // 3. inverse DFT along n1 of G u_{k+1}
-    return Fft::template run<1>(res, res == buf ? buf2 : buf, L, g.ax[0], nsync);
+    __syncthreads();
+    // 3. inverse DFT along n1 of the strain of u_{k+1}
+    return run_fft<R, 1, NF>(res, res == buf ? buf2 : buf, L, L, g.ax[0]);
 }
 
 // At most 384 threads per CTA (set_shapes enforces it): the fused pass keeps
-// the Lanczos operands of a frequency (five Krylov vectors, 60 values) in
+// the Lanczos operands of a frequency in
 // registers, so it is not held to a register cap that would spill them.
 #define HOM_X1L_BOUNDS(R) __launch_bounds__(384, 1)
 
@@ -1253,8 +1330,8 @@ __global__ void HOM_X1L_BOUNDS(R) k_x1_lanczos(Geometry g, cpx<R> *__restrict__ 
     }
     __syncthreads();
     Acc<R> acc;
-    cpx<R> *res = x1_lanczos_tile<R, PassFft<R, NF>, true>(g, T, buf, buf2, g0, c, uk + ko, um + ko, un + ko, wa + ko, wb + ko,
-                                               x + ko, acc, 0);
+    cpx<R> *res = x1_lanczos_tile<R, NF>(g, buf, buf2, g0, c, uk + ko, um + ko, un + ko, wa + ko, wb + ko, x + ko, acc,
+                                          fold.st + cs);
     if (live) {
         cpx<R> *dst = spec + (size_t)g0 * NC + lt;
         for (int e = e0; e < N; e += es) dst[e * sK1] = res[e * L + lt];
@@ -1308,19 +1385,52 @@ __global__ void __launch_bounds__(kEwThreads) k_lanczos_update(int n, int h, int
     if (threadIdx.x == 0) partials[blockIdx.x] = s;
 }
 
-// standard half-spectrum order <-> n1-tile order (see Geometry::kvec):
-// element (k1, col, c) of the standard order, col = k2 h + k3, sits in the
-// tile order at (col / T) n1 6T + k1 6T + (col % T) 6 + c
+// A spectrum in standard order -> a Krylov vector (see Geometry::kvec): q =
+// B^H in, with the weighted partial ||q||^2; frequency (k1, col), col = k2 h +
+// k3, component c sits at (col / T) krylov_tile + c n1 T + k1 T + col % T.
 template <typename R>
-__global__ void k_tiles(long long n, int n1, int cols, int T, int to_tiles, const cpx<R> *__restrict__ in,
-                        cpx<R> *__restrict__ out) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(i % 6);
-        const long long f = i / 6;
-        const int col = (int)(f % cols), k1 = (int)(f / cols);
-        const long long t = (long long)(col / T) * n1 * 6 * T + (long long)k1 * 6 * T + (col % T) * 6 + c;
-        if (to_tiles) out[t] = in[i];
-        else out[i] = in[t];
+__global__ void __launch_bounds__(kEwThreads) k_to_krylov(Geometry g, const cpx<R> *__restrict__ in,
+                                                          cpx<R> *__restrict__ out, double *__restrict__ partials) {
+    const int cols = g.n2 * g.h, T = g.tile1l, NT = g.n1 * T;
+    Acc<R> acc;
+    for (long long f = (long long)blockIdx.x * blockDim.x + threadIdx.x; f < g.S; f += (long long)gridDim.x * blockDim.x) {
+        const int k1 = (int)(f / cols), col = (int)(f - (long long)k1 * cols);
+        const int k2 = col / g.h, k3 = col - k2 * g.h;
+        cpx<R> t[6], q[3];
+#pragma unroll
+        for (int p = 0; p < 3; ++p) Six<R>::load_pair(in + 6 * f, p, t[2 * p], t[2 * p + 1]);
+        gamma_to_q<R>(g, gamma_e<R>(g, k1, k2, k3), t, q);
+        cpx<R> *o = out + (size_t)(col / T) * krylov_tile(g.n1, T) + (size_t)k1 * T + col % T;
+        const R w = (R)pweight(k3, g.n3);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            o[(size_t)c * NT] = q[c];
+            acc.add_prod(w * q[c].x, q[c].x);
+            acc.add_prod(w * q[c].y, q[c].y);
+        }
+    }
+    const double s = block_sum(acc.value());
+    if (threadIdx.x == 0) partials[blockIdx.x] = s;
+}
+
+// and back: out = B q
+template <typename R>
+__global__ void __launch_bounds__(kEwThreads) k_from_krylov(Geometry g, const cpx<R> *__restrict__ in,
+                                                            cpx<R> *__restrict__ out, const MinresState *state) {
+    const int cols = g.n2 * g.h, T = g.tile1l, NT = g.n1 * T;
+    for (long long f = (long long)blockIdx.x * blockDim.x + threadIdx.x; f < g.S; f += (long long)gridDim.x * blockDim.x) {
+        const int k1 = (int)(f / cols), col = (int)(f - (long long)k1 * cols);
+        const int k2 = col / g.h, k3 = col - k2 * g.h;
+        const cpx<R> *o = in + (size_t)(col / T) * krylov_tile(g.n1, T) + (size_t)k1 * T + col % T;
+        const cpx<R> q[3] = {o[0], o[(size_t)NT], o[2 * (size_t)NT]};
+        cpx<R> t[6];
+        gamma_from_q<R>(g, gamma_e<R>(g, k1, k2, k3), q, t);
+        if (f == 0 && state->dc) {
+#pragma unroll
+            for (int c = 0; c < 6; ++c) t[c] = mk<R>((R)state->dc_x[c], 0);
+        }
+#pragma unroll
+        for (int p = 0; p < 3; ++p) Six<R>::store_pair(out + 6 * f, p, t[2 * p], t[2 * p + 1]);
     }
 }
 
@@ -1476,12 +1586,13 @@ int Launch<R>::x3r_grid(const Geometry &g) {
             cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
             if (!k.fn || k.smem + 1024 > (size_t)optin) return 0;
             line_kernel_attr((const void *)k.fn, optin);
+            line_kernel_attr((const void *)k.fn_sums, optin);
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k.fn, k.threads, k.smem);
             return nb * sms;
         }
         const size_t sm = x3r_smem(g.n3);
         if (g.n3 != 256) return 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_x3r<256>, kX3rWarps * 32, sm);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_x3r<256, false>, kX3rWarps * 32, sm);
         return nb * sms;
     }
 }
@@ -1542,7 +1653,8 @@ void Launch<R>::table_init(const Geometry &) {
     HOM_SET_ATTR1((k_x1_tma_expand<R, NF>))
         HOM_SET_TMA(64) HOM_SET_TMA(96) HOM_SET_TMA(128) HOM_SET_TMA(160) HOM_SET_TMA(256) HOM_SET_TMA(512)
 #undef HOM_SET_TMA
-        HOM_SET_ATTR1((k_x3r<256>))
+        HOM_SET_ATTR1((k_x3r<256, false>))
+        HOM_SET_ATTR1((k_x3r<256, true>))
     }
 #undef HOM_SET_ATTR
 #undef HOM_SET_ATTR1
@@ -1596,13 +1708,14 @@ void Launch<R>::tma_grids(Geometry &g) {
         }
         // the fused MINRES n1 pass: the transform group plus the lagged-update
         // warps, whose ring takes as many stages (up to kX1LagMaxStages) as
-        // leave room for two CTAs per SM
+        // leave room for as many CTAs per SM as the registers do
         if (g.grp1l) {
             const X1lLineFn f = x1l_line_kernel(g.n1);
-            const int t = g.grp1l + kX1LagThreads;
-            const size_t tiles = 2 * g.stage1l, ring = 4 * (size_t)kX1LagChunk, fixed = 15 * 1024;   // static + reserved per CTA
+            const int t = g.grp1l + x1l_lag_threads(g.grp1l);
+            const int ctas = t <= 192 ? 4 : 3;
+            const size_t tiles = 2 * g.stage1l, ring = 4 * (size_t)kX1LagChunk, fixed = 2560;   // static + reserved per CTA
             int st = kX1LagMaxStages;
-            while (st > 1 && 2 * (tiles + st * ring + fixed) > (size_t)smem_sm) --st;
+            while (st > 1 && ctas * (tiles + st * ring + fixed) > (size_t)smem_sm) --st;
             g.x1_lag_stages = st;
             g.smem1l_tma = tiles + st * ring;
             int b = 0;
@@ -1621,23 +1734,23 @@ void Launch<R>::x3(const Geometry &g, cudaStream_t st, int in_mode, const void *
                    const double *macro, double scl, int out_mode, void *out, const R *phi,
                    const MinresState *state, double *epart, Fold fold, double *tsum) {
     if constexpr (sizeof(R) == 4) {
-        if (!tsum && g.x3l && g.nc == 6 && in_mode == X3_IN_SPEC && out_mode == X3_OUT_SPEC && scl == 1.0 &&
+        if (g.x3l && g.nc == 6 && in_mode == X3_IN_SPEC && out_mode == X3_OUT_SPEC && scl == 1.0 &&
             (mid == X3_MID_MATERIAL || mid == X3_MID_NONE)) {
             const X3Line k = x3_line_kernel(g.n3);
-            launch_k(g.pdl, k.fn, x3_epart_grid(g), k.threads, k.smem, st, g, reinterpret_cast<const float2 *>(in),
+            launch_k(g.pdl, tsum ? k.fn_sums : k.fn, x3_epart_grid(g), k.threads, k.smem, st, g, reinterpret_cast<const float2 *>(in),
                      reinterpret_cast<float2 *>(out), mid == X3_MID_MATERIAL ? 1 : 0, (float)lam, (float)(2.0 * mu),
-                     (const float *)phi, state, epart, fold);
+                     (const float *)phi, state, epart, fold, tsum);
             return;
         }
-        if (!tsum && g.x3r && g.nc == 6 && in_mode == X3_IN_SPEC && out_mode == X3_OUT_SPEC && scl == 1.0 &&
+        if (g.x3r && g.nc == 6 && in_mode == X3_IN_SPEC && out_mode == X3_OUT_SPEC && scl == 1.0 &&
             (mid == X3_MID_MATERIAL || mid == X3_MID_NONE)) {
             const int grid = g.grid3r;   // persistent: every case's row groups
             const size_t sm = x3r_smem(g.n3);
             const int mat = mid == X3_MID_MATERIAL;
             const float2 *fi = reinterpret_cast<const float2 *>(in);
             float2 *fo = reinterpret_cast<float2 *>(out);
-            launch_k(g.pdl, k_x3r<256>, grid, 128, sm, st, g, fi, fo, mat, (float)lam, (float)(2.0 * mu),
-                     (const float *)phi, state, epart, fold);
+            launch_k(g.pdl, tsum ? k_x3r<256, true> : k_x3r<256, false>, grid, 128, sm + (tsum ? sizeof(double) * 6 * g.nb * kX3rWarps : 0), st, g, fi, fo, mat, (float)lam, (float)(2.0 * mu),
+                     (const float *)phi, state, epart, fold, tsum);
             return;
         }
     }
@@ -1772,7 +1885,7 @@ void Launch<R>::x1_lanczos(const Geometry &g, cudaStream_t st, cpx<R> *spec, con
     if constexpr (sizeof(R) == 4) {
         if (g.grid1l_tma > 0) {
             const CUtensorMap *ts = tma_map(g, spec, TMA_X1L, 1);
-            launch_k(g.pdl, x1l_line_kernel(g.n1), x1_lanczos_grid(g), g.grp1l + kX1LagThreads, g.smem1l_tma, st, g, *ts, uk,
+            launch_k(g.pdl, x1l_line_kernel(g.n1), x1_lanczos_grid(g), g.grp1l + x1l_lag_threads(g.grp1l), g.smem1l_tma, st, g, *ts, uk,
                      um, un, wa, wb, x, state, partials, fold);
             return;
         }
@@ -1786,15 +1899,16 @@ void Launch<R>::x1_lanczos(const Geometry &g, cudaStream_t st, cpx<R> *spec, con
 }
 
 template <typename R>
-void Launch<R>::to_tiles(const Geometry &g, cudaStream_t st, const cpx<R> *in, cpx<R> *out) {
-    const long long n = 6 * g.S;
-    k_tiles<R><<<ew_grid(n), kEwThreads, 0, st>>>(n, g.n1, g.n2 * g.h, g.tile1l, 1, in, out);
+int Launch<R>::to_krylov(const Geometry &g, cudaStream_t st, const cpx<R> *in, cpx<R> *out, double *partials) {
+    const int nb = ew_grid(g.S);
+    k_to_krylov<R><<<nb, kEwThreads, 0, st>>>(g, in, out, partials);
+    return nb;
 }
 
 template <typename R>
-void Launch<R>::from_tiles(const Geometry &g, cudaStream_t st, const cpx<R> *in, cpx<R> *out) {
-    const long long n = 6 * g.S;
-    k_tiles<R><<<ew_grid(n), kEwThreads, 0, st>>>(n, g.n1, g.n2 * g.h, g.tile1l, 0, in, out);
+void Launch<R>::from_krylov(const Geometry &g, cudaStream_t st, const cpx<R> *in, cpx<R> *out,
+                            const MinresState *state) {
+    k_from_krylov<R><<<ew_grid(g.S), kEwThreads, 0, st>>>(g, in, out, state);
 }
 
 template <typename R>

@@ -4,7 +4,7 @@
 namespace hom {
 X1lLineFn x1l_line_kernel_c(int n) {
     switch (n) {
-#define HOM_CASE(N) case N: return k_x1_lanczos_tma<float, N>;
+#define HOM_CASE(N) case N: if constexpr (x1l_cols(N, LinePlan<N>::TPL) > 0) return k_x1_lanczos_tma<float, N>; else return nullptr;
         HOM_LINE_LENGTHS_C(HOM_CASE)
 #undef HOM_CASE
         default: return nullptr;

@@ -83,10 +83,12 @@ template <int N> struct X3Plan {
     static constexpr int CTAS = BY_SMEM < BY_REGS ? BY_SMEM : BY_REGS;
 };
 
-template <int N>
+// SUMS: the per-CTA stress sums (tsum of Launch::x3) too
+template <int N, bool SUMS>
 __global__ void __launch_bounds__(X3Plan<N>::NT, X3Plan<N>::CTAS)
     k_x3_line(Geometry g, const float2 *__restrict__ in, float2 *__restrict__ out, int material, float lam, float mu2,
-              const float *__restrict__ phi, const MinresState *state, double *__restrict__ epart, Fold fold) {
+              const float *__restrict__ phi, const MinresState *state, double *__restrict__ epart, Fold fold,
+              double *__restrict__ tsum) {
     pdl_release();
     pdl_wait();   // predecessor complete (programmatic launch in the MINRES graph)
     using P = X3Plan<N>;
@@ -97,6 +99,8 @@ __global__ void __launch_bounds__(X3Plan<N>::NT, X3Plan<N>::CTAS)
     __shared__ double sacc[kNbMax * (NT / 32)];   // energy of each case, one running sum a warp
     const float4 *stg = reinterpret_cast<const float4 *>(smem_raw);     // [row][k][line]
     float2 *w = reinterpret_cast<float2 *>(smem_raw + P::STAGE);        // exchange buffer
+    __shared__ double ssum[SUMS ? 6 * kNbMax * (NT / 32) : 1];   // the same for the stress components
+    __shared__ Acc<float> sff[SUMS ? 6 * NT : 1];                // and each thread's sums of the running case
     const int tid = threadIdx.x;
     const bool leader = tid == 0;
     const int nrows = g.n1 * g.n2;
@@ -109,6 +113,11 @@ __global__ void __launch_bounds__(X3Plan<N>::NT, X3Plan<N>::CTAS)
         fence_mbar_init();
     }
     for (int i = tid; i < kNbMax * (NT / 32); i += NT) sacc[i] = 0.0;
+    if constexpr (SUMS)
+    {
+        for (int i = tid; i < 6 * kNbMax * (NT / 32); i += NT) ssum[i] = 0.0;
+        for (int c = 0; c < 6; ++c) sff[c * NT + tid] = Acc<float>{};
+    }
     __syncthreads();
     auto live_from = [&](int t) {
         while (t < ntiles && skip_case(state, t / tpc)) t += gridDim.x;
@@ -120,6 +129,7 @@ __global__ void __launch_bounds__(X3Plan<N>::NT, X3Plan<N>::CTAS)
         mbar_expect_tx(&bar, bytes);
         bulk_load(smem_raw, in + ((size_t)cs * nrows + row0) * (H * 6), bytes, &bar);
     };
+    Acc<float> eacc;   // this thread's energy of the running case
     int tile = live_from(blockIdx.x);
     if (leader && tile < ntiles) issue(tile);
     for (int it = 0; tile < ntiles; ++it) {
@@ -175,7 +185,7 @@ __global__ void __launch_bounds__(X3Plan<N>::NT, X3Plan<N>::CTAS)
                 for (int r = 0; r < B; ++r) z[p][r] = o[p * PS + r * A1];
         }
         __syncthreads();
-        float en = 0.f;
+        float en = 0.f, ts[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};   // sums over B voxels
         if (live2) {
             const float2 *twj;
             asm volatile("mov.b64 %0, %1;" : "=l"(twj) : "l"(tw));
@@ -205,7 +215,10 @@ __global__ void __launch_bounds__(X3Plan<N>::NT, X3Plan<N>::CTAS)
                     for (int c = 1; c < 6; ++c) ee += t[c] * t[c];
                     en += ph[r] * (tr * sum + mu2 * ee);
 #pragma unroll
-                    for (int c = 0; c < 6; ++c) t[c] = ph[r] * ((c < 3 ? tr : 0.f) + mu2 * t[c]);
+                    for (int c = 0; c < 6; ++c) {
+                        t[c] = ph[r] * ((c < 3 ? tr : 0.f) + mu2 * t[c]);
+                        if constexpr (SUMS) ts[c] += t[c];
+                    }
 #pragma unroll
                     for (int p = 0; p < 3; ++p) z[p][r] = make_float2(t[2 * p], t[2 * p + 1]);
                 }
@@ -223,9 +236,27 @@ __global__ void __launch_bounds__(X3Plan<N>::NT, X3Plan<N>::CTAS)
                 for (int r = 0; r < B; ++r) o[p * PS + r] = z[p][r];
             }
         }
-        if (epart) {
-            const double ws = warp_sum((double)en);
+        // reduced over the warp once a case, not once a tile: FP64 adds run at
+        // a small rate (six sums a tile took 17 of 50 us at 128^3)
+        const bool last = next >= ntiles || next / tpc != cs;
+        eacc.add(en);
+        if (epart && last) {
+            const double ws = warp_sum(eacc.value());
             if ((tid & 31) == 0) sacc[cs * (NT / 32) + (tid >> 5)] += ws;
+            eacc = Acc<float>{};
+        }
+        if constexpr (SUMS) {
+#pragma unroll
+            for (int c = 0; c < 6; ++c) {
+                Acc<float> s = sff[c * NT + tid];
+                s.add(ts[c]);
+                if (last) {
+                    const double ws = warp_sum(s.value());
+                    if ((tid & 31) == 0) ssum[(c * kNbMax + cs) * (NT / 32) + (tid >> 5)] += ws;
+                    s = Acc<float>{};
+                }
+                sff[c * NT + tid] = s;
+            }
         }
         __syncthreads();
         // ---- 3: forward radix-A butterflies u and v = B - u (mod B) of line p:
@@ -271,6 +302,15 @@ __global__ void __launch_bounds__(X3Plan<N>::NT, X3Plan<N>::CTAS)
             }
         }
         tile = next;   // (the barrier after the next wait: the exchange buffer is read)
+    }
+    if constexpr (SUMS) {
+        __syncthreads();
+        if (tid < 6 * g.nb) {
+            const int c = tid / g.nb, cc = tid - c * g.nb;
+            double t = 0.0;
+            for (int i = 0; i < NT / 32; ++i) t += ssum[(c * kNbMax + cc) * (NT / 32) + i];
+            tsum[(size_t)tid * gridDim.x + blockIdx.x] = t;   // = tsum[(c * nb + case) * grid + block]
+        }
     }
     if (epart) {
         __syncthreads();

@@ -4,7 +4,7 @@
 namespace hom {
 X3Line x3_line_kernel_b(int n) {
     switch (n) {
-#define HOM_CASE(N) case N: return X3Line{k_x3_line<N>, X3Plan<N>::NT, X3Plan<N>::ROWS, X3Plan<N>::SMEM};
+#define HOM_CASE(N) case N: return X3Line{k_x3_line<N, false>, k_x3_line<N, true>, X3Plan<N>::NT, X3Plan<N>::ROWS, X3Plan<N>::SMEM};
         HOM_X3_LENGTHS_B(HOM_CASE)
 #undef HOM_CASE
         default: return X3Line{};
