@@ -4,10 +4,12 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -300,16 +302,30 @@ __global__ void k_colsum_reduce(int nb, int C, int cout, const float *partials, 
     if (lane == 0) out[c] = s;
 }
 
-// dW[t][co][ci] (logical sizes) = sum over splits of the padded partials
-__global__ void k_wgrad_reduce(int S, int cout_p, int cin_s, int cout, int cin, const float *__restrict__ partial,
-                               float *__restrict__ dW) {
-    const long long total = 27LL * cout * cin;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        const int ci = (int)(i % cin);
-        const long long r = i / cin;
-        const int co = (int)(r % cout), t = (int)(r / cout);
-        float s = 0.f;
-        for (int k = 0; k < S; ++k) s += partial[(((long long)k * 27 + t) * cout_p + co) * cin_s + ci];
+// dW[t][co][ci] (logical sizes) = sum over splits of the padded partials: 32
+// values a block, each by eight threads that take every eighth split (one
+// thread a value waited for up to 256 loads in 27 blocks: 53 us at 16 x 16
+// channels and 256 splits, 16 here)
+constexpr int kRedVals = 32, kRedWays = 8;
+__global__ void __launch_bounds__(kRedVals *kRedWays) k_wgrad_reduce(int S, int cout_p, int cin_s, int cout, int cin,
+                                                                     const float *__restrict__ partial,
+                                                                     float *__restrict__ dW) {
+    __shared__ float part[kRedWays][kRedVals];
+    const int lane = threadIdx.x % kRedVals, way = threadIdx.x / kRedVals;
+    const int total = 27 * cout * cin, i = blockIdx.x * kRedVals + lane;
+    const long long stride = 27LL * cout_p * cin_s;
+    float s = 0.f;
+    if (i < total) {
+        const int ci = i % cin, r = i / cin, co = r % cout, t = r / cout;
+        const float *p = partial + ((long long)t * cout_p + co) * cin_s + ci;
+#pragma unroll 8
+        for (int k = way; k < S; k += kRedWays) s += p[k * stride];
+    }
+    part[way][lane] = s;
+    __syncthreads();
+    if (way == 0 && i < total) {
+#pragma unroll
+        for (int q = 1; q < kRedWays; ++q) s += part[q][lane];
         dW[i] = s;
     }
 }
@@ -420,9 +436,34 @@ long long level_vox(const hom_net *n, int B, const int g[3], int level) {
     return (long long)B * (g[0] >> level) * (g[1] >> level) * (g[2] >> level);
 }
 
-int wgrad_splits(long long vox) {
-    long long s = (vox + 4095) / 4096;
-    return (int)(s < 1 ? 1 : (s > 256 ? 256 : s));
+// Scratch of hom_net_conv3d_wgrad: a stream-ordered pool per device, so that
+// a call does not pay for cudaMalloc and cudaFree (about 150 us together); it
+// keeps at most 64 MB between calls.
+cudaMemPool_t scratch_pool() {
+    constexpr int kDevices = 64;
+    static cudaMemPool_t pools[kDevices] = {};
+    static std::mutex m;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev >= kDevices) return nullptr;
+    std::lock_guard<std::mutex> lock(m);
+    if (!pools[dev]) {
+        cudaMemPoolProps pp = {};
+        pp.allocType = cudaMemAllocationTypePinned;
+        pp.location.type = cudaMemLocationTypeDevice;
+        pp.location.id = dev;
+        if (cudaMemPoolCreate(&pools[dev], &pp) != cudaSuccess) return pools[dev] = nullptr;
+        uint64_t keep = 64ull << 20;
+        cudaMemPoolSetAttribute(pools[dev], cudaMemPoolAttrReleaseThreshold, &keep);
+    }
+    return pools[dev];
+}
+
+// Voxel splits of a weight gradient: about one wave of two CTAs per SM over the
+// input chunks and the groups of 16 output channels, a kilovoxel (eight planes
+// of a column) at least (a fixed 4096 left 64 CTAs at 64^3 and four at 20^3 x 2)
+int wgrad_splits(long long vox, int cin_s, int cout) {
+    const long long wave = 304 / std::max(1, (cin_s / 16) * (cout / 16)), s = (vox + 1023) / 1024;
+    return (int)std::max(1LL, std::min(s, wave));
 }
 
 int ensure_ws(hom_net *n, int B, const int g[3]) {
@@ -436,7 +477,7 @@ int ensure_ws(hom_net *n, int B, const int g[3]) {
         else rc = alloc(n, &n->act[l], (size_t)vox * L.cout_p);
         if (!rc) rc = alloc(n, &n->G[l], (size_t)vox * L.cout_p);
         if (!rc && l != E1A) rc = alloc(n, &n->dX[l], (size_t)vox * L.cin_s);
-        const size_t pf = (size_t)wgrad_splits(vox) * 27 * L.cout_p * L.cin_s;
+        const size_t pf = (size_t)wgrad_splits(vox, L.cin_s, L.cout_p) * 27 * L.cout_p * L.cin_s;
         if (pf > n->partial_floats) n->partial_floats = pf;
     }
     for (int k = 0; k < 3 && !rc; ++k) {
@@ -588,9 +629,9 @@ int layer_back(hom_net *n, int l, int B, const int g[3]) {
     w.G = n->G[l];
     w.cout = L.cout_p;
     w.partial = n->partial;
-    w.S = wgrad_splits(vox);
+    w.S = wgrad_splits(vox, L.cin_s, L.cout_p);
     if (conv3_wgrad(w, n->stream)) return set_err(HOM_EINVAL, "weight-gradient shape not supported");
-    k_wgrad_reduce<<<ew_blocks(27LL * L.d.cout * L.d.cin), kEw, 0, n->stream>>>(
+    k_wgrad_reduce<<<(27 * L.d.cout * L.d.cin + kRedVals - 1) / kRedVals, kRedVals * kRedWays, 0, n->stream>>>(
         w.S, L.cout_p, L.cin_s, L.d.cout, L.d.cin, n->partial, n->grads + L.off);
     const int nb = ew_blocks(vox);
     k_colsum<<<nb, kEw, kEw * sizeof(float), n->stream>>>(vox, L.cout_p, n->G[l], n->colpart);
@@ -952,20 +993,23 @@ int hom_net_conv3d_wgrad(int batch, const int grid[3], const unsigned short *G, 
     w.G = reinterpret_cast<const bf16 *>(G);
     w.cout = cout;
     const long long vox = (long long)batch * grid[0] * grid[1] * grid[2];
-    w.S = wgrad_splits(vox);
     const int cin_s = c0s + c1s;
+    w.S = wgrad_splits(vox, cin_s, cout);
     float *partial = nullptr;
     cudaStream_t st = (cudaStream_t)stream;
-    NCU(cudaMalloc(&partial, sizeof(float) * w.S * 27 * cout * cin_s));
+    cudaMemPool_t pool = scratch_pool();
+    const size_t bytes = sizeof(float) * w.S * 27 * cout * cin_s;
+    if (!pool || cudaMallocFromPoolAsync((void **)&partial, bytes, pool, st) != cudaSuccess)
+        return set_err(HOM_ENOMEM, "device allocation failed");
     w.partial = partial;
     if (conv3_wgrad(w, st)) {
-        cudaFree(partial);
+        cudaFreeAsync(partial, st);
         return set_err(HOM_EINVAL, "channel counts must be multiples of 16, cout <= 64");
     }
-    k_wgrad_reduce<<<ew_blocks(27LL * cout * cin_s), kEw, 0, st>>>(w.S, cout, cin_s, cout, cin_s, partial, dW);
+    k_wgrad_reduce<<<(27 * cout * cin_s + kRedVals - 1) / kRedVals, kRedVals * kRedWays, 0, st>>>(w.S, cout, cin_s, cout, cin_s, partial, dW);
     cudaError_t e = cudaGetLastError();
+    cudaFreeAsync(partial, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cudaFree(partial);
     if (e != cudaSuccess) return set_err(HOM_ECUDA, cudaGetErrorString(e));
     return HOM_OK;
 }

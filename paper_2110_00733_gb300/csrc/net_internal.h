@@ -22,6 +22,7 @@ struct ConvArgs {
     int relu;
     __nv_bfloat16 *out_bf16;
     float *out_f32;
+    int *err;               // set when a bounded wait gives up (filled in by the launchers)
 };
 
 // Weight gradient of a convolution whose input is described by `in` (sources
@@ -38,7 +39,7 @@ struct WgradArgs {
 int conv3_forward_tc(const ConvArgs &a, cudaStream_t st);   // tcgen05, cout <= 256
 // nonzero if a tcgen05 convolution gave up a bounded wait (clears it if asked)
 int conv3_tc_error(int clear);
-int conv3_wgrad(const WgradArgs &a, cudaStream_t st);      // tcgen05 where bricks tile the grid, else mma.sync
+int conv3_wgrad(const WgradArgs &a, cudaStream_t st);      // tcgen05, or mma.sync where that does not take the shape
 int conv3_wgrad_tc(const WgradArgs &a, cudaStream_t st);   // -1 if the shape does not suit it
 
 }  // namespace hnet

@@ -16,17 +16,18 @@
 // core matrices of 8 rows x 16 bytes, K-adjacent core matrices LBO = 128 B
 // apart, 8-row groups SBO = 1024 B apart.
 //
-// Every wait is bounded; on a timeout the kernel records it in g_tc_err,
+// Every wait is bounded; on a timeout the kernel records it in *ConvArgs::err,
 // waits (bounded) for its own MMAs, frees its tensor memory and returns.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <initializer_list>
+#include <mutex>
+
 #include "net_internal.h"
 
 namespace hnet {
-
-__device__ int g_tc_err;
 
 namespace {
 
@@ -190,7 +191,7 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tc(ConvArgs a, int ncols) {
                 mma_commit(&done);
             } else {
                 abort_flag = 1;
-                atomicExch(&g_tc_err, 1);
+                atomicExch(a.err, 1);
                 // let the issued MMAs drain (bounded) before the accumulator is freed
                 for (int s = 0; s < kStages; ++s)
                     if (ncommit[s] > 0) mbar_wait(&empty[s], (uint32_t)(ncommit[s] - 1) & 1u);
@@ -273,7 +274,7 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tc(ConvArgs a, int ncols) {
                 }
             }
         } else if (tid == 0) {
-            atomicExch(&g_tc_err, 1);
+            atomicExch(a.err, 1);
         }
     }
     tc_fence_before();
@@ -368,7 +369,7 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tch(ConvArgs a, int ncols) {
                 mma_commit(&done);
             } else {
                 abort_flag = 1;
-                atomicExch(&g_tc_err, 1);
+                atomicExch(a.err, 1);
                 for (int q = 0; q < kHSt; ++q)
                     if (ncommit[q] > 0) mbar_wait(&empty[q], (uint32_t)(ncommit[q] - 1) & 1u);
             }
@@ -467,7 +468,7 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tch(ConvArgs a, int ncols) {
                 }
             }
         } else if (tid == 0) {
-            atomicExch(&g_tc_err, 1);
+            atomicExch(a.err, 1);
         }
     }
     tc_fence_before();
@@ -574,7 +575,7 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tcd(ConvArgs a, int ncols, i
                 mma_commit(&done);
             } else {
                 abort_flag = 1;
-                atomicExch(&g_tc_err, 1);
+                atomicExch(a.err, 1);
                 for (int q = 0; q < 2; ++q)
                     if (ncommit[q] > 0) mbar_wait(&empty[q], (uint32_t)(ncommit[q] - 1) & 1u);
             }
@@ -656,7 +657,7 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tcd(ConvArgs a, int ncols, i
                 }
             }
         } else if (tid == 0) {
-            atomicExch(&g_tc_err, 1);
+            atomicExch(a.err, 1);
         }
     }
     tc_fence_before();
@@ -738,7 +739,7 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tcp(ConvArgs a, int ncols) {
             }
             if (!ok) {
                 abort_flag = 1;
-                atomicExch(&g_tc_err, 1);
+                atomicExch(a.err, 1);
                 for (int q = 0; q < 2; ++q) {
                     if (nh[q] > 0) mbar_wait(&hempty[q], (uint32_t)(nh[q] - 1) & 1u);
                     if (na[q] > 0) mbar_wait(&afull[q], (uint32_t)(na[q] - 1) & 1u);
@@ -847,7 +848,7 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tcp(ConvArgs a, int ncols) {
         asm volatile("cp.async.wait_all;" ::: "memory");
         if (!ok) {
             abort_flag = 1;
-            if (tid == 0) atomicExch(&g_tc_err, 1);
+            if (tid == 0) atomicExch(a.err, 1);
         }
     }
     tc_fence_before();
@@ -857,83 +858,86 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tcp(ConvArgs a, int ncols) {
 }
 
 // ---------------------------------------------------------------------------
-// Weight gradient on tcgen05: dW[t][co][ci] = sum_v G[v][co] X[v + d_t][ci].
-// D rows are (tap, input channel) pairs, 8 taps x 16 channels = 128 per tap
-// group (4 groups cover 27 taps), N = c_out, K = the 128 voxels of a brick.
-// Both operands are MN-major, which is their natural layout: a 16-byte row
-// of a core matrix is 8 channels of one voxel (X rows out of the halo, G
-// rows out of the output gradient), 8 voxels per core matrix; MN-adjacent
-// core matrices 2048 B apart, K-adjacent ones 128 B.  Without swizzling the
-// descriptor of an MN-major operand takes the K-direction stride as its
-// leading byte offset and the MN-direction stride as its stride byte offset
-// (as for K-major operands, where the 8-row groups run along MN).  A CTA takes
-// one 16-channel chunk of the input and a range of bricks, keeps the four
-// group accumulators in tensor memory, and writes its split's partial sums.
+// Column convolution: a CTA marches a tile of 8 x 16 voxels (x, y) through up
+// to zl planes of z.  Every input plane (its periodic halo of 10 x 18 voxels,
+// one 16-channel chunk at a time) is read once and multiplied for all three
+// output planes it reaches: for a tap (dy, dx) one MMA of M = 128 voxels and
+// N = 3 c_out, whose B rows are the weights of dz = +1, 0, -1, and whose
+// accumulator columns are those of the output planes z-1, z, z+1, side by side
+// in tensor memory (plane q at column q c_out).  Nine MMAs a plane and chunk in
+// place of 27: reading A (4 KB an MMA) from shared memory bounds the small-N
+// products of this network, so a third of the reads is a third of the time.
+// The halo of a brick (2.8 loads per voxel) becomes 1.4 (1 + 2/zl).
+// Persistent: four warps load planes, one issues the MMAs, four take an item's
+// accumulators to the output while the next item fills the other half of the
+// tensor memory; a CTA keeps the weights of all chunks where they fit.
+// A in place: plane rows of 16 bytes (8 channels), channel halves kPHalf apart;
+// the 8 voxels of an x run are one core matrix, y runs 160 B apart, and a tap
+// only moves the start.  The plane that a chunk-0 plane reaches first (z+1)
+// starts its accumulator with that plane's first tap.
+// Measured (64^3 x 8, 16 -> 16 channels, a call with its synchronisation): 76 us
+// against 163 with k_conv3_tcp (27 MMAs a brick); 24 us of a call are the
+// launch and the synchronisation.  An MMA of these sizes takes 85 to 100 cycles
+// whatever its N, which makes 53 us of the nine a plane.
 // ---------------------------------------------------------------------------
-constexpr int kWgMn = 2048;        // MN-adjacent core matrices (16 K-groups x 128 B): SBO
-constexpr int kWgK = 128;          // K-adjacent core matrices: LBO
-constexpr int kWgATile = 16 * kWgMn;   // 128 rows x 128 K, 32 KB
+constexpr int kPX = 8, kPY = 16, kPHX = kPX + 2, kPRows = kPHX * (kPY + 2);   // tile, halo rows
+constexpr int kPHalf = kPRows * 16, kPPlane = 2 * kPHalf;
+constexpr int kPSlots = 12, kPDepth = 5;   // most halo planes in shared memory, loads in flight
+constexpr int kColThreads = 2 * kProducers + 32;   // loads, epilogue, MMA issue
 
-__device__ __forceinline__ uint64_t smem_desc_mn(uint32_t addr) {
-    return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)((kWgK >> 4) & 0x3FFF) << 16) |
-           ((uint64_t)((kWgMn >> 4) & 0x3FFF) << 32) | (1ull << 46);
+__device__ __forceinline__ uint64_t smem_desc_p(uint32_t addr) {   // K-major: LBO the channel half, SBO the next y
+    return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)((kPHalf >> 4) & 0x3FFF) << 16) |
+           ((uint64_t)((kPHX * 16 >> 4) & 0x3FFF) << 32) | (1ull << 46);
 }
 
-// kind::f16, FP32 accumulator, BF16 A and B, both MN-major (bits 15, 16)
-__device__ __forceinline__ uint32_t instr_desc_mn(int n) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((uint32_t)(n >> 3) << 17) |
-           ((uint32_t)(kBM >> 4) << 24);
+__device__ __forceinline__ int wrapm(int i, int n) {   // any distance
+    const int r = i % n;
+    return r < 0 ? r + n : r;
 }
 
-// A tile of tap group GRP for one voxel: rows (tap, channel half) of the
-// voxel's column, taken from the two halo planes at the taps' offsets (all
-// loads issued before the stores)
-template <int GRP>
-__device__ __forceinline__ void wg_copy(unsigned char *at, const unsigned char *hv) {
-    constexpr int kNt = GRP < 3 ? 8 : 3;
-    constexpr int kPlane = kHalo * 16;
-    uint4 r[2 * kNt];
+// the nine taps of one plane: B blocks [j0, j1] (output planes), fresh: block 2
+// starts its accumulator
+__device__ __forceinline__ void plane_mmas(uint32_t d, uint32_t ab, uint32_t bb, int N, int j0, int j1, bool fresh) {
+    const uint64_t ad = smem_desc_p(ab), bd = smem_desc_h(bb);
+    const uint64_t bstep = (uint64_t)(6 * N), blk = (uint64_t)(2 * N);   // 96 N and 32 N bytes, >> 4
+    const uint32_t idesc = instr_desc((j1 - j0 + 1) * N);
 #pragma unroll
-    for (int k = 0; k < kNt; ++k) {
-        const int t = GRP * 8 + k;
-        const int off = (((t / 9) * kHY + (t / 3) % 3) * kHX + t % 3) * 16;
-        r[2 * k] = *reinterpret_cast<const uint4 *>(hv + off);
-        r[2 * k + 1] = *reinterpret_cast<const uint4 *>(hv + kPlane + off);
+    for (int s = 0; s < 9; ++s) {
+        const uint64_t as = ad + (uint64_t)((s / 3) * kPHX + s % 3);
+        const uint64_t bs = bd + bstep * s;
+        if (s == 0 && fresh) {
+            if (j0 < 2) mma_bf16(d + j0 * N, as, bs + blk * j0, instr_desc((2 - j0) * N), 1u);
+            mma_bf16(d + 2 * N, as, bs + blk * 2, instr_desc(N), 0u);
+        } else {
+            mma_bf16(d + j0 * N, as, bs + blk * j0, idesc, 1u);
+        }
     }
-#pragma unroll
-    for (int m = 0; m < 2 * kNt; ++m) *reinterpret_cast<uint4 *>(at + m * kWgMn) = r[m];
 }
 
-__global__ void __launch_bounds__(kThreads) k_wgrad3_tc(WgradArgs w, int ncols, int bricks_per_cta) {
+// planes: halo planes in shared memory; wslots: chunks' weights there (all nch
+// of them: loaded once)
+template <int N>
+__global__ void __launch_bounds__(kColThreads) k_conv3_col(ConvArgs a, int ncols, int zl, int nplanes, int wslots) {
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ __align__(8) uint64_t full[2], empty[2], done;
+    __shared__ __align__(8) uint64_t full[kPSlots], empty[kPSlots], wempty[2], afull[2], aempty[2];
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int abort_flag;
-    const ConvArgs &a = w.in;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int N = w.cout;
-    const int cin_s = a.c0s + a.c1s;
-    const int cc = blockIdx.y;
-    const int split = blockIdx.x;
-    const int bx3 = a.n3 / 8, by2 = a.n2 / 4, bz1 = a.n1 / 4;
-    const long long nbricks = (long long)bx3 * by2 * bz1 * a.B;
-    const long long bb0 = (long long)split * bricks_per_cta;
-    const long long bb1 = bb0 + bricks_per_cta < nbricks ? bb0 + bricks_per_cta : nbricks;
-    constexpr int kMma = kProducers / 32;
-    if (bb0 >= bb1) {   // no voxels in this split: its partial sums are zero
-        for (int i = tid; i < 27 * N * 16; i += kThreads) {
-            const int ci = i % 16, r = i / 16, co = r % N, t = r / N;
-            w.partial[(((long long)split * 27 + t) * N + co) * cin_s + cc * 16 + ci] = 0.f;
-        }
-        return;
-    }
-    // two bricks in flight: halo[2] (two planes of 16-byte rows, channels
-    // 0-7 and 8-15), G tile[2], and the two A-tile stages
-    constexpr int kPlane = kHalo * 16;
-    const int gbytes = (N / 8) * kWgMn;
-    unsigned char *halo = smem;                              // 2 x 2 planes
-    unsigned char *gt = smem + 4 * kPlane;                   // 2 x G tile
-    unsigned char *ring = gt + 2 * gbytes;                   // 2 x A tile
+    const int cin_s = a.c0s + a.c1s, nch = cin_s / 16;
+    const bool resident = wslots >= nch;
+    constexpr int w_bytes = 27 * 32 * N;
+    unsigned char *planes = smem + wslots * w_bytes;
+    const int tx = (a.n3 + kPX - 1) / kPX, ty = (a.n2 + kPY - 1) / kPY, tz = (a.n1 + zl - 1) / zl;
+    const int items = tx * ty * tz * a.B;
+    constexpr int kMma = 2 * kProducers / 32;
+    // item -> its first voxel (x0, y0, z0, b) and number of output planes
+    auto decode = [&](int it, int &x0, int &y0, int &z0, int &b) {
+        x0 = it % tx * kPX; it /= tx;
+        y0 = it % ty * kPY; it /= ty;
+        z0 = it % tz * zl;
+        b = it / tz;
+        return a.n1 - z0 < zl ? a.n1 - z0 : zl;
+    };
 
     if (warp == kMma) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr(&tmem_slot)),
@@ -942,11 +946,15 @@ __global__ void __launch_bounds__(kThreads) k_wgrad3_tc(WgradArgs w, int ncols, 
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        for (int q = 0; q < 2; ++q) {
-            mbar_init(&full[q], kProducers);
+        for (int q = 0; q < nplanes; ++q) {
+            mbar_init(&full[q], kProducers / 32);
             mbar_init(&empty[q], 1);
         }
-        mbar_init(&done, 1);
+        for (int q = 0; q < 2; ++q) {
+            mbar_init(&wempty[q], 1);
+            mbar_init(&afull[q], 1);
+            mbar_init(&aempty[q], kProducers / 32);
+        }
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -954,129 +962,435 @@ __global__ void __launch_bounds__(kThreads) k_wgrad3_tc(WgradArgs w, int ncols, 
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
-    const int nst = (int)(bb1 - bb0) * 4;                    // (brick, tap group) stages
 
     if (warp == kMma) {
         if (lane == 0) {
-            int ncommit[2] = {0, 0};
-            const uint32_t idesc = instr_desc_mn(N);
             bool ok = true;
-            for (int c = 0; c < nst && ok; ++c) {
-                const int q = c & 1, grp = c & 3;
-                ok = mbar_wait(&full[q], (uint32_t)(c >> 1) & 1u) && !abort_flag;
+            int k = 0, q = 0, c = 0, n = 0;   // stages, slot, chunks and items done
+            uint32_t ph = 0;
+            for (int it = blockIdx.x; it < items && ok; it += gridDim.x, ++n) {
+                int x0, y0, z0, b;
+                const int nz = decode(it, x0, y0, z0, b), P = nz + 2;
+                if (n >= 2) ok = mbar_wait(&aempty[n & 1], (uint32_t)((n >> 1) - 1) & 1u) && !abort_flag;
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t ab = saddr(ring + q * kWgATile);
-                const uint32_t gb = saddr(gt + ((c >> 2) & 1) * gbytes);
+                const uint32_t acc = tmem + (uint32_t)((n & 1) * zl * N);
+                for (int cc = 0; cc < nch && ok; ++cc, ++c) {
+                    const int ws = resident ? cc : c % wslots;
+                    const uint32_t wb = saddr(smem + ws * w_bytes);
+                    for (int i = 0; i < P; ++i, ++k) {   // input plane z0 - 1 + i reaches outputs i - 2 + j
+                        ok = mbar_wait(&full[q], ph) && !abort_flag;
+                        if (!ok) break;
+                        tc_fence_after();
+                        const int j0 = i < 2 ? 2 - i : 0, j1 = nz + 1 - i < 2 ? nz + 1 - i : 2;
+                        plane_mmas(acc + (uint32_t)((i - 2) * N), saddr(planes + q * kPPlane), wb, N, j0, j1,
+                                   cc == 0 && j1 == 2);
+                        mma_commit(&empty[q]);
+                        if (++q == nplanes) {
+                            q = 0;
+                            ph ^= 1;
+                        }
+                    }
+                    if (ok && !resident) mma_commit(&wempty[ws]);
+                }
+                if (ok) mma_commit(&afull[n & 1]);
+            }
+            if (!ok) {
+                abort_flag = 1;
+                atomicExch(a.err, 1);
+                if (k > 0) mbar_wait(&empty[(k - 1) % nplanes], (uint32_t)((k - 1) / nplanes) & 1u);
+            }
+        }
+        __syncwarp();
+    } else if (tid < kProducers) {
+        // my 16-byte pieces of a plane: piece tid + 128 m, (row, channel half)
+        constexpr int kMine = (2 * kPRows + kProducers - 1) / kProducers;   // 3
+        const int h2 = a.n2 >> 1, h3 = a.n3 >> 1;
+        uint32_t dst[kMine];
 #pragma unroll
-                for (int j = 0; j < 8; ++j)   // K = 16 voxels = 2 K-adjacent core matrices per MMA
-                    mma_bf16(tmem + (uint32_t)(grp * N), smem_desc_mn(ab + j * 2 * kWgK),
-                             smem_desc_mn(gb + j * 2 * kWgK), idesc, (c >= 4 || j > 0) ? 1u : 0u);
-                mma_commit(&empty[q]);
-                ++ncommit[q];
+        for (int m = 0; m < kMine; ++m) {
+            const int p = tid + m * kProducers;
+            dst[m] = saddr(planes) + (p & 1) * kPHalf + (p >> 1) * 16;
+        }
+        const bool mine2 = tid + 2 * kProducers < 2 * kPRows;
+        auto load_weights = [&](int cc, int ws) {   // [tap][3 c_out rows][16 channels] of chunk cc
+            const uint32_t wb = saddr(smem + ws * w_bytes);
+#pragma unroll 2
+            for (int p = tid; p < 54 * N; p += kProducers) {
+                const int s = p / (6 * N), r6 = p - s * 6 * N, j = r6 / (2 * N), r2 = r6 - j * 2 * N;
+                const int co = r2 >> 1, h = r2 & 1, n = j * N + co;
+                const __nv_bfloat16 *src = a.W + (((2 - j) * 9 + s) * N + co) * cin_s + cc * 16 + h * 8;
+                cp_async16(wb + s * 96 * N + (n >> 3) * kHSBO + h * kLBO + (n & 7) * 16, src, 16);
+            }
+        };
+        bool ok = true;
+        int k = 0, q = 0, c = 0, sent = 0, qs = 0;   // stage, slot, chunk; stages handed over and the next one's slot
+        int kprev = 0;                               // first stage of the chunk before
+        uint32_t ph = 1;                             // parity of the slot's previous round
+        auto arrive = [&]() {                        // my pieces of stage `sent` are in: one arrival a warp
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(&full[qs])) : "memory");
+            ++sent;
+            if (++qs == nplanes) qs = 0;
+        };
+        if (resident)
+            for (int cc = 0; cc < nch; ++cc) load_weights(cc, cc);   // joined to the first plane
+        for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
+            int x0, y0, z0, b;
+            const int P = decode(it, x0, y0, z0, b) + 2;
+            int vfull[kMine], vhalf[kMine];
+#pragma unroll
+            for (int m = 0; m < kMine; ++m) {
+                const int p = tid + m * kProducers, row = p >> 1, h = p & 1;
+                const int yy = wrapm(y0 - 1 + row / kPHX, a.n2), xx = wrapm(x0 - 1 + row % kPHX, a.n3);
+                vfull[m] = (yy * a.n3 + xx) * a.c0s + h * 8;
+                vhalf[m] = ((yy >> 1) * h3 + (xx >> 1)) * a.c1s + h * 8;
+            }
+            const __nv_bfloat16 *s0 = a.src0 + (long long)b * a.n1 * a.n2 * a.n3 * a.c0s;
+            const __nv_bfloat16 *s1 = a.c1s ? a.src1 + (long long)b * (a.n1 >> 1) * h2 * h3 * a.c1s : nullptr;
+            const int zfirst = wrapm(z0 - 1, a.n1);
+            for (int cc = 0; cc < nch && ok; ++cc, ++c) {
+                if (!resident) {
+                    // the buffer is free once the planes of the chunk that used it are
+                    // multiplied: those of them still in flight are handed over first
+                    const int need = wslots == 1 ? k : kprev;
+                    kprev = k;
+                    if (c >= wslots && sent < need) {
+                        asm volatile("cp.async.wait_all;" ::: "memory");
+                        while (sent < need) arrive();
+                    }
+                    if (c >= wslots)
+                        ok = mbar_wait(&wempty[c % wslots], (uint32_t)(c / wslots - 1) & 1u) && !abort_flag;
+                    if (!ok) break;
+                    load_weights(cc, c % wslots);
+                }
+                const bool first = cc * 16 < a.c0s;
+                const int o0 = first ? vfull[0] : vhalf[0], o1 = first ? vfull[1] : vhalf[1];
+                const int o2 = first ? vfull[2] : vhalf[2];
+                const __nv_bfloat16 *sc = first ? s0 + cc * 16 : s1 + (cc * 16 - a.c0s);
+                const long long pstride = first ? (long long)a.n2 * a.n3 * a.c0s : (long long)h2 * h3 * a.c1s;
+                int zz = zfirst;
+                for (int i = 0; i < P; ++i, ++k) {
+                    if (k >= nplanes) ok = mbar_wait(&empty[q], ph) && !abort_flag;
+                    if (!ok) break;
+                    const __nv_bfloat16 *src = sc + (first ? zz : zz >> 1) * pstride;
+                    if (++zz == a.n1) zz = 0;
+                    const uint32_t st = q * kPPlane;
+                    cp_async16(dst[0] + st, src + o0, 16);
+                    cp_async16(dst[1] + st, src + o1, 16);
+                    if (mine2) cp_async16(dst[2] + st, src + o2, 16);
+                    cp_async_commit();
+                    if (k - sent >= kPDepth - 1) {
+                        cp_async_wait<kPDepth - 1>();
+                        arrive();
+                    }
+                    if (++q == nplanes) {
+                        q = 0;
+                        ph ^= 1;
+                    }
+                }
+            }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        if (ok)
+            while (sent < k) arrive();
+        if (!ok) {
+            abort_flag = 1;
+            if (tid == 0) atomicExch(a.err, 1);
+        }
+    } else {
+        // epilogue warps: an item's planes while the next item is multiplied
+        const int e = tid - kProducers, quarter = warp - kProducers / 32;
+        float bias[N == 16 ? 16 : 1];   // a 16-channel output's bias stays in registers
+        if constexpr (N == 16) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) bias[i] = a.bias ? __ldg(a.bias + i) : 0.f;
+        }
+        bool ok = true;
+        int n = 0;
+        const long long plane = (long long)a.n2 * a.n3 * N;
+        for (int it = blockIdx.x; it < items && ok; it += gridDim.x, ++n) {
+            int x0, y0, z0, b;
+            const int nz = decode(it, x0, y0, z0, b);
+            ok = mbar_wait(&afull[n & 1], (uint32_t)(n >> 1) & 1u) && !abort_flag;
+            if (!ok) break;
+            tc_fence_after();
+            const int y = y0 + (e >> 3), x = x0 + (e & 7);
+            const bool live = y < a.n2 && x < a.n3;
+            long long m = ((((long long)b * a.n1 + z0) * a.n2 + y) * a.n3 + x) * N;
+            const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)((n & 1) * zl * N);
+            for (int p = 0; p < nz; ++p, m += plane) {
+#pragma unroll
+                for (int c0 = 0; c0 < N; c0 += 16) {
+                    float v[16];
+                    __syncwarp();
+                    tmem_ld16(acc + (uint32_t)(p * N + c0), v);
+                    if (live) {
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) {
+                            if constexpr (N == 16) v[i] += bias[i];
+                            else if (a.bias) v[i] += __ldg(a.bias + c0 + i);
+                            if (a.relu) v[i] = fmaxf(v[i], 0.f);
+                        }
+                        if (a.out_f32) {
+                            float4 *o = reinterpret_cast<float4 *>(a.out_f32 + m + c0);
+#pragma unroll
+                            for (int i = 0; i < 4; ++i)
+                                o[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+                        } else {
+                            __nv_bfloat162 hv[8];
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) hv[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+                            uint4 *o = reinterpret_cast<uint4 *>(a.out_bf16 + m + c0);
+                            o[0] = *reinterpret_cast<uint4 *>(&hv[0]);
+                            o[1] = *reinterpret_cast<uint4 *>(&hv[4]);
+                        }
+                    }
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(&aempty[n & 1])) : "memory");
+        }
+        if (!ok) {
+            abort_flag = 1;
+            if (e == 0) atomicExch(a.err, 1);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == kMma)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
+}
+
+// ---------------------------------------------------------------------------
+// Column weight gradient: dW[t][co][ci] = sum_v G[v][co] X[v + d_t][ci] on the
+// same 8 x 16 columns, 16 output channels and one 16-channel chunk of the
+// input per CTA.  Rows of D are (dx, input channel), 48 of M = 64; its columns
+// are (dz, dy, output channel), N = 144: the G planes z+1, z, z-1 of an X plane z,
+// each as three copies shifted by dy.  So a plane takes 8 MMAs (K = the tile's
+// 128 voxels, 16 at a time) for all 27 taps.  (24 of N = 48, dy in the start of
+// A, took 131 us against 126 at 64^3 x 8, 16 -> 16 channels, and leave the
+// copies' number to the output channels; one CTA per SM with eight stages in
+// flight took 180.  What bounds it is neither: the loads alone, or a eighth of
+// the MMAs, take nearly as long.)
+// Both operands are MN-major in place: A three copies of the X plane, one per
+// dx, [dx][channel half][16 y][8 x] rows of 16 bytes; B a ring of G planes,
+// [plane][dy][channel half][16 y][8 x], whose window of three is one run of
+// column groups except where the ring wraps (then two MMAs).  D stays in
+// tensor memory while the CTA takes its share of columns.  (k_wgrad3_tc, which
+// this replaces, copied 27 taps of every voxel between shared buffers: 258 us
+// at 64^3 x 8, 16 -> 16 channels.)
+// ---------------------------------------------------------------------------
+constexpr int kCHalf = kPY * kPX * 16;              // 2048 B: 8 channels of one copy of a plane
+constexpr int kCPlane = 6 * kCHalf;                 // three copies of 16 channels (X: dx, G: dy)
+constexpr int kCSlots = 3, kCGSlots = 6, kCDepth = 2;   // X planes, G planes (each read for three stages), loads in flight
+constexpr int kCPad = 2 * kCHalf;                   // rows 48..63 of A read past the last X slot
+constexpr int kCTaps = 48;                          // columns of one G plane: dy, 16 output channels
+
+__device__ __forceinline__ uint64_t smem_desc_c(uint32_t addr) {   // MN-major: LBO along K, SBO along MN
+    return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)((128 >> 4) & 0x3FFF) << 16) |
+           ((uint64_t)((kCHalf >> 4) & 0x3FFF) << 32) | (1ull << 46);
+}
+__device__ __forceinline__ uint32_t instr_desc_c(int n) {   // M = 64, both operands MN-major
+    return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((uint32_t)(n >> 3) << 17) | (4u << 24);
+}
+
+// zl: planes of a work item; blockIdx = (split, input chunk, 16 output channels)
+__global__ void __launch_bounds__(kThreads) k_wgrad3_col(WgradArgs w, int ncols, int zl) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ __align__(8) uint64_t full[kCSlots], empty[kCSlots], done;
+    __shared__ uint32_t tmem_slot;
+    __shared__ volatile int abort_flag;
+    const ConvArgs &a = w.in;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int cin_s = a.c0s + a.c1s, cc = blockIdx.y, split = blockIdx.x, co0 = blockIdx.z * 16;
+    unsigned char *xs = smem, *gs = smem + kCSlots * kCPlane + kCPad;
+    const int tx = (a.n3 + kPX - 1) / kPX, ty = (a.n2 + kPY - 1) / kPY, tz = (a.n1 + zl - 1) / zl;
+    const long long items = (long long)tx * ty * tz * a.B;
+    const long long it0 = items * split / w.S, it1 = items * (split + 1) / w.S;
+    constexpr int kMma = kProducers / 32;
+    if (it0 >= it1) {   // no columns in this split: its partial sums are zero
+        for (int i = tid; i < 27 * 16 * 16; i += kThreads) {
+            const int ci = i % 16, r = i / 16, co = r % 16, t = r / 16;
+            w.partial[(((long long)split * 27 + t) * w.cout + co0 + co) * cin_s + cc * 16 + ci] = 0.f;
+        }
+        return;
+    }
+    auto item_z = [&](long long it) { return (int)(it % tz) * zl; };   // z fastest: neighbours share halo planes
+    auto item_nz = [&](long long it) { return a.n1 - item_z(it) < zl ? a.n1 - item_z(it) : zl; };
+
+    if (warp == kMma) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr(&tmem_slot)),
+                     "r"(ncols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (tid == 0) {
+        for (int q = 0; q < kCSlots; ++q) {
+            mbar_init(&full[q], kProducers / 32);
+            mbar_init(&empty[q], 1);
+        }
+        mbar_init(&done, 1);
+        abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    // the pad that A's unused rows read stays finite
+    for (int i = tid; i < kCPad / 16; i += kThreads)
+        reinterpret_cast<uint4 *>(smem + kCSlots * kCPlane)[i] = make_uint4(0, 0, 0, 0);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_slot;
+
+    if (warp == kMma) {
+        if (lane == 0) {
+            bool ok = true;
+            int k = 0, q = 0, g0 = 0;   // stage, its slot, ring slot of the item's G plane 0
+            uint32_t ph = 0;
+            for (long long it = it0; it < it1 && ok; ++it) {
+                const int nz = item_nz(it);
+                for (int i = 0; i < nz + 2; ++i, ++k) {   // X plane z0 - 1 + i meets G planes i - 2 + j
+                    ok = mbar_wait(&full[q], ph) && !abort_flag;
+                    if (!ok) break;
+                    tc_fence_after();
+                    const int j0 = i < 2 ? 2 - i : 0, j1 = nz + 1 - i < 2 ? nz + 1 - i : 2;
+                    const bool fresh = it == it0 && i <= 2;   // block j0 starts its accumulators
+                    const int s0 = (g0 + i - 2 + j0) % kCGSlots, left = kCGSlots - s0;   // planes before the ring wraps
+                    const int ja = j1 - j0 + 1 > left ? j0 + left - 1 : j1;              // last block of the first run
+                    const uint64_t ad = smem_desc_c(saddr(xs + q * kCPlane));
+                    const uint64_t b0 = smem_desc_c(saddr(gs + s0 * kCPlane)), b1 = smem_desc_c(saddr(gs));
+                    const uint32_t d = tmem + (uint32_t)(j0 * kCTaps), d1 = tmem + (uint32_t)((ja + 1) * kCTaps);
+                    const uint32_t n0 = instr_desc_c((ja - j0 + 1) * kCTaps), n1 = instr_desc_c((j1 - ja) * kCTaps);
+#pragma unroll
+                    for (int kk = 0; kk < 8; ++kk) {   // 16 voxels: two y runs of 128 B
+                        const uint64_t o = (uint64_t)(kk * 16);
+                        if (fresh && kk == 0) {
+                            mma_bf16(d, ad + o, b0 + o, instr_desc_c(kCTaps), 0u);
+                            if (ja > j0)
+                                mma_bf16(d + kCTaps, ad + o, b0 + o + (uint64_t)(kCPlane >> 4),
+                                         instr_desc_c((ja - j0) * kCTaps), 1u);
+                        } else {
+                            mma_bf16(d, ad + o, b0 + o, n0, 1u);
+                        }
+                        if (j1 > ja) mma_bf16(d1, ad + o, b1 + o, n1, 1u);
+                    }
+                    mma_commit(&empty[q]);
+                    if (++q == kCSlots) {
+                        q = 0;
+                        ph ^= 1;
+                    }
+                }
+                g0 = (g0 + nz) % kCGSlots;
             }
             if (ok) {
                 mma_commit(&done);
             } else {
                 abort_flag = 1;
-                atomicExch(&g_tc_err, 1);
-                for (int q = 0; q < 2; ++q)
-                    if (ncommit[q] > 0) mbar_wait(&empty[q], (uint32_t)(ncommit[q] - 1) & 1u);
+                atomicExch(a.err, 1);
+                if (k > 0) mbar_wait(&empty[(k - 1) % kCSlots], (uint32_t)((k - 1) / kCSlots) & 1u);
             }
         }
         __syncwarp();
     } else {
-        // producer row = voxel tid of the brick: offsets (bz, by, bx)
-        const int bz = tid >> 5, by = (tid >> 3) & 3, bx = tid & 7;
-        const int hrow = ((bz * kHY + by) * kHX + bx) * 16;   // my voxel's halo row at tap offset 0
+        // my pieces of a plane's copies: piece p = tid + 128 m is (copy, y, x, half)
+        constexpr int kMine = 3 * kPY * kPX * 2 / kProducers;   // 6
+        static_assert(kMine * kProducers == 3 * kPY * kPX * 2, "whole pieces");
         const bool first = cc * 16 < a.c0s;
-        // my halo rows (at most 3 of the 360) and their positions in the halo
-        int hz[3], hy[3], hx[3];
-#pragma unroll
-        for (int r = 0; r < 3; ++r) {
-            const int h = tid + r * kProducers;
-            hx[r] = h % kHX;
-            hy[r] = (h / kHX) % kHY;
-            hz[r] = h / (kHX * kHY);
-        }
-        // the chunk's source: full resolution, or the half-resolution second
-        // source read with nearest-neighbour upsampling
         const int sh = first ? 0 : 1;
         const int m1 = a.n1 >> sh, m2 = a.n2 >> sh, m3 = a.n3 >> sh;
         const int cs = first ? a.c0s : a.c1s;
         const __nv_bfloat16 *sbase = first ? a.src0 + cc * 16 : a.src1 + (cc * 16 - a.c0s);
-        // halo of brick br into halo buffer hb, my G row into G buffer hb
-        auto load_brick = [&](long long br, int hb) {
-            long long rr = br;
-            const int xb = (int)(rr % bx3); rr /= bx3;
-            const int yb = (int)(rr % by2); rr /= by2;
-            const int zb = (int)(rr % bz1);
-            const int b = (int)(rr / bz1);
-            const int z0 = zb * 4, y0 = yb * 4, x0 = xb * 8;
-            const __nv_bfloat16 *src_b = sbase + (long long)b * m1 * m2 * m3 * cs;
-            unsigned char *hp = halo + hb * 2 * kPlane + tid * 16;
+        int off[kMine], goff[kMine];
+        uint32_t dst[kMine];
 #pragma unroll
-            for (int r = 0; r < 3; ++r) {
-                if (tid + r * kProducers < kHalo) {
-                    const int zz = wrapi(z0 - 1 + hz[r], a.n1) >> sh, yy = wrapi(y0 - 1 + hy[r], a.n2) >> sh,
-                              xx = wrapi(x0 - 1 + hx[r], a.n3) >> sh;
-                    const __nv_bfloat16 *src = src_b + (long long)((zz * m2 + yy) * m3 + xx) * cs;
-                    cp_async16(saddr(hp + r * kProducers * 16), src, 16);
-                    cp_async16(saddr(hp + kPlane + r * kProducers * 16), src + 8, 16);
-                }
-            }
-            const long long v = (((long long)b * a.n1 + z0 + bz) * a.n2 + y0 + by) * a.n3 + x0 + bx;
-            const __nv_bfloat16 *g = w.G + v * N;
-            unsigned char *gp = gt + hb * gbytes + (tid >> 3) * kWgK + (tid & 7) * 16;
-            for (int ng = 0; ng < N / 8; ++ng) cp_async16(saddr(gp + ng * kWgMn), g + ng * 8, 16);
-            cp_async_commit();
-        };
+        for (int m = 0; m < kMine; ++m) {
+            const int p = tid + m * kProducers, v = (p >> 1) % (kPY * kPX), copy = p / (2 * kPY * kPX);
+            dst[m] = (2 * copy + (p & 1)) * kCHalf + v * 16;
+        }
         bool ok = true;
-        load_brick(bb0, 0);
-        for (long long br = bb0; br < bb1; ++br) {
-            const int i = (int)(br - bb0), hb = i & 1;
-            asm volatile("cp.async.wait_all;" ::: "memory");
-            bar_producers();     // brick br's halo and G tile are in; brick br-1's copies are done
-            const unsigned char *hp = halo + hb * 2 * kPlane;
-            for (int grp = 0; grp < 4; ++grp) {
-                const int c = 4 * i + grp, q = c & 1;
-                if (!ok) continue;
-                if (c >= 2) ok = mbar_wait(&empty[q], (uint32_t)((c >> 1) - 1) & 1u) && !abort_flag;
-                if (!ok) continue;
-                // stage c-2 is the last MMA of brick br-1: its buffers take brick br+1
-                if (grp == 1 && br + 1 < bb1) load_brick(br + 1, hb ^ 1);
-                unsigned char *at = ring + q * kWgATile + (tid >> 3) * kWgK + (tid & 7) * 16;
-                switch (grp) {
-                    case 0: wg_copy<0>(at, hp + hrow); break;
-                    case 1: wg_copy<1>(at, hp + hrow); break;
-                    case 2: wg_copy<2>(at, hp + hrow); break;
-                    default: wg_copy<3>(at, hp + hrow); break;
+        int k = 0, q = 0, gq = 0, sent = 0, qs = 0;   // stage, X slot, G slot; stages handed over and the next one's slot
+        uint32_t ph = 1;                              // parity of the slot's previous round
+        auto arrive = [&]() {                         // my pieces of stage `sent` are in: one arrival a warp
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(&full[qs])) : "memory");
+            ++sent;
+            if (++qs == kCSlots) qs = 0;
+        };
+        const long long pstride = (long long)m2 * m3 * cs, gstride = (long long)a.n2 * a.n3 * w.cout;
+        for (long long it = it0; it < it1 && ok; ++it) {
+            const int z0 = item_z(it), nz = item_nz(it);
+            long long r = it / tz;
+            const int x0 = (int)(r % tx) * kPX; r /= tx;
+            const int y0 = (int)(r % ty) * kPY;
+            const int b = (int)(r / ty);
+            // X row y of copy dx: X[y][x + dx]; G row y of copy dy: G[y - dy][x], zero
+            // for y or x beyond the grid (each X row, each G column counts once)
+            uint32_t live = 0;
+#pragma unroll
+            for (int m = 0; m < kMine; ++m) {
+                const int p = tid + m * kProducers, v = (p >> 1) % (kPY * kPX), copy = p / (2 * kPY * kPX);
+                const int y = y0 + v / kPX, x = x0 + v % kPX;
+                off[m] = ((wrapm(y, a.n2) >> sh) * m3 + (wrapm(x - 1 + copy, a.n3) >> sh)) * cs + (tid & 1) * 8;
+                const bool in = y < a.n2 && x < a.n3;
+                goff[m] = in ? (wrapm(y + 1 - copy, a.n2) * a.n3 + x) * w.cout + co0 + (tid & 1) * 8 : 0;
+                live |= (in ? 1u : 0u) << m;
+            }
+            const __nv_bfloat16 *src_b = sbase + (long long)b * m1 * pstride;
+            const __nv_bfloat16 *g = w.G + ((long long)b * a.n1 + z0) * gstride;
+            int zz = wrapm(z0 - 1, a.n1);
+            for (int i = 0; i < nz + 2; ++i, ++k) {
+                if (k >= kCSlots) ok = mbar_wait(&empty[q], ph) && !abort_flag;
+                if (!ok) break;
+                const __nv_bfloat16 *src = src_b + (zz >> sh) * pstride;
+                if (++zz == a.n1) zz = 0;
+                const uint32_t st = saddr(xs) + q * kCPlane;
+#pragma unroll
+                for (int m = 0; m < kMine; ++m) cp_async16(st + dst[m], src + off[m], 16);
+                if (i < nz) {   // G plane i (its slot's last reader is no later than the X slot's)
+                    const uint32_t gd = saddr(gs) + gq * kCPlane;
+#pragma unroll
+                    for (int m = 0; m < kMine; ++m) cp_async16(gd + dst[m], g + goff[m], (live >> m) & 1 ? 16 : 0);
+                    g += gstride;
+                    if (++gq == kCGSlots) gq = 0;
                 }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(&full[q])) : "memory");
+                cp_async_commit();
+                if (k - sent >= kCDepth - 1) {
+                    cp_async_wait<kCDepth - 1>();
+                    arrive();
+                }
+                if (++q == kCSlots) {
+                    q = 0;
+                    ph ^= 1;
+                }
             }
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
+        if (ok)
+            while (sent < k) arrive();
         if (!ok) abort_flag = 1;
         if (ok) ok = mbar_wait(&done, 0u) && !abort_flag;
         if (ok) {
             tc_fence_after();
-            const int row = warp * 32 + lane;               // (tap in group, channel)
-            const int tl = row >> 4, ci = row & 15;
-            for (int grp = 0; grp < 4; ++grp) {
-                const int t = grp * 8 + tl;
-                for (int c0 = 0; c0 < N; c0 += 16) {
-                    float v[16];
-                    tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(grp * N + c0), v);
-                    if (t < 27) {
+            // M = 64: rows 16 w .. 16 w + 15 in lanes 0..15 of warp w's quarter; warp w holds dx = w
+#pragma unroll 1
+            for (int jd = 0; jd < 9; ++jd) {   // (dz block j, dy copy)
+                float v[16];
+                __syncwarp();
+                tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(jd * 16), v);
+                if (warp < 3 && lane < 16) {
+                    const int j = jd / 3, t = (2 - j) * 9 + (jd - 3 * j) * 3 + warp;
+                    float *o = w.partial + (((long long)split * 27 + t) * w.cout + co0) * cin_s + cc * 16 + lane;
 #pragma unroll
-                        for (int i = 0; i < 16; ++i)
-                            w.partial[(((long long)split * 27 + t) * N + c0 + i) * cin_s + cc * 16 + ci] = v[i];
-                    }
+                    for (int i = 0; i < 16; ++i) o[(long long)i * cin_s] = v[i];
                 }
             }
         } else if (tid == 0) {
-            atomicExch(&g_tc_err, 1);
+            atomicExch(a.err, 1);
         }
     }
     tc_fence_before();
@@ -1087,7 +1401,26 @@ __global__ void __launch_bounds__(kThreads) k_wgrad3_tc(WgradArgs w, int ncols, 
 
 }  // namespace
 
-int conv3_forward_tc(const ConvArgs &a, cudaStream_t st) {
+// The word a kernel sets when a bounded wait gives up: host memory mapped for
+// every device, so that reading it after a call costs no copy (the copy from a
+// device symbol took about 10 us of every call).
+static int *err_flag() {
+    static int *f = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void *p = nullptr;
+        if (cudaHostAlloc(&p, sizeof(int), cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess) {
+            f = static_cast<int *>(p);
+            *f = 0;
+        }
+    });
+    return f;
+}
+
+int conv3_forward_tc(const ConvArgs &in, cudaStream_t st) {
+    ConvArgs a = in;
+    a.err = err_flag();
+    if (!a.err) return -1;
     if ((a.cout & 15) || a.cout > 256 || a.cout < 16 || (a.c0s & 15) || (a.c1s & 15) || a.c0s <= 0) return -1;
     if (a.c1s && (!a.src1 || (a.n1 | a.n2 | a.n3) & 1)) return -1;
     int ncols = 32;
@@ -1106,7 +1439,40 @@ int conv3_forward_tc(const ConvArgs &a, cudaStream_t st) {
         cudaFuncSetAttribute(k_conv3_tcd, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
         cudaFuncSetAttribute(k_conv3_tcp, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
         cudaFuncSetAttribute(k_conv3_tch, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        for (auto k : {k_conv3_col<16>, k_conv3_col<32>, k_conv3_col<48>, k_conv3_col<64>, k_conv3_col<80>}) {
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lim - 1024);
+            cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        }
         attr = true;
+    }
+    if (3 * a.cout <= 256) {
+        // column march: two CTAs per SM up to 32 output channels, one above;
+        // planes of an item by half of a CTA's tensor memory
+        static int nsm = 0;
+        if (!nsm) {
+            int dev = 0;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        }
+        const int per_sm = a.cout <= 32 ? 2 : 1, nch = (a.c0s + a.c1s) / 16;
+        const int zmax = a.cout <= 32 ? 128 / a.cout : 256 / a.cout, zl = a.n1 < zmax ? a.n1 : zmax;
+        int nc = 32;
+        while (nc < 2 * zl * a.cout) nc <<= 1;
+        const size_t wb = (size_t)27 * 32 * a.cout, room = 233472 / per_sm - 3 * 1024;
+        // all chunks' weights if they leave room for eight planes, else two or one
+        int wslots = nch;
+        while (wslots > 1 && wslots * wb + 8 * (size_t)kPPlane > room) wslots = wslots > 2 ? 2 : 1;
+        int nplanes = (int)((room - wslots * wb) / kPPlane);
+        nplanes = nplanes < kPSlots ? nplanes : kPSlots;
+        size_t smem = wslots * wb + nplanes * (size_t)kPPlane;
+        const size_t floor = 233472 / (512 / nc + 1) + 1024;   // TMEM columns per SM stay <= 512
+        if (smem < floor) smem = floor;
+        const long long items = (long long)((a.n3 + kPX - 1) / kPX) * ((a.n2 + kPY - 1) / kPY) * ((a.n1 + zl - 1) / zl) * a.B;
+        const long long grid = items < (long long)per_sm * nsm ? items : (long long)per_sm * nsm;
+        const auto k = a.cout == 16 ? k_conv3_col<16> : a.cout == 32 ? k_conv3_col<32> : a.cout == 48 ? k_conv3_col<48>
+                     : a.cout == 64 ? k_conv3_col<64> : k_conv3_col<80>;
+        k<<<(unsigned)grid, kColThreads, smem, st>>>(a, nc, zl, nplanes, wslots);
+        return 0;
     }
     const bool bricks_tile = a.n1 % 4 == 0 && a.n2 % 4 == 0 && a.n3 % 8 == 0;
     const size_t w_bytes = (size_t)(a.c0s + a.c1s) / 16 * 27 * 32 * a.cout;
@@ -1167,38 +1533,37 @@ int conv3_forward_tc(const ConvArgs &a, cudaStream_t st) {
     return 0;
 }
 
-int conv3_wgrad_tc(const WgradArgs &w, cudaStream_t st) {
+int conv3_wgrad_tc(const WgradArgs &in, cudaStream_t st) {
+    WgradArgs w = in;
+    w.in.err = err_flag();
     const ConvArgs &a = w.in;
+    if (!a.err) return -1;
     if ((w.cout & 15) || w.cout > 64 || w.cout < 16 || (a.c0s & 15) || (a.c1s & 15) || w.S <= 0) return -1;
-    if (a.n1 % 4 || a.n2 % 4 || a.n3 % 8) return -1;
-    int ncols = 32;
-    while (ncols < 4 * w.cout) ncols <<= 1;
-    static bool attr = false;
-    if (!attr) {
-        int dev = 0, lim = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        cudaFuncSetAttribute(k_wgrad3_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, lim - 1024);
-        cudaFuncSetAttribute(k_wgrad3_tc, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        attr = true;
+    if (!(a.c1s && ((a.n1 | a.n2 | a.n3) & 1))) {
+        static bool cattr = false;
+        if (!cattr) {
+            int dev = 0, lim = 0;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+            cudaFuncSetAttribute(k_wgrad3_col, cudaFuncAttributeMaxDynamicSharedMemorySize, lim - 1024);
+            cudaFuncSetAttribute(k_wgrad3_col, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+            cattr = true;
+        }
+        const int nc = 256;   // 144 columns; two CTAs per SM by tensor and shared memory
+        const int zl = a.n1 < 8 ? a.n1 : 8;
+        size_t smem = (size_t)(kCSlots + kCGSlots) * kCPlane + kCPad;
+        const size_t floor = 233472 / (512 / nc + 1) + 1024;    // TMEM columns per SM stay <= 512
+        if (smem < floor) smem = floor;
+        k_wgrad3_col<<<dim3(w.S, (a.c0s + a.c1s) / 16, w.cout / 16), kThreads, smem, st>>>(w, nc, zl);
+        return 0;
     }
-    size_t smem = 2 * ((size_t)kHalo * 32 + (size_t)(w.cout / 8) * kWgMn) + 2 * (size_t)kWgATile;
-    const size_t floor = 233472 / (512 / ncols + 1) + 1024;    // TMEM columns per SM stay <= 512
-    if (smem < floor) smem = floor;
-    const long long nbricks = (long long)(a.n1 / 4) * (a.n2 / 4) * (a.n3 / 8) * a.B;
-    const int bpc = (int)((nbricks + w.S - 1) / w.S);
-    const dim3 grid(w.S, (a.c0s + a.c1s) / 16);
-    k_wgrad3_tc<<<grid, kThreads, smem, st>>>(w, ncols, bpc);
-    return 0;
+    return -1;
 }
 
 int conv3_tc_error(int clear) {
-    int e = 0;
-    cudaMemcpyFromSymbol(&e, g_tc_err, sizeof(int));
-    if (clear && e) {
-        const int z = 0;
-        cudaMemcpyToSymbol(g_tc_err, &z, sizeof(int));
-    }
+    int *f = err_flag();
+    const int e = f ? *reinterpret_cast<volatile int *>(f) : 0;
+    if (clear && e) *reinterpret_cast<volatile int *>(f) = 0;
     return e;
 }
 
