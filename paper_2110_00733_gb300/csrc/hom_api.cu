@@ -381,35 +381,28 @@ static int engine_init(hom_ctx *ctx, Engine<R> &E) {
     for (int p = 0; p < 3; ++p) {
         const int N = ctx->n[p];
         if (!factor_radices(N, g.ax[p])) return fail(ctx, HOM_EUNSUPPORTED_GRID, "grid size not 2^a3^b5^c");
-        std::vector<R> tw(2 * N), D(2 * N), M(2 * N);
+        std::vector<R> tw(2 * N), D(N), M(N);
         for (int t = 0; t < N; ++t) {
             const double ang = 2.0 * PI * (double)t / (double)N;
             tw[2 * t] = (R)std::cos(ang);
             tw[2 * t + 1] = (R)-std::sin(ang);
             const int m = (2 * t < N) ? t : t - N;        // signed frequency index
             const double q = 2.0 * PI * (double)m / (double)N;
-            if (ctx->deriv == HOM_DERIV_CONTINUOUS) {      // xi_p = i q_p N_p, eq. (freq)
-                D[2 * t] = 0;
-                D[2 * t + 1] = (R)(q * N);
-                M[2 * t] = 1;
-                M[2 * t + 1] = 0;
-            } else {   // rotated scheme, eq. (freqrot): N (e^{iq}-1) and (1+e^{iq})/2
-                D[2 * t] = (R)(N * (std::cos(q) - 1.0));
-                D[2 * t + 1] = (R)(N * std::sin(q));
-                M[2 * t] = (R)(0.5 * (1.0 + std::cos(q)));
-                M[2 * t + 1] = (R)(0.5 * std::sin(q));
-            }
+            // xi_p up to a phase common to the three axes (see gamma_e)
+            const bool cont = ctx->deriv == HOM_DERIV_CONTINUOUS;   // q_p N_p, eq. (freq)
+            D[t] = (R)(cont ? q * N : 2.0 * N * std::sin(0.5 * q));   // else eq. (freqrot)
+            M[t] = (R)(cont ? 1.0 : std::cos(0.5 * q));
         }
         CU(cudaMalloc(&E.tw[p], cs * N));
-        CU(cudaMalloc(&E.D[p], cs * N));
-        CU(cudaMalloc(&E.M[p], cs * N));
+        CU(cudaMalloc(&E.D[p], sizeof(R) * N));
+        CU(cudaMalloc(&E.M[p], sizeof(R) * N));
         CU(cudaMemcpy(E.tw[p], tw.data(), cs * N, cudaMemcpyHostToDevice));
-        CU(cudaMemcpy(E.D[p], D.data(), cs * N, cudaMemcpyHostToDevice));
-        CU(cudaMemcpy(E.M[p], M.data(), cs * N, cudaMemcpyHostToDevice));
+        CU(cudaMemcpy(E.D[p], D.data(), sizeof(R) * N, cudaMemcpyHostToDevice));
+        CU(cudaMemcpy(E.M[p], M.data(), sizeof(R) * N, cudaMemcpyHostToDevice));
         g.ax[p].tw = E.tw[p];
         g.D[p] = E.D[p];
         g.M[p] = E.M[p];
-        ctx->workspace += 3 * (long long)cs * N;
+        ctx->workspace += 2 * (long long)cs * N;
     }
     CU(cudaMalloc(&E.phi, sizeof(R) * ctx->V));
     CU(cudaMalloc(&E.spec, cs * 6 * ctx->S));

@@ -174,8 +174,8 @@ struct Geometry {
     int n1, n2, n3, h;      // h = n3/2 + 1
     long long V, S;         // voxels, half-spectrum points per component
     AxisPlan ax[3];
-    const void *D[3];       // per axis: difference symbol (complex, length n_p)
-    const void *M[3];       // per axis: averaging factor (complex, length n_p)
+    const void *D[3];       // per axis: difference symbol without its phase (real, length n_p; see gamma_e)
+    const void *M[3];       // per axis: averaging factor without its phase (real, length n_p)
     // launch shapes: rows per CTA of the n3 pass, columns per CTA of the n2
     // and n1 passes, threads per CTA, dynamic shared memory, and whether the
     // axis uses the compile-time register FFT (its length, or 0)

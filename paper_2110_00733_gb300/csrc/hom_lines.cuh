@@ -8,18 +8,11 @@
 // plain loads, which ran them, divides by run-time values for every butterfly,
 // holds two buffers per tile and overlaps nothing with its loads: at 192^3 the
 // n2 pass took 187 us (65 here; 50 is the copy rate) and the fused n1 pass
-// 649 us (272 here), at 108^3 39 (14) and 147 us (72).
+// 649 us (173 here), at 108^3 39 (14) and 147 us (38).
 #pragma once
 #include "hom_passes.cuh"
 
 namespace hom {
-
-// 1 / sqrt(n2): the hardware's estimate and one Newton step, within an ulp or
-// two of the correctly rounded quotient and a third of its instructions
-__device__ __forceinline__ float inv_norm(float n2) {
-    const float y = rsqrtf(n2);
-    return fmaf(0.5f * y, fmaf(-n2 * y, y, 1.0f), y);
-}
 
 // Steps 1-3 of the fused pass (see k_x1_lanczos) on the tile of columns [g0, g0
 // + T) held in buf, element e of line l at buf[e * L + l], L = 6 T; the GRP
@@ -40,13 +33,11 @@ __device__ __forceinline__ void x1_lanczos_line(const Geometry &g, cpx<R> *buf, 
         const R w = (R)pweight(k3, g.n3);
         // mode of the column: 0 a Nyquist index of axis 2 or 3, else 1
         const bool nyq = 2 * k2 == g.n2 || 2 * k3 == g.n3;
-        const cpx<R> m1 = __ldg(&reinterpret_cast<const cpx<R> *>(g.M[1])[k2]);
-        const cpx<R> m2 = __ldg(&reinterpret_cast<const cpx<R> *>(g.M[2])[k3]);
-        const cpx<R> m12 = mul<R>(m1, m2);
-        const cpx<R> d1 = mul<R>(__ldg(&reinterpret_cast<const cpx<R> *>(g.D[1])[k2]), m2);
-        const cpx<R> d2 = mul<R>(__ldg(&reinterpret_cast<const cpx<R> *>(g.D[2])[k3]), m1);
-        const cpx<R> *D0 = reinterpret_cast<const cpx<R> *>(g.D[0]);
-        const cpx<R> *M0 = reinterpret_cast<const cpx<R> *>(g.M[0]);
+        const R m1 = __ldg(reinterpret_cast<const R *>(g.M[1]) + k2), m2 = __ldg(reinterpret_cast<const R *>(g.M[2]) + k3);
+        const R m12 = m1 * m2;
+        const R d1 = __ldg(reinterpret_cast<const R *>(g.D[1]) + k2) * m2;
+        const R d2 = __ldg(reinterpret_cast<const R *>(g.D[2]) + k3) * m1;
+        const R *D0 = reinterpret_cast<const R *>(g.D[0]), *M0 = reinterpret_cast<const R *>(g.M[0]);
         const size_t i0 = (size_t)(g0 / T) * krylov_tile(N, T) + t;
 #pragma unroll 1
         for (int e = e0; e < N; e += ES) {
@@ -58,19 +49,18 @@ __device__ __forceinline__ void x1_lanczos_line(const Geometry &g, cpx<R> *buf, 
                 u[c3] = uk[i + c3 * NT];
                 uo[c3] = um[i + c3 * NT];
             }
-            const cpx<R> m0 = __ldg(&M0[e]);
+            const R m0 = __ldg(&M0[e]);
             GammaE<R> ge;
-            ge.e0 = mul<R>(__ldg(&D0[e]), m12);
-            ge.e1 = mul<R>(d1, m0);
-            ge.e2 = mul<R>(d2, m0);
-            const R n2 = ge.e0.x * ge.e0.x + ge.e0.y * ge.e0.y + ge.e1.x * ge.e1.x + ge.e1.y * ge.e1.y +
-                         ge.e2.x * ge.e2.x + ge.e2.y * ge.e2.y;
+            ge.e0 = __ldg(&D0[e]) * m12;
+            ge.e1 = d1 * m0;
+            ge.e2 = d2 * m0;
+            const R n2 = ge.e0 * ge.e0 + ge.e1 * ge.e1 + ge.e2 * ge.e2;
             ge.mode = (nyq || 2 * e == N || !(n2 > (R)0)) ? 0 : 1;
             if (col == 0 && e == 0) ge.mode = 2;
             const R inv = inv_norm(n2);
-            ge.e0 = scale<R>(ge.e0, inv);
-            ge.e1 = scale<R>(ge.e1, inv);
-            ge.e2 = scale<R>(ge.e2, inv);
+            ge.e0 *= inv;
+            ge.e1 *= inv;
+            ge.e2 *= inv;
 #pragma unroll
             for (int p = 0; p < 3; ++p) Six<R>::load_pair(sp, p, v[2 * p], v[2 * p + 1]);
             gamma_to_q<R>(g, ge, v, q);

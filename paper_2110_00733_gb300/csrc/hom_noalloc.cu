@@ -41,7 +41,8 @@ constexpr int kMaxDevices = 64;
 
 // work half spectrum: n1 n2 (n3/2+1) <= V for n3 >= 2, times 6 components
 static __device__ __align__(256) float2 g_scratch_spec[6 * kMaxV];
-// per axis: twiddles exp(-2 pi i t/N), difference symbol D, averaging factor M
+// per axis: twiddles exp(-2 pi i t/N), difference symbol D and averaging factor M
+// (real, the first half of their slots)
 static __device__ __align__(256) float2 g_scratch_tab[3][3][kMaxN];
 
 struct DevicePtrs {
@@ -54,28 +55,24 @@ std::mutex g_mu;
 
 // Frequency tables on the device, FP64 with sincospi, stored in FP32:
 // tw[t] = exp(-2 pi i t/N); D, M of the continuous (eq. freq) or rotated
-// (eq. freqrot) scheme, as in the context-based path.
+// (eq. freqrot) scheme, as in the context-based path (see gamma_e).
 __global__ void k_noalloc_tables(int n1, int n2, int n3, int deriv, float2 *tab) {
     const int ns[3] = {n1, n2, n3};
     for (int p = 0; p < 3; ++p) {
         const int N = ns[p];
         float2 *tw = tab + (p * 3 + 0) * kMaxN;
-        float2 *D = tab + (p * 3 + 1) * kMaxN;
-        float2 *M = tab + (p * 3 + 2) * kMaxN;
+        float *D = reinterpret_cast<float *>(tab + (p * 3 + 1) * kMaxN);
+        float *M = reinterpret_cast<float *>(tab + (p * 3 + 2) * kMaxN);
         for (int t = threadIdx.x; t < N; t += blockDim.x) {
             double s, c;
             sincospi(2.0 * (double)t / (double)N, &s, &c);
             tw[t] = make_float2((float)c, (float)-s);
             const int m = (2 * t < N) ? t : t - N;
-            double sq, cq;
-            sincospi(2.0 * (double)m / (double)N, &sq, &cq);
-            if (deriv == HOM_DERIV_CONTINUOUS) {
-                D[t] = make_float2(0.f, (float)(2.0 * 3.14159265358979323846 * m));   // i q N with q = 2 pi m / N
-                M[t] = make_float2(1.f, 0.f);
-            } else {
-                D[t] = make_float2((float)(N * (cq - 1.0)), (float)(N * sq));
-                M[t] = make_float2((float)(0.5 * (1.0 + cq)), (float)(0.5 * sq));
-            }
+            double sq, cq;   // of half the angle
+            sincospi((double)m / (double)N, &sq, &cq);
+            const bool cont = deriv == HOM_DERIV_CONTINUOUS;
+            D[t] = (float)(cont ? 2.0 * 3.14159265358979323846 * m : 2.0 * N * sq);
+            M[t] = cont ? 1.f : (float)cq;
         }
     }
 }

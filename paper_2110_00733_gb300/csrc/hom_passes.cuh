@@ -108,52 +108,43 @@ __device__ __forceinline__ double sum_partials(const double *part, int count) {
 __device__ __forceinline__ int pweight(int k3, int n3) { return (k3 == 0 || 2 * k3 == n3) ? 1 : 2; }
 
 // ---------------------------------------------------------------------------
-// Projector of eq. (galop) at one frequency, in closed form.  xi may be
-// complex (rotated scheme).  With e = xi/|xi|, the orthogonal projection of a
-// symmetric tau onto {sym(u (x) xi)} is sym(u (x) e) with
+// Projector of eq. (galop) at one frequency, in closed form.  With e = xi/|xi|,
+// the orthogonal projection of a symmetric tau onto {sym(u (x) xi)} is
+// sym(u (x) e) with
 //     u = 2 tau conj(e) - e (conj(e) . tau conj(e))
 // (Sherman-Morrison inverse of the acoustic tensor 1/2 (I + e e^H)).
-// t[6] holds Mandel components, overwritten.
+//
+// Both schemes' xi is a complex factor common to its three components times a
+// real vector: with q_p the angle of axis p, the rotated scheme's
+//     xi_p = N_p (e^{i q_p} - 1) prod_{r != p} (1 + e^{i q_r}) / 2
+//          = e^{i (q_1 + q_2 + q_3) / 2} i 2 N_p sin(q_p / 2) prod_{r != p} cos(q_r / 2),
+// eq. (freqrot), and the continuous scheme's is i q_p N_p, eq. (freq).  The range
+// sym(u (x) xi), u any complex vector, does not change with the factor, so the
+// projector is that of the real vector: real times complex products, half the
+// arithmetic of complex ones.  The tables D and M hold 2 N sin(q/2) and
+// cos(q/2), or N q and 1.  (The fused n1 pass, bound by instruction issue: 400 to
+// 384 us at 256^3, 186 to 173 at 192^3; by the FP64 pipe: 502 to 389 at 96^3.)
+//
+// The part that depends on the frequency only (mode and unit vector e) is kept
+// apart from its application, so that a pass projecting two tensors at the same
+// frequency builds xi once.  mode 0: G = 0 (a Nyquist index, or xi = 0
+// numerically); 1: the projection; 2: xi = 0 (the identity on the
+// stress-controlled components g.mask0, zero on the others).  Mandel
+// components t: with h = sqrt2 e the factors 1/sqrt2 of the shear entries drop
+// out, (sqrt2 tau e)_0 = t0 h0 + t5 e1 + t4 e2.
 // ---------------------------------------------------------------------------
-template <typename R>
-__device__ __forceinline__ void gamma_project(cpx<R> *t, cpx<R> x0, cpx<R> x1, cpx<R> x2) {
-    const R n2 = x0.x * x0.x + x0.y * x0.y + x1.x * x1.x + x1.y * x1.y + x2.x * x2.x + x2.y * x2.y;
-    if (!(n2 > (R)0)) {
-#pragma unroll
-        for (int c = 0; c < 6; ++c) t[c] = mk<R>(0, 0);
-        return;
-    }
-    const R inv = (R)1 / sqrt(n2);
-    const cpx<R> e0 = scale<R>(x0, inv), e1 = scale<R>(x1, inv), e2 = scale<R>(x2, inv);
-    const cpx<R> c0 = conjc<R>(e0), c1 = conjc<R>(e1), c2 = conjc<R>(e2);
-    const R r2 = (R)0.70710678118654752440;   // 1/sqrt(2)
-    const cpx<R> T11 = t[0], T22 = t[1], T33 = t[2];
-    const cpx<R> T23 = scale<R>(t[3], r2), T13 = scale<R>(t[4], r2), T12 = scale<R>(t[5], r2);
-    const cpx<R> v0 = add<R>(add<R>(mul<R>(T11, c0), mul<R>(T12, c1)), mul<R>(T13, c2));
-    const cpx<R> v1 = add<R>(add<R>(mul<R>(T12, c0), mul<R>(T22, c1)), mul<R>(T23, c2));
-    const cpx<R> v2 = add<R>(add<R>(mul<R>(T13, c0), mul<R>(T23, c1)), mul<R>(T33, c2));
-    const cpx<R> s = add<R>(add<R>(mul<R>(c0, v0), mul<R>(c1, v1)), mul<R>(c2, v2));
-    const cpx<R> u0 = sub<R>(scale<R>(v0, (R)2), mul<R>(e0, s));
-    const cpx<R> u1 = sub<R>(scale<R>(v1, (R)2), mul<R>(e1, s));
-    const cpx<R> u2 = sub<R>(scale<R>(v2, (R)2), mul<R>(e2, s));
-    t[0] = mul<R>(u0, e0);
-    t[1] = mul<R>(u1, e1);
-    t[2] = mul<R>(u2, e2);
-    t[3] = scale<R>(add<R>(mul<R>(u1, e2), mul<R>(u2, e1)), r2);
-    t[4] = scale<R>(add<R>(mul<R>(u0, e2), mul<R>(u2, e0)), r2);
-    t[5] = scale<R>(add<R>(mul<R>(u0, e1), mul<R>(u1, e0)), r2);
-}
-
-// The projector of eq. (galop) at one frequency, split into the part that
-// depends on the frequency only (mode and unit vector e = xi / |xi|) and its
-// application, so that a pass projecting two tensors at the same frequency
-// builds xi once.  mode 0: G = 0 (a Nyquist index, or xi = 0 numerically);
-// 1: the projection; 2: xi = 0 (the identity on the stress-controlled
-// components g.mask0, zero on the others).
 template <typename R> struct GammaE {
-    cpx<R> e0, e1, e2;
+    R e0, e1, e2;
     int mode;
 };
+
+// 1 / sqrt(n2): in FP32 the hardware's estimate and one Newton step, within an
+// ulp or two of the correctly rounded quotient and a third of its instructions
+__device__ __forceinline__ float inv_norm(float n2) {
+    const float y = rsqrtf(n2);
+    return fmaf(0.5f * y, fmaf(-n2 * y, y, 1.0f), y);
+}
+__device__ __forceinline__ double inv_norm(double n2) { return rsqrt(n2); }
 
 template <typename R>
 __device__ __forceinline__ GammaE<R> gamma_e(const Geometry &g, int k1, int k2, int k3) {
@@ -163,34 +154,60 @@ __device__ __forceinline__ GammaE<R> gamma_e(const Geometry &g, int k1, int k2, 
         q.mode = 2;
         return q;
     }
-    const bool nyq = ((g.n1 & 1) == 0 && 2 * k1 == g.n1) || ((g.n2 & 1) == 0 && 2 * k2 == g.n2) ||
-                     ((g.n3 & 1) == 0 && 2 * k3 == g.n3);
-    if (nyq) return q;
-    const cpx<R> *D0 = reinterpret_cast<const cpx<R> *>(g.D[0]);
-    const cpx<R> *D1 = reinterpret_cast<const cpx<R> *>(g.D[1]);
-    const cpx<R> *D2 = reinterpret_cast<const cpx<R> *>(g.D[2]);
-    const cpx<R> *M0 = reinterpret_cast<const cpx<R> *>(g.M[0]);
-    const cpx<R> *M1 = reinterpret_cast<const cpx<R> *>(g.M[1]);
-    const cpx<R> *M2 = reinterpret_cast<const cpx<R> *>(g.M[2]);
-    const cpx<R> m0 = __ldg(&M0[k1]), m1 = __ldg(&M1[k2]), m2 = __ldg(&M2[k3]);
-    // xi_p = D_p(k_p) prod_{r != p} M_r(k_r): N_p (e^{iq_p} - 1) prod (1 + e^{iq_r})/2
-    // for the rotated scheme of eq. (freqrot), i q_p N_p for eq. (freq)
-    const cpx<R> x0 = mul<R>(__ldg(&D0[k1]), mul<R>(m1, m2));
-    const cpx<R> x1 = mul<R>(__ldg(&D1[k2]), mul<R>(m0, m2));
-    const cpx<R> x2 = mul<R>(__ldg(&D2[k3]), mul<R>(m0, m1));
-    const R n2 = x0.x * x0.x + x0.y * x0.y + x1.x * x1.x + x1.y * x1.y + x2.x * x2.x + x2.y * x2.y;
+    // (2 k = n holds at a Nyquist index only, of an even n)
+    if (2 * k1 == g.n1 || 2 * k2 == g.n2 || 2 * k3 == g.n3) return q;
+    const R m0 = __ldg(reinterpret_cast<const R *>(g.M[0]) + k1), m1 = __ldg(reinterpret_cast<const R *>(g.M[1]) + k2),
+            m2 = __ldg(reinterpret_cast<const R *>(g.M[2]) + k3);
+    const R x0 = __ldg(reinterpret_cast<const R *>(g.D[0]) + k1) * (m1 * m2);
+    const R x1 = __ldg(reinterpret_cast<const R *>(g.D[1]) + k2) * (m0 * m2);
+    const R x2 = __ldg(reinterpret_cast<const R *>(g.D[2]) + k3) * (m0 * m1);
+    const R n2 = x0 * x0 + x1 * x1 + x2 * x2;
     if (!(n2 > (R)0)) return q;
-    const R inv = (R)1 / sqrt(n2);
-    q.e0 = scale<R>(x0, inv);
-    q.e1 = scale<R>(x1, inv);
-    q.e2 = scale<R>(x2, inv);
+    const R inv = inv_norm(n2);
+    q.e0 = x0 * inv;
+    q.e1 = x1 * inv;
+    q.e2 = x2 * inv;
     q.mode = 1;
     return q;
 }
 
-// Orthogonal projection of a symmetric tau (Mandel, t[6], overwritten) onto
-// {sym(u (x) e)}, |e| = 1: sym(u (x) e) with u = 2 tau conj(e) - e (conj(e) .
-// tau conj(e)) (Sherman-Morrison inverse of the acoustic tensor 1/2 (I + e e^H)).
+// a x + b y + c z for real a, b, c
+template <typename R>
+__device__ __forceinline__ cpx<R> comb3(R a, cpx<R> x, R b, cpx<R> y, R c, cpx<R> z) {
+    return mk<R>(a * x.x + b * y.x + c * z.x, a * x.y + b * y.y + c * z.y);
+}
+
+// w = sqrt2 tau e
+template <typename R>
+__device__ __forceinline__ void gamma_vec(const GammaE<R> &q, const cpx<R> *t, cpx<R> *w) {
+    const R s2 = (R)1.41421356237309504880;
+    w[0] = comb3<R>(s2 * q.e0, t[0], q.e1, t[5], q.e2, t[4]);
+    w[1] = comb3<R>(q.e0, t[5], s2 * q.e1, t[1], q.e2, t[3]);
+    w[2] = comb3<R>(q.e0, t[4], q.e1, t[3], s2 * q.e2, t[2]);
+}
+
+// w += a e (e . w)
+template <typename R>
+__device__ __forceinline__ void gamma_p(const GammaE<R> &q, R a, cpx<R> *w) {
+    const cpx<R> s = scale<R>(comb3<R>(q.e0, w[0], q.e1, w[1], q.e2, w[2]), a);
+    w[0] = mk<R>(w[0].x + q.e0 * s.x, w[0].y + q.e0 * s.y);
+    w[1] = mk<R>(w[1].x + q.e1 * s.x, w[1].y + q.e1 * s.y);
+    w[2] = mk<R>(w[2].x + q.e2 * s.x, w[2].y + q.e2 * s.y);
+}
+
+// t = sym(sqrt2 w (x) e)
+template <typename R>
+__device__ __forceinline__ void gamma_sym(const GammaE<R> &q, const cpx<R> *w, cpx<R> *t) {
+    const R s2 = (R)1.41421356237309504880;
+    t[0] = scale<R>(w[0], s2 * q.e0);
+    t[1] = scale<R>(w[1], s2 * q.e1);
+    t[2] = scale<R>(w[2], s2 * q.e2);
+    t[3] = mk<R>(w[1].x * q.e2 + w[2].x * q.e1, w[1].y * q.e2 + w[2].y * q.e1);
+    t[4] = mk<R>(w[0].x * q.e2 + w[2].x * q.e0, w[0].y * q.e2 + w[2].y * q.e0);
+    t[5] = mk<R>(w[0].x * q.e1 + w[1].x * q.e0, w[0].y * q.e1 + w[1].y * q.e0);
+}
+
+// t (6 Mandel components, overwritten) = G t: u / sqrt2 = w - e (e . w) / 2
 template <typename R>
 __device__ __forceinline__ void gamma_apply(const Geometry &g, const GammaE<R> &q, cpx<R> *t) {
     if (q.mode != 1) {
@@ -199,24 +216,10 @@ __device__ __forceinline__ void gamma_apply(const Geometry &g, const GammaE<R> &
             if (q.mode == 0 || !((g.mask0 >> c) & 1)) t[c] = mk<R>(0, 0);
         return;
     }
-    const cpx<R> e0 = q.e0, e1 = q.e1, e2 = q.e2;
-    const cpx<R> c0 = conjc<R>(e0), c1 = conjc<R>(e1), c2 = conjc<R>(e2);
-    const R r2 = (R)0.70710678118654752440;   // 1/sqrt(2)
-    const cpx<R> T11 = t[0], T22 = t[1], T33 = t[2];
-    const cpx<R> T23 = scale<R>(t[3], r2), T13 = scale<R>(t[4], r2), T12 = scale<R>(t[5], r2);
-    const cpx<R> v0 = add<R>(add<R>(mul<R>(T11, c0), mul<R>(T12, c1)), mul<R>(T13, c2));
-    const cpx<R> v1 = add<R>(add<R>(mul<R>(T12, c0), mul<R>(T22, c1)), mul<R>(T23, c2));
-    const cpx<R> v2 = add<R>(add<R>(mul<R>(T13, c0), mul<R>(T23, c1)), mul<R>(T33, c2));
-    const cpx<R> sc = add<R>(add<R>(mul<R>(c0, v0), mul<R>(c1, v1)), mul<R>(c2, v2));
-    const cpx<R> u0 = sub<R>(scale<R>(v0, (R)2), mul<R>(e0, sc));
-    const cpx<R> u1 = sub<R>(scale<R>(v1, (R)2), mul<R>(e1, sc));
-    const cpx<R> u2 = sub<R>(scale<R>(v2, (R)2), mul<R>(e2, sc));
-    t[0] = mul<R>(u0, e0);
-    t[1] = mul<R>(u1, e1);
-    t[2] = mul<R>(u2, e2);
-    t[3] = scale<R>(add<R>(mul<R>(u1, e2), mul<R>(u2, e1)), r2);
-    t[4] = scale<R>(add<R>(mul<R>(u0, e2), mul<R>(u2, e0)), r2);
-    t[5] = scale<R>(add<R>(mul<R>(u0, e1), mul<R>(u1, e0)), r2);
+    cpx<R> w[3];
+    gamma_vec<R>(q, t, w);
+    gamma_p<R>(q, (R)-0.5, w);
+    gamma_sym<R>(q, w, t);
 }
 
 // G at frequency (k1,k2,k3) on the 6 Mandel components at p[0..5] (stride 1)
@@ -228,23 +231,12 @@ __device__ __forceinline__ void gamma_at(const Geometry &g, int k1, int k2, int 
 
 // The projector's range at a frequency has three degrees of freedom, and the
 // fused MINRES step keeps its Krylov vectors in them: q with |q| = |strain|
-// (Mandel).  With P x = sqrt2 x + (1 - sqrt2) e (e^H x), |e| = 1,
-//   strain = B q = sym(P q (x) e),   q = B^H tau = P (tau conj(e)),
-// B is an isometry onto the range (|sym(u (x) e)|^2 = (|u|^2 + |e^H u|^2) / 2)
+// (Mandel).  With P x = sqrt2 x + (1 - sqrt2) e (e . x), |e| = 1,
+//   strain = B q = sym(P q (x) e),   q = B^H tau = P (tau e),
+// B is an isometry onto the range (|sym(u (x) e)|^2 = (|u|^2 + |e . u|^2) / 2)
 // and G = B B^H, so MINRES on B^H F C F^-1 B is the iteration on G F C F^-1 G
-// in half the storage.  At xi = 0 the six stress-controlled components are
-// real: two to a value.
-template <typename R>
-__device__ __forceinline__ void gamma_p(const GammaE<R> &ge, cpx<R> *x) {
-    const R s2 = (R)1.41421356237309504880, a = (R)-0.41421356237309504880;
-    const cpx<R> s = add<R>(add<R>(mul<R>(conjc<R>(ge.e0), x[0]), mul<R>(conjc<R>(ge.e1), x[1])),
-                            mul<R>(conjc<R>(ge.e2), x[2]));
-    const cpx<R> as = scale<R>(s, a);
-    x[0] = add<R>(scale<R>(x[0], s2), mul<R>(ge.e0, as));
-    x[1] = add<R>(scale<R>(x[1], s2), mul<R>(ge.e1, as));
-    x[2] = add<R>(scale<R>(x[2], s2), mul<R>(ge.e2, as));
-}
-
+// in half the storage.  P x / sqrt2 = x + (1/sqrt2 - 1) e (e . x).  At xi = 0
+// the six stress-controlled components are real: two to a value.
 // q = B^H t
 template <typename R>
 __device__ __forceinline__ void gamma_to_q(const Geometry &g, const GammaE<R> &ge, const cpx<R> *t, cpx<R> *q) {
@@ -255,13 +247,8 @@ __device__ __forceinline__ void gamma_to_q(const Geometry &g, const GammaE<R> &g
                                                       (g.mask0 >> (2 * c + 1)) & 1 ? t[2 * c + 1].x : (R)0);
         return;
     }
-    const cpx<R> c0 = conjc<R>(ge.e0), c1 = conjc<R>(ge.e1), c2 = conjc<R>(ge.e2);
-    const R r2 = (R)0.70710678118654752440;   // 1/sqrt(2)
-    const cpx<R> T23 = scale<R>(t[3], r2), T13 = scale<R>(t[4], r2), T12 = scale<R>(t[5], r2);
-    q[0] = add<R>(add<R>(mul<R>(t[0], c0), mul<R>(T12, c1)), mul<R>(T13, c2));
-    q[1] = add<R>(add<R>(mul<R>(T12, c0), mul<R>(t[1], c1)), mul<R>(T23, c2));
-    q[2] = add<R>(add<R>(mul<R>(T13, c0), mul<R>(T23, c1)), mul<R>(t[2], c2));
-    gamma_p<R>(ge, q);
+    gamma_vec<R>(ge, t, q);
+    gamma_p<R>(ge, (R)-0.29289321881345247560, q);
 }
 
 // t = B q
@@ -273,15 +260,9 @@ __device__ __forceinline__ void gamma_from_q(const Geometry &g, const GammaE<R> 
             t[c] = ge.mode == 0 || !((g.mask0 >> c) & 1) ? mk<R>(0, 0) : mk<R>(c & 1 ? q[c / 2].y : q[c / 2].x, 0);
         return;
     }
-    const R r2 = (R)0.70710678118654752440;   // 1/sqrt(2)
-    cpx<R> u[3] = {q[0], q[1], q[2]};
-    gamma_p<R>(ge, u);
-    t[0] = mul<R>(u[0], ge.e0);
-    t[1] = mul<R>(u[1], ge.e1);
-    t[2] = mul<R>(u[2], ge.e2);
-    t[3] = scale<R>(add<R>(mul<R>(u[1], ge.e2), mul<R>(u[2], ge.e1)), r2);
-    t[4] = scale<R>(add<R>(mul<R>(u[0], ge.e2), mul<R>(u[2], ge.e0)), r2);
-    t[5] = scale<R>(add<R>(mul<R>(u[0], ge.e1), mul<R>(u[1], ge.e0)), r2);
+    cpx<R> w[3] = {q[0], q[1], q[2]};
+    gamma_p<R>(ge, (R)-0.29289321881345247560, w);
+    gamma_sym<R>(ge, w, t);
 }
 
 // Run the transform of the L lines in buf.  Fast engine: in place, returns
