@@ -762,12 +762,12 @@ static int build_cg_graph(hom_ctx *ctx, Engine<R> &E) {
     return HOM_OK;
 }
 
-// PCG on A^alpha x = rhs (ctx->rhs, 3-component spectrum), zero start;
+// PCG on A^alpha x = rhs (ctx->rhs, 3-component spectrum of norm rnorm), zero start;
 // solution in ctx->xs.  As the paper does (section 2.2) the preconditioned CG
 // recurrences are used although A^alpha is not symmetric where chi_v is
 // non-zero; the FP64 true residual checks the result.
 template <typename R>
-static int run_cg(hom_ctx *ctx, Engine<R> &E, double tol, int max_it, int *iters, double *est, int *status) {
+static int run_cg(hom_ctx *ctx, Engine<R> &E, double rnorm, double tol, int max_it, int *iters, double *est, int *status) {
     const long long nr = 6 * ctx->S;   // reals per 3-component spectral vector
     cudaStream_t s = ctx->stream;
     int rc = build_cg_graph<R>(ctx, E);
@@ -782,6 +782,10 @@ static int run_cg(hom_ctx *ctx, Engine<R> &E, double tol, int max_it, int *iters
     CU(cudaMemcpyAsync(r, ctx->rhs, sizeof(R) * nr, cudaMemcpyDeviceToDevice, s));
     // z0 = M r0 and <r0, z0>, ||r0||^2 through one step of length 0
     memset(ctx->h_cg, 0, sizeof(CgState));
+    // powers of two that FP32 holds; 1 where rnorm is 0 or not finite
+    const double rms = rnorm / std::sqrt((double)nr);
+    if (rms > 0.0 && std::isfinite(rms)) ctx->h_cg->sc = std::ldexp(1.0, std::max(-126, std::min(126, -std::ilogb(rms))));
+    else ctx->h_cg->sc = 1.0;
     CU(cudaMemcpyAsync(ctx->d_cg, ctx->h_cg, sizeof(CgState), cudaMemcpyHostToDevice, s));
     const int np = Launch<R>::ew_grid(E.g.S);
     Launch<R>::cg_xr(E.g, s, lam_b, mu_b, x, r, p, q, z, ctx->d_cg, ctx->partials);
@@ -1728,12 +1732,12 @@ static int solve_case_modb(hom_ctx *ctx, int icase, const double *m, double tol,
         double est = 0.0;
         if (ctx->prec == HOM_PREC_FP64) {
             CU(cudaMemcpyAsync(ctx->rhs, ctx->r64, sizeof(double2) * nc3, cudaMemcpyDeviceToDevice, s));
-            rc = run_cg<double>(ctx, ctx->e64, sweep_tol, budget, &it, &est, &st);
+            rc = run_cg<double>(ctx, ctx->e64, tres * bnorm, sweep_tol, budget, &it, &est, &st);
             if (rc) return rc;
             Launch<double>::axpby(2 * nc3, s, 1.0, (const double *)ctx->xs, 1.0, (double *)x);
         } else {
             spec_d2f(nc3, s, ctx->r64, (float2 *)ctx->rhs);
-            rc = run_cg<float>(ctx, ctx->e32, sweep_tol, budget, &it, &est, &st);
+            rc = run_cg<float>(ctx, ctx->e32, tres * bnorm, sweep_tol, budget, &it, &est, &st);
             if (rc) return rc;
             spec_f2d_acc(nc3, s, (const float2 *)ctx->xs, x);
         }

@@ -167,6 +167,7 @@ struct CgState {
     double a, b;       // step length and direction update of this iteration
     double tol;
     double est;        // ||r_k|| / ||r_0||
+    double sc;         // about 1 / rms(r_0), a power of two (MoDBFFT)
 };
 
 // Kernel-side description of one cell for one precision.

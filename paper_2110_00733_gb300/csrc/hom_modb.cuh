@@ -15,7 +15,8 @@
 namespace hom {
 
 // frequency index of half-spectrum point f and its continuous xi / (i 2 pi)
-__device__ __forceinline__ void modb_freq(const Geometry &g, int f, double q[3], int &k3) {
+template <typename R>
+__device__ __forceinline__ void modb_freq(const Geometry &g, int f, R q[3], int &k3) {
     const int hh = g.h;
     k3 = f % hh;
     const int rest = f / hh;
@@ -24,7 +25,7 @@ __device__ __forceinline__ void modb_freq(const Geometry &g, int f, double q[3],
 #pragma unroll
     for (int p = 0; p < 3; ++p) {
         const int n = ns[p], k = ks[p];
-        q[p] = ((n & 1) == 0 && 2 * k == n) ? 0.0 : (double)((2 * k < n) ? k : k - n);
+        q[p] = 2 * k == n ? (R)0 : (R)((2 * k < n) ? k : k - n);
     }
 }
 
@@ -54,12 +55,12 @@ __global__ void __launch_bounds__(kEwThreads) k_modb_contract(Geometry g, const 
     const R r2 = (R)0.70710678118654752440;
     double acc = 0.0;
     for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < (int)g.S; f += gridDim.x * blockDim.x) {
-        double qd[3];
+        R qd[3];
         int k3;
         modb_freq(g, f, qd, k3);
         cpx<R> r[3] = {mk<R>(0, 0), mk<R>(0, 0), mk<R>(0, 0)};
-        if (!(qd[0] == 0.0 && qd[1] == 0.0 && qd[2] == 0.0)) {
-            const R s[3] = {tp * (R)qd[0], tp * (R)qd[1], tp * (R)qd[2]};
+        if (!(qd[0] == 0 && qd[1] == 0 && qd[2] == 0)) {
+            const R s[3] = {tp * qd[0], tp * qd[1], tp * qd[2]};
             const cpx<R> *t = in + (size_t)f * 10;
             const cpx<R> T[3][3] = {{t[0], scale<R>(t[5], r2), scale<R>(t[4], r2)},
                                     {scale<R>(t[5], r2), t[1], scale<R>(t[3], r2)},
@@ -71,7 +72,7 @@ __global__ void __launch_bounds__(kEwThreads) k_modb_contract(Geometry g, const 
                 r[i] = add<R>(mk<R>(-a.y, a.x), t[6 + i]);
             }
         }
-        const double w = (k3 == 0 || 2 * k3 == g.n3) ? 1.0 : 2.0;
+        const double w = (double)pweight(k3, g.n3);
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             out[3 * f + i] = r[i];
@@ -87,53 +88,108 @@ __global__ void __launch_bounds__(kEwThreads) k_modb_contract(Geometry g, const 
     }
 }
 
-// out3 = [xi . Cbar . xi]^-1 in3, Cbar isotropic (lam_b, mu_b): with xi = i s,
-// xi.Cbar.xi = -((lam+mu) s s^T + mu |s|^2 I), inverse in closed form.
-template <typename R>
-__device__ __forceinline__ void modb_precond_point(double lam_b, double mu_b, const double qd[3], const cpx<R> *in,
-                                                   cpx<R> *out) {
-    if (qd[0] == 0.0 && qd[1] == 0.0 && qd[2] == 0.0) {
-        out[0] = out[1] = out[2] = mk<R>(0, 0);
+// out3 = [xi . Cbar . xi]^-1 in3, Cbar isotropic (lam_b, mu_b).  With xi = i 2 pi q,
+// q integers and Q = |q|^2, xi.Cbar.xi = -4 pi^2 ((lam+mu) q q^T + mu Q I), whose
+// inverse is A / Q (I - c q q^T / Q), A = -1 / (4 pi^2 mu), c = (lam+mu) / (lam+2 mu).
+template <typename R> struct PrecondCoef;
+template <> struct PrecondCoef<double> { double A, c; };
+// FP32 fields: the coefficients as sums of two floats
+template <> struct PrecondCoef<float> { float Ah, Al, ch, cl; };
+
+template <typename R> PrecondCoef<R> precond_coef(double lam_b, double mu_b) {
+    const double A = -1.0 / (39.47841760435743447534 * mu_b), c = (lam_b + mu_b) / (lam_b + 2.0 * mu_b);
+    if constexpr (sizeof(R) == 8) return PrecondCoef<R>{A, c};
+    else {
+        const float Ah = (float)A, ch = (float)c;
+        return PrecondCoef<R>{Ah, (float)(A - Ah), ch, (float)(c - ch)};
+    }
+}
+
+__device__ __forceinline__ void modb_precond_point(const PrecondCoef<double> &k, const double q[3], const double2 *v,
+                                                   double2 *out) {
+    const double Q = q[0] * q[0] + q[1] * q[1] + q[2] * q[2];
+    if (Q == 0.0) {
+        out[0] = out[1] = out[2] = mk<double>(0, 0);
         return;
     }
-    const double tp = 6.28318530717958647692;
-    const double s0 = tp * qd[0], s1 = tp * qd[1], s2 = tp * qd[2];
-    const double ss = s0 * s0 + s1 * s1 + s2 * s2;
-    const double a = -1.0 / (mu_b * ss), b = (lam_b + mu_b) / ((lam_b + 2.0 * mu_b) * ss);
-    const cpx<R> v0 = in[0], v1 = in[1], v2 = in[2];
-    const double dre = s0 * v0.x + s1 * v1.x + s2 * v2.x, dim = s0 * v0.y + s1 * v1.y + s2 * v2.y;
-    const double sv[3] = {s0, s1, s2};
-    const cpx<R> vv[3] = {v0, v1, v2};
+    const double iq = 1.0 / Q, a = k.A * iq, b = k.c * iq;
+    const double dre = b * (q[0] * v[0].x + q[1] * v[1].x + q[2] * v[2].x),
+                 dim = b * (q[0] * v[0].y + q[1] * v[1].y + q[2] * v[2].y);
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
-        out[i] = mk<R>((R)(a * (vv[i].x - b * sv[i] * dre)), (R)(a * (vv[i].y - b * sv[i] * dim)));
+    for (int i = 0; i < 3; ++i) out[i] = mk<double>(a * (v[i].x - q[i] * dre), a * (v[i].y - q[i] * dim));
+}
+
+// FP32 fields: the same in sums of two floats (48 bits) rounded to FP32 at the
+// end.  FP64 arithmetic gives the same rounding but runs at 1/64 of the rate:
+// with its two divisions a point it bound the PCG step (see k_cg_xr).
+__device__ __forceinline__ float2 ff_two_sum(float a, float b) {   // (sum, its rounding error)
+    const float s = a + b, t = s - a;
+    return make_float2(s, (a - (s - t)) + (b - t));
+}
+// sum_i q_i v_i as (hi, lo)
+__device__ __forceinline__ float2 ff_dot3(const float q[3], float v0, float v1, float v2) {
+    const float p0 = q[0] * v0, p1 = q[1] * v1, p2 = q[2] * v2;
+    const float e0 = fmaf(q[0], v0, -p0), e1 = fmaf(q[1], v1, -p1), e2 = fmaf(q[2], v2, -p2);
+    const float2 s1 = ff_two_sum(p0, p1), s2 = ff_two_sum(s1.x, p2);
+    const float lo = ((s1.y + s2.y) + (e0 + e1)) + e2, hi = s2.x + lo;   // renormalised
+    return make_float2(hi, lo - (hi - s2.x));
+}
+__device__ __forceinline__ float2 ff_mul(float2 a, float2 b) {
+    const float p = a.x * b.x;
+    return make_float2(p, fmaf(a.x, b.x, -p) + (a.x * b.y + a.y * b.x));
+}
+__device__ __forceinline__ void modb_precond_point(const PrecondCoef<float> &k, const float q[3], const float2 *v,
+                                                   float2 *out) {
+    const float Q = q[0] * q[0] + q[1] * q[1] + q[2] * q[2];   // exact: below 2^24 up to 4096^3
+    if (Q == 0.f) {
+        out[0] = out[1] = out[2] = mk<float>(0, 0);
+        return;
+    }
+    const float y = 1.0f / Q;
+    const float2 iq = make_float2(y, fmaf(-Q, y, 1.0f) * y);
+    const float2 a = ff_mul(make_float2(k.Ah, k.Al), iq), b = ff_mul(make_float2(k.ch, k.cl), iq);
+    const float2 dre = ff_mul(b, ff_dot3(q, v[0].x, v[1].x, v[2].x)), dim = ff_mul(b, ff_dot3(q, v[0].y, v[1].y, v[2].y));
+    auto comp = [&](float x, float qi, float2 d) {   // a (x - q_i d)
+        const float p = qi * d.x, e = fmaf(qi, d.x, -p) + qi * d.y;
+        const float2 s = ff_two_sum(x, -p);
+        const float l = s.y - e;
+        const float h = s.x * a.x;
+        return h + (fmaf(s.x, a.x, -h) + (s.x * a.y + l * a.x));
+    };
+#pragma unroll
+    for (int i = 0; i < 3; ++i) out[i] = mk<float>(comp(v[i].x, q[i], dre), comp(v[i].y, q[i], dim));
 }
 
 template <typename R>
-__global__ void k_modb_precond(Geometry g, double lam_b, double mu_b, const cpx<R> *__restrict__ in,
-                               cpx<R> *__restrict__ out) {
+__global__ void k_modb_precond(Geometry g, PrecondCoef<R> pc, const cpx<R> *__restrict__ in, cpx<R> *__restrict__ out) {
     for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < (int)g.S; f += gridDim.x * blockDim.x) {
-        double qd[3];
+        R q[3];
         int k3;
-        modb_freq(g, f, qd, k3);
-        modb_precond_point<R>(lam_b, mu_b, qd, in + 3 * f, out + 3 * f);
+        modb_freq(g, f, q, k3);
+        modb_precond_point(pc, q, in + 3 * f, out + 3 * f);
     }
 }
 
 // PCG step: x += a p; r -= a q; z = M r; partials <r,z> (first half) and
-// <r,r> (second half), Parseval-weighted
+// <r,r> (second half), Parseval-weighted.  Bound by HBM (seven 3-component
+// vectors); the sums of a thread's points are kept as two floats (Acc: each
+// product exact, a point's rounding 2^-47 of it) and added in FP64 over the
+// grid, where rounding at 2^-53 of the total outweighs the points' random errors;
+// st->sc, a power of two, brings the products into the range of FP32.
+// In FP64 throughout the pass was bound by the FP64 pipe: 191 us at 128^3.
 template <typename R>
-__global__ void __launch_bounds__(kEwThreads) k_cg_xr(Geometry g, double lam_b, double mu_b, cpx<R> *__restrict__ x,
+__global__ void __launch_bounds__(kEwThreads) k_cg_xr(Geometry g, PrecondCoef<R> pc, cpx<R> *__restrict__ x,
                                                       cpx<R> *__restrict__ r, const cpx<R> *__restrict__ p,
                                                       const cpx<R> *__restrict__ q, cpx<R> *__restrict__ z,
                                                       const CgState *st, double *partials) {
     if (st->done) return;
-    const R a = (R)st->a;
-    double rz = 0.0, rr = 0.0;
+    const R a = (R)st->a, sc = (R)st->sc;
+    const double isc2 = 1.0 / (st->sc * st->sc);
+    Acc<R> rz, rr;
     for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < (int)g.S; f += gridDim.x * blockDim.x) {
-        double qd[3];
+        R qv[3];
         int k3;
-        modb_freq(g, f, qd, k3);
+        modb_freq(g, f, qv, k3);
         cpx<R> rv[3], zv[3];
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
@@ -142,19 +198,22 @@ __global__ void __launch_bounds__(kEwThreads) k_cg_xr(Geometry g, double lam_b, 
             rv[i] = mk<R>(rr0.x - a * qq.x, rr0.y - a * qq.y);
             r[3 * f + i] = rv[i];
         }
-        modb_precond_point<R>(lam_b, mu_b, qd, rv, zv);
-        const double w = (k3 == 0 || 2 * k3 == g.n3) ? 1.0 : 2.0;
+        modb_precond_point(pc, qv, rv, zv);
+        const R w = (R)pweight(k3, g.n3);
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             z[3 * f + i] = zv[i];
-            rz += w * ((double)rv[i].x * zv[i].x + (double)rv[i].y * zv[i].y);
-            rr += w * ((double)rv[i].x * rv[i].x + (double)rv[i].y * rv[i].y);
+            const cpx<R> rs = scale<R>(rv[i], sc), zs = scale<R>(zv[i], sc);
+            rz.add_prod(w * rs.x, zs.x);
+            rz.add_prod(w * rs.y, zs.y);
+            rr.add_prod(w * rs.x, rs.x);
+            rr.add_prod(w * rs.y, rs.y);
         }
     }
-    const double s1 = block_sum(rz);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s1;
-    const double s2 = block_sum(rr);
-    if (threadIdx.x == 0) partials[gridDim.x + blockIdx.x] = s2;
+    const double s1 = block_sum(rz.value());
+    if (threadIdx.x == 0) partials[blockIdx.x] = isc2 * s1;
+    const double s2 = block_sum(rr.value());
+    if (threadIdx.x == 0) partials[gridDim.x + blockIdx.x] = isc2 * s2;
 }
 
 // PCG direction: p = z + b p
@@ -182,12 +241,12 @@ void Launch<R>::modb_contract(const Geometry &g, cudaStream_t st, const cpx<R> *
 template <typename R>
 void Launch<R>::modb_precond(const Geometry &g, cudaStream_t st, double lam_b, double mu_b, const cpx<R> *in,
                              cpx<R> *out) {
-    k_modb_precond<R><<<ew_grid(g.S), kEwThreads, 0, st>>>(g, lam_b, mu_b, in, out);
+    k_modb_precond<R><<<ew_grid(g.S), kEwThreads, 0, st>>>(g, precond_coef<R>(lam_b, mu_b), in, out);
 }
 template <typename R>
 void Launch<R>::cg_xr(const Geometry &g, cudaStream_t st, double lam_b, double mu_b, cpx<R> *x, cpx<R> *r,
                       const cpx<R> *p, const cpx<R> *q, cpx<R> *z, const CgState *state, double *partials) {
-    k_cg_xr<R><<<ew_grid(g.S), kEwThreads, 0, st>>>(g, lam_b, mu_b, x, r, p, q, z, state, partials);
+    k_cg_xr<R><<<ew_grid(g.S), kEwThreads, 0, st>>>(g, precond_coef<R>(lam_b, mu_b), x, r, p, q, z, state, partials);
 }
 template <typename R>
 void Launch<R>::cg_p(const Geometry &g, cudaStream_t st, cpx<R> *p, const cpx<R> *z, const CgState *state) {

@@ -904,17 +904,17 @@ template <typename R>
 __device__ __forceinline__ void modb_contract_at(const Geometry &g, int k1, int k2, int k3, const cpx<R> *t,
                                                  cpx<R> r[3]) {
     const int ks[3] = {k1, k2, k3}, ns[3] = {g.n1, g.n2, g.n3};
-    double q[3];
+    R q[3];
 #pragma unroll
     for (int p = 0; p < 3; ++p) {
         const int n = ns[p], k = ks[p];
-        q[p] = ((n & 1) == 0 && 2 * k == n) ? 0.0 : (double)((2 * k < n) ? k : k - n);
+        q[p] = 2 * k == n ? (R)0 : (R)((2 * k < n) ? k : k - n);
     }
     r[0] = r[1] = r[2] = mk<R>(0, 0);
-    if (q[0] == 0.0 && q[1] == 0.0 && q[2] == 0.0) return;
+    if (q[0] == 0 && q[1] == 0 && q[2] == 0) return;
     const R tp = (R)6.28318530717958647692;
     const R r2 = (R)0.70710678118654752440;
-    const R sv[3] = {tp * (R)q[0], tp * (R)q[1], tp * (R)q[2]};
+    const R sv[3] = {tp * q[0], tp * q[1], tp * q[2]};
     const cpx<R> T[3][3] = {{t[0], scale<R>(t[5], r2), scale<R>(t[4], r2)},
                             {scale<R>(t[5], r2), t[1], scale<R>(t[3], r2)},
                             {scale<R>(t[4], r2), scale<R>(t[3], r2), t[2]}};
@@ -935,20 +935,20 @@ template <typename R>
 __device__ __forceinline__ void modb_expand_at(const Geometry &g, int k1, int k2, int k3, const cpx<R> *u, R alpha,
                                                int with_penalty, int nc_out, cpx<R> *o) {
     const int ks[3] = {k1, k2, k3}, ns[3] = {g.n1, g.n2, g.n3};
-    double qd[3];
+    R qd[3];
 #pragma unroll
     for (int p = 0; p < 3; ++p) {
         const int n = ns[p], k = ks[p];
-        qd[p] = ((n & 1) == 0 && 2 * k == n) ? 0.0 : (double)((2 * k < n) ? k : k - n);
+        qd[p] = 2 * k == n ? (R)0 : (R)((2 * k < n) ? k : k - n);
     }
-    if (qd[0] == 0.0 && qd[1] == 0.0 && qd[2] == 0.0) {
+    if (qd[0] == 0 && qd[1] == 0 && qd[2] == 0) {
         for (int c = 0; c < nc_out; ++c) o[c] = mk<R>(0, 0);
         return;
     }
     const R tp = (R)6.28318530717958647692;   // 2 pi
     const R r2 = (R)1.41421356237309504880;
     // xi = i s, s = 2 pi q (real): sym(u (x) xi)_ij = i/2 (u_i s_j + u_j s_i)
-    const R s0 = tp * (R)qd[0], s1 = tp * (R)qd[1], s2 = tp * (R)qd[2];
+    const R s0 = tp * qd[0], s1 = tp * qd[1], s2 = tp * qd[2];
     const cpx<R> u0 = u[0], u1 = u[1], u2 = u[2];
     auto isym = [](cpx<R> a, R sa, cpx<R> b, R sb) {   // i/2 (a sb + b sa)
         const R re = (R)0.5 * (a.x * sb + b.x * sa), im = (R)0.5 * (a.y * sb + b.y * sa);
