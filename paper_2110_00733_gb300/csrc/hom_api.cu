@@ -63,12 +63,14 @@ struct Status {
 template <typename R> struct Engine {
     Geometry g{};
     Geometry gm{};             // MoDBFFT chain: 10 components per frequency
+    Geometry gj{};             // elastoplastic increments: see op_geom
     R *phi = nullptr;
     cpx<R> *spec = nullptr;
     cpx<R> *spec10 = nullptr;  // MoDBFFT work spectrum
     void *tw[3] = {nullptr, nullptr, nullptr};
     void *D[3] = {nullptr, nullptr, nullptr};
     void *M[3] = {nullptr, nullptr, nullptr};
+    void *DMc[3] = {nullptr, nullptr, nullptr};   // FP64: both as complex values
 };
 
 // History and Newton work fields of an elastoplastic cell (hom_j2_*), FP64
@@ -145,6 +147,7 @@ struct hom_ctx {
     bool graph_loops = false;        // graph is a device-side WHILE loop over the body
     bool host_loop = false;          // asked for the host-replayed body
     int pdl = 0;                     // programmatic launches inside the stacked MINRES graph
+    bool j2_ops = false;             // within an elastoplastic increment (op_geom)
     bool tangent_op = false;         // operator of eq. (galnonlin) with the J2 tangent (FP64)
     bool graph_tangent = false;      // the captured graph applies the tangent operator
     J2State j2;
@@ -231,29 +234,49 @@ template <typename R> static size_t cpx_size() { return sizeof(R) * 2; }
 //  fast engine: threads = lines * n / E, one buffer of lines * n values
 //  generic engine: Stockham ping-pong, two buffers
 template <typename R>
-static int set_shapes(hom_ctx *ctx, Geometry &g, int nc) {
+static int set_shapes(hom_ctx *ctx, Geometry &g, int nc, bool lines = true) {
+    constexpr int kSms = 152;
     const size_t cs = cpx_size<R>();
     const int np = nc / 2;   // component pairs of the n3 pass
     g.nc = nc;
+    const bool f64 = sizeof(R) == 8 && lines;   // FP64 on the line engine
+    const int elems3 = sizeof(R) == 4 ? fast_elems_n3(g.n3) : fast_elems(g.n3);
     int rows, t2, t1;
-    if (g.fast[2]) {
-        rows = 48 / (np * (g.n3 / fast_elems_n3r<R>(g.n3)));
+    const int tpl1 = f64 ? f64_line_tpl(g.n1) : 0, tpl2 = f64 ? f64_line_tpl(g.n2) : 0, tpl3 = f64 ? f64_line_tpl(g.n3) : 0;
+    if (tpl3) {
+        // measured (6-component spectra, ms): 96^3 8 rows 0.318, 4 0.324; 108^3 0.490, 0.519;
+        // 128^3 0.699, 0.660 (51 KB of shared memory a CTA against 27); 192^3 2.72, 2.48; 48^3
+        // 8 rows 0.045, 16 0.066
+        rows = (size_t)g.n3 * ((8 * np) | 1) * cs <= 45 * 1024 ? 8 : 4;
+        while (np * rows * tpl3 < 96) rows *= 2;
+        while (rows > 1 && g.n1 * g.n2 < kSms * rows) rows >>= 1;   // small cells: every SM's FP64 pipe
+        while (rows > 1 && (np * rows * tpl3 > 512 || (size_t)g.n3 * ((rows * np) | 1) * cs > 110 * 1024)) rows >>= 1;
+    } else if (g.fast[2]) {
+        rows = 48 / (np * (g.n3 / elems3));
         rows = rows < 1 ? 1 : (rows > 64 ? 64 : rows);
-        // the two-stage FP32 plans at 96 and 160, measured (6-component
-        // spectra): 8 rows at 160 (0.123 against 0.136 ms at 160^3), 2 at 96
-        // (0.027 against 0.029 ms at 96^3)
-        if (fast_elems_n3r<R>(g.n3) != fast_elems(g.n3) && nc == 6) rows = g.n3 == 160 ? 8 : 2;
+        // the two-stage plans at 96 and 160, measured (6-component spectra): 8
+        // rows at 160 (0.123 against 0.136 ms at 160^3), 2 at 96 (0.027 against
+        // 0.029 ms at 96^3)
+        if (sizeof(R) == 4 && fast_elems_n3(g.n3) != fast_elems(g.n3) && nc == 6) rows = g.n3 == 160 ? 8 : 2;
     } else {
         rows = 16;
         while (rows > 1 && 2ull * g.n3 * np * rows * cs > 48 * 1024) rows >>= 1;
     }
-    if (g.fast[1]) {
+    if (tpl2) {
+        t2 = tpl2 <= 8 ? 16 : 8;
+        while (t2 > 4 && g.n1 * nc * g.h < kSms * t2) t2 >>= 1;
+    } else if (g.fast[1]) {
         t2 = g.n2 >= 512 ? 8 : (g.n2 >= 128 ? 16 : 32);
     } else {
         t2 = 32;
         while (t2 > 1 && 2ull * g.n2 * t2 * cs > 64 * 1024) t2 >>= 1;
     }
-    if (g.fast[0]) {
+    if (tpl1) {
+        // powers of two (odd counts cross 128-byte lines: 96^3 four columns 0.394 ms, three 0.453, six 0.484)
+        t1 = 192 / (nc * tpl1);
+        t1 = t1 >= 8 ? 8 : (t1 >= 4 ? 4 : (t1 >= 2 ? 2 : 1));
+        while (t1 > 1 && g.n2 * g.h < kSms * t1) t1 >>= 1;
+    } else if (g.fast[0]) {
         t1 = 192 * fast_elems(g.n1) / (nc * g.n1);
         t1 = t1 < 1 ? 1 : (t1 > 16 ? 16 : t1);
     } else {
@@ -275,14 +298,24 @@ static int set_shapes(hom_ctx *ctx, Geometry &g, int nc) {
     auto round32 = [](int v) { return (v + 31) / 32 * 32; };
     auto clampt = [](int v) { return v < 128 ? 128 : (v > 512 ? 512 : v); };
     const int es3 = (np * rows) | 1;   // element stride of the n3 tile (odd)
-    if (g.fast[2]) {
-        g.threads3 = np * rows * (g.n3 / fast_elems_n3r<R>(g.n3));
+    // FP64: the line engine, unless an explicit shape asks for more threads of it than a CTA takes
+    g.line[0] = tpl1 && nc * t1 * tpl1 <= (nc == 6 ? 384 : 512) ? g.n1 : 0;
+    g.line[1] = tpl2 && t2 * tpl2 <= 512 ? g.n2 : 0;
+    g.line[2] = tpl3 && np * rows * tpl3 <= 512 ? g.n3 : 0;
+    if (g.line[2]) {
+        g.threads3 = np * rows * tpl3;
+        g.smem3 = (size_t)es3 * g.n3 * cs;
+    } else if (g.fast[2]) {
+        g.threads3 = np * rows * (g.n3 / elems3);
         g.smem3 = ((size_t)es3 * g.n3 + g.n3 / 16 + 1) * cs;   // + one pad slot per 16 elements
     } else {
         g.threads3 = clampt(round32(np * rows * g.n3 / 16));
         g.smem3 = 2ull * es3 * g.n3 * cs;
     }
-    if (g.fast[1]) {
+    if (g.line[1]) {
+        g.threads2 = t2 * tpl2;
+        g.smem2 = (size_t)t2 * g.n2 * cs;
+    } else if (g.fast[1]) {
         g.threads2 = t2 * (g.n2 / fast_elems(g.n2));
         g.smem2 = (size_t)t2 * g.n2 * cs;
     } else {
@@ -290,7 +323,10 @@ static int set_shapes(hom_ctx *ctx, Geometry &g, int nc) {
         g.smem2 = 2ull * t2 * g.n2 * cs;
     }
     const int L1 = nc * t1;
-    if (g.fast[0]) {
+    if (g.line[0]) {
+        g.threads1 = L1 * tpl1;
+        g.smem1 = (size_t)L1 * g.n1 * cs;
+    } else if (g.fast[0]) {
         g.threads1 = L1 * (g.n1 / fast_elems(g.n1));
         g.smem1 = (size_t)L1 * g.n1 * cs;
     } else {
@@ -382,6 +418,7 @@ static int engine_init(hom_ctx *ctx, Engine<R> &E) {
         const int N = ctx->n[p];
         if (!factor_radices(N, g.ax[p])) return fail(ctx, HOM_EUNSUPPORTED_GRID, "grid size not 2^a3^b5^c");
         std::vector<R> tw(2 * N), D(N), M(N);
+        std::vector<double2> Dc(N), Mc(N);   // with their phase (FP64)
         for (int t = 0; t < N; ++t) {
             const double ang = 2.0 * PI * (double)t / (double)N;
             tw[2 * t] = (R)std::cos(ang);
@@ -392,6 +429,17 @@ static int engine_init(hom_ctx *ctx, Engine<R> &E) {
             const bool cont = ctx->deriv == HOM_DERIV_CONTINUOUS;   // q_p N_p, eq. (freq)
             D[t] = (R)(cont ? q * N : 2.0 * N * std::sin(0.5 * q));   // else eq. (freqrot)
             M[t] = (R)(cont ? 1.0 : std::cos(0.5 * q));
+            Dc[t] = cont ? make_double2(0.0, q * N) : make_double2(N * (std::cos(q) - 1.0), N * std::sin(q));
+            Mc[t] = cont ? make_double2(1.0, 0.0) : make_double2(0.5 * (1.0 + std::cos(q)), 0.5 * std::sin(q));
+        }
+        if (sizeof(R) == 8) {
+            CU(cudaMalloc(&E.DMc[p], 2 * sizeof(double2) * N));
+            double2 *dm = static_cast<double2 *>(E.DMc[p]);
+            CU(cudaMemcpy(dm, Dc.data(), sizeof(double2) * N, cudaMemcpyHostToDevice));
+            CU(cudaMemcpy(dm + N, Mc.data(), sizeof(double2) * N, cudaMemcpyHostToDevice));
+            g.Dc[p] = dm;
+            g.Mc[p] = dm + N;
+            ctx->workspace += 2 * (long long)sizeof(double2) * N;
         }
         CU(cudaMalloc(&E.tw[p], cs * N));
         CU(cudaMalloc(&E.D[p], sizeof(R) * N));
@@ -410,6 +458,11 @@ static int engine_init(hom_ctx *ctx, Engine<R> &E) {
     Launch<R>::table_init(g);
     int rc = set_shapes<R>(ctx, g, 6);
     if (rc) return rc;
+    E.gj = g;
+    if (sizeof(R) == 8) {
+        rc = set_shapes<R>(ctx, E.gj, 6, false);
+        if (rc) return rc;
+    }
     CU(cudaGetLastError());
     return HOM_OK;
 }
@@ -425,9 +478,16 @@ static void engine_free(Engine<R> &E) {
         cudaFree(E.tw[p]);
         cudaFree(E.D[p]);
         cudaFree(E.M[p]);
+        cudaFree(E.DMc[p]);
     }
     cudaFree(E.phi);
     cudaFree(E.spec);
+}
+
+// The geometry of the unfused operator passes: the elastoplastic increments'
+// FP64 passes keep the engines of old (see run_fft)
+template <typename R> static const Geometry &op_geom(const hom_ctx *ctx, const Engine<R> &E) {
+    return sizeof(R) == 8 && ctx->j2_ops ? E.gj : E.g;
 }
 
 // p = A^ v = G F C F^-1 G v (spectral vectors); optional <v, p> partials.
@@ -435,8 +495,9 @@ template <typename R>
 static void op_spec(hom_ctx *ctx, Engine<R> &E, const cpx<R> *v, cpx<R> *p, bool dot, double *partials,
                     const MinresState *st, double *tsum = nullptr) {
     cudaStream_t s = ctx->stream;
-    Launch<R>::x1(E.g, s, X1_GAMMA_IN, v, E.spec, nullptr, nullptr, st);
-    Launch<R>::x2(E.g, s, 1, E.spec, st);
+    const Geometry &g = op_geom(ctx, E);
+    Launch<R>::x1(g, s, X1_GAMMA_IN, v, E.spec, nullptr, nullptr, st);
+    Launch<R>::x2(g, s, 1, E.spec, st);
     if (ctx->tangent_op) {
         // A_i v = G F (C^{i-1}(x) : F^-1 G v), eq. (galnonlin): the point-wise
         // 6x6 tangent between an inverse and a forward n3 pass (applying it
@@ -448,7 +509,7 @@ static void op_spec(hom_ctx *ctx, Engine<R> &E, const cpx<R> *v, cpx<R> *p, bool
         } else {
             tin = ctx->j2.sig32; tout = ctx->j2.de32;
         }
-        Launch<R>::x3(E.g, s, X3_IN_SPEC, E.spec, X3_MID_NONE, ctx->lam, ctx->mu, nullptr, 1.0, X3_OUT_REAL, tin,
+        Launch<R>::x3(g, s, X3_IN_SPEC, E.spec, X3_MID_NONE, ctx->lam, ctx->mu, nullptr, 1.0, X3_OUT_REAL, tin,
                       E.phi, st);
         // FP64 operator of FP32 fields (their true residual): the FP32 tangent in FP64 arithmetic
         if constexpr (std::is_same<R, double>::value) {
@@ -457,15 +518,15 @@ static void op_spec(hom_ctx *ctx, Engine<R> &E, const cpx<R> *v, cpx<R> *p, bool
         } else {
             j2_tangent_apply<float, float>(ctx->V, ctx->j2.Ct32, tin, tout, s);
         }
-        Launch<R>::x3(E.g, s, X3_IN_REAL, tout, X3_MID_NONE, ctx->lam, ctx->mu, nullptr, 1.0, X3_OUT_SPEC, E.spec,
+        Launch<R>::x3(g, s, X3_IN_REAL, tout, X3_MID_NONE, ctx->lam, ctx->mu, nullptr, 1.0, X3_OUT_SPEC, E.spec,
                       E.phi, st);
         ctx->launches += 2;
     } else {
-        Launch<R>::x3(E.g, s, X3_IN_SPEC, E.spec, X3_MID_MATERIAL, ctx->lam, ctx->mu, nullptr, 1.0, X3_OUT_SPEC,
+        Launch<R>::x3(g, s, X3_IN_SPEC, E.spec, X3_MID_MATERIAL, ctx->lam, ctx->mu, nullptr, 1.0, X3_OUT_SPEC,
                       E.spec, E.phi, st, nullptr, Fold{}, tsum);
     }
-    Launch<R>::x2(E.g, s, 0, E.spec, st);
-    Launch<R>::x1(E.g, s, X1_FWD | X1_GAMMA_OUT | (dot ? X1_DOT : 0), E.spec, p, dot ? v : nullptr, partials, st);
+    Launch<R>::x2(g, s, 0, E.spec, st);
+    Launch<R>::x1(g, s, X1_FWD | X1_GAMMA_OUT | (dot ? X1_DOT : 0), E.spec, p, dot ? v : nullptr, partials, st);
     ctx->launches += 5;
 }
 
@@ -473,10 +534,11 @@ static void op_spec(hom_ctx *ctx, Engine<R> &E, const cpx<R> *v, cpx<R> *p, bool
 template <typename R>
 static void rhs_spec(hom_ctx *ctx, Engine<R> &E, const double *macro_mandel, cpx<R> *b) {
     cudaStream_t s = ctx->stream;
-    Launch<R>::x3(E.g, s, X3_IN_MACRO, nullptr, X3_MID_MATERIAL, ctx->lam, ctx->mu, macro_mandel, -1.0, X3_OUT_SPEC,
+    const Geometry &g = op_geom(ctx, E);
+    Launch<R>::x3(g, s, X3_IN_MACRO, nullptr, X3_MID_MATERIAL, ctx->lam, ctx->mu, macro_mandel, -1.0, X3_OUT_SPEC,
                   E.spec, E.phi, nullptr);
-    Launch<R>::x2(E.g, s, 0, E.spec, nullptr);
-    Launch<R>::x1(E.g, s, X1_FWD | X1_GAMMA_OUT, E.spec, b, nullptr, nullptr, nullptr);
+    Launch<R>::x2(g, s, 0, E.spec, nullptr);
+    Launch<R>::x1(g, s, X1_FWD | X1_GAMMA_OUT, E.spec, b, nullptr, nullptr, nullptr);
     ctx->launches += 3;
 }
 
@@ -484,9 +546,10 @@ static void rhs_spec(hom_ctx *ctx, Engine<R> &E, const double *macro_mandel, cpx
 template <typename R>
 static void real_to_spec(hom_ctx *ctx, Engine<R> &E, const R *in, int mid, bool gamma, cpx<R> *out) {
     cudaStream_t s = ctx->stream;
-    Launch<R>::x3(E.g, s, X3_IN_REAL, in, mid, ctx->lam, ctx->mu, nullptr, 1.0, X3_OUT_SPEC, E.spec, E.phi, nullptr);
-    Launch<R>::x2(E.g, s, 0, E.spec, nullptr);
-    Launch<R>::x1(E.g, s, X1_FWD | (gamma ? X1_GAMMA_OUT : 0), E.spec, out, nullptr, nullptr, nullptr);
+    const Geometry &g = op_geom(ctx, E);
+    Launch<R>::x3(g, s, X3_IN_REAL, in, mid, ctx->lam, ctx->mu, nullptr, 1.0, X3_OUT_SPEC, E.spec, E.phi, nullptr);
+    Launch<R>::x2(g, s, 0, E.spec, nullptr);
+    Launch<R>::x1(g, s, X1_FWD | (gamma ? X1_GAMMA_OUT : 0), E.spec, out, nullptr, nullptr, nullptr);
     ctx->launches += 3;
 }
 
@@ -494,9 +557,10 @@ static void real_to_spec(hom_ctx *ctx, Engine<R> &E, const R *in, int mid, bool 
 template <typename R>
 static void spec_to_real(hom_ctx *ctx, Engine<R> &E, const cpx<R> *in, bool gamma, double scl, R *out) {
     cudaStream_t s = ctx->stream;
-    Launch<R>::x1(E.g, s, gamma ? X1_GAMMA_IN : 0, in, E.spec, nullptr, nullptr, nullptr);
-    Launch<R>::x2(E.g, s, 1, E.spec, nullptr);
-    Launch<R>::x3(E.g, s, X3_IN_SPEC, E.spec, X3_MID_NONE, ctx->lam, ctx->mu, nullptr, scl, X3_OUT_REAL, out, E.phi,
+    const Geometry &g = op_geom(ctx, E);
+    Launch<R>::x1(g, s, gamma ? X1_GAMMA_IN : 0, in, E.spec, nullptr, nullptr, nullptr);
+    Launch<R>::x2(g, s, 1, E.spec, nullptr);
+    Launch<R>::x3(g, s, X3_IN_SPEC, E.spec, X3_MID_NONE, ctx->lam, ctx->mu, nullptr, scl, X3_OUT_REAL, out, E.phi,
                   nullptr);
     ctx->launches += 3;
 }
@@ -526,7 +590,7 @@ static void capture_body(hom_ctx *ctx, Engine<R> &E) {
     cpx<R> *ua = (cpx<R> *)ctx->vbuf[0], *ub = (cpx<R> *)ctx->vbuf[1], *p = (cpx<R> *)ctx->vbuf[2];
     cpx<R> *wc = (cpx<R> *)ctx->wbuf[0], *wd = (cpx<R> *)ctx->wbuf[1];
     cpx<R> *x = (cpx<R> *)ctx->xs;
-    const int np1 = Launch<R>::x1_grid(E.g), npe = Launch<R>::ew_grid(6 * ctx->S);
+    const int np1 = Launch<R>::x1_grid(op_geom(ctx, E)), npe = Launch<R>::ew_grid(6 * ctx->S);
     cudaStream_t s = ctx->stream;
     for (int it = 0; it < ctx->graph_iters; ++it) {
         const bool odd = (it % 2) == 0;          // step k = it + 1 (mod 2)
@@ -827,7 +891,7 @@ static int build_gcg_graph(hom_ctx *ctx, Engine<R> &E) {
     cpx<R> *x = (cpx<R> *)ctx->xs, *r = (cpx<R> *)ctx->vbuf[0], *p = (cpx<R> *)ctx->vbuf[1];
     cpx<R> *q = (cpx<R> *)ctx->vbuf[2];
     const long long n = 6 * ctx->S;
-    const int np1 = Launch<R>::x1_grid(E.g), npc = gcg_blocks(n);
+    const int np1 = Launch<R>::x1_grid(op_geom(ctx, E)), npc = gcg_blocks(n);
     const MinresState *flags = reinterpret_cast<const MinresState *>(ctx->d_cg);
     cudaGraph_t graph;
     CU(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
@@ -1061,8 +1125,10 @@ static int create_impl(hom_ctx *ctx, const int grid[3], const void *phase, int i
     CU(cudaMalloc(&ctx->r64, sizeof(double) * nr));
     ctx->workspace += 6 * (long long)rs * nk + (long long)rs * nr + 2 * (long long)sizeof(double) * nr;
     long long np = 8LL * kEwBlocks;
-    np = std::max(np, (long long)Launch<double>::x1_grid(ctx->e64.g));
-    np = std::max(np, (long long)Launch<double>::x3_grid(ctx->e64.g));
+    for (const Geometry *g : {&ctx->e64.g, &ctx->e64.gj}) {
+        np = std::max(np, (long long)Launch<double>::x1_grid(*g));
+        np = std::max(np, (long long)Launch<double>::x3_grid(*g));
+    }
     np = std::max(np, (long long)Launch<double>::x1_lanczos_grid(ctx->e64.g));
     if (ctx->prec == HOM_PREC_FP32_FIELDS) {
         np = std::max(np, (long long)Launch<float>::x1_grid(ctx->e32.g));
@@ -1073,7 +1139,7 @@ static int create_impl(hom_ctx *ctx, const int grid[3], const void *phase, int i
     CU(cudaMalloc(&ctx->partials, sizeof(double) * ctx->npartials));
     CU(cudaMalloc(&ctx->d_state, sizeof(MinresState)));
     CU(cudaMalloc(&ctx->d_scalar, sizeof(double) * 8));
-    CU(cudaMalloc(&ctx->tsum_part, sizeof(double) * 6 * Launch<double>::x3_grid(ctx->e64.g)));
+    CU(cudaMalloc(&ctx->tsum_part, sizeof(double) * 6 * std::max(Launch<double>::x3_grid(ctx->e64.g), Launch<double>::x3_grid(ctx->e64.gj))));
     CU(cudaMalloc(&ctx->d_flag, sizeof(int)));
     CU(cudaMallocHost(&ctx->h_state, sizeof(MinresState)));
     CU(cudaMallocHost(&ctx->h_scalar, sizeof(double) * 8));
@@ -1647,7 +1713,7 @@ static int true_residual(hom_ctx *ctx, const double2 *x, const double2 *b, doubl
     reduce_to(ctx->stream, ctx->partials, ew_blocks(6 * ctx->S), ctx->d_scalar);
     ctx->launches += 2;
     if (ts) {
-        const int n3 = Launch<double>::x3_grid(ctx->e64.g);
+        const int n3 = Launch<double>::x3_grid(op_geom(ctx, ctx->e64));
         for (int c = 0; c < 6; ++c) reduce_to(ctx->stream, ctx->tsum_part + (size_t)c * n3, n3, ctx->d_scalar + 1 + c);
         ctx->launches += 6;
     }
@@ -2502,7 +2568,7 @@ int solve_cells_one_graph(hom_ctx *const *ctxs, int ncell, const double *macro_s
 // the captured solve graph, whose kernels take the geometry by value
 static void set_stress_mask(hom_ctx *ctx, int mask) {
     if (ctx->e64.g.mask0 == mask && ctx->e32.g.mask0 == mask) return;
-    ctx->e64.g.mask0 = mask;
+    ctx->e64.g.mask0 = ctx->e64.gj.mask0 = mask;
     ctx->e32.g.mask0 = mask;
     if (ctx->graph) {
         cudaGraphExecDestroy(ctx->graph);
@@ -2897,9 +2963,10 @@ int hom_j2_increment(hom_ctx *ctx, const double macro_strain[6], const double ma
     set_stress_mask(ctx, stress_mask);
     ctx->ncase = 0;   // the linear solutions are not kept
     hom_j2_info inf{};
+    ctx->j2_ops = true;
     int rc = j2_increment_impl(ctx, macro_strain, macro_stress, stress_mask, tol_lin, tol_newton, max_newton,
                                max_lin, &inf);
-    ctx->tangent_op = false;
+    ctx->j2_ops = ctx->tangent_op = false;
     if (rc) {
         // the history is written only at the end of an increment: putting
         // the strain at t back leaves the cell as it was

@@ -338,6 +338,8 @@ int line_tpl(int n) {
     }
 }
 
+int f64_line_tpl(int n) { return n == 8 ? LinePlan<8>::TPL : line_tpl(n); }
+
 void line_kernel_attr(const void *kernel, int optin) {
     cudaFuncAttributes fa{};
     cudaFuncGetAttributes(&fa, kernel);

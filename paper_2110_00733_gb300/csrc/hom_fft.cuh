@@ -312,14 +312,6 @@ __host__ __device__ constexpr int fast_elems(int n) {
     return (n == 8 || n == 32 || n == 64) ? 8 : (n == 96 ? 12 : (n == 160 ? 20 : 16));
 }
 __host__ __device__ constexpr int fast_elems_n3(int n) { return n == 96 ? 24 : (n == 160 ? 40 : fast_elems(n)); }
-// the n3 pass's plan by precision: the two-stage plans in FP32 only (FP64
-// elements would not fit in registers)
-template <typename R, int N>
-using PlanN3 = typename std::conditional<sizeof(R) == 4, FastPlanN3<N>, FastPlan<N>>::type;
-template <typename R> __host__ __device__ constexpr int fast_elems_n3r(int n) {
-    return sizeof(R) == 4 ? fast_elems_n3(n) : fast_elems(n);
-}
-
 // Position of element e of a line in a tile with element stride ES; with
 // PAD, one slot is skipped every 16 elements so that the stride-16 writes of
 // a radix-16 stage spread over the shared-memory banks.
@@ -458,6 +450,8 @@ template <int N> struct LinePlan {
     static constexpr int E = line_elems(N, P.r0, P.r1, P.r2, P.tpl);
     static_assert(R0 * R1 * R2 == N, "no plan for this length");
 };
+// (FP64 passes also run 8 on it)
+#define HOM_F64_LENGTHS_A(X) X(8) HOM_LINE_LENGTHS_A(X)
 // threads of a line at run time (0: not a length of the line engine)
 int line_tpl(int n);
 

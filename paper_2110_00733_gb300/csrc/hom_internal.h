@@ -175,6 +175,8 @@ struct Geometry {
     int n1, n2, n3, h;      // h = n3/2 + 1
     long long V, S;         // voxels, half-spectrum points per component
     AxisPlan ax[3];
+    int line[3];            // FP64: length of the axis if the line engine runs it, else 0
+    const double2 *Dc[3], *Mc[3];   // FP64: difference symbol and averaging factor, complex (gamma_at_c)
     const void *D[3];       // per axis: difference symbol without its phase (real, length n_p; see gamma_e)
     const void *M[3];       // per axis: averaging factor without its phase (real, length n_p)
     // launch shapes: rows per CTA of the n3 pass, columns per CTA of the n2
@@ -326,6 +328,19 @@ X1lLineFn x1l_line_kernel(int n);
 // persistent n3 pass of a length, with its threads, rows per tile and shared
 // memory (fn null: none)
 // (fn_sums: with the stress sums)
+// FP64 passes at one line length (hom_f64_*.cu; null members: no such length)
+using F64X1Fn = void (*)(Geometry, int, const double2 *, double2 *, const double2 *, double *, const MinresState *);
+using F64X1lFn = void (*)(Geometry, double2 *, const double2 *, const double2 *, double2 *, const double2 *, double2 *,
+                          double2 *, const MinresState *, double *, Fold);
+using F64X2Fn = void (*)(Geometry, double2 *, const MinresState *);
+using F64X3Fn = void (*)(Geometry, int, const void *, int, double, double, Mac6, double, int, void *, const double *,
+                         const MinresState *, double *, Fold, double *);
+int f64_line_tpl(int n);   // threads of a line (0: the runtime engine)
+F64X1Fn f64_x1_kernel(int n);
+F64X1lFn f64_x1l_kernel(int n);
+F64X2Fn f64_x2_kernel(int n, int inverse);
+F64X3Fn f64_x3_kernel(int n, int pairs);   // pairs of components: 3 or 5
+
 struct X3Line {
     using Fn = void (*)(Geometry, const float2 *, float2 *, int, float, float, const float *, const MinresState *,
                         double *, Fold, double *);

@@ -158,9 +158,10 @@ __device__ __forceinline__ GammaE<R> gamma_e(const Geometry &g, int k1, int k2, 
     if (2 * k1 == g.n1 || 2 * k2 == g.n2 || 2 * k3 == g.n3) return q;
     const R m0 = __ldg(reinterpret_cast<const R *>(g.M[0]) + k1), m1 = __ldg(reinterpret_cast<const R *>(g.M[1]) + k2),
             m2 = __ldg(reinterpret_cast<const R *>(g.M[2]) + k3);
+    // (the factors of axes 2 and 3 first: loops over k1 keep them)
     const R x0 = __ldg(reinterpret_cast<const R *>(g.D[0]) + k1) * (m1 * m2);
-    const R x1 = __ldg(reinterpret_cast<const R *>(g.D[1]) + k2) * (m0 * m2);
-    const R x2 = __ldg(reinterpret_cast<const R *>(g.D[2]) + k3) * (m0 * m1);
+    const R x1 = __ldg(reinterpret_cast<const R *>(g.D[1]) + k2) * m2 * m0;
+    const R x2 = __ldg(reinterpret_cast<const R *>(g.D[2]) + k3) * m1 * m0;
     const R n2 = x0 * x0 + x1 * x1 + x2 * x2;
     if (!(n2 > (R)0)) return q;
     const R inv = inv_norm(n2);
@@ -222,6 +223,47 @@ __device__ __forceinline__ void gamma_apply(const Geometry &g, const GammaE<R> &
     gamma_sym<R>(q, w, t);
 }
 
+// The same projector with the complex vector as it stands (Geometry::Dc, Mc),
+// for the FP64 passes on the engines of old (NF <= 0, see run_fft).
+__device__ __forceinline__ void gamma_at_c(const Geometry &g, int k1, int k2, int k3, double2 *t) {
+    typedef double R;
+    if (k1 == 0 && k2 == 0 && k3 == 0) {
+#pragma unroll
+        for (int c = 0; c < 6; ++c)
+            if (!((g.mask0 >> c) & 1)) t[c] = mk<R>(0, 0);
+        return;
+    }
+    const cpx<R> m0 = __ldg(g.Mc[0] + k1), m1 = __ldg(g.Mc[1] + k2), m2 = __ldg(g.Mc[2] + k3);
+    const cpx<R> x0 = mul<R>(__ldg(g.Dc[0] + k1), mul<R>(m1, m2));
+    const cpx<R> x1 = mul<R>(__ldg(g.Dc[1] + k2), mul<R>(m0, m2));
+    const cpx<R> x2 = mul<R>(__ldg(g.Dc[2] + k3), mul<R>(m0, m1));
+    const R n2 = x0.x * x0.x + x0.y * x0.y + x1.x * x1.x + x1.y * x1.y + x2.x * x2.x + x2.y * x2.y;
+    if (2 * k1 == g.n1 || 2 * k2 == g.n2 || 2 * k3 == g.n3 || !(n2 > (R)0)) {
+#pragma unroll
+        for (int c = 0; c < 6; ++c) t[c] = mk<R>(0, 0);
+        return;
+    }
+    const R inv = (R)1 / sqrt(n2);
+    const cpx<R> e0 = scale<R>(x0, inv), e1 = scale<R>(x1, inv), e2 = scale<R>(x2, inv);
+    const cpx<R> c0 = conjc<R>(e0), c1 = conjc<R>(e1), c2 = conjc<R>(e2);
+    const R r2 = (R)0.70710678118654752440;   // 1/sqrt(2)
+    const cpx<R> T11 = t[0], T22 = t[1], T33 = t[2];
+    const cpx<R> T23 = scale<R>(t[3], r2), T13 = scale<R>(t[4], r2), T12 = scale<R>(t[5], r2);
+    const cpx<R> v0 = add<R>(add<R>(mul<R>(T11, c0), mul<R>(T12, c1)), mul<R>(T13, c2));
+    const cpx<R> v1 = add<R>(add<R>(mul<R>(T12, c0), mul<R>(T22, c1)), mul<R>(T23, c2));
+    const cpx<R> v2 = add<R>(add<R>(mul<R>(T13, c0), mul<R>(T23, c1)), mul<R>(T33, c2));
+    const cpx<R> sc = add<R>(add<R>(mul<R>(c0, v0), mul<R>(c1, v1)), mul<R>(c2, v2));
+    const cpx<R> u0 = sub<R>(scale<R>(v0, (R)2), mul<R>(e0, sc));
+    const cpx<R> u1 = sub<R>(scale<R>(v1, (R)2), mul<R>(e1, sc));
+    const cpx<R> u2 = sub<R>(scale<R>(v2, (R)2), mul<R>(e2, sc));
+    t[0] = mul<R>(u0, e0);
+    t[1] = mul<R>(u1, e1);
+    t[2] = mul<R>(u2, e2);
+    t[3] = scale<R>(add<R>(mul<R>(u1, e2), mul<R>(u2, e1)), r2);
+    t[4] = scale<R>(add<R>(mul<R>(u0, e2), mul<R>(u2, e0)), r2);
+    t[5] = scale<R>(add<R>(mul<R>(u0, e1), mul<R>(u1, e0)), r2);
+}
+
 // G at frequency (k1,k2,k3) on the 6 Mandel components at p[0..5] (stride 1)
 template <typename R>
 __device__ __forceinline__ void gamma_at(const Geometry &g, int k1, int k2, int k3, cpx<R> *t) {
@@ -265,15 +307,28 @@ __device__ __forceinline__ void gamma_from_q(const Geometry &g, const GammaE<R> 
     gamma_sym<R>(ge, w, t);
 }
 
-// Run the transform of the L lines in buf.  Fast engine: in place, returns
-// buf.  Generic engine: ping-pong with buf2, returns the buffer holding the
-// result.
-// nsync != 0 (fast engine only): the first nsync threads run it on named
-// barrier 1.
-template <typename R, int S, int NF, int PAD = 0, typename Plan = FastPlan<NF>>
-__device__ __forceinline__ cpx<R> *run_fft(cpx<R> *buf, cpx<R> *buf2, int L, int ES, const AxisPlan &p, int nsync = 0) {
-    if constexpr (NF > 0) {
-        fast_fft<R, S, NF, PAD, Plan>(buf, L, ES, reinterpret_cast<const cpx<R> *>(p.tw), nsync);
+// Run the transform of the L lines in buf.  Lengths known at compile time (NF):
+// in place, returns buf.  NF > 0: the register engine in FP32; in FP64 the line
+// engine, whose wide butterflies need the fewest operations (the FP64 pipe bounds
+// these passes: 96 = 16 6 takes 19 operations an element, 4 4 2 3 took 22).  NF <
+// 0: FP64 on the register engine of length -NF.  Generic engine (NF = 0):
+// ping-pong with buf2, returns the buffer holding the result.
+//
+// FP64 with NF <= 0 is what the elastoplastic increments run on (and lengths
+// beyond the line engine): they stop their linear solves at a bounded number of
+// steps on nearly singular tangents, where a load changed in its 15th digit
+// moves the strains by 1e-6 to 1e-5 (48^3, three Newton steps), so that their
+// results repeat only if every operation keeps its order.
+template <typename R, int S, int NF, int PAD = 0, typename Plan = void>
+__device__ __forceinline__ cpx<R> *run_fft(cpx<R> *buf, cpx<R> *buf2, int L, int ES, const AxisPlan &p) {
+    if constexpr (NF > 0 && sizeof(R) == 8) {
+        static_assert(PAD == 0, "the line engine does not pad");
+        line_fft<R, S, NF>(buf, L, ES, reinterpret_cast<const cpx<R> *>(p.tw));
+        return buf;
+    } else if constexpr (NF != 0) {
+        constexpr int N = NF < 0 ? -NF : NF;
+        using P = typename std::conditional<std::is_void<Plan>::value, FastPlan<N>, Plan>::type;
+        fast_fft<R, S, N, PAD, P>(buf, L, ES, reinterpret_cast<const cpx<R> *>(p.tw));
         return buf;
     } else {
         return fft_lines<R, S>(buf, buf2, L, ES, p);
@@ -330,7 +385,8 @@ __global__ void HOM_PASS_BOUNDS_N3(R, NF) k_x3(Geometry g, int in_mode, const vo
     // element stride ES = L rounded up to odd: the per-element phases below
     // stride by ES across a warp and stay free of bank conflicts; the fast
     // engine also skips one slot every 16 elements (PAD)
-    constexpr int PAD = NF > 0 ? 1 : 0;
+    constexpr int PAD = (NF > 0 && sizeof(R) == 4) || NF < 0 ? 1 : 0;
+    using Plan = typename std::conditional<NF < 0, FastPlan<(NF < 0 ? -NF : 8)>, FastPlanN3<NF>>::type;
     constexpr int NC = 2 * NP;   // components per frequency
     const int N = g.n3, ROWS = g.rows3, L = NP * ROWS, ES = L | 1, H = g.h;
     auto ep = [ES](int e) { return epos<PAD>(e, ES); };
@@ -369,7 +425,7 @@ __global__ void HOM_PASS_BOUNDS_N3(R, NF) k_x3(Geometry g, int in_mode, const vo
             }
         }
         __syncthreads();
-        cpx<R> *res = run_fft<R, 1, NF, PAD, PlanN3<R, NF>>(buf, buf2, L, ES, g.ax[2]);
+        cpx<R> *res = run_fft<R, 1, NF, PAD, Plan>(buf, buf2, L, ES, g.ax[2]);
         if (res != buf) {   // generic engine ended in the second buffer
             for (int i = threadIdx.x; i < N * ES; i += blockDim.x) buf[i] = res[i];
             __syncthreads();
@@ -393,6 +449,12 @@ __global__ void HOM_PASS_BOUNDS_N3(R, NF) k_x3(Geometry g, int in_mode, const vo
     // ---- scaling and material law on the real-space values
     const R s_in = (in_mode == X3_IN_SPEC) ? (R)(1.0 / (double)g.V) : (R)1;
     const R s_all = s_in * scl;
+    // FP64, bound by the FP64 pipe: the scale, the law's phi and the 1/2 of the
+    // unpacking are one factor on the law's two coefficients (17 operations a
+    // voxel instead of 40), and e : C : e is e . tau
+    constexpr bool kFold = sizeof(R) == 8;
+    const R f_all = kFold && out_mode == X3_OUT_SPEC ? s_all * (R)0.5 : s_all;
+    const R f_lam = lam * f_all, f_mu2 = mu2 * f_all;
     // strain energy sum_x e : C : e of the real-space input (epart): with
     // e = F^-1 G u this is <u, A^ u> / V, the MINRES alpha numerator, so the
     // n1 pass needs no dot product with u
@@ -406,33 +468,46 @@ __global__ void HOM_PASS_BOUNDS_N3(R, NF) k_x3(Geometry g, int in_mode, const vo
 #pragma unroll
             for (int p = 0; p < NP; ++p) {
                 const cpx<R> z = q[p * ROWS];
-                t[2 * p] = z.x * s_all;
-                t[2 * p + 1] = z.y * s_all;
+                t[2 * p] = kFold ? z.x : z.x * s_all;
+                t[2 * p + 1] = kFold ? z.y : z.y * s_all;
             }
             if (mid == X3_MID_MATERIAL || mid == X3_MID_MODB) {
                 const R ph = phi[vbase + e];
                 const R sum = t[0] + t[1] + t[2];
-                const R tr = lam * sum;
-                if (epart) {
-                    R ee = t[0] * t[0];
+                if constexpr (kFold) {
+                    const R m = ph * f_mu2, tr = ph * f_lam * sum;
 #pragma unroll
-                    for (int c = 1; c < 6; ++c) ee += t[c] * t[c];
-                    en += ph * (tr * sum + mu2 * ee);
+                    for (int c = 0; c < 6; ++c) {
+                        const R o = c < 3 ? tr + m * t[c] : m * t[c];
+                        if (epart) en += t[c] * o;   // (times s_all / f_all s_all at the end)
+                        t[c] = o;
+                    }
+                } else {
+                    const R tr = lam * sum;
+                    if (epart) {
+                        R ee = t[0] * t[0];
+#pragma unroll
+                        for (int c = 1; c < 6; ++c) ee += t[c] * t[c];
+                        en += ph * (tr * sum + mu2 * ee);
+                    }
+#pragma unroll
+                    for (int c = 0; c < 6; ++c) t[c] = ph * ((c < 3 ? tr : (R)0) + mu2 * t[c]);
                 }
-#pragma unroll
-                for (int c = 0; c < 6; ++c) t[c] = ph * ((c < 3 ? tr : (R)0) + mu2 * t[c]);
                 if (tsum) {
 #pragma unroll
                     for (int c = 0; c < 6; ++c) ts[c] += (double)t[c];
                 }
                 if constexpr (NC == 10) {
                     // MoDBFFT penalty vector on the empty phase: chi_v g, eq. (modbfftfop)
-                    const R chi = (ph == (R)0) ? (R)1 : (R)0;
+                    const R chi = (ph == (R)0) ? (kFold ? f_all : (R)1) : (R)0;
                     t[6] *= chi;
                     t[7] *= chi;
                     t[8] *= chi;
                     t[9] = 0;
                 }
+            } else if (kFold) {
+#pragma unroll
+                for (int c = 0; c < NC; ++c) t[c] *= f_all;
             }
             if (out_mode == X3_OUT_REAL) {
                 R *real = reinterpret_cast<R *>(out_);
@@ -448,11 +523,11 @@ __global__ void HOM_PASS_BOUNDS_N3(R, NF) k_x3(Geometry g, int in_mode, const vo
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
             const double sum = block_sum(ts[c]);
-            if (threadIdx.x == 0) tsum[(size_t)c * gridDim.x + blockIdx.x] = sum;
+            if (threadIdx.x == 0) tsum[(size_t)c * gridDim.x + blockIdx.x] = kFold ? sum * (s_all / f_all) : sum;
         }
     }
     if (epart) {
-        const double sum = block_sum((double)en);
+        const double sum = block_sum((double)en) * (kFold ? s_all * (s_all / f_all) : 1.0);
         if (threadIdx.x == 0) epart[blockIdx.x] = sum;
         if (fold.cnt && last_of(fold.cnt + cs, bpc)) {   // alpha of case cs
             const double tot = sum_partials(epart + (size_t)cs * bpc, bpc);
@@ -465,7 +540,7 @@ __global__ void HOM_PASS_BOUNDS_N3(R, NF) k_x3(Geometry g, int in_mode, const vo
     if (out_mode == X3_OUT_REAL) return;
     // rows beyond nrows hold zeros already (their inputs were zero)
     __syncthreads();
-    cpx<R> *res = run_fft<R, -1, NF, PAD, PlanN3<R, NF>>(buf, buf2, L, ES, g.ax[2]);
+    cpx<R> *res = run_fft<R, -1, NF, PAD, Plan>(buf, buf2, L, ES, g.ax[2]);
     // unpack the two real transforms of each packed line:
     //   X_a[k] = (Z[k] + conj Z[N-k]) / 2,  X_b[k] = (Z[k] - conj Z[N-k]) / (2i)
     cpx<R> *spec = reinterpret_cast<cpx<R> *>(out_);
@@ -477,8 +552,11 @@ __global__ void HOM_PASS_BOUNDS_N3(R, NF) k_x3(Geometry g, int in_mode, const vo
             for (int p = 0; p < NP; ++p) {
                 const cpx<R> z = res[ep(k) + p * ROWS + r];
                 const cpx<R> zm = conjc<R>(res[ep(km) + p * ROWS + r]);
-                Six<R>::store_pair(row + NC * k, p, mk<R>((R)0.5 * (z.x + zm.x), (R)0.5 * (z.y + zm.y)),
-                                   mk<R>((R)0.5 * (z.y - zm.y), (R)-0.5 * (z.x - zm.x)));
+                if constexpr (kFold)
+                    Six<R>::store_pair(row + NC * k, p, mk<R>(z.x + zm.x, z.y + zm.y), mk<R>(z.y - zm.y, zm.x - z.x));
+                else
+                    Six<R>::store_pair(row + NC * k, p, mk<R>((R)0.5 * (z.x + zm.x), (R)0.5 * (z.y + zm.y)),
+                                       mk<R>((R)0.5 * (z.y - zm.y), (R)-0.5 * (z.x - zm.x)));
             }
         }
     }
@@ -831,16 +909,20 @@ __global__ void HOM_PASS_BOUNDS_NF(R, NF) k_x1(Geometry g, int flags, const cpx<
     const int tg = threadIdx.x % T, eg0 = threadIdx.x / T, egs = blockDim.x / T;
     const int colg = g0 + tg;
     const int k2g = colg / H, k3g = colg - k2g * H;
+    auto gamma = [&](int e, cpx<R> *t) {
+        if constexpr (sizeof(R) == 8 && NF <= 0) gamma_at_c(g, e, k2g, k3g, t);
+        else gamma_at<R>(g, e, k2g, k3g, t);
+    };
     if (flags & X1_GAMMA_IN) {
         if (colg < cols)
-            for (int e = eg0; e < N; e += egs) gamma_at<R>(g, e, k2g, k3g, buf + e * L + tg * NC);
+            for (int e = eg0; e < N; e += egs) gamma(e, buf + e * L + tg * NC);
         __syncthreads();
     }
     cpx<R> *res = (flags & X1_FWD) ? run_fft<R, -1, NF>(buf, buf2, L, L, g.ax[0])
                                    : run_fft<R, 1, NF>(buf, buf2, L, L, g.ax[0]);
     if (flags & X1_GAMMA_OUT) {
         if (colg < cols)
-            for (int e = eg0; e < N; e += egs) gamma_at<R>(g, e, k2g, k3g, res + e * L + tg * NC);
+            for (int e = eg0; e < N; e += egs) gamma(e, res + e * L + tg * NC);
         __syncthreads();
     }
     Acc<R> acc;
@@ -1216,17 +1298,18 @@ __device__ __forceinline__ cpx<R> *x1_lanczos_tile(const Geometry &g, cpx<R> *bu
     // 2. per frequency: q of p, Lanczos step, lagged update, strain of u_{k+1}
     const int NT = N * T;   // one of the three planes of a Krylov tile
     const size_t kb = (size_t)(g0 / T) * krylov_tile(N, T);
-    for (int f = threadIdx.x; f < NT; f += blockDim.x) {
-        const int e = f / T, t = f - e * T;
-        const int col = g0 + t;
+    // a thread keeps one column (blockDim is a multiple of T)
+    const int t = threadIdx.x % T, col = g0 + t;
+    const int k2 = col / H, k3 = col - k2 * H;
+    const R w = (R)pweight(k3, g.n3);
+    for (int e = threadIdx.x / T; e < N; e += blockDim.x / T) {
         cpx<R> *sp = res + e * L + t * NC;
         if (col >= cols) {
 #pragma unroll
             for (int q = 0; q < NC; ++q) sp[q] = mk<R>(0, 0);
             continue;
         }
-        const int k2 = col / H, k3 = col - k2 * H;
-        const size_t i = kb + f;
+        const size_t i = kb + e * T + t;
         cpx<R> v[NC], q[3], u[3], uo[3];
 #pragma unroll
         for (int c3 = 0; c3 < 3; ++c3) {
@@ -1237,7 +1320,6 @@ __device__ __forceinline__ cpx<R> *x1_lanczos_tile(const Geometry &g, cpx<R> *bu
         for (int p = 0; p < 3; ++p) Six<R>::load_pair(sp, p, v[2 * p], v[2 * p + 1]);
         const GammaE<R> ge = gamma_e<R>(g, e, k2, k3);
         gamma_to_q<R>(g, ge, v, q);
-        const R w = (R)pweight(k3, g.n3);
 #pragma unroll
         for (int c3 = 0; c3 < 3; ++c3) {
             q[c3] = mk<R>(c.cp * q[c3].x + c.cu * u[c3].x + c.cv * uo[c3].x,
@@ -1583,6 +1665,20 @@ int Launch<R>::x1_grid(const Geometry &g) {
     return g.tma ? g.grid1d_tma : (g.n2 * g.h + g.tile1 - 1) / g.tile1;
 }
 
+// (FP64: NF = -n, the register engine in its order of old)
+#define HOM_F64_SWITCH(n, CALL)                    \
+    switch (n) {                                   \
+        case 8: CALL(-8); break;                   \
+        case 16: CALL(-16); break;                 \
+        case 32: CALL(-32); break;                 \
+        case 64: CALL(-64); break;                 \
+        case 96: CALL(-96); break;                 \
+        case 128: CALL(-128); break;               \
+        case 160: CALL(-160); break;               \
+        case 256: CALL(-256); break;               \
+        case 512: CALL(-512); break;               \
+        default: CALL(0); break;                   \
+    }
 #define HOM_FAST_SWITCH(n, CALL)                   \
     switch (n) {                                   \
         case 8: CALL(8); break;                    \
@@ -1598,7 +1694,7 @@ int Launch<R>::x1_grid(const Geometry &g) {
     }
 
 template <typename R>
-void Launch<R>::table_init(const Geometry &) {
+void Launch<R>::table_init(const Geometry &g) {
     // The dynamic shared-memory limit of each pass kernel is raised to the
     // device's opt-in maximum (a per-function setting shared by all contexts;
     // the launch's own size still decides occupancy).
@@ -1625,9 +1721,28 @@ void Launch<R>::table_init(const Geometry &) {
     HOM_SET_ATTR1((k_x2<R, 1, NF>))     \
     HOM_SET_ATTR1((k_x1<R, NF>))        \
     HOM_SET_ATTR1((k_x1_lanczos<R, NF>))
-    HOM_SET_ATTR(0) HOM_SET_ATTR(8) HOM_SET_ATTR(16) HOM_SET_ATTR(32) HOM_SET_ATTR(64) HOM_SET_ATTR(96)
-    HOM_SET_ATTR(128) HOM_SET_ATTR(160) HOM_SET_ATTR(256) HOM_SET_ATTR(512)
+    if constexpr (sizeof(R) == 8) {
+        if (f64_line_tpl(g.n1)) {
+            line_kernel_attr((const void *)f64_x1_kernel(g.n1), lim);
+            line_kernel_attr((const void *)f64_x1l_kernel(g.n1), lim);
+        }
+        if (f64_line_tpl(g.n2))
+            for (int inv = 0; inv < 2; ++inv) line_kernel_attr((const void *)f64_x2_kernel(g.n2, inv), lim);
+        if (f64_line_tpl(g.n3))
+            for (int np : {3, 5}) line_kernel_attr((const void *)f64_x3_kernel(g.n3, np), lim);
+#define HOM_F64_ATTR1(NF) line_kernel_attr((const void *)k_x1<R, NF>, lim), line_kernel_attr((const void *)k_x1_lanczos<R, NF>, lim)
+#define HOM_F64_ATTR2(NF) line_kernel_attr((const void *)k_x2<R, -1, NF>, lim), line_kernel_attr((const void *)k_x2<R, 1, NF>, lim)
+#define HOM_F64_ATTR3(NF) line_kernel_attr((const void *)k_x3<R, NF, 3>, lim), line_kernel_attr((const void *)k_x3<R, NF, 5>, lim)
+        HOM_F64_SWITCH(g.fast[0], HOM_F64_ATTR1)
+        HOM_F64_SWITCH(g.fast[1], HOM_F64_ATTR2)
+        HOM_F64_SWITCH(g.fast[2], HOM_F64_ATTR3)
+#undef HOM_F64_ATTR1
+#undef HOM_F64_ATTR2
+#undef HOM_F64_ATTR3
+    }
     if constexpr (sizeof(R) == 4) {
+        HOM_SET_ATTR(0) HOM_SET_ATTR(8) HOM_SET_ATTR(16) HOM_SET_ATTR(32) HOM_SET_ATTR(64) HOM_SET_ATTR(96)
+        HOM_SET_ATTR(128) HOM_SET_ATTR(160) HOM_SET_ATTR(256) HOM_SET_ATTR(512)
 #define HOM_SET_TMA(NF)                   \
     HOM_SET_ATTR1((k_x1_tma<R, NF>))      \
     HOM_SET_ATTR1((k_x1_tma<R, NF, true>)) \
@@ -1739,6 +1854,17 @@ void Launch<R>::x3(const Geometry &g, cudaStream_t st, int in_mode, const void *
     if (macro)
         for (int c = 0; c < 6; ++c) m.v[c] = macro[c];
     const int grid = x3_grid(g) * g.nb;
+    if constexpr (sizeof(R) == 8) {
+        F64X3Fn f = nullptr;
+#define HOM_X3(NF) f = g.nc == 10 ? k_x3<R, NF, 5> : k_x3<R, NF, 3>
+        if (g.line[2]) f = f64_x3_kernel(g.n3, g.nc / 2);
+        else HOM_F64_SWITCH(g.fast[2], HOM_X3)
+#undef HOM_X3
+        if (g.nc == 10) epart = tsum = nullptr, fold = Fold{};
+        launch_k(g.pdl, f, grid, g.threads3, g.smem3, st, g, in_mode, in, mid, lam, 2.0 * mu, m, scl, out_mode, out, phi,
+                 state, epart, fold, tsum);
+        return;
+    } else {
 #define HOM_X3(NF)                                                                                          \
     if (g.nc == 10)                                                                                         \
         launch_k(g.pdl, k_x3<R, NF, 5>, grid, g.threads3, g.smem3, st, g, in_mode, in, mid, (R)lam, (R)(2.0 * mu), m, \
@@ -1748,6 +1874,7 @@ void Launch<R>::x3(const Geometry &g, cudaStream_t st, int in_mode, const void *
                                                             (R)scl, out_mode, out, phi, state, epart, fold, tsum)
     HOM_FAST_SWITCH(g.fast[2], HOM_X3)
 #undef HOM_X3
+    }
 }
 
 template <typename R>
@@ -1764,11 +1891,20 @@ void Launch<R>::x2(const Geometry &g, cudaStream_t st, int inverse, cpx<R> *spec
         }
     }
     const int grid = (g.n1 * g.nb * g.nc * g.h + g.tile2 - 1) / g.tile2;
+    if constexpr (sizeof(R) == 8) {
+        F64X2Fn f = nullptr;
+#define HOM_X2(NF) f = inverse ? k_x2<R, 1, NF> : k_x2<R, -1, NF>
+        if (g.line[1]) f = f64_x2_kernel(g.n2, inverse);
+        else HOM_F64_SWITCH(g.fast[1], HOM_X2)
+#undef HOM_X2
+        launch_k(g.pdl, f, grid, g.threads2, g.smem2, st, g, spec, state);
+    } else {
 #define HOM_X2(NF)                                                                  \
     if (inverse) launch_k(g.pdl, k_x2<R, 1, NF>, grid, g.threads2, g.smem2, st, g, spec, state); \
     else launch_k(g.pdl, k_x2<R, -1, NF>, grid, g.threads2, g.smem2, st, g, spec, state)
     HOM_FAST_SWITCH(g.fast[1], HOM_X2)
 #undef HOM_X2
+    }
 }
 
 template <typename R>
@@ -1796,9 +1932,18 @@ void Launch<R>::x1(const Geometry &g, cudaStream_t st, int flags, const cpx<R> *
         }
     }
     const int grid = (g.n2 * g.h + g.tile1 - 1) / g.tile1;
+    if constexpr (sizeof(R) == 8) {
+        F64X1Fn f = nullptr;
+#define HOM_X1(NF) f = k_x1<R, NF>
+        if (g.line[0]) f = f64_x1_kernel(g.n1);
+        else HOM_F64_SWITCH(g.fast[0], HOM_X1)
+#undef HOM_X1
+        f<<<grid, g.threads1, g.smem1, st>>>(g, flags, in, out, dotv, partials, state);
+    } else {
 #define HOM_X1(NF) k_x1<R, NF><<<grid, g.threads1, g.smem1, st>>>(g, flags, in, out, dotv, partials, state)
     HOM_FAST_SWITCH(g.fast[0], HOM_X1)
 #undef HOM_X1
+    }
 }
 
 template <typename R>
@@ -1872,11 +2017,20 @@ void Launch<R>::x1_lanczos(const Geometry &g, cudaStream_t st, cpx<R> *spec, con
         }
     }
     const int grid = (g.n2 * g.h + g.tile1 - 1) / g.tile1 * g.nb;
+    if constexpr (sizeof(R) == 8) {
+        F64X1lFn f = nullptr;
+#define HOM_X1L(NF) f = k_x1_lanczos<R, NF>
+        if (g.line[0]) f = f64_x1l_kernel(g.n1);
+        else HOM_F64_SWITCH(g.fast[0], HOM_X1L)
+#undef HOM_X1L
+        launch_k(g.pdl, f, grid, g.threads1, g.smem1, st, g, spec, uk, um, un, wa, wb, x, state, partials, fold);
+    } else {
 #define HOM_X1L(NF) \
     launch_k(g.pdl, k_x1_lanczos<R, NF>, grid, g.threads1, g.smem1, st, g, spec, uk, um, un, wa, wb, x, state, partials, \
              fold)
     HOM_FAST_SWITCH(g.fast[0], HOM_X1L)
 #undef HOM_X1L
+    }
 }
 
 template <typename R>
