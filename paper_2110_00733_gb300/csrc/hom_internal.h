@@ -287,7 +287,8 @@ enum X3Mid { X3_MID_NONE = 0, X3_MID_MATERIAL = 1,
              X3_MID_MODB = 2 };   // 10 components: tau = phi C_m eps (0-5), chi_v g (6-8), 0 (9)
 enum X3Out { X3_OUT_SPEC = 0, X3_OUT_REAL = 1 };
 // n1 pass (x1) flags
-enum X1Flags { X1_FWD = 1, X1_GAMMA_IN = 2, X1_GAMMA_OUT = 4, X1_DOT = 8 };
+// (X1_BACK: the inverse transform after the projection, FP32 plain-load form)
+enum X1Flags { X1_FWD = 1, X1_GAMMA_IN = 2, X1_GAMMA_OUT = 4, X1_DOT = 8, X1_BACK = 16 };
 
 constexpr int kEwBlocks = 152 * 8;   // grid of the element-wise Krylov kernels
 constexpr int kNbMax = 8;            // load cases of one stacked MINRES batch

@@ -56,25 +56,25 @@ std::mutex g_mu;
 // Frequency tables on the device, FP64 with sincospi, stored in FP32:
 // tw[t] = exp(-2 pi i t/N); D, M of the continuous (eq. freq) or rotated
 // (eq. freqrot) scheme, as in the context-based path (see gamma_e).
-__global__ void k_noalloc_tables(int n1, int n2, int n3, int deriv, float2 *tab) {
-    const int ns[3] = {n1, n2, n3};
-    for (int p = 0; p < 3; ++p) {
-        const int N = ns[p];
-        float2 *tw = tab + (p * 3 + 0) * kMaxN;
-        float *D = reinterpret_cast<float *>(tab + (p * 3 + 1) * kMaxN);
-        float *M = reinterpret_cast<float *>(tab + (p * 3 + 2) * kMaxN);
-        for (int t = threadIdx.x; t < N; t += blockDim.x) {
-            double s, c;
-            sincospi(2.0 * (double)t / (double)N, &s, &c);
-            tw[t] = make_float2((float)c, (float)-s);
-            const int m = (2 * t < N) ? t : t - N;
-            double sq, cq;   // of half the angle
-            sincospi((double)m / (double)N, &sq, &cq);
-            const bool cont = deriv == HOM_DERIV_CONTINUOUS;
-            D[t] = (float)(cont ? 2.0 * 3.14159265358979323846 * m : 2.0 * N * sq);
-            M[t] = cont ? 1.f : (float)cq;
-        }
+// One CTA an axis, its first kMaxN threads the twiddles, the others D and M, so
+// that one FP64 sincospi deep is all the kernel takes (a single CTA that went
+// through them in turn was an eighth of the call).
+__global__ void __launch_bounds__(2 * kMaxN) k_noalloc_tables(int n1, int n2, int n3, int deriv, float2 *tab) {
+    pdl_release();
+    const int p = blockIdx.x, N = p == 0 ? n1 : (p == 1 ? n2 : n3);
+    const bool first = threadIdx.x < kMaxN;
+    const int t = first ? threadIdx.x : threadIdx.x - kMaxN;
+    if (t >= N) return;
+    const int m = (2 * t < N) ? t : t - N;
+    double s, c;   // of the whole angle, or of half of it
+    sincospi((first ? 2.0 * (double)t : (double)m) / (double)N, &s, &c);
+    if (first) {
+        tab[(p * 3 + 0) * kMaxN + t] = make_float2((float)c, (float)-s);
+        return;
     }
+    const bool cont = deriv == HOM_DERIV_CONTINUOUS;
+    reinterpret_cast<float *>(tab + (p * 3 + 1) * kMaxN)[t] = (float)(cont ? 2.0 * 3.14159265358979323846 * m : 2.0 * N * s);
+    reinterpret_cast<float *>(tab + (p * 3 + 2) * kMaxN)[t] = cont ? 1.f : (float)c;
 }
 
 bool radices(int n, AxisPlan &p) {
@@ -247,12 +247,17 @@ int hom_apply_noalloc(const int grid[3], const float *phi, double E, double nu, 
     const double lam = nu / ((1.0 + nu) * (1.0 - 2.0 * nu));   // lambda / E
     const double mu = 1.0 / (2.0 * (1.0 + nu));                // mu / E
     float2 *spec = d->spec;
-    k_noalloc_tables<<<1, 64, 0, st>>>(g.n1, g.n2, g.n3, derivative, d->tab);
+    // programmatic launches: a pass's CTAs are placed while the one before it
+    // still runs, and wait for its end before they touch memory.  (The tables'
+    // launch is an ordinary one: nothing here starts before earlier work of the
+    // stream is complete, nor later work before this.)  With the tables on three
+    // CTAs and the two n1 transforms in one pass: 32^3 53 -> 30 us.
+    g.pdl = 1;
+    k_noalloc_tables<<<3, 2 * kMaxN, 0, st>>>(g.n1, g.n2, g.n3, derivative, d->tab);
     // A(eps) = F^-1 G F (phi C_m : eps), eq. (linearOp), C_m in units of E
     Launch<float>::x3(g, st, X3_IN_REAL, eps, X3_MID_MATERIAL, lam, mu, nullptr, 1.0, X3_OUT_SPEC, spec, phi, nullptr);
     Launch<float>::x2(g, st, 0, spec, nullptr);
-    Launch<float>::x1(g, st, X1_FWD | X1_GAMMA_OUT, spec, spec, nullptr, nullptr, nullptr);
-    Launch<float>::x1(g, st, 0, spec, spec, nullptr, nullptr, nullptr);
+    Launch<float>::x1(g, st, X1_FWD | X1_GAMMA_OUT | X1_BACK, spec, spec, nullptr, nullptr, nullptr);
     Launch<float>::x2(g, st, 1, spec, nullptr);
     Launch<float>::x3(g, st, X3_IN_SPEC, spec, X3_MID_NONE, lam, mu, nullptr, 1.0, X3_OUT_REAL, out, phi, nullptr);
     // launch errors only: the call does not wait for its kernels

@@ -888,6 +888,8 @@ template <typename R, int NF>
 __global__ void HOM_PASS_BOUNDS_NF(R, NF) k_x1(Geometry g, int flags, const cpx<R> *__restrict__ in,
                                             cpx<R> *__restrict__ out, const cpx<R> *__restrict__ dotv,
                                             double *__restrict__ partials, const MinresState *state) {
+    pdl_release();
+    pdl_wait();   // predecessor complete (programmatic launch)
     if (skip(state)) return;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int NC = g.nc, N = g.n1, T = g.tile1, H = g.h, L = NC * T;
@@ -924,6 +926,9 @@ __global__ void HOM_PASS_BOUNDS_NF(R, NF) k_x1(Geometry g, int flags, const cpx<
         if (colg < cols)
             for (int e = eg0; e < N; e += egs) gamma(e, res + e * L + tg * NC);
         __syncthreads();
+    }
+    if constexpr (sizeof(R) == 4) {
+        if (flags & X1_BACK) res = run_fft<R, 1, NF>(res, res == buf ? buf2 : buf, L, L, g.ax[0]);
     }
     Acc<R> acc;
     if (live) {
@@ -1940,7 +1945,7 @@ void Launch<R>::x1(const Geometry &g, cudaStream_t st, int flags, const cpx<R> *
 #undef HOM_X1
         f<<<grid, g.threads1, g.smem1, st>>>(g, flags, in, out, dotv, partials, state);
     } else {
-#define HOM_X1(NF) k_x1<R, NF><<<grid, g.threads1, g.smem1, st>>>(g, flags, in, out, dotv, partials, state)
+#define HOM_X1(NF) launch_k(g.pdl, k_x1<R, NF>, grid, g.threads1, g.smem1, st, g, flags, in, out, dotv, partials, state)
     HOM_FAST_SWITCH(g.fast[0], HOM_X1)
 #undef HOM_X1
     }
