@@ -63,7 +63,8 @@ struct Status {
 template <typename R> struct Engine {
     Geometry g{};
     Geometry gm{};             // MoDBFFT chain: 10 components per frequency
-    Geometry gj{};             // elastoplastic increments: see op_geom
+    Geometry gj{};             // elastoplastic increments: see op_geom, ordered_shapes
+    Geometry gd{};             // the launch shape of their dot products
     R *phi = nullptr;
     cpx<R> *spec = nullptr;
     cpx<R> *spec10 = nullptr;  // MoDBFFT work spectrum
@@ -402,6 +403,42 @@ static int set_shapes(hom_ctx *ctx, Geometry &g, int nc, bool lines = true) {
     return HOM_OK;
 }
 
+// The launch shapes of the elastoplastic increments' FP64 passes: ordered_fft
+// where it has the length, and tiles narrow enough for every SM.  Neither moves a
+// bit of a transform, nor of the dot product, which x1_dot takes with the former
+// shape (gd).  48^3: n1 pass 53 us on 75 CTAs of the runtime engine.
+static void ordered_shapes(Geometry &g) {
+    constexpr int kSms = 152;
+    const int cs = sizeof(double2);
+    g.ord[0] = f64_ord_x1_kernel(g.n1) ? g.n1 : 0;
+    g.ord[1] = f64_ord_x2_kernel(g.n2, 0) ? g.n2 : 0;
+    g.ord[2] = f64_ord_x3_kernel(g.n3) ? g.n3 : 0;
+    if (g.ord[0] || g.fast[0]) {
+        const int tpl = g.ord[0] ? ordered_tpl(g.n1) : g.n1 / fast_elems(g.n1);
+        int t = 8;
+        while (t > 1 && (6 * t * tpl > 192 || g.n2 * g.h < kSms * t)) t >>= 1;
+        g.tile1 = t;
+        g.threads1 = 6 * t * tpl;
+        g.smem1 = (size_t)6 * t * g.n1 * cs;
+    }
+    if (g.ord[1]) {
+        const int tpl = ordered_tpl(g.n2);
+        int t = tpl <= 8 ? 16 : 8;
+        while (t > 4 && g.n1 * 6 * g.h < kSms * t) t >>= 1;
+        g.tile2 = t;
+        g.threads2 = t * tpl;
+        g.smem2 = (size_t)t * g.n2 * cs;
+    }
+    if (g.ord[2]) {
+        const int tpl = ordered_tpl(g.n3);
+        int rows = 8;
+        while (rows > 1 && (3 * rows * tpl > 192 || g.n1 * g.n2 < kSms * rows)) rows >>= 1;
+        g.rows3 = rows;
+        g.threads3 = 3 * rows * tpl;
+        g.smem3 = (size_t)((3 * rows) | 1) * g.n3 * cs;
+    }
+}
+
 template <typename R>
 static int engine_init(hom_ctx *ctx, Engine<R> &E) {
     Geometry &g = E.g;
@@ -462,6 +499,8 @@ static int engine_init(hom_ctx *ctx, Engine<R> &E) {
     if (sizeof(R) == 8) {
         rc = set_shapes<R>(ctx, E.gj, 6, false);
         if (rc) return rc;
+        E.gd = E.gj;
+        if (!ctx->shape[0] && !ctx->shape[1] && !ctx->shape[2]) ordered_shapes(E.gj);
     }
     CU(cudaGetLastError());
     return HOM_OK;
@@ -526,7 +565,13 @@ static void op_spec(hom_ctx *ctx, Engine<R> &E, const cpx<R> *v, cpx<R> *p, bool
                       E.spec, E.phi, st, nullptr, Fold{}, tsum);
     }
     Launch<R>::x2(g, s, 0, E.spec, st);
-    Launch<R>::x1(g, s, X1_FWD | X1_GAMMA_OUT | (dot ? X1_DOT : 0), E.spec, p, dot ? v : nullptr, partials, st);
+    if (sizeof(R) == 8 && ctx->j2_ops && dot) {
+        Launch<R>::x1(g, s, X1_FWD | X1_GAMMA_OUT, E.spec, p, nullptr, nullptr, st);
+        Launch<R>::x1_dot(E.gd, s, p, v, partials, st);
+        ctx->launches += 1;
+    } else {
+        Launch<R>::x1(g, s, X1_FWD | X1_GAMMA_OUT | (dot ? X1_DOT : 0), E.spec, p, dot ? v : nullptr, partials, st);
+    }
     ctx->launches += 5;
 }
 
@@ -590,7 +635,7 @@ static void capture_body(hom_ctx *ctx, Engine<R> &E) {
     cpx<R> *ua = (cpx<R> *)ctx->vbuf[0], *ub = (cpx<R> *)ctx->vbuf[1], *p = (cpx<R> *)ctx->vbuf[2];
     cpx<R> *wc = (cpx<R> *)ctx->wbuf[0], *wd = (cpx<R> *)ctx->wbuf[1];
     cpx<R> *x = (cpx<R> *)ctx->xs;
-    const int np1 = Launch<R>::x1_grid(op_geom(ctx, E)), npe = Launch<R>::ew_grid(6 * ctx->S);
+    const int np1 = Launch<R>::x1_grid(sizeof(R) == 8 && ctx->j2_ops ? E.gd : E.g), npe = Launch<R>::ew_grid(6 * ctx->S);
     cudaStream_t s = ctx->stream;
     for (int it = 0; it < ctx->graph_iters; ++it) {
         const bool odd = (it % 2) == 0;          // step k = it + 1 (mod 2)
@@ -891,7 +936,7 @@ static int build_gcg_graph(hom_ctx *ctx, Engine<R> &E) {
     cpx<R> *x = (cpx<R> *)ctx->xs, *r = (cpx<R> *)ctx->vbuf[0], *p = (cpx<R> *)ctx->vbuf[1];
     cpx<R> *q = (cpx<R> *)ctx->vbuf[2];
     const long long n = 6 * ctx->S;
-    const int np1 = Launch<R>::x1_grid(op_geom(ctx, E)), npc = gcg_blocks(n);
+    const int np1 = Launch<R>::x1_grid(E.g), npc = gcg_blocks(n);
     const MinresState *flags = reinterpret_cast<const MinresState *>(ctx->d_cg);
     cudaGraph_t graph;
     CU(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
@@ -1125,7 +1170,7 @@ static int create_impl(hom_ctx *ctx, const int grid[3], const void *phase, int i
     CU(cudaMalloc(&ctx->r64, sizeof(double) * nr));
     ctx->workspace += 6 * (long long)rs * nk + (long long)rs * nr + 2 * (long long)sizeof(double) * nr;
     long long np = 8LL * kEwBlocks;
-    for (const Geometry *g : {&ctx->e64.g, &ctx->e64.gj}) {
+    for (const Geometry *g : {&ctx->e64.g, &ctx->e64.gj, &ctx->e64.gd}) {
         np = std::max(np, (long long)Launch<double>::x1_grid(*g));
         np = std::max(np, (long long)Launch<double>::x3_grid(*g));
     }

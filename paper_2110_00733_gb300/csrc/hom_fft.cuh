@@ -509,4 +509,30 @@ __device__ __forceinline__ void line_fft(cpx<R> *buf, int L, int ES, const cpx<R
     if constexpr (P::R2 > 1) line_stage<R, S, N, P::R2, P::R0 * P::R1, P::TPL>(buf, ES, l, j0, tw, nsync);
 }
 
+// The runtime engine's transform (its radices in its order: powers of two from
+// the largest, then threes, then fives) with everything but the data known at
+// compile time and the line engine's in-place stages: the same operations on the
+// same values, so the same bits, without the second buffer and the divisions by
+// run-time values.
+constexpr int ordered_radix(int n, int s) {
+    int a = 0, b = 0, c = 0;
+    while (n % 2 == 0) { n /= 2; ++a; }
+    while (n % 3 == 0) { n /= 3; ++b; }
+    while (n % 5 == 0) { n /= 5; ++c; }
+    const int st2 = (a + 3) / 4;
+    if (s < st2) return 1 << (a / st2 + (s < a % st2 ? 1 : 0));
+    return s < st2 + b ? 3 : (s < st2 + b + c ? 5 : 1);
+}
+// threads of a line: 12 to 16 elements each
+__host__ __device__ constexpr int ordered_tpl(int n) { return (n + 11) / 12; }
+
+template <typename R, int S, int N, int STAGE = 0, int NSB = 1>
+__device__ __forceinline__ void ordered_fft(cpx<R> *buf, int L, int ES, const cpx<R> *__restrict__ tw) {
+    constexpr int RAD = ordered_radix(N, STAGE);
+    if constexpr (RAD > 1) {
+        line_stage<R, S, N, RAD, NSB, ordered_tpl(N)>(buf, ES, (int)threadIdx.x % L, (int)threadIdx.x / L, tw, 0);
+        ordered_fft<R, S, N, STAGE + 1, NSB * RAD>(buf, L, ES, tw);
+    }
+}
+
 }  // namespace hom

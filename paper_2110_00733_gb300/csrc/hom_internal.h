@@ -176,6 +176,7 @@ struct Geometry {
     long long V, S;         // voxels, half-spectrum points per component
     AxisPlan ax[3];
     int line[3];            // FP64: length of the axis if the line engine runs it, else 0
+    int ord[3];             // FP64: the same for ordered_fft
     const double2 *Dc[3], *Mc[3];   // FP64: difference symbol and averaging factor, complex (gamma_at_c)
     const void *D[3];       // per axis: difference symbol without its phase (real, length n_p; see gamma_e)
     const void *M[3];       // per axis: averaging factor without its phase (real, length n_p)
@@ -341,6 +342,10 @@ F64X1Fn f64_x1_kernel(int n);
 F64X1lFn f64_x1l_kernel(int n);
 F64X2Fn f64_x2_kernel(int n, int inverse);
 F64X3Fn f64_x3_kernel(int n, int pairs);   // pairs of components: 3 or 5
+// the same on ordered_fft (6 components)
+F64X1Fn f64_ord_x1_kernel(int n);
+F64X2Fn f64_ord_x2_kernel(int n, int inverse);
+F64X3Fn f64_ord_x3_kernel(int n);
 
 struct X3Line {
     using Fn = void (*)(Geometry, const float2 *, float2 *, int, float, float, const float *, const MinresState *,
@@ -397,6 +402,8 @@ template <typename R> struct Launch {
                    const cpx<R> *dotv, double *partials, const MinresState *state);
     // MoDBFFT: forward n1 pass of the 10-component spectrum in10 with the
     // contraction to 3 components fused (out3 = tau xi + g, eq. modbfftfop;
+    static void x1_dot(const Geometry &g, cudaStream_t st, const cpx<R> *z, const cpx<R> *dotv, double *partials,
+                       const MinresState *state);
     // with dot3, the weighted <dot3, out3> partials).  Returns the number of
     // partials written, or 0 without launching where the fused form does not
     // apply (not the TMA-staged FP32 pass, or more partials than max_partials).

@@ -311,8 +311,9 @@ __device__ __forceinline__ void gamma_from_q(const Geometry &g, const GammaE<R> 
 // in place, returns buf.  NF > 0: the register engine in FP32; in FP64 the line
 // engine, whose wide butterflies need the fewest operations (the FP64 pipe bounds
 // these passes: 96 = 16 6 takes 19 operations an element, 4 4 2 3 took 22).  NF <
-// 0: FP64 on the register engine of length -NF.  Generic engine (NF = 0):
-// ping-pong with buf2, returns the buffer holding the result.
+// 0: FP64 on the register engine of length -NF, or in the runtime engine's order
+// (ordered_fft).  Generic engine (NF = 0): ping-pong with buf2, returns the buffer
+// holding the result.
 //
 // FP64 with NF <= 0 is what the elastoplastic increments run on (and lengths
 // beyond the line engine): they stop their linear solves at a bounded number of
@@ -324,6 +325,9 @@ __device__ __forceinline__ cpx<R> *run_fft(cpx<R> *buf, cpx<R> *buf2, int L, int
     if constexpr (NF > 0 && sizeof(R) == 8) {
         static_assert(PAD == 0, "the line engine does not pad");
         line_fft<R, S, NF>(buf, L, ES, reinterpret_cast<const cpx<R> *>(p.tw));
+        return buf;
+    } else if constexpr (NF < 0 && !is_fast_length(-NF)) {
+        ordered_fft<R, S, -NF>(buf, L, ES, reinterpret_cast<const cpx<R> *>(p.tw));
         return buf;
     } else if constexpr (NF != 0) {
         constexpr int N = NF < 0 ? -NF : NF;
@@ -385,7 +389,8 @@ __global__ void HOM_PASS_BOUNDS_N3(R, NF) k_x3(Geometry g, int in_mode, const vo
     // element stride ES = L rounded up to odd: the per-element phases below
     // stride by ES across a warp and stay free of bank conflicts; the fast
     // engine also skips one slot every 16 elements (PAD)
-    constexpr int PAD = (NF > 0 && sizeof(R) == 4) || NF < 0 ? 1 : 0;
+    constexpr bool kOrdered = NF < 0 && !is_fast_length(-NF);
+    constexpr int PAD = (NF > 0 && sizeof(R) == 4) || (NF < 0 && !kOrdered) ? 1 : 0;
     using Plan = typename std::conditional<NF < 0, FastPlan<(NF < 0 ? -NF : 8)>, FastPlanN3<NF>>::type;
     constexpr int NC = 2 * NP;   // components per frequency
     const int N = g.n3, ROWS = g.rows3, L = NP * ROWS, ES = L | 1, H = g.h;
@@ -953,6 +958,32 @@ __global__ void HOM_PASS_BOUNDS_NF(R, NF) k_x1(Geometry g, int flags, const cpx<
     }
 }
 
+// the X1_DOT sum of k_x1 alone, over z as it was stored: the same partials bit
+// for bit, with k_x1's own launch free to take narrower tiles
+template <typename R>
+__global__ void k_x1_dot(Geometry g, const cpx<R> *__restrict__ z, const cpx<R> *__restrict__ dotv,
+                         double *__restrict__ partials, const MinresState *state) {
+    if (skip(state)) return;
+    const int NC = g.nc, N = g.n1, T = g.tile1, H = g.h, L = NC * T;
+    const int cols = g.n2 * H, g0 = blockIdx.x * T;
+    const size_t sK1 = (size_t)cols * NC;
+    const int lt = threadIdx.x % L, e0 = threadIdx.x / L, es = blockDim.x / L;
+    const int col = g0 + lt / NC;
+    Acc<R> acc;
+    if (col < cols) {
+        const R w = (R)pweight(col - (col / H) * H, g.n3);
+        const size_t o = (size_t)g0 * NC + lt;
+#pragma unroll 4
+        for (int e = e0; e < N; e += es) {
+            const cpx<R> a = z[o + e * sK1], d = dotv[o + e * sK1];
+            acc.add_prod(w * a.x, d.x);
+            acc.add_prod(w * a.y, d.y);
+        }
+    }
+    const double s = block_sum(acc.value());
+    if (threadIdx.x == 0) partials[blockIdx.x] = s;
+}
+
 // A TMA box dimension holds at most 256 elements: a tile of n > 256 rows moves
 // as n / box consecutive boxes of box rows (tma_box_rows); rowb is the bytes of
 // one row of the tile in shared memory.
@@ -1429,8 +1460,17 @@ __global__ void __launch_bounds__(kEwThreads) k_lanczos_update(int n, int h, int
                                                                cpx<R> *__restrict__ x, const MinresState *st,
                                                                double *__restrict__ partials) {
     if (skip(st)) return;
-    const double bk = st->beta, bkm = st->beta_prev;
-    const R cp = (R)(1.0 / bk), cu = (R)(-st->alpha / bk), cv = (R)(bkm > 0.0 ? -bk / bkm : 0.0);
+    // the coefficients once a CTA: three FP64 divisions in every thread, of one
+    // or two elements each, were half of this kernel (33 us at 48^3 in FP64)
+    __shared__ R sc[3];
+    if (threadIdx.x == 0) {
+        const double bk = st->beta, bkm = st->beta_prev;
+        sc[0] = (R)(1.0 / bk);
+        sc[1] = (R)(-st->alpha / bk);
+        sc[2] = (R)(bkm > 0.0 ? -bk / bkm : 0.0);
+    }
+    __syncthreads();
+    const R cp = sc[0], cu = sc[1], cv = sc[2];
     const bool lagged = st->k > 0;
     const R d = (R)st->u_delta, e = (R)st->u_eps, ig = (R)st->u_inv_gamma, tau = (R)st->u_tau,
             ib = (R)st->u_inv_beta;
@@ -1735,6 +1775,10 @@ void Launch<R>::table_init(const Geometry &g) {
             for (int inv = 0; inv < 2; ++inv) line_kernel_attr((const void *)f64_x2_kernel(g.n2, inv), lim);
         if (f64_line_tpl(g.n3))
             for (int np : {3, 5}) line_kernel_attr((const void *)f64_x3_kernel(g.n3, np), lim);
+        if (f64_ord_x1_kernel(g.n1)) line_kernel_attr((const void *)f64_ord_x1_kernel(g.n1), lim);
+        for (int inv = 0; inv < 2; ++inv)
+            if (f64_ord_x2_kernel(g.n2, inv)) line_kernel_attr((const void *)f64_ord_x2_kernel(g.n2, inv), lim);
+        if (f64_ord_x3_kernel(g.n3)) line_kernel_attr((const void *)f64_ord_x3_kernel(g.n3), lim);
 #define HOM_F64_ATTR1(NF) line_kernel_attr((const void *)k_x1<R, NF>, lim), line_kernel_attr((const void *)k_x1_lanczos<R, NF>, lim)
 #define HOM_F64_ATTR2(NF) line_kernel_attr((const void *)k_x2<R, -1, NF>, lim), line_kernel_attr((const void *)k_x2<R, 1, NF>, lim)
 #define HOM_F64_ATTR3(NF) line_kernel_attr((const void *)k_x3<R, NF, 3>, lim), line_kernel_attr((const void *)k_x3<R, NF, 5>, lim)
@@ -1863,6 +1907,7 @@ void Launch<R>::x3(const Geometry &g, cudaStream_t st, int in_mode, const void *
         F64X3Fn f = nullptr;
 #define HOM_X3(NF) f = g.nc == 10 ? k_x3<R, NF, 5> : k_x3<R, NF, 3>
         if (g.line[2]) f = f64_x3_kernel(g.n3, g.nc / 2);
+        else if (g.ord[2]) f = f64_ord_x3_kernel(g.n3);
         else HOM_F64_SWITCH(g.fast[2], HOM_X3)
 #undef HOM_X3
         if (g.nc == 10) epart = tsum = nullptr, fold = Fold{};
@@ -1900,6 +1945,7 @@ void Launch<R>::x2(const Geometry &g, cudaStream_t st, int inverse, cpx<R> *spec
         F64X2Fn f = nullptr;
 #define HOM_X2(NF) f = inverse ? k_x2<R, 1, NF> : k_x2<R, -1, NF>
         if (g.line[1]) f = f64_x2_kernel(g.n2, inverse);
+        else if (g.ord[1]) f = f64_ord_x2_kernel(g.n2, inverse);
         else HOM_F64_SWITCH(g.fast[1], HOM_X2)
 #undef HOM_X2
         launch_k(g.pdl, f, grid, g.threads2, g.smem2, st, g, spec, state);
@@ -1941,6 +1987,7 @@ void Launch<R>::x1(const Geometry &g, cudaStream_t st, int flags, const cpx<R> *
         F64X1Fn f = nullptr;
 #define HOM_X1(NF) f = k_x1<R, NF>
         if (g.line[0]) f = f64_x1_kernel(g.n1);
+        else if (g.ord[0]) f = f64_ord_x1_kernel(g.n1);
         else HOM_F64_SWITCH(g.fast[0], HOM_X1)
 #undef HOM_X1
         f<<<grid, g.threads1, g.smem1, st>>>(g, flags, in, out, dotv, partials, state);
@@ -1949,6 +1996,12 @@ void Launch<R>::x1(const Geometry &g, cudaStream_t st, int flags, const cpx<R> *
     HOM_FAST_SWITCH(g.fast[0], HOM_X1)
 #undef HOM_X1
     }
+}
+
+template <typename R>
+void Launch<R>::x1_dot(const Geometry &g, cudaStream_t st, const cpx<R> *z, const cpx<R> *dotv, double *partials,
+                       const MinresState *state) {
+    k_x1_dot<R><<<(g.n2 * g.h + g.tile1 - 1) / g.tile1, g.threads1, 0, st>>>(g, z, dotv, partials, state);
 }
 
 template <typename R>
