@@ -77,6 +77,7 @@ template <typename R> struct Engine {
 // History and Newton work fields of an elastoplastic cell (hom_j2_*), FP64
 // real fields 6 x V Mandel, component-major.
 struct J2State {
+    double2 *etab = nullptr;   // unit frequency vectors, 3 S (FP64 contexts; null: formed in the passes)
     bool active = false;
     J2Material mat{};          // units of E (E = 1)
     double *eps = nullptr;     // total strain at the current iterate
@@ -245,9 +246,9 @@ static int set_shapes(hom_ctx *ctx, Geometry &g, int nc, bool lines = true) {
     int rows, t2, t1;
     const int tpl1 = f64 ? f64_line_tpl(g.n1) : 0, tpl2 = f64 ? f64_line_tpl(g.n2) : 0, tpl3 = f64 ? f64_line_tpl(g.n3) : 0;
     if (tpl3) {
-        // measured (6-component spectra, ms): 96^3 8 rows 0.318, 4 0.324; 108^3 0.490, 0.519;
-        // 128^3 0.699, 0.660 (51 KB of shared memory a CTA against 27); 192^3 2.72, 2.48; 48^3
-        // 8 rows 0.045, 16 0.066
+        // measured (6-component spectra, ms): 96^3 8 rows 0.293, 4 0.316; 108^3 0.453, 0.505;
+        // 128^3 0.652, 0.631 (51 KB of shared memory a CTA against 27); 192^3 2.49, 2.41; 48^3
+        // 8 rows 0.035, 4 0.045
         rows = (size_t)g.n3 * ((8 * np) | 1) * cs <= 45 * 1024 ? 8 : 4;
         while (np * rows * tpl3 < 96) rows *= 2;
         while (rows > 1 && g.n1 * g.n2 < kSms * rows) rows >>= 1;   // small cells: every SM's FP64 pipe
@@ -1067,6 +1068,8 @@ static void j2_free(hom_ctx *ctx) {
     float *fbufs[] = {j.Ct32, j.sig32, j.de32};
     for (float *p : fbufs) cudaFree(p);
     cudaFree(j.x64);
+    cudaFree(j.etab);
+    ctx->e64.gj.etab = nullptr;
     if (j.h_partials) cudaFreeHost(j.h_partials);
     j = J2State{};
     ctx->tangent_op = false;
@@ -2777,7 +2780,7 @@ int hom_fields(hom_ctx *ctx, int icase, void *strain, void *stress) {
 // device bytes of the history and Newton work fields
 static long long j2_bytes(const hom_ctx *ctx) {
     const long long V = ctx->V;
-    return (long long)sizeof(double) * 37 * V +
+    return (long long)sizeof(double) * 37 * V + (ctx->j2.etab ? (long long)sizeof(double2) * 3 * ctx->S : 0) +
            (ctx->prec == HOM_PREC_FP64 ? (long long)sizeof(double) * 36 * V
                                         : (long long)sizeof(float) * 48 * V + (long long)sizeof(double2) * 6 * ctx->S);
 }
@@ -2815,6 +2818,17 @@ int hom_j2_begin(hom_ctx *ctx, double yield_stress, double hardening) {
         if (rc) {
             j2_free(ctx);
             return rc;
+        }
+        // the increments' projector table, where memory allows it
+        if (ctx->prec == HOM_PREC_FP64) {
+            if (cudaMalloc(&j.etab, sizeof(double2) * 3 * ctx->S) == cudaSuccess) {
+                Launch<double>::gamma_table(ctx->e64.gj, ctx->stream, j.etab);
+                ctx->e64.gj.etab = j.etab;
+                ctx->launches += 1;
+            } else {
+                j.etab = nullptr;
+                cudaGetLastError();
+            }
         }
         ctx->workspace += j2_bytes(ctx);
         j.active = true;

@@ -178,6 +178,7 @@ struct Geometry {
     int line[3];            // FP64: length of the axis if the line engine runs it, else 0
     int ord[3];             // FP64: the same for ordered_fft
     const double2 *Dc[3], *Mc[3];   // FP64: difference symbol and averaging factor, complex (gamma_at_c)
+    const double2 *etab = nullptr;  // unit vectors of every frequency, or null: formed in the pass
     const void *D[3];       // per axis: difference symbol without its phase (real, length n_p; see gamma_e)
     const void *M[3];       // per axis: averaging factor without its phase (real, length n_p)
     // launch shapes: rows per CTA of the n3 pass, columns per CTA of the n2
@@ -402,6 +403,7 @@ template <typename R> struct Launch {
                    const cpx<R> *dotv, double *partials, const MinresState *state);
     // MoDBFFT: forward n1 pass of the 10-component spectrum in10 with the
     // contraction to 3 components fused (out3 = tau xi + g, eq. modbfftfop;
+    static void gamma_table(const Geometry &g, cudaStream_t st, double2 *out);   // FP64
     static void x1_dot(const Geometry &g, cudaStream_t st, const cpx<R> *z, const cpx<R> *dotv, double *partials,
                        const MinresState *state);
     // with dot3, the weighted <dot3, out3> partials).  Returns the number of

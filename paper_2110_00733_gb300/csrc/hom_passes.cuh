@@ -223,8 +223,36 @@ __device__ __forceinline__ void gamma_apply(const Geometry &g, const GammaE<R> &
     gamma_sym<R>(q, w, t);
 }
 
-// The same projector with the complex vector as it stands (Geometry::Dc, Mc),
-// for the FP64 passes on the engines of old (NF <= 0, see run_fft).
+// The same projector with the complex vector as it stands (Geometry::Dc, Mc), for
+// the FP64 passes on the engines of old (NF <= 0, see run_fft).  e = xi / |xi|, or
+// 0 where G = 0 or xi = 0.
+__device__ __forceinline__ void gamma_e_c(const Geometry &g, int k1, int k2, int k3, double2 *e) {
+    typedef double R;
+    const cpx<R> m0 = __ldg(g.Mc[0] + k1), m1 = __ldg(g.Mc[1] + k2), m2 = __ldg(g.Mc[2] + k3);
+    const cpx<R> x0 = mul<R>(__ldg(g.Dc[0] + k1), mul<R>(m1, m2));
+    const cpx<R> x1 = mul<R>(__ldg(g.Dc[1] + k2), mul<R>(m0, m2));
+    const cpx<R> x2 = mul<R>(__ldg(g.Dc[2] + k3), mul<R>(m0, m1));
+    const R n2 = x0.x * x0.x + x0.y * x0.y + x1.x * x1.x + x1.y * x1.y + x2.x * x2.x + x2.y * x2.y;
+    if (2 * k1 == g.n1 || 2 * k2 == g.n2 || 2 * k3 == g.n3 || !(n2 > (R)0)) {
+        e[0] = e[1] = e[2] = mk<R>(0, 0);
+        return;
+    }
+    const R inv = (R)1 / sqrt(n2);
+    e[0] = scale<R>(x0, inv);
+    e[1] = scale<R>(x1, inv);
+    e[2] = scale<R>(x2, inv);
+}
+// e of every frequency (Geometry::etab): a third of the projector's FP64
+// operations are the square root and the division that e takes
+template <typename R> __global__ void k_gamma_table(Geometry g, cpx<R> *__restrict__ out) {
+    for (long long f = (long long)blockIdx.x * blockDim.x + threadIdx.x; f < g.S; f += (long long)gridDim.x * blockDim.x) {
+        const int k3 = (int)(f % g.h), r = (int)(f / g.h);
+        cpx<R> e[3];
+        gamma_e_c(g, r / g.n2, r % g.n2, k3, e);
+        for (int c = 0; c < 3; ++c) out[3 * f + c] = e[c];
+    }
+}
+
 __device__ __forceinline__ void gamma_at_c(const Geometry &g, int k1, int k2, int k3, double2 *t) {
     typedef double R;
     if (k1 == 0 && k2 == 0 && k3 == 0) {
@@ -233,18 +261,21 @@ __device__ __forceinline__ void gamma_at_c(const Geometry &g, int k1, int k2, in
             if (!((g.mask0 >> c) & 1)) t[c] = mk<R>(0, 0);
         return;
     }
-    const cpx<R> m0 = __ldg(g.Mc[0] + k1), m1 = __ldg(g.Mc[1] + k2), m2 = __ldg(g.Mc[2] + k3);
-    const cpx<R> x0 = mul<R>(__ldg(g.Dc[0] + k1), mul<R>(m1, m2));
-    const cpx<R> x1 = mul<R>(__ldg(g.Dc[1] + k2), mul<R>(m0, m2));
-    const cpx<R> x2 = mul<R>(__ldg(g.Dc[2] + k3), mul<R>(m0, m1));
-    const R n2 = x0.x * x0.x + x0.y * x0.y + x1.x * x1.x + x1.y * x1.y + x2.x * x2.x + x2.y * x2.y;
-    if (2 * k1 == g.n1 || 2 * k2 == g.n2 || 2 * k3 == g.n3 || !(n2 > (R)0)) {
+    cpx<R> ev[3];
+    if (g.etab) {
+        const double2 *et = g.etab + 3 * (((size_t)k1 * g.n2 + k2) * g.h + k3);
+        ev[0] = __ldg(et);
+        ev[1] = __ldg(et + 1);
+        ev[2] = __ldg(et + 2);
+    } else {
+        gamma_e_c(g, k1, k2, k3, ev);
+    }
+    const cpx<R> e0 = ev[0], e1 = ev[1], e2 = ev[2];
+    if (e0.x == 0 && e0.y == 0 && e1.x == 0 && e1.y == 0 && e2.x == 0 && e2.y == 0) {
 #pragma unroll
         for (int c = 0; c < 6; ++c) t[c] = mk<R>(0, 0);
         return;
     }
-    const R inv = (R)1 / sqrt(n2);
-    const cpx<R> e0 = scale<R>(x0, inv), e1 = scale<R>(x1, inv), e2 = scale<R>(x2, inv);
     const cpx<R> c0 = conjc<R>(e0), c1 = conjc<R>(e1), c2 = conjc<R>(e2);
     const R r2 = (R)0.70710678118654752440;   // 1/sqrt(2)
     const cpx<R> T11 = t[0], T22 = t[1], T33 = t[2];
@@ -393,7 +424,9 @@ __global__ void HOM_PASS_BOUNDS_N3(R, NF) k_x3(Geometry g, int in_mode, const vo
     constexpr int PAD = (NF > 0 && sizeof(R) == 4) || (NF < 0 && !kOrdered) ? 1 : 0;
     using Plan = typename std::conditional<NF < 0, FastPlan<(NF < 0 ? -NF : 8)>, FastPlanN3<NF>>::type;
     constexpr int NC = 2 * NP;   // components per frequency
-    const int N = g.n3, ROWS = g.rows3, L = NP * ROWS, ES = L | 1, H = g.h;
+    constexpr int NCT = NF < 0 ? -NF : NF;   // the length, where it is known
+    const int N = NCT ? NCT : g.n3, H = N / 2 + 1;
+    const int ROWS = g.rows3, L = NP * ROWS, ES = L | 1;
     auto ep = [ES](int e) { return epos<PAD>(e, ES); };
     cpx<R> *buf = reinterpret_cast<cpx<R> *>(smem_raw);
     cpx<R> *buf2 = buf + ep(N);   // second buffer of the generic engine only
@@ -415,18 +448,19 @@ __global__ void HOM_PASS_BOUNDS_N3(R, NF) k_x3(Geometry g, int in_mode, const vo
         // Z[k] = X_a[k] + i X_b[k] and Z[N-k] = conj X_a[k] + i conj X_b[k];
         // the self-conjugate bins keep their real parts, as a C2R does
         const cpx<R> *spec = reinterpret_cast<const cpx<R> *>(in_);
-        for (int r = 0; r < ROWS; ++r) {
+        // all rows' elements as one range: a row alone has fewer than the CTA
+        // threads (FP64 pass, row by row and so: 48^3 45 to 35 us, 96^3 318 to 293)
+        for (int i = threadIdx.x; i < ROWS * H; i += blockDim.x) {
+            const int r = i / H, k = i - r * H;
             const cpx<R> *row = spec + (size_t)(row0 + r) * H * NC;
-            for (int k = threadIdx.x; k < H; k += blockDim.x) {
-                const bool selfc = (k == 0) || (2 * k == N);
+            const bool selfc = (k == 0) || (2 * k == N);
 #pragma unroll
-                for (int p = 0; p < NP; ++p) {
-                    cpx<R> xa = mk<R>(0, 0), xb = mk<R>(0, 0);
-                    if (r < nr) Six<R>::load_pair(row + NC * k, p, xa, xb);
-                    if (selfc) { xa.y = 0; xb.y = 0; }
-                    buf[ep(k) + p * ROWS + r] = mk<R>(xa.x - xb.y, xa.y + xb.x);
-                    if (!selfc) buf[ep(N - k) + p * ROWS + r] = mk<R>(xa.x + xb.y, xb.x - xa.y);
-                }
+            for (int p = 0; p < NP; ++p) {
+                cpx<R> xa = mk<R>(0, 0), xb = mk<R>(0, 0);
+                if (r < nr) Six<R>::load_pair(row + NC * k, p, xa, xb);
+                if (selfc) { xa.y = 0; xb.y = 0; }
+                buf[ep(k) + p * ROWS + r] = mk<R>(xa.x - xb.y, xa.y + xb.x);
+                if (!selfc) buf[ep(N - k) + p * ROWS + r] = mk<R>(xa.x + xb.y, xb.x - xa.y);
             }
         }
         __syncthreads();
@@ -437,17 +471,16 @@ __global__ void HOM_PASS_BOUNDS_N3(R, NF) k_x3(Geometry g, int in_mode, const vo
         }
     } else {
         const R *real = reinterpret_cast<const R *>(in_);
-        for (int r = 0; r < ROWS; ++r) {
+        for (int i = threadIdx.x; i < ROWS * N; i += blockDim.x) {
+            const int r = i / N, e = i - r * N;
             const int vbase = (row0 + r) * N;
-            for (int e = threadIdx.x; e < N; e += blockDim.x) {
-                R t[NC];
+            R t[NC];
 #pragma unroll
-                for (int c = 0; c < NC; ++c)
-                    t[c] = (r >= nr || c >= 6) ? (R)0
-                                               : (in_mode == X3_IN_MACRO ? (R)mac.v[c] : real[c * V + vbase + e]);
+            for (int c = 0; c < NC; ++c)
+                t[c] = (r >= nr || c >= 6) ? (R)0
+                                           : (in_mode == X3_IN_MACRO ? (R)mac.v[c] : real[c * V + vbase + e]);
 #pragma unroll
-                for (int p = 0; p < NP; ++p) buf[ep(e) + p * ROWS + r] = mk<R>(t[2 * p], t[2 * p + 1]);
-            }
+            for (int p = 0; p < NP; ++p) buf[ep(e) + p * ROWS + r] = mk<R>(t[2 * p], t[2 * p + 1]);
         }
         __syncthreads();
     }
@@ -465,63 +498,62 @@ __global__ void HOM_PASS_BOUNDS_N3(R, NF) k_x3(Geometry g, int in_mode, const vo
     // n1 pass needs no dot product with u
     R en = 0;   // non-negative terms: a short per-thread sum in R is accurate to ~1e-6
     double ts[6] = {0, 0, 0, 0, 0, 0};   // stress sums (tsum)
-    for (int r = 0; r < nr; ++r) {
+    for (int i = threadIdx.x; i < nr * N; i += blockDim.x) {
+        const int r = i / N, e = i - r * N;
         const int vbase = (row0 + r) * N;
-        for (int e = threadIdx.x; e < N; e += blockDim.x) {
-            cpx<R> *q = buf + ep(e) + r;
-            R t[NC];
+        cpx<R> *q = buf + ep(e) + r;
+        R t[NC];
 #pragma unroll
-            for (int p = 0; p < NP; ++p) {
-                const cpx<R> z = q[p * ROWS];
-                t[2 * p] = kFold ? z.x : z.x * s_all;
-                t[2 * p + 1] = kFold ? z.y : z.y * s_all;
-            }
-            if (mid == X3_MID_MATERIAL || mid == X3_MID_MODB) {
-                const R ph = phi[vbase + e];
-                const R sum = t[0] + t[1] + t[2];
-                if constexpr (kFold) {
-                    const R m = ph * f_mu2, tr = ph * f_lam * sum;
+        for (int p = 0; p < NP; ++p) {
+            const cpx<R> z = q[p * ROWS];
+            t[2 * p] = kFold ? z.x : z.x * s_all;
+            t[2 * p + 1] = kFold ? z.y : z.y * s_all;
+        }
+        if (mid == X3_MID_MATERIAL || mid == X3_MID_MODB) {
+            const R ph = phi[vbase + e];
+            const R sum = t[0] + t[1] + t[2];
+            if constexpr (kFold) {
+                const R m = ph * f_mu2, tr = ph * f_lam * sum;
 #pragma unroll
-                    for (int c = 0; c < 6; ++c) {
-                        const R o = c < 3 ? tr + m * t[c] : m * t[c];
-                        if (epart) en += t[c] * o;   // (times s_all / f_all s_all at the end)
-                        t[c] = o;
-                    }
-                } else {
-                    const R tr = lam * sum;
-                    if (epart) {
-                        R ee = t[0] * t[0];
-#pragma unroll
-                        for (int c = 1; c < 6; ++c) ee += t[c] * t[c];
-                        en += ph * (tr * sum + mu2 * ee);
-                    }
-#pragma unroll
-                    for (int c = 0; c < 6; ++c) t[c] = ph * ((c < 3 ? tr : (R)0) + mu2 * t[c]);
+                for (int c = 0; c < 6; ++c) {
+                    const R o = c < 3 ? tr + m * t[c] : m * t[c];
+                    if (epart) en += t[c] * o;   // (times s_all / f_all s_all at the end)
+                    t[c] = o;
                 }
-                if (tsum) {
-#pragma unroll
-                    for (int c = 0; c < 6; ++c) ts[c] += (double)t[c];
-                }
-                if constexpr (NC == 10) {
-                    // MoDBFFT penalty vector on the empty phase: chi_v g, eq. (modbfftfop)
-                    const R chi = (ph == (R)0) ? (kFold ? f_all : (R)1) : (R)0;
-                    t[6] *= chi;
-                    t[7] *= chi;
-                    t[8] *= chi;
-                    t[9] = 0;
-                }
-            } else if (kFold) {
-#pragma unroll
-                for (int c = 0; c < NC; ++c) t[c] *= f_all;
-            }
-            if (out_mode == X3_OUT_REAL) {
-                R *real = reinterpret_cast<R *>(out_);
-#pragma unroll
-                for (int c = 0; c < 6; ++c) real[c * V + vbase + e] = t[c];   // (NC == 6 only)
             } else {
+                const R tr = lam * sum;
+                if (epart) {
+                    R ee = t[0] * t[0];
 #pragma unroll
-                for (int p = 0; p < NP; ++p) q[p * ROWS] = mk<R>(t[2 * p], t[2 * p + 1]);
+                    for (int c = 1; c < 6; ++c) ee += t[c] * t[c];
+                    en += ph * (tr * sum + mu2 * ee);
+                }
+#pragma unroll
+                for (int c = 0; c < 6; ++c) t[c] = ph * ((c < 3 ? tr : (R)0) + mu2 * t[c]);
             }
+            if (tsum) {
+#pragma unroll
+                for (int c = 0; c < 6; ++c) ts[c] += (double)t[c];
+            }
+            if constexpr (NC == 10) {
+                // MoDBFFT penalty vector on the empty phase: chi_v g, eq. (modbfftfop)
+                const R chi = (ph == (R)0) ? (kFold ? f_all : (R)1) : (R)0;
+                t[6] *= chi;
+                t[7] *= chi;
+                t[8] *= chi;
+                t[9] = 0;
+            }
+        } else if (kFold) {
+#pragma unroll
+            for (int c = 0; c < NC; ++c) t[c] *= f_all;
+        }
+        if (out_mode == X3_OUT_REAL) {
+            R *real = reinterpret_cast<R *>(out_);
+#pragma unroll
+            for (int c = 0; c < 6; ++c) real[c * V + vbase + e] = t[c];   // (NC == 6 only)
+        } else {
+#pragma unroll
+            for (int p = 0; p < NP; ++p) q[p * ROWS] = mk<R>(t[2 * p], t[2 * p + 1]);
         }
     }
     if (tsum) {
@@ -549,20 +581,19 @@ __global__ void HOM_PASS_BOUNDS_N3(R, NF) k_x3(Geometry g, int in_mode, const vo
     // unpack the two real transforms of each packed line:
     //   X_a[k] = (Z[k] + conj Z[N-k]) / 2,  X_b[k] = (Z[k] - conj Z[N-k]) / (2i)
     cpx<R> *spec = reinterpret_cast<cpx<R> *>(out_);
-    for (int r = 0; r < nr; ++r) {
+    for (int i = threadIdx.x; i < nr * H; i += blockDim.x) {
+        const int r = i / H, k = i - r * H;
         cpx<R> *row = spec + (size_t)(row0 + r) * H * NC;
-        for (int k = threadIdx.x; k < H; k += blockDim.x) {
-            const int km = (k == 0) ? 0 : N - k;
+        const int km = (k == 0) ? 0 : N - k;
 #pragma unroll
-            for (int p = 0; p < NP; ++p) {
-                const cpx<R> z = res[ep(k) + p * ROWS + r];
-                const cpx<R> zm = conjc<R>(res[ep(km) + p * ROWS + r]);
-                if constexpr (kFold)
-                    Six<R>::store_pair(row + NC * k, p, mk<R>(z.x + zm.x, z.y + zm.y), mk<R>(z.y - zm.y, zm.x - z.x));
-                else
-                    Six<R>::store_pair(row + NC * k, p, mk<R>((R)0.5 * (z.x + zm.x), (R)0.5 * (z.y + zm.y)),
-                                       mk<R>((R)0.5 * (z.y - zm.y), (R)-0.5 * (z.x - zm.x)));
-            }
+        for (int p = 0; p < NP; ++p) {
+            const cpx<R> z = res[ep(k) + p * ROWS + r];
+            const cpx<R> zm = conjc<R>(res[ep(km) + p * ROWS + r]);
+            if constexpr (kFold)
+                Six<R>::store_pair(row + NC * k, p, mk<R>(z.x + zm.x, z.y + zm.y), mk<R>(z.y - zm.y, zm.x - z.x));
+            else
+                Six<R>::store_pair(row + NC * k, p, mk<R>((R)0.5 * (z.x + zm.x), (R)0.5 * (z.y + zm.y)),
+                                   mk<R>((R)0.5 * (z.y - zm.y), (R)-0.5 * (z.x - zm.x)));
         }
     }
 }
@@ -1996,6 +2027,11 @@ void Launch<R>::x1(const Geometry &g, cudaStream_t st, int flags, const cpx<R> *
     HOM_FAST_SWITCH(g.fast[0], HOM_X1)
 #undef HOM_X1
     }
+}
+
+template <typename R>
+void Launch<R>::gamma_table(const Geometry &g, cudaStream_t st, double2 *out) {
+    if constexpr (sizeof(R) == 8) k_gamma_table<R><<<ew_grid(g.S), kEwThreads, 0, st>>>(g, out);
 }
 
 template <typename R>
