@@ -254,7 +254,7 @@ static int set_shapes(hom_ctx *ctx, Geometry &g, int nc, bool lines = true) {
         while (rows > 1 && g.n1 * g.n2 < kSms * rows) rows >>= 1;   // small cells: every SM's FP64 pipe
         while (rows > 1 && (np * rows * tpl3 > 512 || (size_t)g.n3 * ((rows * np) | 1) * cs > 110 * 1024)) rows >>= 1;
     } else if (g.fast[2]) {
-        rows = 48 / (np * (g.n3 / elems3));
+        rows = (nc == 10 && sizeof(R) == 4 ? 160 : 48) / (np * (g.n3 / elems3));   // (MoDBFFT 128^3: 4 rows 0.400 ms a step, 1 0.417)
         rows = rows < 1 ? 1 : (rows > 64 ? 64 : rows);
         // the two-stage plans at 96 and 160, measured (6-component spectra): 8
         // rows at 160 (0.123 against 0.136 ms at 160^3), 2 at 96 (0.027 against
@@ -493,9 +493,10 @@ static int engine_init(hom_ctx *ctx, Engine<R> &E) {
     CU(cudaMalloc(&E.phi, sizeof(R) * ctx->V));
     CU(cudaMalloc(&E.spec, cs * 6 * ctx->S));
     ctx->workspace += sizeof(R) * ctx->V + cs * 6 * ctx->S;
-    Launch<R>::table_init(g);
+    if (sizeof(R) == 4) Launch<R>::table_init(g);   // before the occupancy queries of set_shapes
     int rc = set_shapes<R>(ctx, g, 6);
     if (rc) return rc;
+    if (sizeof(R) == 8) Launch<R>::table_init(g);   // after it chose the engines
     E.gj = g;
     if (sizeof(R) == 8) {
         rc = set_shapes<R>(ctx, E.gj, 6, false);
@@ -776,6 +777,7 @@ static int engine_init_modb(hom_ctx *ctx, Engine<R> &E) {
     E.gm.tma_cache = nullptr;
     int rc = set_shapes<R>(ctx, E.gm, 10);
     if (rc) return rc;
+    if (sizeof(R) == 8) Launch<R>::table_init(E.gm);
     CU(cudaMalloc(&E.spec10, cpx_size<R>() * 10 * ctx->S));
     ctx->workspace += cpx_size<R>() * 10 * ctx->S;
     return HOM_OK;
@@ -2819,6 +2821,7 @@ int hom_j2_begin(hom_ctx *ctx, double yield_stress, double hardening) {
             j2_free(ctx);
             return rc;
         }
+        Launch<double>::table_init(ctx->e64.gj);
         // the increments' projector table, where memory allows it
         if (ctx->prec == HOM_PREC_FP64) {
             if (cudaMalloc(&j.etab, sizeof(double2) * 3 * ctx->S) == cudaSuccess) {

@@ -120,8 +120,11 @@ int setup_device(int dev, DevicePtrs **out) {
             return HOM_ECUDA;
         }
         d.tab = static_cast<float2 *>(p);
-        Geometry g{};
-        Launch<float>::table_init(g);   // shared-memory limits of the pass kernels
+        Geometry g{};   // shared-memory limits of the pass kernels, every length up to 64
+        for (int n : {0, 8, 16, 32, 64}) {
+            g.fast[0] = g.fast[1] = g.fast[2] = n;
+            Launch<float>::table_init(g);
+        }
         e = cudaGetLastError();
         if (e != cudaSuccess) {
             hom_set_error((std::string("hom_apply_noalloc: device set-up failed: ") + cudaGetErrorString(e)).c_str());

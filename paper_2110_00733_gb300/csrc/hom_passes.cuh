@@ -12,8 +12,11 @@
 //   x2(forward)               forward along n2
 //   x1(forward, G on output)  forward along n1 + projector, with the MINRES
 //                             dot product <v, A^ v> fused into the store
-// Lengths 8..512 that are powers of two use the compile-time register FFT
-// (fast_fft); other 2^a 3^b 5^c lengths use the runtime Stockham engine.
+// The unfused FP32 passes here use the compile-time register FFT (fast_fft) at
+// powers of two, 96 and 160 and the runtime Stockham engine at other 2^a 3^b 5^c
+// lengths; the FP64 ones the line engine at every length from 16 to 512 and 8
+// (see run_fft).  The passes of the FP32 MINRES step at those lengths are in
+// hom_lines.cuh (n2 and fused n1) and hom_x3.cuh (n3).
 #pragma once
 #include <math.h>
 
@@ -1769,6 +1772,44 @@ int Launch<R>::x1_grid(const Geometry &g) {
         default: CALL(0); break;                   \
     }
 
+// the FP64 kernels of a geometry: the line engine, the ordered plans, the register
+// engine in its order of old, or the runtime engine
+template <typename R> F64X3Fn f64_x3_of(const Geometry &g) {
+    F64X3Fn f = nullptr;
+#define HOM_X3(NF) f = g.nc == 10 ? k_x3<R, NF, 5> : k_x3<R, NF, 3>
+    if (g.line[2]) f = f64_x3_kernel(g.n3, g.nc / 2);
+    else if (g.ord[2]) f = f64_ord_x3_kernel(g.n3);
+    else HOM_F64_SWITCH(g.fast[2], HOM_X3)
+#undef HOM_X3
+    return f;
+}
+template <typename R> F64X2Fn f64_x2_of(const Geometry &g, int inverse) {
+    F64X2Fn f = nullptr;
+#define HOM_X2(NF) f = inverse ? k_x2<R, 1, NF> : k_x2<R, -1, NF>
+    if (g.line[1]) f = f64_x2_kernel(g.n2, inverse);
+    else if (g.ord[1]) f = f64_ord_x2_kernel(g.n2, inverse);
+    else HOM_F64_SWITCH(g.fast[1], HOM_X2)
+#undef HOM_X2
+    return f;
+}
+template <typename R> F64X1Fn f64_x1_of(const Geometry &g) {
+    F64X1Fn f = nullptr;
+#define HOM_X1(NF) f = k_x1<R, NF>
+    if (g.line[0]) f = f64_x1_kernel(g.n1);
+    else if (g.ord[0]) f = f64_ord_x1_kernel(g.n1);
+    else HOM_F64_SWITCH(g.fast[0], HOM_X1)
+#undef HOM_X1
+    return f;
+}
+template <typename R> F64X1lFn f64_x1l_of(const Geometry &g) {
+    F64X1lFn f = nullptr;
+#define HOM_X1L(NF) f = k_x1_lanczos<R, NF>
+    if (g.line[0]) f = f64_x1l_kernel(g.n1);
+    else HOM_F64_SWITCH(g.fast[0], HOM_X1L)
+#undef HOM_X1L
+    return f;
+}
+
 template <typename R>
 void Launch<R>::table_init(const Geometry &g) {
     // The dynamic shared-memory limit of each pass kernel is raised to the
@@ -1790,49 +1831,39 @@ void Launch<R>::table_init(const Geometry &g) {
         cudaFuncSetAttribute(K, cudaFuncAttributePreferredSharedMemoryCarveout,                 \
                              cudaSharedmemCarveoutMaxShared);                                   \
     }
-#define HOM_SET_ATTR(NF)                \
-    HOM_SET_ATTR1((k_x3<R, NF, 3>))     \
-    HOM_SET_ATTR1((k_x3<R, NF, 5>))     \
-    HOM_SET_ATTR1((k_x2<R, -1, NF>))    \
-    HOM_SET_ATTR1((k_x2<R, 1, NF>))     \
-    HOM_SET_ATTR1((k_x1<R, NF>))        \
-    HOM_SET_ATTR1((k_x1_lanczos<R, NF>))
+    // the kernels of this geometry only: the first touch of a kernel loads it
     if constexpr (sizeof(R) == 8) {
-        if (f64_line_tpl(g.n1)) {
-            line_kernel_attr((const void *)f64_x1_kernel(g.n1), lim);
-            line_kernel_attr((const void *)f64_x1l_kernel(g.n1), lim);
+        line_kernel_attr((const void *)f64_x3_of<R>(g), lim);
+        for (int inv = 0; inv < 2; ++inv) line_kernel_attr((const void *)f64_x2_of<R>(g, inv), lim);
+        line_kernel_attr((const void *)f64_x1_of<R>(g), lim);
+        if (g.nc == 6) line_kernel_attr((const void *)f64_x1l_of<R>(g), lim);
+    } else {
+#define HOM_SET_X1(NF) HOM_SET_ATTR1((k_x1<R, NF>)) HOM_SET_ATTR1((k_x1_lanczos<R, NF>))
+#define HOM_SET_X2(NF) HOM_SET_ATTR1((k_x2<R, -1, NF>)) HOM_SET_ATTR1((k_x2<R, 1, NF>))
+#define HOM_SET_X3(NF) HOM_SET_ATTR1((k_x3<R, NF, 3>)) HOM_SET_ATTR1((k_x3<R, NF, 5>))
+#define HOM_SET_TMA(NF) \
+    HOM_SET_ATTR1((k_x1_tma<R, NF>)) HOM_SET_ATTR1((k_x1_tma<R, NF, true>)) HOM_SET_ATTR1((k_x1_tma_expand<R, NF>))
+        HOM_FAST_SWITCH(g.fast[0], HOM_SET_X1)
+        HOM_FAST_SWITCH(g.fast[1], HOM_SET_X2)
+        HOM_FAST_SWITCH(g.fast[2], HOM_SET_X3)
+        switch (g.fast[0]) {
+            case 64: HOM_SET_TMA(64) break;
+            case 96: HOM_SET_TMA(96) break;
+            case 128: HOM_SET_TMA(128) break;
+            case 160: HOM_SET_TMA(160) break;
+            case 256: HOM_SET_TMA(256) break;
+            case 512: HOM_SET_TMA(512) break;
+            default: break;
         }
-        if (f64_line_tpl(g.n2))
-            for (int inv = 0; inv < 2; ++inv) line_kernel_attr((const void *)f64_x2_kernel(g.n2, inv), lim);
-        if (f64_line_tpl(g.n3))
-            for (int np : {3, 5}) line_kernel_attr((const void *)f64_x3_kernel(g.n3, np), lim);
-        if (f64_ord_x1_kernel(g.n1)) line_kernel_attr((const void *)f64_ord_x1_kernel(g.n1), lim);
-        for (int inv = 0; inv < 2; ++inv)
-            if (f64_ord_x2_kernel(g.n2, inv)) line_kernel_attr((const void *)f64_ord_x2_kernel(g.n2, inv), lim);
-        if (f64_ord_x3_kernel(g.n3)) line_kernel_attr((const void *)f64_ord_x3_kernel(g.n3), lim);
-#define HOM_F64_ATTR1(NF) line_kernel_attr((const void *)k_x1<R, NF>, lim), line_kernel_attr((const void *)k_x1_lanczos<R, NF>, lim)
-#define HOM_F64_ATTR2(NF) line_kernel_attr((const void *)k_x2<R, -1, NF>, lim), line_kernel_attr((const void *)k_x2<R, 1, NF>, lim)
-#define HOM_F64_ATTR3(NF) line_kernel_attr((const void *)k_x3<R, NF, 3>, lim), line_kernel_attr((const void *)k_x3<R, NF, 5>, lim)
-        HOM_F64_SWITCH(g.fast[0], HOM_F64_ATTR1)
-        HOM_F64_SWITCH(g.fast[1], HOM_F64_ATTR2)
-        HOM_F64_SWITCH(g.fast[2], HOM_F64_ATTR3)
-#undef HOM_F64_ATTR1
-#undef HOM_F64_ATTR2
-#undef HOM_F64_ATTR3
-    }
-    if constexpr (sizeof(R) == 4) {
-        HOM_SET_ATTR(0) HOM_SET_ATTR(8) HOM_SET_ATTR(16) HOM_SET_ATTR(32) HOM_SET_ATTR(64) HOM_SET_ATTR(96)
-        HOM_SET_ATTR(128) HOM_SET_ATTR(160) HOM_SET_ATTR(256) HOM_SET_ATTR(512)
-#define HOM_SET_TMA(NF)                   \
-    HOM_SET_ATTR1((k_x1_tma<R, NF>))      \
-    HOM_SET_ATTR1((k_x1_tma<R, NF, true>)) \
-    HOM_SET_ATTR1((k_x1_tma_expand<R, NF>))
-        HOM_SET_TMA(64) HOM_SET_TMA(96) HOM_SET_TMA(128) HOM_SET_TMA(160) HOM_SET_TMA(256) HOM_SET_TMA(512)
+        if (g.n3 == 256) {
+            HOM_SET_ATTR1((k_x3r<256, false>))
+            HOM_SET_ATTR1((k_x3r<256, true>))
+        }
+#undef HOM_SET_X1
+#undef HOM_SET_X2
+#undef HOM_SET_X3
 #undef HOM_SET_TMA
-        HOM_SET_ATTR1((k_x3r<256, false>))
-        HOM_SET_ATTR1((k_x3r<256, true>))
     }
-#undef HOM_SET_ATTR
 #undef HOM_SET_ATTR1
 }
 
@@ -1935,12 +1966,7 @@ void Launch<R>::x3(const Geometry &g, cudaStream_t st, int in_mode, const void *
         for (int c = 0; c < 6; ++c) m.v[c] = macro[c];
     const int grid = x3_grid(g) * g.nb;
     if constexpr (sizeof(R) == 8) {
-        F64X3Fn f = nullptr;
-#define HOM_X3(NF) f = g.nc == 10 ? k_x3<R, NF, 5> : k_x3<R, NF, 3>
-        if (g.line[2]) f = f64_x3_kernel(g.n3, g.nc / 2);
-        else if (g.ord[2]) f = f64_ord_x3_kernel(g.n3);
-        else HOM_F64_SWITCH(g.fast[2], HOM_X3)
-#undef HOM_X3
+        const F64X3Fn f = f64_x3_of<R>(g);
         if (g.nc == 10) epart = tsum = nullptr, fold = Fold{};
         launch_k(g.pdl, f, grid, g.threads3, g.smem3, st, g, in_mode, in, mid, lam, 2.0 * mu, m, scl, out_mode, out, phi,
                  state, epart, fold, tsum);
@@ -1973,12 +1999,7 @@ void Launch<R>::x2(const Geometry &g, cudaStream_t st, int inverse, cpx<R> *spec
     }
     const int grid = (g.n1 * g.nb * g.nc * g.h + g.tile2 - 1) / g.tile2;
     if constexpr (sizeof(R) == 8) {
-        F64X2Fn f = nullptr;
-#define HOM_X2(NF) f = inverse ? k_x2<R, 1, NF> : k_x2<R, -1, NF>
-        if (g.line[1]) f = f64_x2_kernel(g.n2, inverse);
-        else if (g.ord[1]) f = f64_ord_x2_kernel(g.n2, inverse);
-        else HOM_F64_SWITCH(g.fast[1], HOM_X2)
-#undef HOM_X2
+        const F64X2Fn f = f64_x2_of<R>(g, inverse);
         launch_k(g.pdl, f, grid, g.threads2, g.smem2, st, g, spec, state);
     } else {
 #define HOM_X2(NF)                                                                  \
@@ -2015,12 +2036,7 @@ void Launch<R>::x1(const Geometry &g, cudaStream_t st, int flags, const cpx<R> *
     }
     const int grid = (g.n2 * g.h + g.tile1 - 1) / g.tile1;
     if constexpr (sizeof(R) == 8) {
-        F64X1Fn f = nullptr;
-#define HOM_X1(NF) f = k_x1<R, NF>
-        if (g.line[0]) f = f64_x1_kernel(g.n1);
-        else if (g.ord[0]) f = f64_ord_x1_kernel(g.n1);
-        else HOM_F64_SWITCH(g.fast[0], HOM_X1)
-#undef HOM_X1
+        const F64X1Fn f = f64_x1_of<R>(g);
         f<<<grid, g.threads1, g.smem1, st>>>(g, flags, in, out, dotv, partials, state);
     } else {
 #define HOM_X1(NF) launch_k(g.pdl, k_x1<R, NF>, grid, g.threads1, g.smem1, st, g, flags, in, out, dotv, partials, state)
@@ -2112,11 +2128,7 @@ void Launch<R>::x1_lanczos(const Geometry &g, cudaStream_t st, cpx<R> *spec, con
     }
     const int grid = (g.n2 * g.h + g.tile1 - 1) / g.tile1 * g.nb;
     if constexpr (sizeof(R) == 8) {
-        F64X1lFn f = nullptr;
-#define HOM_X1L(NF) f = k_x1_lanczos<R, NF>
-        if (g.line[0]) f = f64_x1l_kernel(g.n1);
-        else HOM_F64_SWITCH(g.fast[0], HOM_X1L)
-#undef HOM_X1L
+        const F64X1lFn f = f64_x1l_of<R>(g);
         launch_k(g.pdl, f, grid, g.threads1, g.smem1, st, g, spec, uk, um, un, wa, wb, x, state, partials, fold);
     } else {
 #define HOM_X1L(NF) \

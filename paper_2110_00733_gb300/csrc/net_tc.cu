@@ -2,6 +2,10 @@
 // generation tensor cores: tcgen05.mma (kind::f16, BF16 operands, FP32
 // accumulator in tensor memory), issued by one thread, completion tracked on
 // mbarriers with tcgen05.commit, the result read back with tcgen05.ld.
+// Kernels: column marches for up to 80 output channels (k_conv3_col and the
+// weight gradient k_wgrad3_col), halo bricks for more (k_conv3_tcp, k_conv3_tcd,
+// k_conv3_tch), and for grids that bricks do not tile the gathering kernel
+// k_conv3_tc, described here.
 //
 // CTA tile: M = 128 output voxels x N = all output channels (<= 256, a
 // multiple of 16) x K = 27 taps x input channels, consumed 64 K at a time
