@@ -58,7 +58,7 @@
  *   - HOM_X1_L2PF=0 in the environment at hom_create turns off the L2
  *     prefetch of each tile's Lanczos blocks in the fused FP32 n1 pass.
  *   - HOM_FOLD_ALPHA=1 in the environment at the first solve folds the
- *     MINRES alpha reduction into the register n3 pass (one launch fewer
+ *     MINRES alpha reduction into the persistent n3 pass (one launch fewer
  *     per step; off by default).
  */
 #ifndef HOM_H
@@ -109,8 +109,9 @@ typedef struct {
     int tile2;          /* launch shape: n2-pass columns per CTA (0 = automatic; power of 2, <= 32) */
     int tile1;          /* launch shape: n1-pass columns per CTA (0 = automatic, <= 16) */
     int staging;        /* 0: persistent TMA-staged n1/n2 passes where supported
-                           (FP32, n1 and n2 in {64, 96, 128, 160, 256, 512});
-                           1: plain loads */
+                           (FP32: the n2 pass and the fused MINRES n1 pass at
+                           most lengths from 16 to 512, the unfused n1 pass at
+                           64, 96, 128, 160, 256 and 512); 1: plain loads */
     double alpha;       /* MoDBFFT penalty alpha / E (0: 1e-4, section 4.2) */
     int autotune;       /* nonzero (and no explicit rows3/tile2/tile1): launch
                            shapes from hom_autotune for this grid and precision */

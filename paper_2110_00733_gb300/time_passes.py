@@ -38,7 +38,8 @@ from paper_2110_00733_gb300 import hom  # noqa: E402
 def bytes_per_voxel(n3: int) -> dict:
     spec = 48.0 * (n3 // 2 + 1) / n3
     return {"x2_inv": 2 * spec, "x3_c2r_law_energy_r2c": 2 * spec + 4, "x2_fwd": 2 * spec,
-            "x1_fwd_lanczos_inv": (8 + 2 / 3) * spec}   # x read and written on one step in three
+            # the work spectrum and 6 2/3 vectors of three components: x read and written on one step in three
+            "x1_fwd_lanczos_inv": (2 + (6 + 2 / 3) / 2) * spec}
 
 
 def main():
@@ -85,7 +86,7 @@ def write_traffic(csv_path, shape):
     # each twice: warm-up, then --reps 1; the fused n1 pass four times, see
     # below); FP64 launches of context creation and the first inverse n1 pass
     # are skipped
-    patterns = {"x2_inv": ("k_x2_tma<float, 1,", "k_x2<float, 1,"), "x3_c2r_law_energy_r2c": ("k_x3r<", "k_x3<float"),
+    patterns = {"x2_inv": ("k_x2_tma<float, 1,", "k_x2<float, 1,"), "x3_c2r_law_energy_r2c": ("k_x3r<", "k_x3_line<", "k_x3<float"),
                 "x2_fwd": ("k_x2_tma<float, -1,", "k_x2_tma<float, (int)-1", "k_x2<float, -1,", "k_x2<float, (int)-1"),
                 "x1_fwd_lanczos_inv": ("k_x1_lanczos",)}
     firsts = []
@@ -124,7 +125,7 @@ def source_hash():
     import hashlib
     h = hashlib.sha256()
     cdir = os.path.join(ROOT, "paper_2110_00733_gb300", "csrc")
-    for fn in ("hom_fft.cuh", "hom_tma.cuh", "hom_passes.cuh", "hom_modb.cuh", "hom_internal.h",
+    for fn in ("hom_fft.cuh", "hom_tma.cuh", "hom_passes.cuh", "hom_lines.cuh", "hom_x3.cuh", "hom_modb.cuh", "hom_internal.h",
                "hom_kernels_f32.cu", "hom_kernels_f64.cu"):
         with open(os.path.join(cdir, fn), "rb") as f:
             h.update(fn.encode())
