@@ -400,9 +400,8 @@ template <> struct Six<double> {
 // Register cap of the pass kernels: FP32 kernels are held to 64 registers
 // (two 512-thread CTAs' worth per SM) so that more CTAs stay resident to hide
 // HBM latency; FP64 kernels keep their data in registers instead.
-#define HOM_PASS_BOUNDS(R) __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1)
-// the same, except for the register FFT lengths with more than 16 elements
-// per thread (160: 20), which keep their elements in registers instead
+// Except for the register FFT lengths with more than 16 elements per thread
+// (160: 20), which keep their elements in registers instead.
 #define HOM_PASS_BOUNDS_NF(R, NF) __launch_bounds__(512, (sizeof(R) == 4 && fast_elems(NF) <= 16) ? 2 : 1)
 // the n3 pass, by its own plan's elements per thread
 #define HOM_PASS_BOUNDS_N3(R, NF) __launch_bounds__(512, (sizeof(R) == 4 && fast_elems_n3(NF) <= 16) ? 2 : 1)
