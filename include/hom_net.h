@@ -103,7 +103,8 @@ int hom_net_conv3d(int batch, const int grid[3], const unsigned short *src0, int
                    int c1s, const unsigned short *W, const float *bias, int relu, int cout, void *out, int out_f32,
                    void *stream);
 /* dW[t][co][ci] = sum_v G[v][co] in[v + d_t][ci] (FP32 [27][cout][c0s+c1s]),
- * cout <= 64. */
+ * cout <= 64.  Both calls refuse an odd grid size with a second source, whose
+ * half-resolution grid has no voxel for the last plane. */
 int hom_net_conv3d_wgrad(int batch, const int grid[3], const unsigned short *G, int cout, const unsigned short *src0,
                          int c0s, const unsigned short *src1, int c1s, float *dW, void *stream);
 

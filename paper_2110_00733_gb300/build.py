@@ -20,7 +20,7 @@ SOURCES = ["hom_kernels_f32.cu", "hom_kernels_f64.cu", "hom_x1l_a.cu", "hom_x1l_
            "hom_f64_x2_a.cu", "hom_f64_x2_b.cu", "hom_f64_x2_c.cu", "hom_f64_x3_a.cu", "hom_f64_x3_b.cu", "hom_f64_x3_c.cu",
            "hom_f64_ord_a.cu", "hom_f64_ord_b.cu",
            "hom_x2_a.cu", "hom_x2_b.cu", "hom_x2_c.cu", "hom_x3_a.cu", "hom_x3_b.cu", "hom_x3_c.cu", "hom_common.cu", "hom_api.cu", "hom_noalloc.cu",
-           "hom_batch.cu", "hom_cg.cu", "hom_pfs.cu", "hom_j2.cu", "net_kernels.cu", "net.cu", "net_tc.cu"]
+           "hom_batch.cu", "hom_cg.cu", "hom_pfs.cu", "hom_j2.cu", "net.cu", "net_tc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 

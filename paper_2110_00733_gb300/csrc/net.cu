@@ -1,5 +1,5 @@
 // net.cu -- the warm-start network: point-wise kernels, the U-Net forward and
-// backward passes over the convolution kernels of net_kernels.cu, Adam, and
+// backward passes over the convolution kernels of net_tc.cu, Adam, and
 // the C ABI of hom_net.h.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -992,6 +992,8 @@ int hom_net_conv3d_wgrad(int batch, const int grid[3], const unsigned short *G, 
     w.in.c1s = c1s;
     w.G = reinterpret_cast<const bf16 *>(G);
     w.cout = cout;
+    if (!conv3_wgrad_takes(w))
+        return set_err(HOM_EINVAL, "channel counts must be multiples of 16, cout <= 64, and the grid even with a second source");
     const long long vox = (long long)batch * grid[0] * grid[1] * grid[2];
     const int cin_s = c0s + c1s;
     w.S = wgrad_splits(vox, cin_s, cout);
@@ -1004,7 +1006,7 @@ int hom_net_conv3d_wgrad(int batch, const int grid[3], const unsigned short *G, 
     w.partial = partial;
     if (conv3_wgrad(w, st)) {
         cudaFreeAsync(partial, st);
-        return set_err(HOM_EINVAL, "channel counts must be multiples of 16, cout <= 64");
+        return set_err(HOM_ENOMEM, "no error word for the kernel's bounded waits");
     }
     k_wgrad_reduce<<<(27 * cout * cin_s + kRedVals - 1) / kRedVals, kRedVals * kRedWays, 0, st>>>(w.S, cout, cin_s, cout, cin_s, partial, dW);
     cudaError_t e = cudaGetLastError();

@@ -39,7 +39,10 @@ struct WgradArgs {
 int conv3_forward_tc(const ConvArgs &a, cudaStream_t st);   // tcgen05, cout <= 256
 // nonzero if a tcgen05 convolution gave up a bounded wait (clears it if asked)
 int conv3_tc_error(int clear);
-int conv3_wgrad(const WgradArgs &a, cudaStream_t st);      // tcgen05, or mma.sync where that does not take the shape
-int conv3_wgrad_tc(const WgradArgs &a, cudaStream_t st);   // -1 if the shape does not suit it
+// whether the shape is one of the weight gradient's: channel counts multiples of
+// 16, 16 <= cout <= 64, and even grid sizes where there is a second source (its
+// half-resolution grid has no voxel for the last plane of an odd one)
+bool conv3_wgrad_takes(const WgradArgs &a);
+int conv3_wgrad(const WgradArgs &a, cudaStream_t st);   // tcgen05; -1 if not
 
 }  // namespace hnet

@@ -15,8 +15,8 @@
 // waits on it, issues the MMAs and commits to the stage's "empty" barrier,
 // which the producers wait on before reusing the stage.
 // Each K chunk is staged by cp.async (16-byte rows, the gathered input rows
-// with periodic wrap and the half-resolution second source as in the
-// mma.sync kernel) into the canonical no-swizzle K-major layout of the MMA:
+// with periodic wrap and the half-resolution second source) into the
+// canonical no-swizzle K-major layout of the MMA:
 // core matrices of 8 rows x 16 bytes, K-adjacent core matrices LBO = 128 B
 // apart, 8-row groups SBO = 1024 B apart.
 //
@@ -1537,31 +1537,34 @@ int conv3_forward_tc(const ConvArgs &in, cudaStream_t st) {
     return 0;
 }
 
-int conv3_wgrad_tc(const WgradArgs &in, cudaStream_t st) {
+bool conv3_wgrad_takes(const WgradArgs &w) {
+    const ConvArgs &a = w.in;
+    if ((w.cout & 15) || w.cout > 64 || w.cout < 16 || a.c0s < 0 || a.c1s < 0 || ((a.c0s | a.c1s) & 15)) return false;
+    if (a.c0s + a.c1s <= 0) return false;
+    return !(a.c1s && ((a.n1 | a.n2 | a.n3) & 1));
+}
+
+int conv3_wgrad(const WgradArgs &in, cudaStream_t st) {
     WgradArgs w = in;
     w.in.err = err_flag();
     const ConvArgs &a = w.in;
-    if (!a.err) return -1;
-    if ((w.cout & 15) || w.cout > 64 || w.cout < 16 || (a.c0s & 15) || (a.c1s & 15) || w.S <= 0) return -1;
-    if (!(a.c1s && ((a.n1 | a.n2 | a.n3) & 1))) {
-        static bool cattr = false;
-        if (!cattr) {
-            int dev = 0, lim = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-            cudaFuncSetAttribute(k_wgrad3_col, cudaFuncAttributeMaxDynamicSharedMemorySize, lim - 1024);
-            cudaFuncSetAttribute(k_wgrad3_col, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-            cattr = true;
-        }
-        const int nc = 256;   // 144 columns; two CTAs per SM by tensor and shared memory
-        const int zl = a.n1 < 8 ? a.n1 : 8;
-        size_t smem = (size_t)(kCSlots + kCGSlots) * kCPlane + kCPad;
-        const size_t floor = 233472 / (512 / nc + 1) + 1024;    // TMEM columns per SM stay <= 512
-        if (smem < floor) smem = floor;
-        k_wgrad3_col<<<dim3(w.S, (a.c0s + a.c1s) / 16, w.cout / 16), kThreads, smem, st>>>(w, nc, zl);
-        return 0;
+    if (!a.err || w.S <= 0 || !conv3_wgrad_takes(w)) return -1;
+    static bool cattr = false;
+    if (!cattr) {
+        int dev = 0, lim = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        cudaFuncSetAttribute(k_wgrad3_col, cudaFuncAttributeMaxDynamicSharedMemorySize, lim - 1024);
+        cudaFuncSetAttribute(k_wgrad3_col, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        cattr = true;
     }
-    return -1;
+    const int nc = 256;   // 144 columns; two CTAs per SM by tensor and shared memory
+    const int zl = a.n1 < 8 ? a.n1 : 8;
+    size_t smem = (size_t)(kCSlots + kCGSlots) * kCPlane + kCPad;
+    const size_t floor = 233472 / (512 / nc + 1) + 1024;    // TMEM columns per SM stay <= 512
+    if (smem < floor) smem = floor;
+    k_wgrad3_col<<<dim3(w.S, (a.c0s + a.c1s) / 16, w.cout / 16), kThreads, smem, st>>>(w, nc, zl);
+    return 0;
 }
 
 int conv3_tc_error(int clear) {
