@@ -113,7 +113,7 @@ __global__ void k_dc_start(MinresState *st, const float2 *rhs, int mask) {
     const int c = threadIdx.x;
     if (c >= 6) return;
     st->dc_u[c] = (mask >> c) & 1 ? (double)rhs[c].x : 0.0;
-    st->dc_tau[c] = st->dc_um[c] = st->dc_un[c] = st->dc_w1[c] = st->dc_w2[c] = st->dc_x[c] = 0.0;
+    st->dc_tau[c] = st->dc_um[c] = st->dc_un[c] = st->dc_w1[c] = st->dc_w2[c] = st->dc_x[c] = st->dc_keep[c] = 0.0;
     if (c == 0) st->dc = 1;
 }
 

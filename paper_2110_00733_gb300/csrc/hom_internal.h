@@ -61,7 +61,11 @@ struct MinresState {
     // restatement, 48^3 octet).  Six real components each (Mandel).
     int dc;
     double dc_tau[6], dc_u[6], dc_um[6], dc_un[6], dc_w1[6], dc_w2[6], dc_x[6];
+    double dc_keep[6];   // x there as of the FP32 vectors' last update of x
 };
+
+// the fused step updates x when the iterations done (the state's k) are a multiple of 3
+__host__ __device__ constexpr bool minres_xstep(int k) { return k > 0 && k % 3 == 0; }
 
 // the step's w and x at xi = 0, and u_{k+1} in u_k's place (one thread; ib =
 // 1 / beta_k, ig = 1 / gamma; the values are loaded together, one memory
@@ -126,7 +130,16 @@ __device__ __forceinline__ void givens_step(MinresState *st, double bn2) {
     const double cn = gbar / gamma, sn = beta_next / gamma;
     const double tau = cn * st->phibar;
     const double phibar = sn * st->phibar;
-    if (st->dc) dc_step(st, 1.0 / st->beta, delta, st->eps, 1.0 / gamma, tau);
+    const bool finite = isfinite(alpha) && isfinite(beta_next) && isfinite(phibar);
+    if (st->dc) {
+        // this step's n1 pass took x to the iterations done so far; a breakdown
+        // keeps the iterate of the last such pass, at xi = 0 as everywhere else
+        if (minres_xstep(st->k))
+            for (int i = 0; i < 6; ++i) st->dc_keep[i] = st->dc_x[i];
+        if (finite) dc_step(st, 1.0 / st->beta, delta, st->eps, 1.0 / gamma, tau);
+        else
+            for (int i = 0; i < 6; ++i) st->dc_x[i] = st->dc_keep[i];
+    }
     st->u_delta = delta;
     st->u_eps = st->eps;            // epsilon_k multiplies w_{k-2}
     st->u_inv_gamma = 1.0 / gamma;
@@ -143,7 +156,7 @@ __device__ __forceinline__ void givens_step(MinresState *st, double bn2) {
     st->beta = beta_next;
     st->k += 1;
     st->est = phibar / st->beta1;
-    if (!isfinite(alpha) || !isfinite(beta_next) || !isfinite(phibar)) {
+    if (!finite) {
         st->status = -5;
         st->done = 1;
         st->done_update = 1;        // keep the last finite iterate

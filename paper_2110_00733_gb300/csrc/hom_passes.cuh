@@ -1323,9 +1323,6 @@ template <typename R> struct LzCoef {
     bool dc;                 // the state carries xi = 0 in FP64
 };
 
-// x is updated when the iterations done (the state's k) are a multiple of 3
-__host__ __device__ constexpr bool minres_xstep(int k) { return k > 0 && k % 3 == 0; }
-
 template <typename R>
 __device__ __forceinline__ LzCoef<R> lz_coef(const MinresState *st) {
     LzCoef<R> c;
