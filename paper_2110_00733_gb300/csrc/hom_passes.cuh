@@ -23,6 +23,7 @@
 #include <type_traits>
 
 #include "hom_internal.h"
+#include "hom_warp.h"
 
 namespace hom {
 
@@ -65,11 +66,23 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// Sum over the block in a fixed order; the result is valid in thread 0.
+// the same over the first n lanes of a warp, which are all it has; valid in lane 0
+__device__ __forceinline__ double warp_sum(double v, int n) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double t = __shfl_xor_sync(0xffffffffu, v, o);
+        if (sum_takes(lane, o, n)) v += t;   // (what a lane that is not there holds is dropped)
+    }
+    return v;
+}
+
+// Sum over the block in a fixed order; the result is valid in thread 0.  (The
+// passes' blocks are not all whole warps: 6 t1 TPL or 3 rows TPL threads.)
 __device__ __forceinline__ double block_sum(double v) {
     __shared__ double red[32];
-    v = warp_sum(v);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    v = warp_sum(v, warp_lanes(blockDim.x, wid));
     __syncthreads();
     if (lane == 0) red[wid] = v;
     __syncthreads();
@@ -77,7 +90,7 @@ __device__ __forceinline__ double block_sum(double v) {
     if (wid == 0) {
         const int nw = (blockDim.x + 31) >> 5;
         r = (lane < nw) ? red[lane] : 0.0;
-        r = warp_sum(r);
+        r = warp_sum(r, warp_lanes(blockDim.x, 0));
     }
     return r;
 }
