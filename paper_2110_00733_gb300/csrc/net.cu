@@ -1013,5 +1013,5 @@ int hom_net_conv3d_wgrad(int batch, const int grid[3], const unsigned short *G, 
     cudaFreeAsync(partial, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return set_err(HOM_ECUDA, cudaGetErrorString(e));
-    return HOM_OK;
+    return tc_status();   // a wait given up leaves partial sums unwritten
 }

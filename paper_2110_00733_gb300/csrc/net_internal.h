@@ -37,6 +37,7 @@ struct WgradArgs {
 };
 
 int conv3_forward_tc(const ConvArgs &a, cudaStream_t st);   // tcgen05, cout <= 256
+int *conv3_tc_error_word();   // the word such a wait sets (null: it could not be allocated)
 // nonzero if a tcgen05 convolution gave up a bounded wait (clears it if asked)
 int conv3_tc_error(int clear);
 // whether the shape is one of the weight gradient's: channel counts multiples of

@@ -1408,7 +1408,7 @@ __global__ void __launch_bounds__(kThreads) k_wgrad3_col(WgradArgs w, int ncols,
 // The word a kernel sets when a bounded wait gives up: host memory mapped for
 // every device, so that reading it after a call costs no copy (the copy from a
 // device symbol took about 10 us of every call).
-static int *err_flag() {
+int *conv3_tc_error_word() {
     static int *f = nullptr;
     static std::once_flag once;
     std::call_once(once, [] {
@@ -1423,7 +1423,7 @@ static int *err_flag() {
 
 int conv3_forward_tc(const ConvArgs &in, cudaStream_t st) {
     ConvArgs a = in;
-    a.err = err_flag();
+    a.err = conv3_tc_error_word();
     if (!a.err) return -1;
     if ((a.cout & 15) || a.cout > 256 || a.cout < 16 || (a.c0s & 15) || (a.c1s & 15) || a.c0s <= 0) return -1;
     if (a.c1s && (!a.src1 || (a.n1 | a.n2 | a.n3) & 1)) return -1;
@@ -1546,7 +1546,7 @@ bool conv3_wgrad_takes(const WgradArgs &w) {
 
 int conv3_wgrad(const WgradArgs &in, cudaStream_t st) {
     WgradArgs w = in;
-    w.in.err = err_flag();
+    w.in.err = conv3_tc_error_word();
     const ConvArgs &a = w.in;
     if (!a.err || w.S <= 0 || !conv3_wgrad_takes(w)) return -1;
     static bool cattr = false;
@@ -1568,7 +1568,7 @@ int conv3_wgrad(const WgradArgs &in, cudaStream_t st) {
 }
 
 int conv3_tc_error(int clear) {
-    int *f = err_flag();
+    int *f = conv3_tc_error_word();
     const int e = f ? *reinterpret_cast<volatile int *>(f) : 0;
     if (clear && e) *reinterpret_cast<volatile int *>(f) = 0;
     return e;
