@@ -1332,8 +1332,9 @@ __global__ void __launch_bounds__(kThreads) k_wgrad3_col(WgradArgs w, int ncols,
             const int x0 = (int)(r % tx) * kPX; r /= tx;
             const int y0 = (int)(r % ty) * kPY;
             const int b = (int)(r / ty);
-            // X row y of copy dx: X[y][x + dx]; G row y of copy dy: G[y - dy][x], zero
-            // for y or x beyond the grid (each X row, each G column counts once)
+            // X row y of copy dx: X[y][x + dx]; G row y of copy dy: G[y - dy][x]; both zero
+            // for y or x beyond the grid (each X row, each G column counts once, and
+            // an infinite X or G there must not meet the other's zero)
             uint32_t live = 0;
 #pragma unroll
             for (int m = 0; m < kMine; ++m) {
@@ -1354,7 +1355,7 @@ __global__ void __launch_bounds__(kThreads) k_wgrad3_col(WgradArgs w, int ncols,
                 if (++zz == a.n1) zz = 0;
                 const uint32_t st = saddr(xs) + q * kCPlane;
 #pragma unroll
-                for (int m = 0; m < kMine; ++m) cp_async16(st + dst[m], src + off[m], 16);
+                for (int m = 0; m < kMine; ++m) cp_async16(st + dst[m], src + off[m], (live >> m) & 1 ? 16 : 0);
                 if (i < nz) {   // G plane i (its slot's last reader is no later than the X slot's)
                     const uint32_t gd = saddr(gs) + gq * kCPlane;
 #pragma unroll
