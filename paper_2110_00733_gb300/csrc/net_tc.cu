@@ -75,6 +75,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
     return false;
 }
 
+// The outcome of a wait that every lane of a warp made, the same in all: lanes that
+// part after a time-out would meet neither at the collectives that follow a wait
+// (tcgen05.ld, __syncwarp) nor, those that stay behind at one, at the block's end.
+__device__ __forceinline__ bool warp_agrees(bool ok) { return __all_sync(0xffffffffu, ok); }
+
 // shared-memory matrix descriptor: start >> 4, LBO >> 4, SBO >> 4, version 1
 // (bit 46), no swizzle
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
@@ -217,7 +222,7 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tc(ConvArgs a, int ncols) {
         for (int c = 0; c < nk + kStages - 2 && ok; ++c) {
             if (c < nk) {
                 const int s = c % kStages;
-                if (c >= kStages) ok = mbar_wait(&empty[s], (uint32_t)(c / kStages - 1) & 1u) && !abort_flag;
+                if (c >= kStages) ok = warp_agrees(mbar_wait(&empty[s], (uint32_t)(c / kStages - 1) & 1u) && !abort_flag);
                 if (!ok) break;
                 unsigned char *base = smem + s * stage_bytes;
                 const uint32_t ab = saddr(base), bb = saddr(base + a_bytes);
@@ -250,7 +255,7 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tc(ConvArgs a, int ncols) {
         cp_async_wait<0>();
         if (!ok) abort_flag = 1;
         // ---- epilogue: all MMAs done -> TMEM -> bias, ReLU -> global
-        if (ok) ok = mbar_wait(&done, 0u) && !abort_flag;
+        ok = warp_agrees(ok && mbar_wait(&done, 0u) && !abort_flag);
         if (ok) {
             tc_fence_after();
             const long long m = m0 + tid;
@@ -421,7 +426,7 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tch(ConvArgs a, int ncols) {
             for (int t = 0; t < 27; ++t, ++stage) {
                 if (!ok) continue;
                 const int q = stage % kHSt;
-                if (stage >= kHSt) ok = mbar_wait(&empty[q], (uint32_t)(stage / kHSt - 1) & 1u) && !abort_flag;
+                if (stage >= kHSt) ok = warp_agrees(mbar_wait(&empty[q], (uint32_t)(stage / kHSt - 1) & 1u) && !abort_flag);
                 if (!ok) continue;
                 unsigned char *base = ring + q * stage_bytes;
                 // A: my row's 16 channels at the tap's halo position
@@ -446,7 +451,7 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tch(ConvArgs a, int ncols) {
         asm volatile("cp.async.wait_all;" ::: "memory");
         if (ok) arrive_upto(nst);
         if (!ok) abort_flag = 1;
-        if (ok) ok = mbar_wait(&done, 0u) && !abort_flag;
+        ok = warp_agrees(ok && mbar_wait(&done, 0u) && !abort_flag);
         if (ok) {
             tc_fence_after();
             const long long m = (((long long)b * a.n1 + z0 + bz) * a.n2 + y0 + by) * a.n3 + x0 + bx;
@@ -608,7 +613,7 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tcd(ConvArgs a, int ncols, i
         for (int cc = 0; cc < nch; ++cc) {
             const int q = cc % ring;
             if (!ok) continue;
-            if (cc >= ring) ok = mbar_wait(&empty[q], (uint32_t)(cc / ring - 1) & 1u) && !abort_flag;
+            if (cc >= ring) ok = warp_agrees(mbar_wait(&empty[q], (uint32_t)(cc / ring - 1) & 1u) && !abort_flag);
             if (!ok) continue;
             unsigned char *st = smem + q * stage_bytes;
             const bool first = cc * 16 < a.c0s;
@@ -634,7 +639,7 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tcd(ConvArgs a, int ncols, i
             asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(&full[q])) : "memory");
         }
         if (!ok) abort_flag = 1;
-        if (ok) ok = mbar_wait(&done, 0u) && !abort_flag;
+        ok = warp_agrees(ok && mbar_wait(&done, 0u) && !abort_flag);
         if (ok) {
             tc_fence_after();
             const int bz = tid >> 5, by = (tid >> 3) & 3, bx = tid & 7;
@@ -781,7 +786,7 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tcp(ConvArgs a, int ncols) {
         int pb = 0, pz0 = 0, py0 = 0, px0 = 0;              // the previous brick, for its epilogue
         auto epilogue = [&](int j) {                        // brick j's accumulator to the output
             const int s = j & 1;
-            ok = mbar_wait(&afull[s], (uint32_t)(j >> 1) & 1u) && !abort_flag;
+            ok = warp_agrees(mbar_wait(&afull[s], (uint32_t)(j >> 1) & 1u) && !abort_flag);
             if (!ok) return;
             tc_fence_after();
             const long long m = (((long long)pb * a.n1 + pz0 + bz) * a.n2 + py0 + by) * a.n3 + px0 + bx;
@@ -826,7 +831,7 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tcp(ConvArgs a, int ncols) {
             const __nv_bfloat16 *s1 = a.c1s ? a.src1 + (long long)b * h1 * h2 * h3 * a.c1s : nullptr;
             for (int cc = 0; cc < nch && ok; ++cc) {
                 const int k = j * nch + cc, q = k & 1;
-                if (k >= 2) ok = mbar_wait(&hempty[q], (uint32_t)((k >> 1) - 1) & 1u) && !abort_flag;
+                if (k >= 2) ok = warp_agrees(mbar_wait(&hempty[q], (uint32_t)((k >> 1) - 1) & 1u) && !abort_flag);
                 if (!ok) break;
                 unsigned char *st = halo + q * kDHalo;
                 const bool first = cc * 16 < a.c0s;
@@ -1065,7 +1070,7 @@ __global__ void __launch_bounds__(kColThreads) k_conv3_col(ConvArgs a, int ncols
                         while (sent < need) arrive();
                     }
                     if (c >= wslots)
-                        ok = mbar_wait(&wempty[c % wslots], (uint32_t)(c / wslots - 1) & 1u) && !abort_flag;
+                        ok = warp_agrees(mbar_wait(&wempty[c % wslots], (uint32_t)(c / wslots - 1) & 1u) && !abort_flag);
                     if (!ok) break;
                     load_weights(cc, c % wslots);
                 }
@@ -1076,7 +1081,7 @@ __global__ void __launch_bounds__(kColThreads) k_conv3_col(ConvArgs a, int ncols
                 const long long pstride = first ? (long long)a.n2 * a.n3 * a.c0s : (long long)h2 * h3 * a.c1s;
                 int zz = zfirst;
                 for (int i = 0; i < P; ++i, ++k) {
-                    if (k >= nplanes) ok = mbar_wait(&empty[q], ph) && !abort_flag;
+                    if (k >= nplanes) ok = warp_agrees(mbar_wait(&empty[q], ph) && !abort_flag);
                     if (!ok) break;
                     const __nv_bfloat16 *src = sc + (first ? zz : zz >> 1) * pstride;
                     if (++zz == a.n1) zz = 0;
@@ -1117,7 +1122,7 @@ __global__ void __launch_bounds__(kColThreads) k_conv3_col(ConvArgs a, int ncols
         for (int it = blockIdx.x; it < items && ok; it += gridDim.x, ++n) {
             int x0, y0, z0, b;
             const int nz = decode(it, x0, y0, z0, b);
-            ok = mbar_wait(&afull[n & 1], (uint32_t)(n >> 1) & 1u) && !abort_flag;
+            ok = warp_agrees(mbar_wait(&afull[n & 1], (uint32_t)(n >> 1) & 1u) && !abort_flag);
             if (!ok) break;
             tc_fence_after();
             const int y = y0 + (e >> 3), x = x0 + (e & 7);
@@ -1349,7 +1354,7 @@ __global__ void __launch_bounds__(kThreads) k_wgrad3_col(WgradArgs w, int ncols,
             const __nv_bfloat16 *g = w.G + ((long long)b * a.n1 + z0) * gstride;
             int zz = wrapm(z0 - 1, a.n1);
             for (int i = 0; i < nz + 2; ++i, ++k) {
-                if (k >= kCSlots) ok = mbar_wait(&empty[q], ph) && !abort_flag;
+                if (k >= kCSlots) ok = warp_agrees(mbar_wait(&empty[q], ph) && !abort_flag);
                 if (!ok) break;
                 const __nv_bfloat16 *src = src_b + (zz >> sh) * pstride;
                 if (++zz == a.n1) zz = 0;
@@ -1378,7 +1383,7 @@ __global__ void __launch_bounds__(kThreads) k_wgrad3_col(WgradArgs w, int ncols,
         if (ok)
             while (sent < k) arrive();
         if (!ok) abort_flag = 1;
-        if (ok) ok = mbar_wait(&done, 0u) && !abort_flag;
+        ok = warp_agrees(ok && mbar_wait(&done, 0u) && !abort_flag);
         if (ok) {
             tc_fence_after();
             // M = 64: rows 16 w .. 16 w + 15 in lanes 0..15 of warp w's quarter; warp w holds dx = w
