@@ -1197,6 +1197,7 @@ constexpr int kCHalf = kPY * kPX * 16;              // 2048 B: 8 channels of one
 constexpr int kCPlane = 6 * kCHalf;                 // three copies of 16 channels (X: dx, G: dy)
 constexpr int kCSlots = 3, kCGSlots = 6, kCDepth = 2;   // X planes, G planes (each read for three stages), loads in flight
 constexpr int kCPad = 2 * kCHalf;                   // rows 48..63 of A read past the last X slot
+constexpr int kCRun = 4;                            // items whose products an accumulator takes at least
 constexpr int kCTaps = 48;                          // columns of one G plane: dy, 16 output channels
 
 __device__ __forceinline__ uint64_t smem_desc_c(uint32_t addr) {   // MN-major: LBO along K, SBO along MN
@@ -1208,9 +1209,18 @@ __device__ __forceinline__ uint32_t instr_desc_c(int n) {   // M = 64, both oper
 }
 
 // zl: planes of a work item; blockIdx = (split, input chunk, 16 output channels)
-__global__ void __launch_bounds__(kThreads) k_wgrad3_col(WgradArgs w, int ncols, int zl) {
+// The tensor core adds to its FP32 accumulators with about 2^-24 of them lost each
+// time, in one direction, so that a sum over many voxels is off in proportion to
+// their number (64 -> 64 channels, 64^3 x 8: 19 splits of 110 k voxels 1.2e-4 off the
+// FP64 gradient).  So a CTA works through its split in runs of at most `run` items,
+// starts the accumulators afresh in each and adds the runs up in FP32 arithmetic in
+// its partial sums (7e-6; the first run is stored).  That takes 1853 us there against
+// 1774 in one run, and more splits instead, of as few voxels, 2465.  Splits that are
+// one run anyway (RUNS false) do without: 143 us against 149 at 16 -> 16 channels.
+template <bool RUNS>
+__global__ void __launch_bounds__(kThreads, 2) k_wgrad3_col(WgradArgs w, int ncols, int zl, int run) {
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ __align__(8) uint64_t full[kCSlots], empty[kCSlots], done;
+    __shared__ __align__(8) uint64_t full[kCSlots], empty[kCSlots], done, taken;   // done, taken: once a run
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int abort_flag;
     const ConvArgs &a = w.in;
@@ -1228,6 +1238,8 @@ __global__ void __launch_bounds__(kThreads) k_wgrad3_col(WgradArgs w, int ncols,
         }
         return;
     }
+    // runs of a split, alike: their number and items
+    const int n = (int)(it1 - it0), nruns = RUNS ? (n + run - 1) / run : 1, per = RUNS ? (n + nruns - 1) / nruns : n;
     auto item_z = [&](long long it) { return (int)(it % tz) * zl; };   // z fastest: neighbours share halo planes
     auto item_nz = [&](long long it) { return a.n1 - item_z(it) < zl ? a.n1 - item_z(it) : zl; };
 
@@ -1243,6 +1255,7 @@ __global__ void __launch_bounds__(kThreads) k_wgrad3_col(WgradArgs w, int ncols,
             mbar_init(&empty[q], 1);
         }
         mbar_init(&done, 1);
+        mbar_init(&taken, kProducers / 32);
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -1260,14 +1273,24 @@ __global__ void __launch_bounds__(kThreads) k_wgrad3_col(WgradArgs w, int ncols,
             bool ok = true;
             int k = 0, q = 0, g0 = 0;   // stage, its slot, ring slot of the item's G plane 0
             uint32_t ph = 0;
+            int left = per, r = 0;      // items left of the run, runs done
             for (long long it = it0; it < it1 && ok; ++it) {
                 const int nz = item_nz(it);
+                if (RUNS && left == 0) {   // the next run: its accumulators once this one's are read
+                    mma_commit(&done);
+                    ok = mbar_wait(&taken, (uint32_t)r & 1u) && !abort_flag;
+                    if (!ok) break;
+                    tc_fence_after();
+                    left = per;
+                    ++r;
+                }
+                const bool starts = RUNS ? left-- == per : it == it0;
                 for (int i = 0; i < nz + 2; ++i, ++k) {   // X plane z0 - 1 + i meets G planes i - 2 + j
                     ok = mbar_wait(&full[q], ph) && !abort_flag;
                     if (!ok) break;
                     tc_fence_after();
                     const int j0 = i < 2 ? 2 - i : 0, j1 = nz + 1 - i < 2 ? nz + 1 - i : 2;
-                    const bool fresh = it == it0 && i <= 2;   // block j0 starts its accumulators
+                    const bool fresh = starts && i <= 2;   // block j0 starts its accumulators
                     const int s0 = (g0 + i - 2 + j0) % kCGSlots, left = kCGSlots - s0;   // planes before the ring wraps
                     const int ja = j1 - j0 + 1 > left ? j0 + left - 1 : j1;              // last block of the first run
                     const uint64_t ad = smem_desc_c(saddr(xs + q * kCPlane));
@@ -1330,8 +1353,51 @@ __global__ void __launch_bounds__(kThreads) k_wgrad3_col(WgradArgs w, int ncols,
             ++sent;
             if (++qs == kCSlots) qs = 0;
         };
+        // the run's accumulators: M = 64, rows 16 w .. 16 w + 15 in lanes 0..15 of warp
+        // w's quarter; warp w holds dx = w
+        float *const out = w.partial + (((long long)split * 27 + (warp < 3 ? warp : 0)) * w.cout + co0) * cin_s + cc * 16 + (lane & 15);
+        const long long tstride = (long long)w.cout * cin_s;
+        auto take = [&](bool add) {
+            const bool mine = warp < 3 && lane < 16;
+            auto at = [&](int jd) { return out + ((2 - jd / 3) * 9 + jd % 3 * 3) * tstride; };   // (dz block, dy copy)
+            float sum[16];   // of the runs before, a copy ahead
+            auto fetch = [&](int jd) {
+#pragma unroll
+                for (int i = 0; i < 16; ++i) sum[i] = at(jd)[(long long)i * cin_s];
+            };
+            if (add && mine) fetch(0);
+#pragma unroll 1
+            for (int jd = 0; jd < 9; ++jd) {
+                float v[16];
+                __syncwarp();
+                tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(jd * 16), v);
+                if (mine) {
+                    if (add) {
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) v[i] += sum[i];
+                        if (jd < 8) fetch(jd + 1);
+                    }
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) at(jd)[(long long)i * cin_s] = v[i];
+                }
+            }
+        };
         const long long pstride = (long long)m2 * m3 * cs, gstride = (long long)a.n2 * a.n3 * w.cout;
-        for (long long it = it0; it < it1 && ok; ++it) {
+        int left = per, nr = 0;   // items left of the run, runs done
+        for (long long it = it0; it < it1 && ok; ++it, --left) {
+            if (RUNS && left == 0) {   // the run before is loaded: hand it over, and take its sums
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                while (sent < k) arrive();
+                ok = warp_agrees(mbar_wait(&done, (uint32_t)nr & 1u) && !abort_flag);
+                if (!ok) break;
+                tc_fence_after();
+                take(nr > 0);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(&taken)) : "memory");
+                left = per;
+                ++nr;
+            }
             const int z0 = item_z(it), nz = item_nz(it);
             long long r = it / tz;
             const int x0 = (int)(r % tx) * kPX; r /= tx;
@@ -1383,22 +1449,10 @@ __global__ void __launch_bounds__(kThreads) k_wgrad3_col(WgradArgs w, int ncols,
         if (ok)
             while (sent < k) arrive();
         if (!ok) abort_flag = 1;
-        ok = warp_agrees(ok && mbar_wait(&done, 0u) && !abort_flag);
+        ok = warp_agrees(ok && mbar_wait(&done, (uint32_t)(nruns - 1) & 1u) && !abort_flag);
         if (ok) {
             tc_fence_after();
-            // M = 64: rows 16 w .. 16 w + 15 in lanes 0..15 of warp w's quarter; warp w holds dx = w
-#pragma unroll 1
-            for (int jd = 0; jd < 9; ++jd) {   // (dz block j, dy copy)
-                float v[16];
-                __syncwarp();
-                tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(jd * 16), v);
-                if (warp < 3 && lane < 16) {
-                    const int j = jd / 3, t = (2 - j) * 9 + (jd - 3 * j) * 3 + warp;
-                    float *o = w.partial + (((long long)split * 27 + t) * w.cout + co0) * cin_s + cc * 16 + lane;
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) o[(long long)i * cin_s] = v[i];
-                }
-            }
+            take(nruns > 1);
         } else if (tid == 0) {
             atomicExch(a.err, 1);
         }
@@ -1560,8 +1614,10 @@ int conv3_wgrad(const WgradArgs &in, cudaStream_t st) {
         int dev = 0, lim = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        cudaFuncSetAttribute(k_wgrad3_col, cudaFuncAttributeMaxDynamicSharedMemorySize, lim - 1024);
-        cudaFuncSetAttribute(k_wgrad3_col, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        for (auto k : {k_wgrad3_col<false>, k_wgrad3_col<true>}) {
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lim - 1024);
+            cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        }
         cattr = true;
     }
     const int nc = 256;   // 144 columns; two CTAs per SM by tensor and shared memory
@@ -1569,7 +1625,12 @@ int conv3_wgrad(const WgradArgs &in, cudaStream_t st) {
     size_t smem = (size_t)(kCSlots + kCGSlots) * kCPlane + kCPad;
     const size_t floor = 233472 / (512 / nc + 1) + 1024;    // TMEM columns per SM stay <= 512
     if (smem < floor) smem = floor;
-    k_wgrad3_col<<<dim3(w.S, (a.c0s + a.c1s) / 16, w.cout / 16), kThreads, smem, st>>>(w, nc, zl);
+    // four items of 1024 voxels, or 1/256 of all voxels where that is more
+    const long long vox = (long long)a.B * a.n1 * a.n2 * a.n3, per256 = vox / (256 * 1024);
+    const int run = (int)(per256 < kCRun ? kCRun : (per256 > 1 << 20 ? 1 << 20 : per256));
+    const long long items = (long long)((a.n3 + kPX - 1) / kPX) * ((a.n2 + kPY - 1) / kPY) * ((a.n1 + zl - 1) / zl) * a.B;
+    const auto k = (items + w.S - 1) / w.S > run ? k_wgrad3_col<true> : k_wgrad3_col<false>;
+    k<<<dim3(w.S, (a.c0s + a.c1s) / 16, w.cout / 16), kThreads, smem, st>>>(w, nc, zl, run);
     return 0;
 }
 
