@@ -9,13 +9,13 @@
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
-#include <mutex>
 #include <string>
 #include <vector>
 
 #include "../../include/hom.h"
 #include "../../include/hom_net.h"
 #include "net_internal.h"
+#include "per_device.h"
 
 using namespace hnet;
 using bf16 = __nv_bfloat16;
@@ -27,6 +27,13 @@ thread_local std::string g_err;
 int set_err(int code, const std::string &msg) {
     g_err = msg;
     return code;
+}
+
+// of a convolution launcher's result (see net_internal.h)
+int launch_err(int rc, const char *shape) {
+    if (rc == 0) return HOM_OK;
+    return rc == -2 ? set_err(HOM_ENOMEM, "no host memory mapped for the error word of the kernels' bounded waits")
+                    : set_err(HOM_EINVAL, shape);
 }
 
 #define NCU(call)                                                                        \
@@ -440,22 +447,20 @@ long long level_vox(const hom_net *n, int B, const int g[3], int level) {
 // a call does not pay for cudaMalloc and cudaFree (about 150 us together); it
 // keeps at most 64 MB between calls.
 cudaMemPool_t scratch_pool() {
-    constexpr int kDevices = 64;
-    static cudaMemPool_t pools[kDevices] = {};
-    static std::mutex m;
+    static PerDevice<cudaMemPool_t> pools;
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev >= kDevices) return nullptr;
-    std::lock_guard<std::mutex> lock(m);
-    if (!pools[dev]) {
+    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    cudaMemPool_t *p = pools.get(dev, [dev](cudaMemPool_t &pool) {
         cudaMemPoolProps pp = {};
         pp.allocType = cudaMemAllocationTypePinned;
         pp.location.type = cudaMemLocationTypeDevice;
         pp.location.id = dev;
-        if (cudaMemPoolCreate(&pools[dev], &pp) != cudaSuccess) return pools[dev] = nullptr;
+        if (cudaMemPoolCreate(&pool, &pp) != cudaSuccess) return false;
         uint64_t keep = 64ull << 20;
-        cudaMemPoolSetAttribute(pools[dev], cudaMemPoolAttrReleaseThreshold, &keep);
-    }
-    return pools[dev];
+        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        return true;
+    });
+    return p ? *p : nullptr;
 }
 
 // Voxel splits of a weight gradient: about one wave of two CTAs per SM over the
@@ -564,7 +569,7 @@ ConvArgs layer_args(hom_net *n, int l, int B, const int g[3]) {
 }
 
 int run_conv(hom_net *n, const ConvArgs &a) {
-    if (conv3_forward_tc(a, n->stream)) return set_err(HOM_EINVAL, "convolution shape not supported");
+    if (int rc = launch_err(conv3_forward_tc(a, n->stream), "convolution shape not supported")) return rc;
     ++n->launches;
     return HOM_OK;
 }
@@ -630,7 +635,7 @@ int layer_back(hom_net *n, int l, int B, const int g[3]) {
     w.cout = L.cout_p;
     w.partial = n->partial;
     w.S = wgrad_splits(vox, L.cin_s, L.cout_p);
-    if (conv3_wgrad(w, n->stream)) return set_err(HOM_EINVAL, "weight-gradient shape not supported");
+    if (int rc = launch_err(conv3_wgrad(w, n->stream), "weight-gradient shape not supported")) return rc;
     k_wgrad_reduce<<<(27 * L.d.cout * L.d.cin + kRedVals - 1) / kRedVals, kRedVals * kRedWays, 0, n->stream>>>(
         w.S, L.cout_p, L.cin_s, L.d.cout, L.d.cin, n->partial, n->grads + L.off);
     const int nb = ew_blocks(vox);
@@ -970,8 +975,8 @@ int hom_net_conv3d(int batch, const int grid[3], const unsigned short *src0, int
     if (out_f32) a.out_f32 = static_cast<float *>(out);
     else a.out_bf16 = static_cast<bf16 *>(out);
     if (grid[0] <= 0 || grid[1] <= 0 || grid[2] <= 0) return set_err(HOM_EUNSUPPORTED_GRID, "empty grid");
-    if (conv3_forward_tc(a, (cudaStream_t)stream))
-        return set_err(HOM_EINVAL, "channel counts must be multiples of 16 (cout <= 256)");
+    if (int rc = launch_err(conv3_forward_tc(a, (cudaStream_t)stream), "channel counts must be multiples of 16 (cout <= 256)"))
+        return rc;
     NCU(cudaGetLastError());
     NCU(cudaStreamSynchronize((cudaStream_t)stream));
     return tc_status();
@@ -1001,12 +1006,14 @@ int hom_net_conv3d_wgrad(int batch, const int grid[3], const unsigned short *G, 
     cudaStream_t st = (cudaStream_t)stream;
     cudaMemPool_t pool = scratch_pool();
     const size_t bytes = sizeof(float) * w.S * 27 * cout * cin_s;
-    if (!pool || cudaMallocFromPoolAsync((void **)&partial, bytes, pool, st) != cudaSuccess)
+    if (!pool || cudaMallocFromPoolAsync((void **)&partial, bytes, pool, st) != cudaSuccess) {
+        cudaGetLastError();   // (not for a later call to find)
         return set_err(HOM_ENOMEM, "device allocation failed");
+    }
     w.partial = partial;
-    if (conv3_wgrad(w, st)) {
+    if (int rc = launch_err(conv3_wgrad(w, st), "weight-gradient shape not supported")) {
         cudaFreeAsync(partial, st);
-        return set_err(HOM_ENOMEM, "no error word for the kernel's bounded waits");
+        return rc;
     }
     k_wgrad_reduce<<<(27 * cout * cin_s + kRedVals - 1) / kRedVals, kRedVals * kRedWays, 0, st>>>(w.S, cout, cin_s, cout, cin_s, partial, dW);
     cudaError_t e = cudaGetLastError();

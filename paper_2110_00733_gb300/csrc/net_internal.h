@@ -36,14 +36,18 @@ struct WgradArgs {
     int S;
 };
 
+// the launchers return -1 for a shape that they do not take, -2 without an error word
 int conv3_forward_tc(const ConvArgs &a, cudaStream_t st);   // tcgen05, cout <= 256
-int *conv3_tc_error_word();   // the word such a wait sets (null: it could not be allocated)
-// nonzero if a tcgen05 convolution gave up a bounded wait (clears it if asked)
+// the word of the current device, or of another, that a bounded wait of a tcgen05
+// convolution sets as it gives up (null: it could not be allocated)
+int *conv3_tc_error_word();
+int *conv3_tc_error_word_of(int dev);
+// nonzero if one did on the current device (clears it if asked)
 int conv3_tc_error(int clear);
 // whether the shape is one of the weight gradient's: channel counts multiples of
 // 16, 16 <= cout <= 64, and even grid sizes where there is a second source (its
 // half-resolution grid has no voxel for the last plane of an odd one)
 bool conv3_wgrad_takes(const WgradArgs &a);
-int conv3_wgrad(const WgradArgs &a, cudaStream_t st);   // tcgen05; -1 if not
+int conv3_wgrad(const WgradArgs &a, cudaStream_t st);   // tcgen05
 
 }  // namespace hnet

@@ -27,9 +27,9 @@
 #include <stdint.h>
 
 #include <initializer_list>
-#include <mutex>
 
 #include "net_internal.h"
+#include "per_device.h"
 
 namespace hnet {
 
@@ -1465,28 +1465,39 @@ __global__ void __launch_bounds__(kThreads, 2) k_wgrad3_col(WgradArgs w, int nco
 
 }  // namespace
 
-// The word a kernel sets when a bounded wait gives up: host memory mapped for
-// every device, so that reading it after a call costs no copy (the copy from a
-// device symbol took about 10 us of every call).
-int *conv3_tc_error_word() {
-    static int *f = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void *p = nullptr;
-        if (cudaHostAlloc(&p, sizeof(int), cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess) {
-            f = static_cast<int *>(p);
-            *f = 0;
+// The word a kernel sets when a bounded wait gives up, one per device: host memory
+// that the device maps, so that reading it after a call costs no copy (the copy
+// from a device symbol took about 10 us of every call).
+int *conv3_tc_error_word_of(int dev) {
+    static PerDevice<int *> words;
+    int **w = words.get(dev, [](int *&p) {
+        void *q = nullptr;
+        if (cudaHostAlloc(&q, sizeof(int), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+            cudaGetLastError();   // (not for a later call to find)
+            return false;
         }
+        p = static_cast<int *>(q);
+        *p = 0;
+        return true;
     });
-    return f;
+    return w ? *w : nullptr;
+}
+
+int *conv3_tc_error_word() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return conv3_tc_error_word_of(dev);
 }
 
 int conv3_forward_tc(const ConvArgs &in, cudaStream_t st) {
     ConvArgs a = in;
-    a.err = conv3_tc_error_word();
-    if (!a.err) return -1;
     if ((a.cout & 15) || a.cout > 256 || a.cout < 16 || (a.c0s & 15) || (a.c1s & 15) || a.c0s <= 0) return -1;
     if (a.c1s && (!a.src1 || (a.n1 | a.n2 | a.n3) & 1)) return -1;
+    a.err = conv3_tc_error_word();
+    if (!a.err) return -2;
     int ncols = 32;
     while (ncols < a.cout) ncols <<= 1;
     static bool attr = false;
@@ -1608,7 +1619,8 @@ int conv3_wgrad(const WgradArgs &in, cudaStream_t st) {
     WgradArgs w = in;
     w.in.err = conv3_tc_error_word();
     const ConvArgs &a = w.in;
-    if (!a.err || w.S <= 0 || !conv3_wgrad_takes(w)) return -1;
+    if (w.S <= 0 || !conv3_wgrad_takes(w)) return -1;
+    if (!a.err) return -2;
     static bool cattr = false;
     if (!cattr) {
         int dev = 0, lim = 0;
@@ -1636,9 +1648,8 @@ int conv3_wgrad(const WgradArgs &in, cudaStream_t st) {
 
 int conv3_tc_error(int clear) {
     int *f = conv3_tc_error_word();
-    const int e = f ? *reinterpret_cast<volatile int *>(f) : 0;
-    if (clear && e) *reinterpret_cast<volatile int *>(f) = 0;
-    return e;
+    if (!f) return 0;
+    return clear ? __atomic_exchange_n(f, 0, __ATOMIC_ACQ_REL) : __atomic_load_n(f, __ATOMIC_ACQUIRE);
 }
 
 }  // namespace hnet

@@ -38,3 +38,18 @@ def test_the_call_reports_its_timeout(env, name):
     assert e.value.code == hom.HOM_ETIMEOUT
     assert word()[0] == 0
     call()
+
+
+def test_another_devices_timeout_is_left_to_it(env):
+    """Each device has its own word (host memory: no second device is needed to hold one)."""
+    torch, hom, net, word = env
+    of = getattr(net.load_library(), "_ZN4hnet22conv3_tc_error_word_ofEi")   # int *hnet::conv3_tc_error_word_of(int)
+    of.restype, of.argtypes = ctypes.POINTER(ctypes.c_int), [ctypes.c_int]
+    here = torch.cuda.current_device()
+    assert ctypes.addressof(of(here).contents) == ctypes.addressof(word().contents)
+    other = of(here + 1)
+    other[0] = 1
+    for call in calls(torch, net).values():
+        call()
+    assert other[0] == 1
+    other[0] = 0

@@ -27,3 +27,16 @@ def test_weight_gradient_refuses(net, grid, cout, c0, c1):
     from paper_2110_00733_gb300 import hom
     assert rc == hom.HOM_EINVAL, lib.hom_net_last_error()
     assert b"even with a second source" in lib.hom_net_last_error()
+
+
+def test_convolution_without_a_device_does_not_blame_the_shape(net):
+    """Without a device there is no error word for the kernel's waits: HOM_ENOMEM, and before any launch."""
+    import torch
+    if torch.cuda.is_available():
+        pytest.skip("host buffers stand in for device ones")
+    from paper_2110_00733_gb300 import hom
+    buf = np.zeros(4096, np.float32)
+    p = ctypes.c_void_p(buf.ctypes.data)
+    lib = net.load_library()
+    rc = lib.hom_net_conv3d(1, (ctypes.c_int * 3)(1, 1, 1), p, 16, None, 0, p, None, 0, 16, p, 1, None)
+    assert rc == hom.HOM_ENOMEM and b"error word" in lib.hom_net_last_error()
