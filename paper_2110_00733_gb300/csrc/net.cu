@@ -32,6 +32,7 @@ int set_err(int code, const std::string &msg) {
 // of a convolution launcher's result (see net_internal.h)
 int launch_err(int rc, const char *shape) {
     if (rc == 0) return HOM_OK;
+    if (rc == -3) return set_err(HOM_ECUDA, "the kernels' shared-memory limits could not be raised on this device");
     return rc == -2 ? set_err(HOM_ENOMEM, "no host memory mapped for the error word of the kernels' bounded waits")
                     : set_err(HOM_EINVAL, shape);
 }

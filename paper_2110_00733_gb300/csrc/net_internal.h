@@ -36,7 +36,8 @@ struct WgradArgs {
     int S;
 };
 
-// the launchers return -1 for a shape that they do not take, -2 without an error word
+// the launchers return -1 for a shape that they do not take, -2 without an error
+// word, -3 where the device could not be set up
 int conv3_forward_tc(const ConvArgs &a, cudaStream_t st);   // tcgen05, cout <= 256
 // the word of the current device, or of another, that a bounded wait of a tcgen05
 // convolution sets as it gives up (null: it could not be allocated)

@@ -1492,6 +1492,33 @@ int *conv3_tc_error_word() {
     return conv3_tc_error_word_of(dev);
 }
 
+// SMs of the current device, whose kernels' shared-memory limits (and carve-outs: all
+// of the unified L1/shared array, so that the CTAs that the budget allows are
+// resident together) are raised at the first call on it; 0 where that failed
+static int device_sms() {
+    static PerDevice<int> sms;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    const int *n = sms.get(dev, [dev](int &count) {
+        int lim = 0;
+        cudaError_t e = cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        auto raise = [&](const void *k, bool carveout) {
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lim - 1024);
+            if (e == cudaSuccess && carveout) e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        };
+        raise((const void *)k_conv3_tc, false);
+        for (auto k : {k_conv3_tch, k_conv3_tcp}) raise((const void *)k, true);
+        raise((const void *)k_conv3_tcd, true);
+        for (auto k : {k_conv3_col<16>, k_conv3_col<32>, k_conv3_col<48>, k_conv3_col<64>, k_conv3_col<80>})
+            raise((const void *)k, true);
+        for (auto k : {k_wgrad3_col<false>, k_wgrad3_col<true>}) raise((const void *)k, true);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&count, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) cudaGetLastError();
+        return e == cudaSuccess;
+    });
+    return n ? *n : 0;
+}
+
 int conv3_forward_tc(const ConvArgs &in, cudaStream_t st) {
     ConvArgs a = in;
     if ((a.cout & 15) || a.cout > 256 || a.cout < 16 || (a.c0s & 15) || (a.c1s & 15) || a.c0s <= 0) return -1;
@@ -1500,35 +1527,11 @@ int conv3_forward_tc(const ConvArgs &in, cudaStream_t st) {
     if (!a.err) return -2;
     int ncols = 32;
     while (ncols < a.cout) ncols <<= 1;
-    static bool attr = false;
-    if (!attr) {
-        int dev = 0, lim = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        cudaFuncSetAttribute(k_conv3_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, lim - 1024);
-        cudaFuncSetAttribute(k_conv3_tch, cudaFuncAttributeMaxDynamicSharedMemorySize, lim - 1024);
-        cudaFuncSetAttribute(k_conv3_tcd, cudaFuncAttributeMaxDynamicSharedMemorySize, lim - 1024);
-        cudaFuncSetAttribute(k_conv3_tcp, cudaFuncAttributeMaxDynamicSharedMemorySize, lim - 1024);
-        // all of the unified L1/shared array as shared memory, so that the
-        // CTAs that the shared-memory budget allows are resident together
-        cudaFuncSetAttribute(k_conv3_tcd, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        cudaFuncSetAttribute(k_conv3_tcp, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        cudaFuncSetAttribute(k_conv3_tch, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        for (auto k : {k_conv3_col<16>, k_conv3_col<32>, k_conv3_col<48>, k_conv3_col<64>, k_conv3_col<80>}) {
-            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lim - 1024);
-            cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        }
-        attr = true;
-    }
+    const int nsm = device_sms();
+    if (!nsm) return -3;
     if (3 * a.cout <= 256) {
         // column march: two CTAs per SM up to 32 output channels, one above;
         // planes of an item by half of a CTA's tensor memory
-        static int nsm = 0;
-        if (!nsm) {
-            int dev = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        }
         const int per_sm = a.cout <= 32 ? 2 : 1, nch = (a.c0s + a.c1s) / 16;
         const int zmax = a.cout <= 32 ? 128 / a.cout : 256 / a.cout, zl = a.n1 < zmax ? a.n1 : zmax;
         int nc = 32;
@@ -1558,19 +1561,12 @@ int conv3_forward_tc(const ConvArgs &in, cudaStream_t st) {
         size_t smem = w_bytes + 2 * (size_t)kDHalo;
         const size_t floor = 233472 / (512 / ncols2 + 1) + 1024;
         if (smem < floor) smem = floor;
-        static int nsm = 0;
-        if (!nsm) {
-            int dev = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        }
         // CTAs per SM that shared memory, registers and tensor memory allow
-        static int regs = 0;
-        if (!regs) {
+        static const int regs = [] {   // the compiler's, the same on every device
             cudaFuncAttributes fa{};
-            cudaFuncGetAttributes(&fa, k_conv3_tcp);
-            regs = fa.numRegs > 0 ? (fa.numRegs + 7) / 8 * 8 : 255;
-        }
+            if (cudaFuncGetAttributes(&fa, k_conv3_tcp) != cudaSuccess) cudaGetLastError();
+            return fa.numRegs > 0 ? (fa.numRegs + 7) / 8 * 8 : 255;
+        }();
         int per_sm = (int)(233472 / (smem + 2048));
         per_sm = per_sm < 65536 / (regs * kThreads) ? per_sm : 65536 / (regs * kThreads);
         per_sm = per_sm < 512 / ncols2 ? per_sm : 512 / ncols2;
@@ -1621,17 +1617,7 @@ int conv3_wgrad(const WgradArgs &in, cudaStream_t st) {
     const ConvArgs &a = w.in;
     if (w.S <= 0 || !conv3_wgrad_takes(w)) return -1;
     if (!a.err) return -2;
-    static bool cattr = false;
-    if (!cattr) {
-        int dev = 0, lim = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        for (auto k : {k_wgrad3_col<false>, k_wgrad3_col<true>}) {
-            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lim - 1024);
-            cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        }
-        cattr = true;
-    }
+    if (!device_sms()) return -3;
     const int nc = 256;   // 144 columns; two CTAs per SM by tensor and shared memory
     const int zl = a.n1 < 8 ? a.n1 : 8;
     size_t smem = (size_t)(kCSlots + kCGSlots) * kCPlane + kCPad;

@@ -39,3 +39,13 @@ def test_once_per_device(tmp_path):
     subprocess.run(["g++", "-std=c++17", "-pthread", "-I", os.path.join(ROOT, "paper_2110_00733_gb300", "csrc"), str(src),
                     "-o", str(exe)], check=True)
     assert subprocess.run([str(exe)]).returncode == 0
+
+
+def test_network_launchers_keep_no_other_static():
+    """What the launchers keep between calls is made per device and under a lock: kernel attributes and
+    the number of SMs belong to a device, and a plain flag is written by every thread that finds it unset."""
+    import re
+    for name in ("net.cu", "net_tc.cu"):
+        src = open(os.path.join(ROOT, "paper_2110_00733_gb300", "csrc", name)).read()
+        kept = re.findall(r"^\s+static (?!constexpr)([^;(]*)", src, re.M)
+        assert all(k.startswith(("PerDevice<", "const int regs")) for k in kept), kept
