@@ -105,9 +105,11 @@ typedef struct {
     void *stream;       /* cudaStream_t to run on; NULL: a stream the context creates */
     int device;         /* CUDA device ordinal; -1: the current device */
     int refine;         /* FP32 fields: max FP64 iterative-refinement sweeps (default 3) */
-    int rows3;          /* launch shape: n3-pass rows per CTA (0 = automatic, <= 64) */
+    int rows3;          /* launch shape: n3-pass rows per CTA (0 = automatic, <= 64; other
+                           values select the shared-memory pass, the slower one) */
     int tile2;          /* launch shape: n2-pass columns per CTA (0 = automatic; power of 2, <= 32) */
-    int tile1;          /* launch shape: n1-pass columns per CTA (0 = automatic, <= 16) */
+    int tile1;          /* launch shape: n1-pass columns per CTA (0 = automatic, <= 16);
+                           the TMA-staged fused MINRES pass keeps its own */
     int staging;        /* 0: persistent TMA-staged n1/n2 passes where supported
                            (FP32: the n2 pass and the fused MINRES n1 pass at
                            most lengths from 16 to 512, the unfused n1 pass at

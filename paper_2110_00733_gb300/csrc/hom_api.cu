@@ -387,10 +387,11 @@ static int set_shapes(hom_ctx *ctx, Geometry &g, int nc, bool lines = true) {
             const char *e = getenv("HOM_X1_L2PF");
             g.x1_l2pf = e ? atoi(e) : 1;
         }
-        // the fused pass's tile width is the plan's; an explicit tile1 other
-        // than it selects the plain-load form
+        // the fused pass's tile width is the plan's, whatever tile1 the unfused
+        // passes take (the plain-load form, which would take it, is slower at any:
+        // 160^3 step 521 us at tile1 = 4 against 245)
         const int tpl = line_tpl(g.n1), t = tpl > 0 && nc == 6 ? x1l_cols(g.n1, tpl) : 0;
-        if (t > 0 && (ctx->shape[2] == 0 || ctx->shape[2] == t)) {
+        if (t > 0) {
             g.box1l = tma_box_rows(g.n1, 48 * t);
             g.tile1l = t;
             g.grp1l = x1l_group(g.n1, tpl);
