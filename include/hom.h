@@ -425,8 +425,9 @@ int hom_solve_batch(hom_ctx *const *ctxs, int ncell, const double *macro_strain,
  * MINRES iteration (scratch contexts, random phase map, CUDA events) for
  * candidate tiles of each FFT pass and write the fastest
  * (rows3, tile2, tile1) to shape[3].  Cached per process and, when the
- * environment variable HOM_TUNE_CACHE names a file, on disk.  Allocates and
- * frees scratch contexts. */
+ * environment variable HOM_TUNE_CACHE names a file, on disk (shapes timed on
+ * other kernels than this library's are timed again).  Allocates and frees
+ * scratch contexts. */
 int hom_autotune(const int grid[3], int precision, int shape[3]);
 
 /* Grid, precision and workspace size of a context. */
