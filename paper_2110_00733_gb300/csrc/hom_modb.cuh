@@ -10,6 +10,7 @@
 // unknown and no equation.  The preconditioner is eq. (precf) with the mean
 // stiffness of eq. (avstiff).
 #pragma once
+#include "hom_sum3.h"
 #include "hom_internal.h"
 
 namespace hom {
@@ -172,10 +173,10 @@ __global__ void k_modb_precond(Geometry g, PrecondCoef<R> pc, const cpx<R> *__re
 
 // PCG step: x += a p; r -= a q; z = M r; partials <r,z> (first half) and
 // <r,r> (second half), Parseval-weighted.  Bound by HBM (seven 3-component
-// vectors); the sums of a thread's points are kept as two floats (Acc: each
-// product exact, a point's rounding 2^-47 of it) and added in FP64 over the
-// grid, where rounding at 2^-53 of the total outweighs the points' random errors;
-// st->sc, a power of two, brings the products into the range of FP32.
+// vectors); the sums of a thread's points are kept as three floats (Sum3: as good
+// as exact) and added in FP64 over the grid, so that they are as far off as FP64
+// sums of the points (1e-16 rms, 24^3 to 256^3); st->sc, a power of two, brings the
+// products into the range of FP32.
 // In FP64 throughout the pass was bound by the FP64 pipe: 191 us at 128^3.
 template <typename R>
 __global__ void __launch_bounds__(kEwThreads) k_cg_xr(Geometry g, PrecondCoef<R> pc, cpx<R> *__restrict__ x,
@@ -185,7 +186,7 @@ __global__ void __launch_bounds__(kEwThreads) k_cg_xr(Geometry g, PrecondCoef<R>
     if (st->done) return;
     const R a = (R)st->a, sc = (R)st->sc;
     const double isc2 = 1.0 / (st->sc * st->sc);
-    Acc<R> rz, rr;
+    typename std::conditional<sizeof(R) == 4, Sum3, Acc<R>>::type rz, rr;
     for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < (int)g.S; f += gridDim.x * blockDim.x) {
         R qv[3];
         int k3;
