@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(x1l_threads(N, LinePlan<N>::TPL),
     if (!xform) {
         x1_lagged<R, GRP, x1l_lag_threads(GRP)>(g, scoef, live_from, ntiles, tpc, kper, smem_raw + 2 * g.stage1l, lbar, um, wa, wb, x);
     } else {
-        Acc<R> acc;   // this thread's ||u_{k+1}||^2 of the running case
+        double run = 0.0;   // this thread's ||u_{k+1}||^2 of the running case
         int tile = live_from(blockIdx.x);
         if (leader && tile < ntiles) {
             mbar_expect_tx(&bar[0], bytes);
@@ -372,11 +372,15 @@ __global__ void __launch_bounds__(x1l_threads(N, LinePlan<N>::TPL),
             }
             const LzCoef<R> c = scoef[cs];
             cpx<R> *buf = base + s * sper;
+            // a tile's products as two floats, the tiles in FP64: two floats over all
+            // tiles of a case lose 1e-13 of the thread's sum (36 tiles), 2e-15 so
+            Acc<R> acc;
             x1_lanczos_line<R, N, T, GRP>(g, buf, tc * T, c, uk + ko, um + ko, un + ko, acc, fold.st + cs);
+            run += acc.value();
             if (next >= ntiles || next / tpc != cs) {   // the last tile of the case here
-                const double ws = warp_sum(acc.value());
+                const double ws = warp_sum(run);
                 if ((threadIdx.x & 31) == 0) sacc[cs * (kX1Group / 32) + (threadIdx.x >> 5)] += ws;
-                acc = Acc<R>{};
+                run = 0.0;
             }
             fence_proxy_async_smem();
             group_sync(GRP);

@@ -736,7 +736,7 @@ __global__ void __launch_bounds__(kX3rWarps * 32, 3)
     const int lane0 = lane & ~(P - 1);
     const int partner = lane0 + ((P - j) & (P - 1));
     const float sV = 1.0f / (float)g.V;
-    Acc<float> eacc;   // this lane's energy of the running case
+    double eacc = 0.0;   // this lane's energy of the running case
     int q = live_from(blockIdx.x * kX3rWarps + warp);
     if (q < ngroups) prefetch(q);
     while (q < ngroups) {
@@ -862,11 +862,11 @@ __global__ void __launch_bounds__(kX3rWarps * 32, 3)
             }
         }
         // (reduced over the warp once a case: FP64 adds run at a small rate)
-        eacc.add(en);
+        eacc += (double)en;
         if (epart && (qn >= ngroups || qn / gpc != cs)) {
-            const double ws = warp_sum(eacc.value());
+            const double ws = warp_sum(eacc);
             if (lane == 0) sacc[cs * kX3rWarps + warp] += ws;
-            eacc = Acc<float>{};
+            eacc = 0.0;
         }
         if constexpr (SUMS) {
 #pragma unroll

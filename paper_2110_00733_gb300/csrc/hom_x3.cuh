@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(X3Plan<N>::NT, X3Plan<N>::CTAS)
         mbar_expect_tx(&bar, bytes);
         bulk_load(smem_raw, in + ((size_t)cs * nrows + row0) * (H * 6), bytes, &bar);
     };
-    Acc<float> eacc;   // this thread's energy of the running case
+    double eacc = 0.0;   // this thread's energy of the running case
     int tile = live_from(blockIdx.x);
     if (leader && tile < ntiles) issue(tile);
     for (int it = 0; tile < ntiles; ++it) {
@@ -239,11 +239,11 @@ __global__ void __launch_bounds__(X3Plan<N>::NT, X3Plan<N>::CTAS)
         // reduced over the warp once a case, not once a tile: FP64 adds run at
         // a small rate (six sums a tile took 17 of 50 us at 128^3)
         const bool last = next >= ntiles || next / tpc != cs;
-        eacc.add(en);
+        eacc += (double)en;
         if (epart && last) {
-            const double ws = warp_sum(eacc.value());
+            const double ws = warp_sum(eacc);
             if ((tid & 31) == 0) sacc[cs * (NT / 32) + (tid >> 5)] += ws;
-            eacc = Acc<float>{};
+            eacc = 0.0;
         }
         if constexpr (SUMS) {
 #pragma unroll
