@@ -3153,6 +3153,7 @@ template <typename R>
 static int j2_time_impl(hom_ctx *ctx, Engine<R> &E, int reps, double *ms, int nmax) {
     J2State &j = ctx->j2;
     cudaStream_t s = ctx->stream;
+    const Geometry &g = op_geom(ctx, E);
     R *tin, *tout;
     if constexpr (std::is_same<R, double>::value) {
         tin = j.sig; tout = j.de;
@@ -3175,11 +3176,11 @@ static int j2_time_impl(hom_ctx *ctx, Engine<R> &E, int reps, double *ms, int nm
                         else j2_tangent_apply<float, float>(ctx->V, j.Ct32, tin, tout, s);
                         break;
                     case 2:
-                        Launch<R>::x3(E.g, s, X3_IN_SPEC, E.spec, X3_MID_NONE, ctx->lam, ctx->mu, nullptr, 1.0, X3_OUT_REAL,
+                        Launch<R>::x3(g, s, X3_IN_SPEC, E.spec, X3_MID_NONE, ctx->lam, ctx->mu, nullptr, 1.0, X3_OUT_REAL,
                                       tin, E.phi, nullptr);
                         break;
                     default:
-                        Launch<R>::x3(E.g, s, X3_IN_REAL, tout, X3_MID_NONE, ctx->lam, ctx->mu, nullptr, 1.0, X3_OUT_SPEC,
+                        Launch<R>::x3(g, s, X3_IN_REAL, tout, X3_MID_NONE, ctx->lam, ctx->mu, nullptr, 1.0, X3_OUT_SPEC,
                                       E.spec, E.phi, nullptr);
                         break;
                 }
@@ -3199,8 +3200,10 @@ int hom_j2_time_kernels(hom_ctx *ctx, int reps, double *ms, int nmax) {
     if (!ctx || !ms || reps <= 0 || nmax <= 0) return fail(ctx, HOM_EINVAL, "bad argument");
     if (!ctx->j2.active) return fail(ctx, HOM_EINVAL, "hom_j2_begin first");
     cudaSetDevice(ctx->device);
+    ctx->j2_ops = true;   // the passes of the increments
     int r = (ctx->prec == HOM_PREC_FP64) ? j2_time_impl<double>(ctx, ctx->e64, reps, ms, nmax)
                                          : j2_time_impl<float>(ctx, ctx->e32, reps, ms, nmax);
+    ctx->j2_ops = false;
     if (r < 0) return r;
     int rc = finish(ctx);
     return rc ? rc : r;

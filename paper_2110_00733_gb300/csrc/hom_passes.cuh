@@ -366,7 +366,9 @@ __device__ __forceinline__ void gamma_from_q(const Geometry &g, const GammaE<R> 
 // beyond the line engine): they stop their linear solves at a bounded number of
 // steps on nearly singular tangents, where a load changed in its 15th digit
 // moves the strains by 1e-6 to 1e-5 (48^3, three Newton steps), so that their
-// results repeat only if every operation keeps its order.
+// results repeat only if every operation keeps its order.  (Increments of FP32
+// fields solve their linear systems with the FP32 passes, as every FP32 operator
+// does; there only the FP64 residuals keep it.)
 template <typename R, int S, int NF, int PAD = 0, typename Plan = void>
 __device__ __forceinline__ cpx<R> *run_fft(cpx<R> *buf, cpx<R> *buf2, int L, int ES, const AxisPlan &p) {
     if constexpr (NF > 0 && sizeof(R) == 8) {
