@@ -57,6 +57,10 @@
  *     the TMA ring of the FP32 n2 pass (default 3 at n2 >= 256, else 2).
  *   - HOM_X1_L2PF=0 in the environment at hom_create turns off the L2
  *     prefetch of each tile's Lanczos blocks in the fused FP32 n1 pass.
+ *   - HOM_J2_TABLE=0 in the environment at hom_j2_begin keeps the unit
+ *     frequency vectors of an FP64 elastoplastic context out of memory (48
+ *     bytes a frequency): the increments form them in their passes, as where
+ *     that memory cannot be had (the same results, more slowly).
  *   - HOM_FOLD_ALPHA=1 in the environment at the first solve folds the
  *     MINRES alpha reduction into the persistent n3 pass (one launch fewer
  *     per step; off by default).

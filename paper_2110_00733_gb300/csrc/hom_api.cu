@@ -2823,8 +2823,9 @@ int hom_j2_begin(hom_ctx *ctx, double yield_stress, double hardening) {
             return rc;
         }
         Launch<double>::table_init(ctx->e64.gj);
-        // the increments' projector table, where memory allows it
-        if (ctx->prec == HOM_PREC_FP64) {
+        // the increments' projector table, where memory allows it and the caller wants it
+        const char *et = std::getenv("HOM_J2_TABLE");
+        if (ctx->prec == HOM_PREC_FP64 && !(et && std::atoi(et) == 0)) {
             if (cudaMalloc(&j.etab, sizeof(double2) * 3 * ctx->S) == cudaSuccess) {
                 Launch<double>::gamma_table(ctx->e64.gj, ctx->stream, j.etab);
                 ctx->e64.gj.etab = j.etab;
