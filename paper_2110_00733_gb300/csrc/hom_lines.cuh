@@ -91,11 +91,21 @@ __device__ __forceinline__ void x1_lanczos_line(const Geometry &g, cpx<R> *buf, 
 // up, where that room is two or three CTAs anyway: there the twiddles stay in
 // registers across the loop (141 against 146 us at 256^3, 118 against 127 at
 // 240^3; at 192^3 68 against 66).
+// At 512 the register engine runs the same plan, at 64 registers: its stages have no
+// idle threads to tell apart.  The tiles' rows are 64 bytes there, half of the lines
+// they come from, and neighbouring tiles find the other half in L2 only as long as
+// their CTAs stay together: on the line engine the pass read 0.96 to 0.99 GB of DRAM
+// at 256 x 512 x 256 where the register engine reads the 0.81 it needs, and took 0.36
+// against 0.275 ms, 1.9 against 1.06 at 512^3.  (At 256, whose rows are whole lines,
+// the line engine is the faster, 141 against 148 us at 256^3.)
+template <int N> constexpr bool x2_register_engine() { return N == 512; }
+
 template <typename R, int S, int N>
-__global__ void __launch_bounds__(512, LinePlan<N>::E <= 16 && N < 225 ? 2 : 1) k_x2_tma(Geometry g, const __grid_constant__ CUtensorMap tm, int qtiles,
+__global__ void __launch_bounds__(512, LinePlan<N>::E <= 16 && (N < 225 || x2_register_engine<N>()) ? 2 : 1) k_x2_tma(Geometry g, const __grid_constant__ CUtensorMap tm, int qtiles,
                                             const MinresState *state) {
     pdl_release();
     pdl_wait();   // predecessor complete (programmatic launch in the MINRES graph)
+    if constexpr (x2_register_engine<N>()) static_assert(LinePlan<N>::TPL == N / FastPlan<N>::E, "every thread in the transform");
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bar[kX2MaxStages];
     const int T = g.tile2, NS = g.x2_stages;
@@ -146,7 +156,8 @@ __global__ void __launch_bounds__(512, LinePlan<N>::E <= 16 && N < 225 ? 2 : 1) 
             return;
         }
         cpx<R> *buf = base + q * per;
-        line_fft<R, S, N>(buf, T, T, tw);
+        if constexpr (x2_register_engine<N>()) fast_fft<R, S, N>(buf, T, T, tw);
+        else line_fft<R, S, N>(buf, T, T, tw);
         fence_proxy_async_smem();
         __syncthreads();
         if (leader) {
