@@ -244,7 +244,10 @@ static int set_shapes(hom_ctx *ctx, Geometry &g, int nc, bool lines = true) {
     const bool f64 = sizeof(R) == 8 && lines;   // FP64 on the line engine
     const int elems3 = sizeof(R) == 4 ? fast_elems_n3(g.n3) : fast_elems(g.n3);
     int rows, t2, t1;
-    const int tpl1 = f64 ? f64_line_tpl(g.n1) : 0, tpl2 = f64 ? f64_line_tpl(g.n2) : 0, tpl3 = f64 ? f64_line_tpl(g.n3) : 0;
+    // (384 in the n2 pass: the runtime engine's 253 us at 64 x 384 x 64 against 287,
+    // whose 24 butterflies of the first stage leave 2 of a line's 26 threads idle)
+    const int tpl1 = f64 ? f64_line_tpl(g.n1) : 0, tpl2 = f64 && g.n2 != 384 ? f64_line_tpl(g.n2) : 0,
+              tpl3 = f64 ? f64_line_tpl(g.n3) : 0;
     if (tpl3) {
         // measured (6-component spectra, ms): 96^3 8 rows 0.293, 4 0.316; 108^3 0.453, 0.505;
         // 128^3 0.652, 0.631 (51 KB of shared memory a CTA against 27); 192^3 2.49, 2.41; 48^3
@@ -265,7 +268,13 @@ static int set_shapes(hom_ctx *ctx, Geometry &g, int nc, bool lines = true) {
         while (rows > 1 && 2ull * g.n3 * np * rows * cs > 48 * 1024) rows >>= 1;
     }
     if (tpl2) {
-        t2 = tpl2 <= 8 ? 16 : 8;
+        // whole warps, five of them at most: both passes (us) with 8, 16, 32 columns at
+        // 128 x n x 128: 25 (5 threads a line) 147, 115, 101; 75 512, 392, 345; 96 (8)
+        // 426, 369, 390; 90 (10) 501, 422, 427; 162 (9) 1074, 910, 1122; 200 (10) 1142,
+        // 966, 1276; 108 (12) 513, 500, 639, but 144 (12) 569, 613, 781.  (9 and 10
+        // threads with three CTAs an SM or more: at 32 x 90 x 32 50 us with 8, 53 with 16)
+        const bool many = (long long)g.n1 * nc * g.h >= 16LL * 3 * kSms;
+        t2 = tpl2 <= 5 && (tpl2 & 1) ? 32 : (tpl2 <= 8 || (tpl2 <= 10 && many) ? 16 : 8);
         while (t2 > 4 && g.n1 * nc * g.h < kSms * t2) t2 >>= 1;
     } else if (g.fast[1]) {
         t2 = g.n2 >= 512 ? 8 : (g.n2 >= 128 ? 16 : 32);
