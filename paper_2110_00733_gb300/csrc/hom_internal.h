@@ -119,8 +119,12 @@ __device__ __forceinline__ void alpha_step(MinresState *st, double sum, double s
 // beta_{k+1} = 0, or k reaches max_it.  bn2 = ||u_{k+1}||^2.
 __device__ __forceinline__ void givens_step(MinresState *st, double bn2) {
     if (st->done) return;
+    // everything the step reads, before it writes: one memory latency and not one
+    // after each group of stores
+    const double alpha = st->alpha, c = st->c, s = st->s, dbar = st->dbar, eps = st->eps, beta = st->beta;
+    const double phibar0 = st->phibar, beta1 = st->beta1, tol = st->tol, u_tau = st->u_tau, u_tau1 = st->u_tau1;
+    const int k = st->k, max_it = st->max_it, dc = st->dc;
     const double beta_next = sqrt(bn2 > 0 ? bn2 : 0.0);
-    const double alpha = st->alpha, c = st->c, s = st->s, dbar = st->dbar;
     const double delta = c * dbar + s * alpha;
     const double gbar = s * dbar - c * alpha;
     const double eps_next = s * beta_next;
@@ -128,43 +132,44 @@ __device__ __forceinline__ void givens_step(MinresState *st, double bn2) {
     double gamma = hypot(gbar, beta_next);
     if (gamma == 0.0) gamma = 1e-300;
     const double cn = gbar / gamma, sn = beta_next / gamma;
-    const double tau = cn * st->phibar;
-    const double phibar = sn * st->phibar;
+    const double tau = cn * phibar0;
+    const double phibar = sn * phibar0;
+    const double inv_gamma = 1.0 / gamma, inv_beta = 1.0 / beta, est = phibar / beta1;
     const bool finite = isfinite(alpha) && isfinite(beta_next) && isfinite(phibar);
-    if (st->dc) {
+    if (dc) {
         // this step's n1 pass took x to the iterations done so far; a breakdown
         // keeps the iterate of the last such pass, at xi = 0 as everywhere else
-        if (minres_xstep(st->k))
+        if (minres_xstep(k))
             for (int i = 0; i < 6; ++i) st->dc_keep[i] = st->dc_x[i];
-        if (finite) dc_step(st, 1.0 / st->beta, delta, st->eps, 1.0 / gamma, tau);
+        if (finite) dc_step(st, inv_beta, delta, eps, inv_gamma, tau);
         else
             for (int i = 0; i < 6; ++i) st->dc_x[i] = st->dc_keep[i];
     }
     st->u_delta = delta;
-    st->u_eps = st->eps;            // epsilon_k multiplies w_{k-2}
-    st->u_inv_gamma = 1.0 / gamma;
-    st->u_tau2 = st->u_tau1;
-    st->u_tau1 = st->u_tau;
+    st->u_eps = eps;            // epsilon_k multiplies w_{k-2}
+    st->u_inv_gamma = inv_gamma;
+    st->u_tau2 = u_tau1;
+    st->u_tau1 = u_tau;
     st->u_tau = tau;
-    st->u_inv_beta = 1.0 / st->beta;   // v_k = u_k / beta_k in the lagged update
+    st->u_inv_beta = inv_beta;   // v_k = u_k / beta_k in the lagged update
     st->c = cn;
     st->s = sn;
     st->dbar = dbar_next;
     st->eps = eps_next;
     st->phibar = phibar;
-    st->beta_prev = st->beta;
+    st->beta_prev = beta;
     st->beta = beta_next;
-    st->k += 1;
-    st->est = phibar / st->beta1;
+    st->k = k + 1;
+    st->est = est;
     if (!finite) {
         st->status = -5;
         st->done = 1;
         st->done_update = 1;        // keep the last finite iterate
         return;
     }
-    if (st->est <= st->tol || beta_next == 0.0) {
+    if (est <= tol || beta_next == 0.0) {
         st->done = 1;               // the flush still applies this step's update
-    } else if (st->k >= st->max_it) {
+    } else if (k + 1 >= max_it) {
         st->status = 1;
         st->done = 1;
     }
