@@ -247,8 +247,8 @@ def source_hash():
     import hashlib
     h = hashlib.sha256()
     cdir = os.path.join(ROOT, "paper_2110_00733_gb300", "csrc")
-    for fn in ("hom_fft.cuh", "hom_tma.cuh", "hom_passes.cuh", "hom_lines.cuh", "hom_x3.cuh", "hom_modb.cuh", "hom_internal.h",
-               "hom_kernels_f32.cu", "hom_kernels_f64.cu"):
+    for fn in ("hom_fft.cuh", "hom_tma.cuh", "hom_passes.cuh", "hom_lines.cuh", "hom_x3.cuh", "hom_modb.cuh",
+               "hom_sum3.h", "hom_warp.h", "hom_internal.h", "hom_kernels_f32.cu", "hom_kernels_f64.cu"):
         with open(os.path.join(cdir, fn), "rb") as f:
             h.update(fn.encode())
             h.update(f.read())

@@ -325,8 +325,7 @@ __device__ __forceinline__ void group_sync(int n) {
 }
 
 template <typename R, int S, int N, int RAD, int NS_BEFORE, int PAD, typename Plan = FastPlan<N>>
-__device__ __forceinline__ void fast_stage(cpx<R> *buf, int ES, int l, int j0, const cpx<R> *__restrict__ tw,
-                                           int nsync) {
+__device__ __forceinline__ void fast_stage(cpx<R> *buf, int ES, int l, int j0, const cpx<R> *__restrict__ tw) {
     constexpr int E = Plan::E;
     constexpr int BPT = E / RAD;
     constexpr int nb = N / RAD;
@@ -339,7 +338,7 @@ __device__ __forceinline__ void fast_stage(cpx<R> *buf, int ES, int l, int j0, c
 #pragma unroll
         for (int r = 0; r < RAD; ++r) v[i][r] = buf[epos<PAD>(j + r * nb, ES) + l];
     }
-    group_sync(nsync);
+    __syncthreads();
 #pragma unroll
     for (int i = 0; i < BPT; ++i) {
         const int j = j0 + i * jstep;
@@ -357,22 +356,20 @@ __device__ __forceinline__ void fast_stage(cpx<R> *buf, int ES, int l, int j0, c
 #pragma unroll
         for (int r = 0; r < RAD; ++r) buf[epos<PAD>(o + r * NS_BEFORE, ES) + l] = v[i][r];
     }
-    group_sync(nsync);
+    __syncthreads();
 }
 
 // Transform of L interleaved lines in buf (in place), element e of line l
-// at buf[epos<PAD>(e, ES) + l] (ES >= L).  With nsync = 0 the CTA must have
-// exactly L * N / E threads (every thread takes part in every barrier);
-// otherwise threads 0 .. nsync-1 (= L * N / E) run it and synchronise on
-// named barrier 1, and the CTA's other warps are free for other work.
+// at buf[epos<PAD>(e, ES) + l] (ES >= L).  The CTA has exactly L * N / E threads:
+// every thread takes part in every barrier.
 template <typename R, int S, int N, int PAD = 0, typename P = FastPlan<N>>
-__device__ __forceinline__ void fast_fft(cpx<R> *buf, int L, int ES, const cpx<R> *__restrict__ tw, int nsync = 0) {
+__device__ __forceinline__ void fast_fft(cpx<R> *buf, int L, int ES, const cpx<R> *__restrict__ tw) {
     const int l = (int)threadIdx.x % L;
     const int j0 = (int)threadIdx.x / L;
-    fast_stage<R, S, N, P::R0, 1, PAD, P>(buf, ES, l, j0, tw, nsync);
-    if constexpr (P::NS > 1) fast_stage<R, S, N, P::R1, P::R0, PAD, P>(buf, ES, l, j0, tw, nsync);
-    if constexpr (P::NS > 2) fast_stage<R, S, N, P::R2, P::R0 * P::R1, PAD, P>(buf, ES, l, j0, tw, nsync);
-    if constexpr (P::NS > 3) fast_stage<R, S, N, P::R3, P::R0 * P::R1 * P::R2, PAD, P>(buf, ES, l, j0, tw, nsync);
+    fast_stage<R, S, N, P::R0, 1, PAD, P>(buf, ES, l, j0, tw);
+    if constexpr (P::NS > 1) fast_stage<R, S, N, P::R1, P::R0, PAD, P>(buf, ES, l, j0, tw);
+    if constexpr (P::NS > 2) fast_stage<R, S, N, P::R2, P::R0 * P::R1, PAD, P>(buf, ES, l, j0, tw);
+    if constexpr (P::NS > 3) fast_stage<R, S, N, P::R3, P::R0 * P::R1 * P::R2, PAD, P>(buf, ES, l, j0, tw);
 }
 
 // ---------------------------------------------------------------------------

@@ -233,10 +233,13 @@ struct Geometry {
     int grid2_tma, grid1_tma, grid1d_tma;
     int grid1l_tma = 0;     // persistent grid of the fused MINRES n1 pass (0: plain-load form)
     size_t smem2_tma, smem1_tma, smem1d_tma;
-    // TMA-staged n2 pass and fused n1 pass, every length of the line engine:
-    // x2t enables the n2 pass (threads2t threads); the fused n1 pass has
-    // grp1l transform threads (0: plain-load form), tiles of tile1l columns
-    // and stage1l bytes per shared-memory stage; rows per TMA box
+    // TMA-staged n2 pass and fused n1 pass, the line engine's lengths (the n2 pass
+    // but 375 and 405, the fused pass but 270, 300, 324, 375, 405, 450, 486 and 500:
+    // beyond 256 a tile moves in boxes, and those lengths have no division whose
+    // boxes start on 128-byte boundaries): x2t enables the n2 pass (threads2t
+    // threads); the fused n1 pass has grp1l transform threads (0: plain-load form),
+    // tiles of tile1l columns and stage1l bytes per shared-memory stage; rows per
+    // TMA box
     int x2t = 0, threads2t = 0, grp1l = 0;
     int tile1l;             // columns of a Krylov-vector tile (tile1 where the plain-load form runs)
     size_t stage1l = 0;
@@ -346,9 +349,6 @@ using X1lLineFn = void (*)(Geometry, CUtensorMap, const float2 *, const float2 *
                            float2 *, const MinresState *, double *, Fold);
 X2LineFn x2_line_kernel(int n, int inverse);
 X1lLineFn x1l_line_kernel(int n);
-// persistent n3 pass of a length, with its threads, rows per tile and shared
-// memory (fn null: none)
-// (fn_sums: with the stress sums)
 // FP64 passes at one line length (hom_f64_*.cu; null members: no such length)
 using F64X1Fn = void (*)(Geometry, int, const double2 *, double2 *, const double2 *, double *, const MinresState *);
 using F64X1lFn = void (*)(Geometry, double2 *, const double2 *, const double2 *, double2 *, const double2 *, double2 *,
@@ -366,6 +366,8 @@ F64X1Fn f64_ord_x1_kernel(int n);
 F64X2Fn f64_ord_x2_kernel(int n, int inverse);
 F64X3Fn f64_ord_x3_kernel(int n);
 
+// persistent n3 pass of a length (fn_sums: with the stress sums), with its threads,
+// rows per tile and shared memory (fn null: none)
 struct X3Line {
     using Fn = void (*)(Geometry, const float2 *, float2 *, int, float, float, const float *, const MinresState *,
                         double *, Fold, double *);
@@ -419,11 +421,13 @@ template <typename R> struct Launch {
     // the weighted partial sum <dotv, out> per CTA
     static void x1(const Geometry &g, cudaStream_t st, int flags, const cpx<R> *in, cpx<R> *out,
                    const cpx<R> *dotv, double *partials, const MinresState *state);
-    // MoDBFFT: forward n1 pass of the 10-component spectrum in10 with the
-    // contraction to 3 components fused (out3 = tau xi + g, eq. modbfftfop;
-    static void gamma_table(const Geometry &g, cudaStream_t st, double2 *out);   // FP64
+    // the elastoplastic increments' (FP64): the unit frequency vectors (Geometry::
+    // etab), and x1's weighted partial sum <dotv, z> alone
+    static void gamma_table(const Geometry &g, cudaStream_t st, double2 *out);
     static void x1_dot(const Geometry &g, cudaStream_t st, const cpx<R> *z, const cpx<R> *dotv, double *partials,
                        const MinresState *state);
+    // MoDBFFT: forward n1 pass of the 10-component spectrum in10 with the
+    // contraction to 3 components fused (out3 = tau xi + g, eq. modbfftfop;
     // with dot3, the weighted <dot3, out3> partials).  Returns the number of
     // partials written, or 0 without launching where the fused form does not
     // apply (not the TMA-staged FP32 pass, or more partials than max_partials).

@@ -1,9 +1,11 @@
 // hom_lines.cuh -- the persistent TMA-staged n2 pass and fused MINRES n1 pass
-// (FP32) at every length of the line engine (hom_fft.cuh).  The kernels of a
+// (FP32) at the lengths of the line engine (hom_fft.cuh) whose tiles TMA boxes can
+// move: all but 375 and 405 in the n2 pass, all but 270, 300, 324, 375, 405, 450,
+// 486 and 500 in the n1 pass, which run the plain-load kernels.  The kernels of a
 // length are reached through x2_line_kernel / x1l_line_kernel, whose tables
 // are built in the translation units that include this file.
 //
-// Why every length: grids between the powers of two are as common as these
+// Why lengths between the powers of two: grids between the powers of two are as common as these
 // (the paper's own are 90, 108 and 160).  The runtime Stockham engine with
 // plain loads, which ran them, divides by run-time values for every butterfly,
 // holds two buffers per tile and overlaps nothing with its loads: at 192^3 the
@@ -306,8 +308,8 @@ __device__ __forceinline__ bool x1_lagged(const Geometry &g, const LzCoef<R> *sc
 // the DRAM reads: the lines were evicted before use; the current tile's are
 // used within microseconds.)  Tiles are numbered case-major over the stacked
 // batch; tiles of converged cases are skipped; each transform thread keeps
-// one running sum per case in shared memory, and the CTA writes one partial
-// per case (partials[case * gridDim + block]).
+// the running sum of a case, reduced over its warp into shared memory at the
+// case's last tile, and the CTA writes one partial per case (partials[case * gridDim + block]).
 template <typename R, int N>
 __global__ void __launch_bounds__(x1l_threads(N, LinePlan<N>::TPL),
                                   LinePlan<N>::E > 16 ? 2 : (x1l_threads(N, LinePlan<N>::TPL) <= 192 ? 4 : 3))

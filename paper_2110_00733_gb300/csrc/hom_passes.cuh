@@ -1053,7 +1053,7 @@ __device__ __forceinline__ void tma_store_rows_2d(const CUtensorMap *tm, int x, 
 }
 
 // ---------------------------------------------------------------------------
-// Persistent TMA-staged n2 and n1 passes (FP32, register-FFT n in [64, 512]).
+// Persistent TMA-staged unfused n1 pass (FP32, register-FFT n1 and n2 in [64, 512]).
 // Each CTA loops over tiles with two shared-memory stages: while the FFT runs
 // on stage s, the TMA load of the next tile fills stage s^1; results leave by
 // TMA store.  One thread issues all copies; completion is tracked by one
