@@ -386,7 +386,8 @@ static int set_shapes(hom_ctx *ctx, Geometry &g, int nc, bool lines = true) {
         g.smem2_tma = (size_t)g.x2_stages * g.n2 * t2 * cs;
         g.threads2t = round32(t2 * line_tpl(g.n2));
         g.box2 = tma_box_rows(g.n2, t2 * (int)cs);
-        g.x2t = line_tpl(g.n2) > 0 && g.box2 > 0 && g.threads2t <= 512 &&
+        // (t2 % 2: a TMA copy starts and ends on a 16-byte boundary, two columns)
+        g.x2t = line_tpl(g.n2) > 0 && t2 % 2 == 0 && g.box2 > 0 && g.threads2t <= 512 &&
                 (size_t)g.n2 * t2 * cs % 128 == 0;   // every ring stage on a 128-byte boundary
         // fused n1 pass: bulk L2 prefetch of each tile's u_k and u_{k-1}
         // blocks at the tile's start (0.625 against 0.647 ms at 256^3; the
